@@ -206,12 +206,12 @@ h2_status setup_device(h2_ctx* c) {
       slot[(size_t)i * lf.D + (t - H.leaf_offsets[i])] = H.perm[t];
   CKS(upload(c, &c->slot_pt, slot));
   CKC(dalloc(c, &c->A64, (size_t)lf.NP * lf.D * lf.D));
-  launch_eval_blocks(c->kfn, c->pts, lf.NP, lf.near_i, lf.near_j, c->slot_pt, lf.D, lf.D, lf.D, c->A64, 0);
+  launch_eval_blocks(c->kfn, c->pts, lf.NP, lf.near_ptr, lf.near_i, lf.near_j, c->slot_pt, lf.D, c->A64, 0);
   CKC(cudaGetLastError());
   for (int l = 1; l <= L; ++l) {
     DevLevel& d = c->lv[l];
     CKC(dalloc(c, &d.S, (size_t)std::max<int64_t>(d.FP, 1) * d.K * d.K));
-    launch_eval_blocks(c->kfn, c->pts, d.FP, d.far_i, d.far_j, d.SK, d.K, d.K, d.K, d.S, 0);
+    launch_eval_blocks(c->kfn, c->pts, d.FP, d.far_ptr, d.far_i, d.far_j, d.SK, d.K, d.S, 0);
     CKC(cudaGetLastError());
   }
   // vectors and scratch

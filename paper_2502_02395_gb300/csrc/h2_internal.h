@@ -101,8 +101,8 @@ struct RankRecord {
 // (fptr / fidx), close boxes (nptr / nidx: the near list, j == i skipped),
 // close samples of each box (cptr / cidx), rank K, m sketch + probe columns
 // (ms of them sketch), q = m - ms probes, Gauss-Seidel sweeps gs (0: exact
-// solve).  Outputs: X (nb * D * K row-major), SK (nb * K), piv (nb * D),
-// the pivot ratio rho and probe error err per box.
+// solve).  Outputs: X (nb * D * K row-major), SK (nb * K), the pivot ratio
+// rho and probe error err per box.
 struct GpuLevelJob {
   int nb = 0, D = 0, K = 0, m = 0, ms = 0, q = 0, gs = 0;
   uint64_t seed = 0;
@@ -111,7 +111,6 @@ struct GpuLevelJob {
   std::vector<int32_t> nidx;
   std::vector<double> X, rho, err;
   std::vector<int64_t> SK;
-  std::vector<int32_t> piv;
   double flops_prefactor = 0, flops_far = 0;
 };
 struct GpuCompressor {

@@ -28,9 +28,8 @@ extern std::atomic<int> g_box_ctas_per_sm;
 extern std::atomic<int> g_pair_ctas_per_sm;
 
 // kernels_factor.cu
-void launch_eval_blocks(const KernelFn& G, const double* pts, int64_t npairs, const int32_t* pi,
-                        const int32_t* pj, const int64_t* idx, int idx_stride, int rows, int cols,
-                        double* out, cudaStream_t st);
+void launch_eval_blocks(const KernelFn& G, const double* pts, int64_t npairs, const int64_t* ptr, const int32_t* pi,
+                        const int32_t* pj, const int64_t* idx, int n, double* out, cudaStream_t st);
 template <typename S, typename T>
 void launch_convert(const S* in, T* out, int64_t n, cudaStream_t st);
 template <typename T, typename TB>
