@@ -578,7 +578,7 @@ void launch_cc_weights(const KernelFn& G, const double* pts, int nb, const int64
   ++g_launches;
   if (gs > 0) {
     const size_t sm = sizeof(double) * (size_t)GC_MAXS * (GC_MAXS + m);
-    cudaFuncSetAttribute(cc_sweeps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem((const void*)cc_sweeps_kernel);
     cc_sweeps_kernel<<<nb, 256, sm, st>>>(G, pts, cptr, cidx, m, seed, gs, W);
     return;
   }
@@ -604,7 +604,7 @@ void launch_sketch(const KernelFn& G, const double* pts, int nb, int D, int m, i
                    double* Y, cudaStream_t st) {
   const size_t sm = sizeof(double) * ((size_t)GC_ROWS * (GC_CHUNK + 1) + (size_t)GC_CHUNK * m + GC_ROWS * 3) +
                     sizeof(int64_t) * GC_CHUNK;
-  cudaFuncSetAttribute(sketch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)sketch_kernel);
   const int halves = (D + GC_ROWS - 1) / GC_ROWS;
   ++g_launches;
   sketch_kernel<<<dim3(halves * nb, nz), 256, sm, st>>>(G, pts, D, m, nbox, bpts, fptr, fidx, nptr, nidx, cptr, cidx,
@@ -616,7 +616,7 @@ cudaError_t launch_pivqr_t(int C, int nb, int D, int m, int ms, int q, int K, in
                            const int64_t* bpts, double* Y, double* X, int64_t* SK, double* rho, double* err,
                            cudaStream_t st) {
   const size_t sm = sizeof(double) * (size_t)K * K;
-  cudaFuncSetAttribute(pivqr_id_kernel<CW, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)pivqr_id_kernel<CW, NR>);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(nb * C));
   cfg.blockDim = dim3(512);

@@ -27,6 +27,10 @@ extern std::atomic<int> g_box_stream;
 extern std::atomic<int> g_box_ctas_per_sm;
 extern std::atomic<int> g_pair_ctas_per_sm;
 
+// Lets kernel f be launched with as much dynamic shared memory as the device
+// allows (once per kernel and device; safe from several threads).
+void allow_smem(const void* f);
+
 // kernels_factor.cu
 void launch_eval_blocks(const KernelFn& G, const double* pts, int64_t npairs, const int64_t* ptr, const int32_t* pi,
                         const int32_t* pj, const int64_t* idx, int n, double* out, cudaStream_t st);

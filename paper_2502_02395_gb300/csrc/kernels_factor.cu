@@ -949,7 +949,7 @@ bool launch_qr_panel(int nb, int D, int K, const T* Xin, T* Vout, T* tau, T* Tm,
     while (Kp < K) Kp *= 2;
     const size_t nscr = std::max<size_t>(32 * 129, (size_t)Kp * Kp / 4);
     const size_t sm = sizeof(float) * (2 * 256 + 4 + Kp + nscr + (Tw ? (size_t)Kp * (Kp + 1) : 0));
-    if (sm > 48 * 1024) cudaFuncSetAttribute(qr_reg_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem((const void*)qr_reg_kernel<8>);
     ++g_launches;
     qr_reg_kernel<8><<<nb, 512, sm, st>>>(D, K, Kp, reinterpret_cast<const float*>(Xin),
                                           reinterpret_cast<float*>(Vout), reinterpret_cast<float*>(tau),
@@ -958,7 +958,7 @@ bool launch_qr_panel(int nb, int D, int K, const T* Xin, T* Vout, T* tau, T* Tm,
   }
   const size_t sm = sizeof(T) * (size_t)D * K;
   const int use = sm <= 200 * 1024;
-  if (use) cudaFuncSetAttribute(qr_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)qr_panel_kernel<T>);
   ++g_launches;
   qr_panel_kernel<T><<<nb, 512, use ? sm : 0, st>>>(D, K, Xin, Vout, tau, Tm, gscr, use);
   return false;
@@ -970,7 +970,7 @@ void launch_wy_tfactor(int nb, int K, const T* S, const T* tau, T* Tw, cudaStrea
     int Kp = 8;
     while (Kp < K) Kp *= 2;
     const size_t sm = sizeof(T) * ((size_t)Kp * (Kp + 1) + (size_t)Kp * Kp / 4);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(wy_tinv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem((const void*)wy_tinv_kernel<T>);
     ++g_launches;
     wy_tinv_kernel<T><<<nb, 256, sm, st>>>(K, Kp, S, tau, Tw);
     return;
@@ -978,7 +978,7 @@ void launch_wy_tfactor(int nb, int K, const T* S, const T* tau, T* Tw, cudaStrea
   size_t sm = sizeof(T) * ((size_t)K * K + K);
   const int use = sm <= 200 * 1024;
   if (!use) sm = sizeof(T) * (size_t)K;
-  if (sm > 48 * 1024) cudaFuncSetAttribute(wy_tfactor_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)wy_tfactor_kernel<T>);
   ++g_launches;
   wy_tfactor_kernel<T><<<nb, 256, sm, st>>>(K, S, tau, Tw, use);
 }
@@ -1841,7 +1841,7 @@ void launch_lu_inverse(int nb, int D, int R, const T* Ablk, const int32_t* diag_
   const size_t cap = 220 * 1024;
   size_t sm1 = sizeof(T) * (size_t)R * (R + 1);
   int use = sm1 <= cap;
-  if (use) cudaFuncSetAttribute(lu_factor_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
+  allow_smem((const void*)lu_factor_kernel<T>);
   ++g_launches;
   lu_factor_kernel<T><<<nb, 256, use ? sm1 : 0, st>>>(D, R, Ablk, diag_idx, luT, piv, status, level, use);
   if (R > 1024) return;  // the permutation table holds 1024 rows; larger blocks are rejected by the caller
@@ -1849,7 +1849,7 @@ void launch_lu_inverse(int nb, int D, int R, const T* Ablk, const int32_t* diag_
     const int Rp = (R + 31) / 32 * 32;
     const size_t smf = sizeof(float) * 2 * (size_t)Rp * Rp;
     if (smf <= 200 * 1024 && Rp <= 256) {
-      cudaFuncSetAttribute(lu_inverse_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smf);
+      allow_smem((const void*)lu_inverse_f32_kernel);
       ++g_launches;
       lu_inverse_f32_kernel<<<nb, Rp, smf, st>>>(R, Rp, reinterpret_cast<const float*>(luT), piv,
                                                   reinterpret_cast<float*>(Ainv));
@@ -1859,7 +1859,7 @@ void launch_lu_inverse(int nb, int D, int R, const T* Ablk, const int32_t* diag_
   size_t f = sizeof(T) * (size_t)R * (R + 1), y = sizeof(T) * (size_t)R * R;
   int mode = (f + y <= cap) ? 2 : (f <= cap ? 1 : 0);
   size_t sm = mode == 2 ? f + y : (mode == 1 ? f : 0);
-  if (sm) cudaFuncSetAttribute(lu_inverse_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)lu_inverse_kernel<T>);
   ++g_launches;
   lu_inverse_kernel<T><<<nb, 256, sm, st>>>(R, luT, piv, Ainv, mode);
 }
@@ -2033,13 +2033,13 @@ void launch_lu_inverse_f64_for_f32(int nb, int D, int R, const float* Ablk, cons
   const size_t cap = 220 * 1024;
   const size_t sm1 = sizeof(double) * (size_t)R * (R + 1);
   const int use = sm1 <= cap;
-  if (use) cudaFuncSetAttribute(lu_factor_kernel<double, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
+  allow_smem((const void*)lu_factor_kernel<double, float>);
   ++g_launches;
   lu_factor_kernel<double, float><<<nb, 256, use ? sm1 : 0, st>>>(D, R, Ablk, diag_idx, lu, piv, status, level, use);
   const size_t f = sizeof(double) * (size_t)R * (R + 1), y = sizeof(double) * (size_t)R * R;
   const int mode = (f + y <= cap) ? 2 : (f <= cap ? 1 : 0);
   const size_t sm = mode == 2 ? f + y : (mode == 1 ? f : 0);
-  if (sm) cudaFuncSetAttribute(lu_inverse_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem((const void*)lu_inverse_kernel<double>);
   ++g_launches;
   lu_inverse_kernel<double><<<nb, 256, sm, st>>>(R, lu, piv, inv, mode);
   launch_convert<double, float>(inv, Ainv, (int64_t)nb * R * R, st);

@@ -19,6 +19,8 @@
 // S_ij x^_j on every level, downward pass, leaf y_i = X_i y^_i +
 // sum_near A_ij x_j.
 #include <atomic>
+#include <mutex>
+#include <set>
 
 #include "h2_internal.h"
 #include "kernels.h"
@@ -1027,8 +1029,27 @@ void launch_transpose_pairs(int D, int64_t n, const int32_t* dst, const int32_t*
   transpose_pairs_kernel<T><<<grid, dim3(32, 8), 0, st>>>(D, n, dst, src, A);
 }
 
+// The largest dynamic shared memory a kernel may be launched with, raised to
+// what the device allows, once per kernel and device.  (Set to each launch's
+// own size it was a race: with two contexts in two threads, one could lower
+// the limit between the other's call and its launch, which then failed.)
+void allow_smem(const void* f) {
+  static std::mutex mu;
+  static std::set<std::pair<int, const void*>> done;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(mu);
+  if (done.count({dev, f})) return;
+  int optin = 0;
+  cudaFuncAttributes a{};
+  if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaFuncGetAttributes(&a, f) != cudaSuccess ||
+      cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes) != cudaSuccess)
+    return;
+  done.insert({dev, f});
+}
 static void set_smem(const void* f, size_t sm) {
-  if (sm > 48 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (sm > 32 * 1024) allow_smem(f);
 }
 
 // Launch with programmatic stream serialization (see griddep_wait).
@@ -1450,7 +1471,7 @@ template <typename T>
 void launch_gemv_rows(int nb, int n, const T* M, const T* x, T* y, cudaStream_t st) {
   if (n == 0 || nb == 0) return;
   const size_t sm = sizeof(T) * 2 * (size_t)n;
-  if (sm > 48 * 1024) cudaFuncSetAttribute(gemv_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  set_smem((const void*)gemv_rows_kernel<T>, sm);
   ++g_launches;
   gemv_rows_kernel<T><<<nb, 256, sm, st>>>(n, M, x, y);
 }

@@ -662,7 +662,7 @@ bool gemm_tc(int ab_bf16, int M, int N, int K, const void* A, int64_t nA, int ro
   const size_t per_sm = 228 * 1024;
   const size_t max_ctas = 512 / cols;
   smem = std::max(smem, per_sm / (max_ctas + 1) + 1024);
-  cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem((const void*)tc_gemm_kernel);
   int dev = 0, nsm = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -671,7 +671,7 @@ bool gemm_tc(int ab_bf16, int M, int N, int K, const void* A, int64_t nA, int ro
     // persistent warp-specialized kernel: one CTA per SM (TMEM holds two
     // accumulators), WS_STAGES-deep ring
     const size_t sm_ws = (size_t)WS_STAGES * (TC_BM * TC_BK * 2 + (size_t)N * TC_BK * 2) + 1024;
-    cudaFuncSetAttribute(tc_gemm_ws_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_ws);
+    allow_smem((const void*)tc_gemm_ws_kernel);
     const int64_t ntiles = batch * (M / TC_BM);
     ++g_launches;
     tc_gemm_ws_kernel<<<(unsigned)std::min<int64_t>(ntiles, nsm), 192, sm_ws, st>>>(ta, tb, p, batch);
