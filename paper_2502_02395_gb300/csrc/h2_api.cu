@@ -84,7 +84,7 @@ h2_status make_leaf_lowp(h2_ctx* c, int bf16) {
   // couplings, per level, with max |S| scaled to sqrt(32768 / K): the
   // tensor-core coupling products then stay inside FP16 (|S T^T| <= 32768)
   for (int l = 1; l <= c->L; ++l) {
-    DevLevel& d = c->lv[l];
+    DevLevel& d = c->pv[l];
     if (d.FP == 0 || d.K == 0) continue;
     const int64_t ns = d.FP * (int64_t)d.K * d.K;
     CKC(dalloc(c, &d.S16_scale[bf16], 2));
@@ -97,6 +97,86 @@ h2_status make_leaf_lowp(h2_ctx* c, int bf16) {
   CKC(cudaGetLastError());
   CKC(cudaStreamSynchronize(c->stream));
   return H2_OK;
+}
+
+// The dimensions of the FP32 arrays (pv) of an instance: K and R of every
+// level rounded up to multiples of 4, with D = K + R at the leaves and 2 K of
+// the level below above them, so that every row of every block starts on 16
+// bytes and the kernels take their vector loads (a point count that fills no
+// leaf gives leaves of, say, 196 points and ranks of 98).  Padding entries are
+// zero in the bases and couplings and 1 on the diagonal of the near blocks, so
+// that they are decoupled unknowns, as a ragged leaf's are.  From the root
+// down, K_l+1 must also leave room for R_l: 2 K_l+1 >= R_l + K_l.  Instances
+// with a level that fits the tensor-core shapes or above 256 keep their
+// dimensions, and so do those that need no padding.
+void padded_dims(h2_ctx* c) {
+  const int L = c->L;
+  for (int l = 0; l <= L; ++l) c->pv[l].D = c->lv[l].D, c->pv[l].K = c->lv[l].K, c->pv[l].R = c->lv[l].R;
+  auto up4 = [](int v) { return (v + 3) & ~3; };
+  if (L < 1) return;
+  std::vector<int> K(L + 1, 0), D(L + 1, 0);
+  for (int l = 1; l <= L; ++l) {
+    const DevLevel& d = c->lv[l];
+    if (d.K == 0 || gemm_tc_supported(d.D, d.D, d.D, d.D, d.D, d.D)) return;
+    K[l] = up4(l == 1 ? d.K : std::max(d.K, (c->lv[l - 1].R + K[l - 1] + 1) / 2));
+  }
+  for (int l = 0; l <= L; ++l) {
+    D[l] = l < L ? 2 * K[l + 1] : K[L] + up4(c->lv[L].R);
+    if (D[l] > 256) return;
+  }
+  for (int l = 0; l <= L; ++l) c->pv[l].D = D[l], c->pv[l].K = K[l], c->pv[l].R = D[l] - K[l];
+}
+// where a level's logical rows (its points, or its children's skeletons) lie
+// in the padded arrays
+PadSeg row_seg(const h2_ctx* c, int l) {
+  if (l == c->L) return {c->lv[l].D, c->pv[l].D};
+  return {c->lv[l + 1].K, c->pv[l + 1].K};
+}
+PadSeg skel_seg(const h2_ctx* c, int l) { return {c->lv[l].K, c->pv[l].K}; }
+// a leaf vector's boxes
+PadSeg leaf_seg(const h2_ctx* c) { return {c->lv[c->L].D, c->pv[c->L].D}; }
+
+// The stored pairs of a symmetric list of n x n blocks, and per box the list
+// of partial products it receives.
+struct StoredPairs {
+  std::vector<int32_t> q, i, j, ent;
+  std::vector<int64_t> ptr;
+  StoredPairs(const std::vector<int32_t>& pi, const std::vector<int32_t>& pj, int nb, bool diag) {
+    for (size_t k = 0; k < pi.size(); ++k)
+      if (pi[k] < pj[k] || (diag && pi[k] == pj[k])) q.push_back((int32_t)k), i.push_back(pi[k]), j.push_back(pj[k]);
+    std::vector<std::vector<std::pair<int32_t, int32_t>>> lists(nb);  // (partner box, entry)
+    for (size_t k = 0; k < q.size(); ++k) {
+      lists[i[k]].push_back({j[k], (int32_t)(2 * k)});
+      if (i[k] != j[k]) lists[j[k]].push_back({i[k], (int32_t)(2 * k + 1)});
+    }
+    ptr.assign(nb + 1, 0);
+    for (int b = 0; b < nb; ++b) {
+      std::sort(lists[b].begin(), lists[b].end());
+      for (auto& pe : lists[b]) ent.push_back(pe.second);
+      ptr[b + 1] = (int64_t)ent.size();
+    }
+  }
+  // descriptors of the pairs: blocks from m0, partial products from p0 on,
+  // box b's vector slice at x0 + b n
+  void describe(std::vector<SymPair>& out, int n, int64_t m0, int64_t p0, int64_t x0) const {
+    for (size_t k = 0; k < q.size(); ++k)
+      out.push_back({m0 + (int64_t)k * n * n, p0 + (int64_t)k * 2 * n, (int32_t)(x0 + (int64_t)i[k] * n),
+                     (int32_t)(x0 + (int64_t)j[k] * n), n, 0});
+  }
+};
+
+// The mirror (j, i) of every pair (i, j) of a sorted list (CSR ptr over i):
+// false if one is missing.
+bool mirrors(const std::vector<int32_t>& pi, const std::vector<int32_t>& pj, const std::vector<int64_t>& ptr,
+             std::vector<int32_t>& m) {
+  m.assign(pi.size(), -1);
+  for (size_t q = 0; q < pi.size(); ++q) {
+    const auto b = pj.begin() + ptr[pj[q]], e = pj.begin() + ptr[pj[q] + 1];
+    const auto it = std::lower_bound(b, e, pi[q]);
+    if (it == e || *it != pi[q] || pi[it - pj.begin()] != pj[q]) return false;
+    m[q] = (int32_t)(it - pj.begin());
+  }
+  return true;
 }
 
 h2_status setup_device(h2_ctx* c) {
@@ -223,79 +303,81 @@ h2_status setup_device(h2_ctx* c) {
   for (int l = 1; l <= L; ++l) c->hat_off[l + 1] = c->hat_off[l] + (int64_t)c->lv[l].nb * c->lv[l].K;
   CKC(dalloc(c, &c->xhat, c->hat_off[L + 1]));
   CKC(dalloc(c, &c->yhat, c->hat_off[L + 1]));
+  // upper / lower split of each level's near and far lists (the kernels are
+  // symmetric: blocks (j, i) are blocks (i, j) transposed)
+  bool far_closed = true;
+  for (int l = 1; l <= L; ++l) {
+    DevLevel& d = c->lv[l];
+    if (mirrors(d.h_near_i, d.h_near_j, d.h_near_ptr, d.h_mirror)) {
+      std::vector<int32_t> uq, ui, uj, lq, lm;
+      for (int64_t q = 0; q < d.NP; ++q) {
+        const int32_t i = d.h_near_i[q], j = d.h_near_j[q];
+        if (i <= j) uq.push_back((int32_t)q), ui.push_back(i), uj.push_back(j);
+        else lq.push_back((int32_t)q), lm.push_back(d.h_mirror[q]);
+      }
+      d.near_sym = true;
+      d.n_up = (int64_t)uq.size();
+      d.n_lw = (int64_t)lq.size();
+      CKS(upload(c, &d.su_q, uq));
+      CKS(upload(c, &d.su_i, ui));
+      CKS(upload(c, &d.su_j, uj));
+      CKS(upload(c, &d.mirror, d.h_mirror));
+      if (d.n_lw) {
+        CKS(upload(c, &d.lw_q, lq));
+        CKS(upload(c, &d.lw_m, lm));
+      }
+    }
+    std::vector<int32_t> fm;
+    if (d.FP > 0 && mirrors(d.h_far_i, d.h_far_j, d.h_far_ptr, fm)) {
+      std::vector<int32_t> uq, ui, uj, lq, lm;
+      for (int64_t q = 0; q < d.FP; ++q) {
+        if (d.h_far_i[q] < d.h_far_j[q]) uq.push_back((int32_t)q), ui.push_back(d.h_far_i[q]), uj.push_back(d.h_far_j[q]);
+        else lq.push_back((int32_t)q), lm.push_back(fm[q]);
+      }
+      d.far_mirrored = lq.size() == uq.size();
+      d.n_fu = (int64_t)uq.size();
+      CKS(upload(c, &d.fu_q, uq));
+      CKS(upload(c, &d.fu_i, ui));
+      CKS(upload(c, &d.fu_j, uj));
+      CKS(upload(c, &d.fl_q, lq));
+      CKS(upload(c, &d.fl_m, lm));
+    }
+    if (d.FP > 0 && !d.far_mirrored) far_closed = false;
+  }
   // FP32 copy of the H^2 matrix: the operator of the inner solver of the
   // mixed-precision refinement (part of the instance)
-  CKC(dalloc(c, &c->xhat32, c->hat_off[L + 1]));
-  CKC(dalloc(c, &c->yhat32, c->hat_off[L + 1]));
-  for (float** p : {&c->xdf_h, &c->xdf_l}) CKC(dalloc(c, p, nslot));
-  for (float** p : {&c->hdf_h, &c->hdf_l, &c->ydf_h, &c->ydf_l}) CKC(dalloc(c, p, c->hat_off[L + 1]));
-  c->sym = sym_leaf_supported(lf.D);
+  c->pv = c->lv;
+  padded_dims(c);
+  c->hat_off32.assign(L + 2, 0);
+  for (int l = 1; l <= L; ++l) c->hat_off32[l + 1] = c->hat_off32[l] + (int64_t)c->pv[l].nb * c->pv[l].K;
+  const int64_t nhat32 = c->hat_off32[L + 1];
+  const DevLevel& pf = c->pv[L];
+  CKC(dalloc(c, &c->xhat32, nhat32));
+  CKC(dalloc(c, &c->yhat32, nhat32));
+  for (float** p : {&c->xdf_h, &c->xdf_l}) CKC(dalloc(c, p, (size_t)pf.nb * pf.D));
+  for (float** p : {&c->hdf_h, &c->hdf_l, &c->ydf_h, &c->ydf_l}) CKC(dalloc(c, p, nhat32));
+  const int64_t DD = (int64_t)pf.D * pf.D;
+  const PadSeg ls = leaf_seg(c);
+  c->sym = sym_supported(pf.D) && (L == 0 || lf.near_sym);
+  size_t npart = 0;
   if (c->sym) {
     // the kernels' near blocks are symmetric (A_ji = A_ij^T): keep i <= j
-    std::vector<int32_t> uq, ui, uj;
-    for (int64_t q = 0; q < lf.NP; ++q)
-      if (lf.h_near_i[q] <= lf.h_near_j[q])
-        uq.push_back((int32_t)q), ui.push_back(lf.h_near_i[q]), uj.push_back(lf.h_near_j[q]);
-    c->npu = (int64_t)uq.size();
-    std::vector<std::vector<std::pair<int32_t, int32_t>>> lists(lf.nb);  // (partner box, entry)
-    for (int64_t k = 0; k < c->npu; ++k) {
-      lists[ui[k]].push_back({uj[k], (int32_t)(2 * k)});
-      if (ui[k] != uj[k]) lists[uj[k]].push_back({ui[k], (int32_t)(2 * k + 1)});
-    }
-    std::vector<int64_t> ptr(lf.nb + 1, 0);
-    std::vector<int32_t> ent;
-    for (int i = 0; i < lf.nb; ++i) {
-      std::sort(lists[i].begin(), lists[i].end());
-      for (auto& pe : lists[i]) ent.push_back(pe.second);
-      ptr[i + 1] = (int64_t)ent.size();
-    }
-    CKS(upload(c, &c->sym_q, uq));
-    CKS(upload(c, &c->sym_i, ui));
-    CKS(upload(c, &c->sym_j, uj));
-    CKS(upload(c, &c->sym_ptr, ptr));
-    CKS(upload(c, &c->sym_ent, ent));
-    const int64_t DD = (int64_t)lf.D * lf.D;
+    const StoredPairs sp(lf.h_near_i, lf.h_near_j, lf.nb, true);
+    c->npu = (int64_t)sp.q.size();
+    std::vector<SymPair> ds;
+    sp.describe(ds, pf.D, 0, 0, 0);
+    CKS(upload(c, &c->sym_q, sp.q));
+    CKS(upload(c, &c->sym_desc, ds));
+    CKS(upload(c, &c->sym_ptr, sp.ptr));
+    CKS(upload(c, &c->sym_ent, sp.ent));
     CKC(dalloc(c, &c->A32, (size_t)(c->npu * DD)));
     CKC(dalloc(c, &c->Alo, (size_t)(c->npu * DD)));
-    launch_gather_blocks(c->A64, c->sym_q, DD, c->npu, c->A32, 0);
-    launch_gather_split_lo(c->A64, c->sym_q, DD, c->npu, c->A32, c->Alo, 0);
+    launch_pad_blocks<double>(c->A64, c->sym_q, c->npu, pf.D, ls, pf.D, ls, c->A32, c->Alo, lf.near_i, lf.near_j, 0);
+    npart = (size_t)c->npu * 2 * pf.D;
   } else {
-    CKC(dalloc(c, &c->A32, (size_t)lf.NP * lf.D * lf.D));
-    launch_convert<double, float>(c->A64, c->A32, (int64_t)lf.NP * lf.D * lf.D, 0);
-    CKC(dalloc(c, &c->Alo, (size_t)lf.NP * lf.D * lf.D));
-    launch_split_lo(c->A64, c->A32, c->Alo, (int64_t)lf.NP * lf.D * lf.D, 0);
-  }
-  // upper / lower split of each level's near list (symmetric kernels)
-  for (int l = 1; l <= L && c->sym; ++l) {
-    DevLevel& d = c->lv[l];
-    std::map<std::pair<int32_t, int32_t>, int32_t> at;
-    for (int64_t q = 0; q < d.NP; ++q) at[{d.h_near_i[q], d.h_near_j[q]}] = (int32_t)q;
-    d.h_mirror.assign(d.NP, -1);
-    bool closed = true;
-    std::vector<int32_t> uq, ui, uj, lq, lm;
-    for (int64_t q = 0; q < d.NP; ++q) {
-      const int32_t i = d.h_near_i[q], j = d.h_near_j[q];
-      auto it = at.find({j, i});
-      if (it == at.end()) {
-        closed = false;
-        break;
-      }
-      d.h_mirror[q] = it->second;
-      if (i <= j) uq.push_back((int32_t)q), ui.push_back(i), uj.push_back(j);
-      else lq.push_back((int32_t)q), lm.push_back(it->second);
-    }
-    if (!closed) continue;
-    d.near_sym = true;
-    d.n_up = (int64_t)uq.size();
-    d.n_lw = (int64_t)lq.size();
-    CKS(upload(c, &d.su_q, uq));
-    CKS(upload(c, &d.su_i, ui));
-    CKS(upload(c, &d.su_j, uj));
-    CKS(upload(c, &d.mirror, d.h_mirror));
-    if (d.n_lw) {
-      CKS(upload(c, &d.lw_q, lq));
-      CKS(upload(c, &d.lw_m, lm));
-    }
+    CKC(dalloc(c, &c->A32, (size_t)(lf.NP * DD)));
+    CKC(dalloc(c, &c->Alo, (size_t)(lf.NP * DD)));
+    launch_pad_blocks<double>(c->A64, nullptr, lf.NP, pf.D, ls, pf.D, ls, c->A32, c->Alo, lf.near_i, lf.near_j, 0);
   }
   c->X64p.assign(L + 1, nullptr);
   c->S64p.assign(L + 1, nullptr);
@@ -303,88 +385,62 @@ h2_status setup_device(h2_ctx* c) {
   c->S32p.assign(L + 1, nullptr);
   c->Slo.assign(L + 1, nullptr);
   c->Xlo.assign(L + 1, nullptr);
-  size_t npart = c->sym ? (size_t)c->npu * 2 * lf.D : 0;
-  // one batch of all levels' stored coupling pairs when every level with
-  // couplings qualifies for the symmetric form with one common rank
-  std::vector<int64_t> goff(L + 1, 0);
-  {
-    bool ok = true;
-    int K0 = -1;
-    int64_t tot = 0;
-    for (int l = 1; l <= L && ok; ++l) {
-      const DevLevel& d = c->lv[l];
+  // the couplings i < j of all levels as one batch
+  c->cb_ok = L >= 1 && far_closed;
+  for (int l = 1; l <= L; ++l)
+    if (c->pv[l].FP > 0 && !sym_supported(c->pv[l].K)) c->cb_ok = false;
+  std::vector<SymPair> cb;
+  std::vector<int32_t*> fsq(L + 1, nullptr);
+  int64_t cb_m = 0, cb_p = 0;
+  for (int l = 1; l <= L && c->cb_ok; ++l) {
+    DevLevel& d = c->pv[l];
+    if (d.FP == 0) continue;
+    const StoredPairs sp(d.h_far_i, d.h_far_j, d.nb, false);
+    d.fpu = (int64_t)sp.q.size();
+    d.fs_poff = cb_p;
+    sp.describe(cb, d.K, cb_m, cb_p, c->hat_off32[l]);
+    CKS(upload(c, &fsq[l], sp.q));
+    CKS(upload(c, &d.fs_ptr, sp.ptr));
+    CKS(upload(c, &d.fs_ent, sp.ent));
+    cb_m += d.fpu * (int64_t)d.K * d.K;
+    cb_p += d.fpu * 2 * (int64_t)d.K;
+    c->cb_max = std::max(c->cb_max, d.K);
+  }
+  c->cb_n = (int64_t)cb.size();
+  if (c->cb_ok) {
+    CKS(upload(c, &c->cb, cb));
+    CKC(dalloc(c, &c->S32u_all, (size_t)cb_m));
+    CKC(dalloc(c, &c->part32c, (size_t)cb_p));
+    int64_t m0 = 0;
+    for (int l = 1; l <= L; ++l) {
+      const DevLevel& d = c->pv[l];
       if (d.FP == 0) continue;
-      if (!sym_leaf_supported(d.K) || (K0 >= 0 && d.K != K0) || c->hat_off[l] % d.K != 0) ok = false;
-      K0 = d.K;
-      goff[l] = tot;
-      for (int64_t q = 0; q < d.FP; ++q) tot += d.h_far_i[q] < d.h_far_j[q];
-    }
-    c->cb_ok = ok && tot > 0;
-    if (c->cb_ok) {
-      c->cb_K = K0;
-      c->cb_n = tot;
-      CKC(dalloc(c, &c->S32u_all, (size_t)tot * K0 * K0));
+      launch_pad_blocks<double>(d.S, fsq[l], d.fpu, d.K, skel_seg(c, l), d.K, skel_seg(c, l), c->S32u_all + m0, nullptr,
+                                nullptr, nullptr, 0);
+      m0 += d.fpu * (int64_t)d.K * d.K;
     }
   }
-  std::vector<int32_t> cbi, cbj;
   for (int l = 1; l <= L; ++l) {
-    DevLevel& d = c->lv[l];
+    DevLevel& d = c->pv[l];
+    const DevLevel& g = c->lv[l];
     const size_t nx = (size_t)d.nb * d.D * d.K, ns = (size_t)std::max<int64_t>(d.FP, 1) * d.K * d.K;
+    const PadSeg rs = row_seg(c, l), ks = skel_seg(c, l);
     CKC(dalloc(c, &d.X32, nx));
     CKC(dalloc(c, &d.S32, ns));
-    launch_convert<double, float>(d.X, d.X32, (int64_t)nx, 0);
-    launch_convert<double, float>(d.S, d.S32, (int64_t)ns, 0);
-    d.far_sym = d.FP > 0 && sym_leaf_supported(d.K);
-    if (d.far_sym) {
-      // couplings of a symmetric kernel: S_ji = S_ij^T; keep i < j
-      std::vector<int32_t> fq, fi, fj;
-      for (int64_t q = 0; q < d.FP; ++q)
-        if (d.h_far_i[q] < d.h_far_j[q]) fq.push_back((int32_t)q), fi.push_back(d.h_far_i[q]), fj.push_back(d.h_far_j[q]);
-      d.fpu = (int64_t)fq.size();
-      std::vector<std::vector<std::pair<int32_t, int32_t>>> lists(d.nb);
-      for (int64_t k = 0; k < d.fpu; ++k) {
-        lists[fi[k]].push_back({fj[k], (int32_t)(2 * k)});
-        lists[fj[k]].push_back({fi[k], (int32_t)(2 * k + 1)});
-      }
-      std::vector<int64_t> ptr(d.nb + 1, 0);
-      std::vector<int32_t> ent;
-      for (int i = 0; i < d.nb; ++i) {
-        std::sort(lists[i].begin(), lists[i].end());
-        for (auto& pe : lists[i]) ent.push_back(pe.second);
-        ptr[i + 1] = (int64_t)ent.size();
-      }
-      int32_t* fsq = nullptr;
-      CKS(upload(c, &fsq, fq));
-      CKS(upload(c, &d.fs_i, fi));
-      CKS(upload(c, &d.fs_j, fj));
-      CKS(upload(c, &d.fs_ptr, ptr));
-      CKS(upload(c, &d.fs_ent, ent));
-      const int64_t KK = (int64_t)d.K * d.K;
-      if (c->cb_ok) {
-        d.fs_goff = goff[l];
-        d.S32u = c->S32u_all + goff[l] * KK;
-        const int32_t s0 = (int32_t)(c->hat_off[l] / d.K);
-        for (int64_t k = 0; k < d.fpu; ++k) cbi.push_back(s0 + fi[k]), cbj.push_back(s0 + fj[k]);
-      } else {
-        CKC(dalloc(c, &d.S32u, (size_t)(d.fpu * KK)));
-      }
-      launch_gather_blocks(d.S, fsq, KK, d.fpu, d.S32u, 0);
-      npart = std::max(npart, (size_t)d.fpu * 2 * d.K);
-    }
-    // the residual's FP32-pair matvec reads the couplings in full
-    CKC(dalloc(c, &c->Slo[l], ns));
-    launch_split_lo(d.S, d.S32, c->Slo[l], (int64_t)d.FP * d.K * d.K, 0);
     CKC(dalloc(c, &c->Xlo[l], nx));
-    launch_split_lo(d.X, d.X32, c->Xlo[l], (int64_t)nx, 0);
+    CKC(dalloc(c, &c->Slo[l], ns));
+    launch_pad_blocks<double>(d.X, nullptr, d.nb, d.D, rs, d.K, ks, d.X32, c->Xlo[l], nullptr, nullptr, 0);
+    // (the residual's FP32-pair matvec reads the couplings in full)
+    launch_pad_blocks<double>(d.S, nullptr, d.FP, d.K, ks, d.K, ks, d.S32, c->Slo[l], nullptr, nullptr, 0);
+    d.X32q = d.X32;
+    if (d.D != g.D || d.K != g.K) {
+      CKC(dalloc(c, &d.X32q, (size_t)g.nb * g.D * g.K));
+      launch_convert<double, float>(g.X, d.X32q, (int64_t)g.nb * g.D * g.K, 0);
+    }
     c->X64p[l] = d.X;
     c->S64p[l] = d.S;
     c->X32p[l] = d.X32;
     c->S32p[l] = d.S32;
-  }
-  if (c->cb_ok) {
-    CKS(upload(c, &c->cb_i, cbi));
-    CKS(upload(c, &c->cb_j, cbj));
-    CKC(dalloc(c, &c->part32c, (size_t)c->cb_n * 2 * c->cb_K));
   }
   if (npart) {
     CKC(dalloc(c, &c->part32, npart));
@@ -411,30 +467,44 @@ struct Ev {
 template <typename T>
 void release_factor(h2_ctx* c, Factor<T>& F);
 
+// the levels as the arrays of storage type T hold them
+template <typename T>
+const std::vector<DevLevel>& levels(const h2_ctx* c) {
+  if constexpr (std::is_same<T, double>::value) return c->lv;
+  else return c->pv;
+}
+
+// whether the FP32 path's leaf level takes its input from the stored halves
+// A32 (the pairs i <= j) instead of a copy of all its blocks
+bool leaf_in_halves(const h2_ctx* c) { return c->sym && c->lv[c->L].near_sym && c->lv[c->L].n_lw > 0; }
+
 template <typename T>
 h2_status alloc_factor_arrays(h2_ctx* c, Factor<T>& F) {
   AllocSink sink(c, &F.allocs);
   const int L = c->L;
   F.lv.assign(L + 1, FacLevel<T>());
   size_t wk = 0, wk16 = 0, wq = 0, wc = 0, wc16 = 0;
+  const std::vector<DevLevel>& LV = levels<T>(c);
   for (int l = 0; l <= L; ++l) {
-    const DevLevel& d = c->lv[l];
+    const DevLevel& d = LV[l];
+    const size_t Dq = c->lv[l].D, Kq = c->lv[l].K;  // the QR runs without padding
     FacLevel<T>& f = F.lv[l];
     const size_t nb = d.nb, D = d.D, K = d.K, R = d.R;
     wk = std::max(wk, (size_t)d.NP * D * D);
     const bool mixed = !std::is_same<T, double>::value;
-    f.tc = mixed && l >= 1 && gemm_tc_supported(d.D, d.D, d.D, d.D, d.D, d.D);
+    // (padded levels stay off the 16-bit path, as their logical shapes do)
+    f.tc = mixed && l >= 1 && D == Dq && K == Kq && gemm_tc_supported(d.D, d.D, d.D, d.D, d.D, d.D);
     bool leaf64 = (l == L) && !mixed;
     if (!leaf64 && !(f.tc && l == L)) {
       if (f.tc) CKC(dalloc(c, reinterpret_cast<uint16_t**>(&f.Ain16), (size_t)d.NP * D * D));
-      else CKC(dalloc(c, &f.Ain, (size_t)d.NP * D * D));
+      else if (!(mixed && l == L && l >= 1 && leaf_in_halves(c))) CKC(dalloc(c, &f.Ain, (size_t)d.NP * D * D));
     }
     if (l == 0) continue;
     if (f.tc) {
       CKC(dalloc(c, reinterpret_cast<uint16_t**>(&f.U16), nb * D * D));
       wk16 = std::max(wk16, (size_t)d.NP * D * D);
     }
-    f.tc_coup = mixed && d.FP > 0 && gemm_tc_supported(d.K, d.K, d.K, d.K, d.K, d.K);
+    f.tc_coup = mixed && d.FP > 0 && K == Kq && gemm_tc_supported(d.K, d.K, d.K, d.K, d.K, d.K);
     if (f.tc_coup) {
       CKC(dalloc(c, reinterpret_cast<uint16_t**>(&f.T16), nb * K * K));
       wc16 = std::max(wc16, (size_t)d.FP * K * K);
@@ -443,13 +513,15 @@ h2_status alloc_factor_arrays(h2_ctx* c, Factor<T>& F) {
     }
     CKC(dalloc(c, &f.U, nb * D * D));
     CKC(dalloc(c, &f.Ur, nb * D * D));
-    CKC(dalloc(c, &f.Tm, nb * K * K));
-    CKC(dalloc(c, &f.Xo, nb * D * K));
-    CKC(dalloc(c, &f.Vq, nb * D * K));
-    CKC(dalloc(c, &f.tau, nb * std::max<size_t>(K, 1)));
-    CKC(dalloc(c, &f.Tw, nb * K * K));
-    if (sizeof(T) * D * K > 200 * 1024) CKC(dalloc(c, &f.Qs, nb * D * K));
-    wq = std::max(wq, nb * (K * K + D * K));
+    CKC(dalloc(c, &f.Tm, nb * Kq * Kq));
+    f.Tp = f.Tm;
+    if (K != Kq) CKC(dalloc(c, &f.Tp, nb * K * K));
+    CKC(dalloc(c, &f.Xo, nb * Dq * Kq));
+    CKC(dalloc(c, &f.Vq, nb * Dq * Kq));
+    CKC(dalloc(c, &f.tau, nb * std::max<size_t>(Kq, 1)));
+    CKC(dalloc(c, &f.Tw, nb * Kq * Kq));
+    if (sizeof(T) * Dq * Kq > 200 * 1024) CKC(dalloc(c, &f.Qs, nb * Dq * Kq));
+    wq = std::max(wq, nb * (Kq * Kq + Dq * Kq));
     CKC(dalloc(c, &f.Ahat, (size_t)d.NP * D * D));
     if (f.tc) CKC(dalloc(c, reinterpret_cast<uint16_t**>(&f.Ahat16), (size_t)d.NP * D * D));
     CKC(dalloc(c, &f.Shat, (size_t)std::max<int64_t>(d.FP, 1) * K * K));
@@ -467,10 +539,10 @@ h2_status alloc_factor_arrays(h2_ctx* c, Factor<T>& F) {
     CKC(dalloc(c, &f.M1, std::max<size_t>(nb * R * D, 1)));
     for (T** p : {&f.u, &f.v, &f.om}) CKC(dalloc(c, p, nb * std::max<size_t>(R, 1)));
   }
-  const int D0 = c->lv[0].D;
+  const int D0 = LV[0].D;
   size_t npart = 1;
   for (int l = 1; l <= L; ++l) {
-    const DevLevel& d = c->lv[l];
+    const DevLevel& d = LV[l];
     npart = std::max(npart, (size_t)d.NP * (size_t)std::max(d.R, d.K));
   }
   CKC(dalloc(c, &F.part, npart));
@@ -533,6 +605,7 @@ template <typename T>
 h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
   CKS(alloc_factor(c, F));
   const int L = c->L;
+  const std::vector<DevLevel>& LV = levels<T>(c);
   cudaStream_t st = c->stream;
   if (!c->basis_stream) {
     // the highest priority: the other chain waits for each level's bases
@@ -584,8 +657,8 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
   const bool lu64_mixed = mixed && c->rr_lu64;
   if (lu64_mixed && !F.rr_lu) {
     AllocSink sink(c, &F.allocs);
-    size_t n = (size_t)c->lv[0].nb * c->lv[0].D * c->lv[0].D;
-    for (int l = 1; l <= L; ++l) n = std::max(n, (size_t)c->lv[l].nb * c->lv[l].R * c->lv[l].R);
+    size_t n = (size_t)LV[0].nb * LV[0].D * LV[0].D;
+    for (int l = 1; l <= L; ++l) n = std::max(n, (size_t)LV[l].nb * LV[l].R * LV[l].R);
     CKC(dalloc(c, &F.rr_lu, n));
     CKC(dalloc(c, &F.rr_inv, n));
   }
@@ -598,31 +671,42 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
   wait_for(st, sc);
   wait_for(st, sp);
   mark();
+  // (the FP32 projection of the upper pairs reads them from the instance's
+  // stored halves, which list them in the same order)
+  const bool leaf_halves = mixed && L >= 1 && leaf_in_halves(c);
   const T* Aleaf = nullptr;
   if (!mixed) {
     Aleaf = reinterpret_cast<const T*>(c->A64);
   } else if (L == 0 || !F.lv[L].tc) {
     if (!c->A64) return fail(H2_ERR_STATE, "the leaf level needs the FP64 leaf blocks, which were released");
-    launch_convert<double, T>(c->A64, F.lv[L].Ain, (int64_t)c->lv[L].NP * c->lv[L].D * c->lv[L].D, st);
-    Aleaf = F.lv[L].Ain;
+    const DevLevel& lf = LV[L];
+    if constexpr (std::is_same<T, float>::value) {
+      if (leaf_halves) {
+        Aleaf = c->A32;
+      } else {
+        launch_pad_blocks<double>(c->A64, nullptr, lf.NP, lf.D, leaf_seg(c), lf.D, leaf_seg(c), F.lv[L].Ain, nullptr,
+                                  lf.near_i, lf.near_j, st);
+        Aleaf = F.lv[L].Ain;
+      }
+    }
   }
   mark();
 
   // ---- basis stream: a1 (and the 16-bit copy of U), a2' per level
   std::string coup_err;
   for (int l = L; l >= 1; --l) {
-    const DevLevel& d = c->lv[l];
+    const DevLevel& d = LV[l];
     FacLevel<T>& f = F.lv[l];
-    const int D = d.D, K = d.K, R = d.R;
-    const int64_t DD = (int64_t)D * D;
     mark_on(evb, sb);
     // a1: complement bases.  X^orth = X (leaf) or blockdiag(T_2p, T_2p+1) X,
     // then Householder QR, the compact WY factor and U = P (I - V Tw V^T).
+    // The QR runs on the logical dimensions; U takes the padded ones.
     {
-      const int nb = d.nb;
-      const int64_t DK = (int64_t)D * K, KK = (int64_t)K * K;
+      const DevLevel& dq = c->lv[l];
+      const int nb = d.nb, D = dq.D, K = dq.K, R = dq.R;
+      const int64_t DD = (int64_t)D * D, DK = (int64_t)D * K, KK = (int64_t)K * K;
       // X in T, row-major D x K per box (the instance keeps FP64 and FP32 copies)
-      const T* Xc = std::is_same<T, double>::value ? reinterpret_cast<const T*>(d.X) : reinterpret_cast<const T*>(d.X32);
+      const T* Xc = std::is_same<T, double>::value ? reinterpret_cast<const T*>(d.X) : reinterpret_cast<const T*>(d.X32q);
       const T* Xin = Xc;
       if (l < L) {
         const int Kc = c->lv[l + 1].K;
@@ -647,23 +731,21 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
         gemm<T>(prec, D, K, K, f.Vq, DK, nullptr, D, true, f.Tw, KK, nullptr, K, false, W1, DK, nullptr, K, T(1), T(0),
                 nb, sb);
       }
+      bool formed = false;
       if constexpr (std::is_same<T, float>::value) {
-        // one pass: U, its row-major copy and the 16-bit copy
-        if (K > 0 && D % 4 == 0 && K % 4 == 0) {
-          launch_form_u(nb, D, K, W1, f.Vq, f.U, f.Ur, f.tc ? f.U16 : nullptr, bf16, sb);
-        } else {
-          launch_perm_identity<T>(nb, D, K, f.U, sb);
-          if (K > 0) {
-            if (R > 0)
-              gemm<T>(prec, R, D, K, f.Vq + K, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U, DD, nullptr, D,
-                      T(-1), T(1), nb, sb);
-            gemm<T>(prec, K, D, K, f.Vq, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U + (int64_t)R * D, DD,
-                    nullptr, D, T(-1), T(1), nb, sb);
-          }
-          launch_transpose_blocks<T>(nb, D, f.U, f.Ur, sb);
-          if (f.tc) launch_to_lowp<T>(bf16, f.U, f.U16, (int64_t)d.nb * DD, nullptr, sb);
+        if (K > 0) {
+          // one pass: U, its row-major copy and the 16-bit copy
+          const bool u16 = f.tc && D % 4 == 0 && K % 4 == 0;
+          launch_form_u(nb, D, K, W1, f.Vq, f.U, f.Ur, u16 ? f.U16 : nullptr, bf16, d.D, d.K, row_seg(c, l), sb);
+          if (d.D != D) launch_form_u_pads(nb, d.D, d.R, R, K, row_seg(c, l), f.U, f.Ur, sb);
+          if (f.tc && !u16) launch_to_lowp<T>(bf16, f.U, f.U16, (int64_t)d.nb * DD, nullptr, sb);
+          if (d.K != K)
+            launch_pad_blocks<float>(f.Tm, nullptr, nb, d.K, skel_seg(c, l), d.K, skel_seg(c, l), f.Tp, nullptr, nullptr,
+                                     nullptr, sb);
+          formed = true;
         }
-      } else {
+      }
+      if (!formed) {
         launch_perm_identity<T>(nb, D, K, f.U, sb);
         if (K > 0) {
           if (R > 0)
@@ -676,6 +758,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
         if (f.tc) launch_to_lowp<T>(bf16, f.U, f.U16, (int64_t)d.nb * DD, nullptr, sb);
       }
     }
+    const int K = d.K;
     mark_on(evb, sb);
     // the couplings of level l follow its bases on the coupling stream
     CKC(cudaStreamWaitEvent(sc, evb.back(), 0));
@@ -686,9 +769,9 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       const int64_t KK = (int64_t)K * K;
       unsigned int* am = F.amax + (L + 1) + l;
       CKC(cudaMemsetAsync(am, 0, sizeof(unsigned int), sc));
-      launch_amax_blocks<T>(f.Tm, d.nb, KK, K, K, K, am, sc);
+      launch_amax_blocks<T>(f.Tp, d.nb, KK, K, K, K, am, sc);
       launch_pow2_scale(am, std::sqrt(32768.0f / K), F.tscale + 2 * l, sc);
-      launch_to_lowp<T>(bf16, f.Tm, f.T16, d.nb * KK, F.tscale + 2 * l, sc);
+      launch_to_lowp<T>(bf16, f.Tp, f.T16, d.nb * KK, F.tscale + 2 * l, sc);
       launch_inv_scale_product(d.S16_scale[bf16], F.tscale + 2 * l, F.cscale + l, sc);
       bool ok = gemm_tc(bf16, K, K, K, d.S16[bf16], d.FP, K, K, nullptr, f.T16, d.nb, K, K, d.far_j, F.W16c, KK,
                         nullptr, K, 1, bf16, 1.0f, nullptr, d.FP, c->status + 2, sc, nullptr, -1, nullptr, nullptr,
@@ -703,10 +786,13 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
     } else if (d.FP > 0 && K > 0) {
       const int64_t KK = (int64_t)K * K;
       const T* Sc = std::is_same<T, double>::value ? reinterpret_cast<const T*>(d.S) : reinterpret_cast<const T*>(d.S32);
-      gemm<T>(prec, K, K, K, Sc, KK, nullptr, K, false, f.Tm, KK, d.far_j, K, true, F.Wc, KK, nullptr, K, T(1),
-              T(0), d.FP, sc);
-      gemm<T>(prec, K, K, K, f.Tm, KK, d.far_i, K, false, F.Wc, KK, nullptr, K, false, f.Shat, KK, nullptr, K, T(1),
-              T(0), d.FP, sc);
+      // (symmetric lists: the pairs i < j, and the others as their transposes)
+      const bool up = d.far_mirrored;
+      const int64_t n = up ? d.n_fu : d.FP;
+      const int32_t *pq = up ? d.fu_q : nullptr, *pi = up ? d.fu_i : d.far_i, *pj = up ? d.fu_j : d.far_j;
+      gemm<T>(prec, K, K, K, Sc, KK, pq, K, false, f.Tp, KK, pj, K, true, F.Wc, KK, nullptr, K, T(1), T(0), n, sc);
+      gemm<T>(prec, K, K, K, f.Tp, KK, pi, K, false, F.Wc, KK, nullptr, K, false, f.Shat, KK, pq, K, T(1), T(0), n, sc);
+      if (up) launch_transpose_pairs<T>(K, n, d.fl_q, d.fl_m, f.Shat, sc);
     }
     // max |Shat| for the 16-bit merge's scale, beside the main chain
     if (mixed && F.lv[l - 1].tc && std::is_same<T, float>::value) {
@@ -727,13 +813,13 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
   // bits (the merge reads the lower pairs' SS from their mirrors)
   for (int l = 0; l <= L; ++l) F.lv[l].proj_sym = false;
   for (int l = 2; l <= L; ++l) {
-    const DevLevel& d = c->lv[l];
+    const DevLevel& d = LV[l];
     F.lv[l].proj_sym = d.near_sym && F.lv[l].tc && F.lv[l - 1].tc && (bf16 || d.D <= 256) && d.R > 0 &&
                        d.R % 32 == 0 && d.K > 0;
   }
   // ---- the context's stream: a2, a3, a4/a5, a6 per level
   for (int l = L; l >= 1; --l) {
-    const DevLevel& d = c->lv[l];
+    const DevLevel& d = LV[l];
     FacLevel<T>& f = F.lv[l];
     const int D = d.D, K = d.K, R = d.R;
     const int64_t DD = (int64_t)D * D;
@@ -789,11 +875,11 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
         launch_transpose16_blocks(D, R, d.n_lw, d.lw_q, d.lw_m, f.Ahat16, sp);
       }
       if (!ok) return fail(H2_ERR_CUDA, "tensor-core GEMM setup failed at level " + std::to_string(l));
-    } else if (!mixed && d.near_sym && d.n_lw > 0) {
-      // FP64, symmetric near list: project the upper pairs i <= j, then
+    } else if (d.near_sym && d.n_lw > 0) {
+      // symmetric near list: project the upper pairs i <= j, then
       // Ahat_ji = Ahat_ij^T for the lower ones (the kernels are symmetric)
       const T* Ain = (l == L) ? Aleaf : f.Ain;
-      gemm<T>(prec, D, D, D, Ain, DD, d.su_q, D, false, f.U, DD, d.su_j, D, true, F.Wk, DD, nullptr, D, T(1), T(0),
+      gemm<T>(prec, D, D, D, Ain, DD, l == L && leaf_halves ? nullptr : d.su_q, D, false, f.U, DD, d.su_j, D, true, F.Wk, DD, nullptr, D, T(1), T(0),
               d.n_up, st);
       gemm<T>(prec, D, D, D, f.U, DD, d.su_i, D, false, F.Wk, DD, nullptr, D, false, f.Ahat, DD, d.su_q, D, T(1),
               T(0), d.n_up, st);
@@ -900,7 +986,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
   if (L >= 1) CKC(cudaStreamWaitEvent(st, evb.back(), 0));
   wait_for(sp, st);
   // a7: root
-  const int D0 = c->lv[0].D;
+  const int D0 = LV[0].D;
   const T* Aroot = (L == 0) ? Aleaf : F.lv[0].Ain;
   const int nr = c->lv[0].nb;  // one root per system (the level-0 blocks are in box order)
   if (lu64_mixed)
@@ -983,12 +1069,13 @@ void with_ahat(const FacLevel<T>& f, int bf16, Fn&& fn) {
 template <typename T>
 void ulv_sweep(h2_ctx* c, Factor<T>& F) {
   const int L = c->L;
+  const std::vector<DevLevel>& LV = levels<T>(c);
   cudaStream_t st = c->stream;
   // the children's input of level l (below the leaf level: their SR sums)
   auto child_in = [&](int l) {
     ChildIn<T> ch;
     if (l < L) {
-      const DevLevel& dc = c->lv[l + 1];
+      const DevLevel& dc = LV[l + 1];
       const FacLevel<T>& fc = F.lv[l + 1];
       ch.c = fc.c;
       ch.part = fc.part;
@@ -999,7 +1086,7 @@ void ulv_sweep(h2_ctx* c, Factor<T>& F) {
     return ch;
   };
   auto fwd = [&](int l) {
-    const DevLevel& d = c->lv[l];
+    const DevLevel& d = LV[l];
     FacLevel<T>& f = F.lv[l];
     launch_fwd1<T>(d, f, child_in(l), st);
     with_ahat(f, F.bf16, [&](auto A, const float* isc) {
@@ -1009,7 +1096,7 @@ void ulv_sweep(h2_ctx* c, Factor<T>& F) {
     });
   };
   auto bwd = [&](int l) {
-    const DevLevel& d = c->lv[l];
+    const DevLevel& d = LV[l];
     FacLevel<T>& f = F.lv[l];
     const T* px = (l > 1) ? F.lv[l - 1].xs : F.root_x;
     with_ahat(f, F.bf16, [&](auto A, const float* isc) {
@@ -1019,7 +1106,7 @@ void ulv_sweep(h2_ctx* c, Factor<T>& F) {
     });
   };
   for (int l = L; l >= 1; --l) fwd(l);
-  launch_gemv_rows<T>(c->lv[0].nb, c->lv[0].D, F.root_inv, F.root_vec, F.root_x, st);
+  launch_gemv_rows<T>(LV[0].nb, LV[0].D, F.root_inv, F.root_vec, F.root_x, st);
   for (int l = 1; l <= L; ++l) bwd(l);
 }
 template <typename T>
@@ -1028,15 +1115,22 @@ template <typename T>
 T* ulv_out(h2_ctx* c, Factor<T>& F) { return c->L >= 1 ? F.lv[c->L].xs : F.root_x; }
 
 int64_t nslots(const h2_ctx* c) { return (int64_t)c->lv[c->L].nb * c->lv[c->L].D; }
+// the same of the FP32 vectors (padded boxes)
+int64_t nslots32(const h2_ctx* c) { return (int64_t)c->pv[c->L].nb * c->pv[c->L].D; }
+template <typename T>
+PadSeg vec_seg(const h2_ctx* c) {
+  const int D = c->lv[c->L].D;
+  return std::is_same<T, double>::value ? PadSeg{D, D} : leaf_seg(c);
+}
 
 // x += ULV^-1 r for FP64 tree vectors; the sweep runs in T on r / ||r||.
 template <typename T>
 void ulv_apply_impl(h2_ctx* c, Factor<T>& F, const double* r, double* x) {
   const int64_t n = nslots(c);
   launch_norm2<double>(r, n, c->red, c->stream);
-  launch_scale_to<T>(r, c->red, ulv_in(c, F), n, c->stream);
+  launch_scale_to<T>(r, c->red, ulv_in(c, F), n, vec_seg<T>(c), c->stream);
   ulv_sweep<T>(c, F);
-  launch_axpy_from<T>(ulv_out(c, F), c->red, x, n, c->stream);
+  launch_axpy_from<T>(ulv_out(c, F), c->red, x, n, vec_seg<T>(c), c->stream);
 }
 
 // Capture fn's work on the context's stream into a CUDA graph (on a private
@@ -1075,7 +1169,7 @@ void drop_graphs(h2_ctx* c) {
 // z = ULV^-1 v for FP32 tree vectors (mixed-precision factorization); the
 // sweep (about a hundred dependent launches) replays as one CUDA graph.
 void ulv_apply_f32(h2_ctx* c, const float* v, float* z) {
-  const int64_t n = nslots(c);
+  const int64_t n = nslots32(c);
   Factor<float>& F = c->f32;
   cudaMemcpyAsync(ulv_in(c, F), v, n * sizeof(float), cudaMemcpyDeviceToDevice, c->stream);
   if (c->use_graphs && !c->g_ulv) c->g_ulv = capture_graph(c, c->g_ulv_kernels, [&] { ulv_sweep<float>(c, F); });
@@ -1100,6 +1194,7 @@ template <typename T>
 void matvec_t(h2_ctx* c, const T* A, T* const* X, T* const* S, T* xh, T* yh, const T* x, T* y,
               EventPairs* leaf_ev = nullptr) {
   const int L = c->L;
+  const std::vector<DevLevel>& LV = levels<T>(c);
   cudaStream_t st = c->stream;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (leaf_ev) {
@@ -1111,23 +1206,23 @@ void matvec_t(h2_ctx* c, const T* A, T* const* X, T* const* S, T* xh, T* yh, con
   auto leaf = [&](const T* XL, const T* yhL) {
     if constexpr (std::is_same<T, float>::value) {
       if (c->sym) {
-        const DevLevel& lf = c->lv[L];
+        const DevLevel& lf = LV[L];
         if (leaf_ev) cudaEventRecord(e0, st);
-        launch_matvec_sym_pairs(lf.D, c->npu, c->sym_i, c->sym_j, A, x, c->part32, false, st);
+        launch_matvec_sym_pairs(lf.D, c->npu, c->sym_desc, A, x, c->part32, false, st);
         if (leaf_ev) cudaEventRecord(e1, st), leaf_ev->push_back({e0, e1});
         launch_matvec_sym_sum<float>(lf.nb, lf.D, L ? lf.K : 0, c->sym_ptr, c->sym_ent, XL, yhL, c->part32, y, st);
         return;
       }
     }
     if (leaf_ev) cudaEventRecord(e0, st);
-    launch_matvec_leaf<T>(c->lv[L], A, XL, x, yhL, y, st);
+    launch_matvec_leaf<T>(LV[L], A, XL, x, yhL, y, st);
     if (leaf_ev) cudaEventRecord(e1, st), leaf_ev->push_back({e0, e1});
   };
   if (L == 0) {
     leaf(nullptr, nullptr);
     return;
   }
-  const std::vector<int64_t>& off = c->hat_off;
+  const std::vector<int64_t>& off = std::is_same<T, double>::value ? c->hat_off : c->hat_off32;
   if constexpr (std::is_same<T, float>::value) {
     if (c->cb_ok && c->sym) {
       // the leaf near-field products need only x: they run on the leaf
@@ -1140,27 +1235,27 @@ void matvec_t(h2_ctx* c, const T* A, T* const* X, T* const* S, T* xh, T* yh, con
         cudaEventCreateWithFlags(&c->mv_join, cudaEventDisableTiming);
       }
       cudaStream_t sl = c->leaf_stream;
-      const DevLevel& lf = c->lv[L];
+      const DevLevel& lf = LV[L];
       cudaEventRecord(c->mv_fork, st);
       cudaStreamWaitEvent(sl, c->mv_fork, 0);
       if (leaf_ev) cudaEventRecord(e0, sl);
-      launch_matvec_sym_pairs(lf.D, c->npu, c->sym_i, c->sym_j, A, x, c->part32, false, sl);
+      launch_matvec_sym_pairs(lf.D, c->npu, c->sym_desc, A, x, c->part32, false, sl);
       if (leaf_ev) cudaEventRecord(e1, sl), leaf_ev->push_back({e0, e1});
       cudaEventRecord(c->mv_join, sl);
-      launch_matvec_up<T>(c->lv[L], X[L], x, xh + off[L], st);
-      for (int l = L - 1; l >= 1; --l) launch_matvec_up<T>(c->lv[l], X[l], xh + off[l + 1], xh + off[l], st);
-      launch_matvec_sym_pairs(c->cb_K, c->cb_n, c->cb_i, c->cb_j, c->S32u_all, xh, c->part32c, true, st);
-      const DevLevel& d1 = c->lv[1];
+      launch_matvec_up<T>(LV[L], X[L], x, xh + off[L], st);
+      for (int l = L - 1; l >= 1; --l) launch_matvec_up<T>(LV[l], X[l], xh + off[l + 1], xh + off[l], st);
+      launch_matvec_sym_pairs(c->cb_max, c->cb_n, c->cb, c->S32u_all, xh, c->part32c, true, st);
+      const DevLevel& d1 = LV[1];
       if (d1.FP > 0 && d1.K > 0)
         launch_matvec_sym_sum<float>(d1.nb, d1.K, 0, d1.fs_ptr, d1.fs_ent, nullptr, nullptr,
-                                     c->part32c + d1.fs_goff * 2 * d1.K, yh + off[1], st);
+                                     c->part32c + d1.fs_poff, yh + off[1], st);
       else
         cudaMemsetAsync(yh + off[1], 0, sizeof(T) * (size_t)d1.nb * d1.K, st);
       for (int l = 1; l < L; ++l) {
-        const DevLevel& dc = c->lv[l + 1];
+        const DevLevel& dc = LV[l + 1];
         const bool has = dc.FP > 0 && dc.K > 0;
-        launch_matvec_down_far<float>(c->lv[l], X[l], yh + off[l], yh + off[l + 1], has ? dc.fs_ptr : nullptr,
-                                      has ? dc.fs_ent : nullptr, c->part32c + dc.fs_goff * 2 * dc.K, st);
+        launch_matvec_down_far<float>(LV[l], X[l], yh + off[l], yh + off[l + 1], has ? dc.fs_ptr : nullptr,
+                                      has ? dc.fs_ent : nullptr, c->part32c + dc.fs_poff, st);
       }
       cudaStreamWaitEvent(st, c->mv_join, 0);
       launch_matvec_sym_sum<float>(lf.nb, lf.D, lf.K, c->sym_ptr, c->sym_ent, X[L], yh + off[L], c->part32, y, st,
@@ -1168,20 +1263,13 @@ void matvec_t(h2_ctx* c, const T* A, T* const* X, T* const* S, T* xh, T* yh, con
       return;
     }
   }
-  launch_matvec_up<T>(c->lv[L], X[L], x, xh + off[L], st);
-  for (int l = L - 1; l >= 1; --l) launch_matvec_up<T>(c->lv[l], X[l], xh + off[l + 1], xh + off[l], st);
+  launch_matvec_up<T>(LV[L], X[L], x, xh + off[L], st);
+  for (int l = L - 1; l >= 1; --l) launch_matvec_up<T>(LV[l], X[l], xh + off[l + 1], xh + off[l], st);
   for (int l = 1; l <= L; ++l) {
-    const DevLevel& d = c->lv[l];
-    if constexpr (std::is_same<T, float>::value) {
-      if (d.far_sym) {  // stored halves of the symmetric couplings
-        launch_matvec_sym_pairs(d.K, d.fpu, d.fs_i, d.fs_j, d.S32u, xh + off[l], c->part32, true, st);
-        launch_matvec_sym_sum<float>(d.nb, d.K, 0, d.fs_ptr, d.fs_ent, nullptr, nullptr, c->part32, yh + off[l], st);
-        continue;
-      }
-    }
+    const DevLevel& d = LV[l];
     launch_matvec_far<T>(d, S[l], xh + off[l], yh + off[l], st);
   }
-  for (int l = 1; l < L; ++l) launch_matvec_down<T>(c->lv[l], X[l], yh + off[l], yh + off[l + 1], st);
+  for (int l = 1; l < L; ++l) launch_matvec_down<T>(LV[l], X[l], yh + off[l], yh + off[l + 1], st);
   leaf(X[L], yh + off[L]);
 }
 
@@ -1194,25 +1282,26 @@ void matvec_impl(h2_ctx* c, const double* x, double* y) {
 void matvec_df(h2_ctx* c, const double* x, double* y) {
   const int L = c->L;
   cudaStream_t st = c->stream;
-  const DevLevel& lf = c->lv[L];
-  const std::vector<int64_t>& off = c->hat_off;
-  launch_split_df(x, c->xdf_h, c->xdf_l, nslots(c), st);
+  const std::vector<DevLevel>& LV = c->pv;
+  const DevLevel& lf = LV[L];
+  const std::vector<int64_t>& off = c->hat_off32;
+  launch_split_df(x, c->xdf_h, c->xdf_l, nslots(c), leaf_seg(c), st);
   if (L >= 1) {
     // upward pass, couplings of all levels in one launch, downward pass
     launch_matvec_up_df(lf, c->X32p[L], c->Xlo[L], c->xdf_h, c->xdf_l, c->hdf_h + off[L], c->hdf_l + off[L], st);
     for (int l = L - 1; l >= 1; --l)
-      launch_matvec_up_df(c->lv[l], c->X32p[l], c->Xlo[l], c->hdf_h + off[l + 1], c->hdf_l + off[l + 1],
+      launch_matvec_up_df(LV[l], c->X32p[l], c->Xlo[l], c->hdf_h + off[l + 1], c->hdf_l + off[l + 1],
                           c->hdf_h + off[l], c->hdf_l + off[l], st);
     // levels with the longest far lists first (their CTAs take longest)
     std::vector<int> order;
     for (int l = 1; l <= L; ++l) order.push_back(l);
     std::stable_sort(order.begin(), order.end(), [&](int u, int v) {
-      return c->lv[u].FP * (int64_t)c->lv[v].nb > c->lv[v].FP * (int64_t)c->lv[u].nb;
+      return LV[u].FP * (int64_t)LV[v].nb > LV[v].FP * (int64_t)LV[u].nb;
     });
     FarDfArgs fa{};
     int cta = 0;
     for (int l : order) {
-      const DevLevel& d = c->lv[l];
+      const DevLevel& d = LV[l];
       if (d.FP == 0 || d.K == 0) {
         // no couplings: yhat starts at zero
         cudaMemsetAsync(c->ydf_h + off[l], 0, sizeof(float) * d.nb * d.K, st);
@@ -1231,7 +1320,7 @@ void matvec_df(h2_ctx* c, const double* x, double* y) {
     }
     launch_matvec_far_df_all(fa, st);
     for (int l = 1; l < L; ++l)
-      launch_matvec_down_df(c->lv[l], c->X32p[l], c->Xlo[l], c->ydf_h + off[l], c->ydf_l + off[l],
+      launch_matvec_down_df(LV[l], c->X32p[l], c->Xlo[l], c->ydf_h + off[l], c->ydf_l + off[l],
                             c->ydf_h + off[l + 1], c->ydf_l + off[l + 1], st);
   }
   const float* yhh = L ? c->ydf_h + off[L] : nullptr;
@@ -1240,9 +1329,9 @@ void matvec_df(h2_ctx* c, const double* x, double* y) {
     // the partial products as FP32 pairs in the space of the FP64 ones
     float* ph = reinterpret_cast<float*>(c->part64);
     float* pl = ph + c->npu * 2 * lf.D;
-    launch_matvec_sym_pairs_df(lf.D, c->npu, c->sym_i, c->sym_j, c->A32, c->Alo, c->xdf_h, c->xdf_l, ph, pl, st);
+    launch_matvec_sym_pairs_df(lf.D, c->npu, c->sym_desc, c->A32, c->Alo, c->xdf_h, c->xdf_l, ph, pl, st);
     launch_matvec_sym_sum_df(lf.nb, lf.D, L ? lf.K : 0, c->sym_ptr, c->sym_ent, L ? c->X32p[L] : nullptr,
-                             L ? c->Xlo[L] : nullptr, yhh, yhl, ph, pl, y, st);
+                             L ? c->Xlo[L] : nullptr, yhh, yhl, ph, pl, y, c->lv[L].D, st);
   } else {
     launch_matvec_leaf_df(lf, c->A32, c->Alo, L ? c->X32p[L] : nullptr, L ? c->Xlo[L] : nullptr, c->xdf_h, c->xdf_l,
                           yhh, yhl, y, st);
@@ -1273,7 +1362,7 @@ h2_status subst_check(h2_ctx* c) {
 // mixed-precision Ahat (host, FP32) from the 16-bit copy.
 h2_status export_ahat_quadrants(const h2_ctx* c, int level, float* out) {
   const FacLevel<float>& f = c->f32.lv[level];
-  const DevLevel& d = c->lv[level];
+  const DevLevel& d = c->pv[level];
   const size_t D = d.D, R = d.R, n = (size_t)d.NP * D * D;
   std::vector<uint16_t> h(n);
   float isc = 1.0f;
@@ -1309,6 +1398,50 @@ h2_status export_ahat_quadrants(const h2_ctx* c, int level, float* out) {
         out[e] = v * isc;
       }
   }
+  return H2_OK;
+}
+
+// An array of a padded mixed factorization without its padding (4-byte
+// entries; a pivot sequence's rows renumbered: padding never swaps with a
+// logical row, as its entries beside the diagonal are zero).
+h2_status export_unpadded(const h2_ctx* c, const std::string& n, int level, const void* src, size_t cnt, char* dst,
+                          size_t cap, size_t* count, int32_t* elem_size) {
+  const DevLevel &g = c->lv[level], &d = c->pv[level];
+  // places of the logical indices: rows of the level's input blocks, columns
+  // of U (complement, then skeleton), complement and skeleton alone
+  std::vector<int> in, uc, rr, ss;
+  const PadSeg rs = row_seg(c, level);
+  for (int r = 0; r < d.D; ++r)
+    if (r % rs.str < rs.len) in.push_back(r);
+  for (int r = 0; r < g.R; ++r) uc.push_back(r), rr.push_back(r);
+  for (int k = 0; k < g.K; ++k) uc.push_back(d.R + k), ss.push_back(k);
+  const std::vector<int> one{0};
+  const std::vector<int>*rows, *cols;
+  size_t ld, blk;
+  if (n == "U") rows = &uc, cols = &in, ld = d.D, blk = (size_t)d.D * d.D;
+  else if (n == "Ahat") rows = cols = &uc, ld = d.D, blk = (size_t)d.D * d.D;
+  else if (n == "Ainv") rows = cols = &rr, ld = d.R, blk = (size_t)d.R * d.R;
+  else if (n == "Shat") rows = cols = &ss, ld = d.K, blk = (size_t)d.K * d.K;
+  else if (n == "A" || n == "root_inv") rows = cols = &in, ld = d.D, blk = (size_t)d.D * d.D;
+  else if (n == "piv") rows = &one, cols = &rr, ld = blk = d.R;
+  else if (n == "root_piv") rows = &one, cols = &in, ld = blk = d.D;
+  else return H2_ERR_INVALID_ARG;
+  const size_t nblk = blk ? cnt / blk : 0, per = rows->size() * cols->size();
+  *count = nblk * per;
+  *elem_size = 4;
+  if (!dst) return H2_OK;
+  if (!src) return H2_ERR_STATE;
+  if (cap < *count * 4) return H2_ERR_INVALID_ARG;
+  std::vector<int32_t> h(cnt);
+  if (cudaMemcpy(h.data(), src, cnt * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return H2_ERR_CUDA;
+  int32_t* out = reinterpret_cast<int32_t*>(dst);
+  for (size_t b = 0; b < nblk; ++b)
+    for (size_t r = 0; r < rows->size(); ++r)
+      for (size_t k = 0; k < cols->size(); ++k) {
+        int32_t v = h[b * blk + (size_t)(*rows)[r] * ld + (*cols)[k]];
+        if (n == "root_piv") v = (int32_t)(std::lower_bound(in.begin(), in.end(), v) - in.begin());
+        out[b * per + r * cols->size() + k] = v;
+      }
   return H2_OK;
 }
 
@@ -1391,7 +1524,7 @@ template <typename T, class Prec, class Mv>
 h2_status fgmres_cycle(h2_ctx* c, GmresWork& W, int m, double beta, const T* r, double tol_abs, T* V, T* Z, int& k,
                        int& its, Prec prec, Mv mv) {
   cudaStream_t st = c->stream;
-  const int64_t n = nslots(c);
+  const int64_t n = std::is_same<T, double>::value ? nslots(c) : nslots32(c);
   const int m0 = W.m0;
   launch_norm2<T>(r, n, W.nrm, st);
   launch_scaled_copy<T, T>(r, W.nrm, true, V, n, st);
@@ -1451,9 +1584,10 @@ h2_status gmres_work(h2_ctx* c, GmresWork& W) {
   if (c->gm_cap < m0) {
     CKC(dalloc(c, &c->gm_V, (size_t)(m0 + 1) * n));
     CKC(dalloc(c, &c->gm_Z, (size_t)m0 * n));
-    CKC(dalloc(c, &c->gm_V32, (size_t)(m0 + 1) * n));
-    CKC(dalloc(c, &c->gm_Z32, (size_t)m0 * n));
-    CKC(dalloc(c, &c->gm_r32, (size_t)n));
+    const int64_t n32 = nslots32(c);
+    CKC(dalloc(c, &c->gm_V32, (size_t)(m0 + 1) * n32));
+    CKC(dalloc(c, &c->gm_Z32, (size_t)m0 * n32));
+    CKC(dalloc(c, &c->gm_r32, (size_t)n32));
     CKC(dalloc(c, &c->gm_h, 3 * (size_t)(m0 + 2) + 257));
     if (c->gm_host) cudaFreeHost(c->gm_host);
     CKC(cudaMallocHost(&c->gm_host, (2 * (size_t)(m0 + 2) + 1) * sizeof(double)));
@@ -1541,14 +1675,14 @@ h2_status nested_refine(h2_ctx* c, SolveTimer& tm, double bnorm, double target, 
   auto mv = [&](const float* z, float* w) { tm.run(tm.mv32, [&] { matvec32(c, z, w, &tm.leaf32); }); };
   while (its < max_iters && (target <= 0 || beta > target * bnorm)) {
     launch_norm2<double>(c->r64, n, c->red, st);
-    launch_scaled_copy<double, float>(c->r64, c->red, true, c->gm_r32, n, st);
+    launch_pad_scaled_copy(c->r64, c->red, c->gm_r32, n, leaf_seg(c), st);
     const double tol_in = std::max(c->inner_tol, target > 0 ? 0.5 * target * bnorm / beta : 0.0);
     int k = 0;
     CKS(fgmres_cycle<float>(c, W, std::min(W.m0, max_iters - its), 1.0, c->gm_r32, tol_in, c->gm_V32, c->gm_Z32, k,
                             its, prec, mv));
     for (int i = 0; i < k; ++i) W.y[i] *= beta;
     CKC(cudaMemcpyAsync(W.yv, W.y.data(), k * sizeof(double), cudaMemcpyHostToDevice, st));
-    launch_multi_axpy<float, double>(c->gm_Z32, n, k, W.yv, 1.0, c->x64, n, st);
+    launch_pad_axpy(c->gm_Z32, nslots32(c), k, W.yv, c->x64, n, leaf_seg(c), st);
     CKS(fp64_residual(c, tm, beta, !c->resid64));
     rel = beta / bnorm;
     c->times.history.push_back(rel);
@@ -2118,12 +2252,12 @@ h2_status h2_matvec_arith(h2_ctx* c, const double* x, double* y, int32_t arith) 
     matvec_df(c, c->x64, c->y64);
   } else {
     if (!c->mv32_x) {
-      CKC(dalloc(c, &c->mv32_x, (size_t)n));
-      CKC(dalloc(c, &c->mv32_y, (size_t)n));
+      CKC(dalloc(c, &c->mv32_x, (size_t)nslots32(c)));
+      CKC(dalloc(c, &c->mv32_y, (size_t)nslots32(c)));
     }
-    launch_convert<double, float>(c->x64, c->mv32_x, n, c->stream);
+    launch_split_df(c->x64, c->mv32_x, c->xdf_l, n, leaf_seg(c), c->stream);
     matvec32(c, c->mv32_x, c->mv32_y);
-    launch_convert<float, double>(c->mv32_y, c->y64, n, c->stream);
+    launch_unpad(c->mv32_y, c->y64, n, leaf_seg(c), c->stream);
   }
   CKC(cudaGetLastError());
   CKS(vec_out(c, c->y64, y));
@@ -2522,11 +2656,13 @@ h2_status h2_export(const h2_ctx* c, const char* name, int32_t level, void* dst,
     return H2_OK;
   }
   if (level < 0 || level > c->L) return H2_ERR_INVALID_ARG;
-  const DevLevel& d = c->lv[level];
+  const bool f64 = c->prec == H2_PREC_FP64;
+  // a mixed factorization's arrays may be padded; what leaves is not
+  const DevLevel& g = c->lv[level];
+  const DevLevel& d = (f64 || n == "X" || n == "T" || (n == "A" && level == c->L)) ? g : c->pv[level];
   const void* src = nullptr;
   size_t cnt = 0;
   int es = 8;
-  const bool f64 = c->prec == H2_PREC_FP64;
   const bool ready = factor_ready(c);
   auto pick = [&](const void* p64, const void* p32, size_t k, bool need_factor) -> h2_status {
     if (need_factor && !ready) return H2_ERR_STATE;
@@ -2566,7 +2702,7 @@ h2_status h2_export(const h2_ctx* c, const char* name, int32_t level, void* dst,
     cnt = (n == "lu") ? nb * R * R : nb * R;
   } else if (n == "root" || n == "root_piv" || n == "root_inv") {
     if (!ready) return H2_ERR_STATE;
-    const size_t D0 = c->lv[0].D, nr = c->lv[0].nb;  // nr roots (one per system of a forest)
+    const size_t D0 = d.D, nr = d.nb;  // nr roots (one per system of a forest)
     if (n == "root" && !f64) return H2_ERR_INVALID_ARG;  // as for "lu"
     if (n == "root") {
       src = f64 ? (const void*)c->f64.root_lu : (const void*)c->f32.root_luT;
@@ -2583,6 +2719,7 @@ h2_status h2_export(const h2_ctx* c, const char* name, int32_t level, void* dst,
     return H2_ERR_INVALID_ARG;
   }
   if (s != H2_OK) return s;
+  if (d.D != g.D || d.K != g.K) return export_unpadded(c, n, level, src, cnt, static_cast<char*>(dst), cap_bytes, count, elem_size);
   *count = cnt;
   *elem_size = es;
   if (dst) {

@@ -162,6 +162,21 @@ GpuCompressor* make_gpu_compressor(const KernelFn& G, const double* pts, int64_t
 // ---------------------------------------------------------------------------
 // Device-side state.
 // ---------------------------------------------------------------------------
+// One stored block of a symmetric pair (a, b): an n x n block at element
+// offset m of the block array, the two boxes' slices of the input vector at
+// xa and xb, its partial products [M x_b; M^T x_a] at offset p.
+struct SymPair {
+  int64_t m, p;
+  int32_t xa, xb, n, pad;
+};
+
+// Where the entries of a logical vector or block lie in its padded form:
+// segments of len entries (a leaf's points, or one child's skeletons) at a
+// stride of str.
+struct PadSeg {
+  int len, str;
+};
+
 struct DevLevel {
   int nb = 0, D = 0, K = 0, R = 0;
   int64_t NP = 0, FP = 0;
@@ -186,17 +201,21 @@ struct DevLevel {
   int64_t* SK = nullptr;  // nb * K
   double* S = nullptr;    // FP * K * K couplings G(SK_i, SK_j)
   float* X32 = nullptr;   // FP32 copies for the inner solver of the mixed refinement
+  float* X32q = nullptr;  // the unpadded FP32 bases (X32 itself without padding): the QR's input
   float* S32 = nullptr;
   // symmetric coupling storage for the FP32 matvec (S_ji = S_ij^T): the far
-  // pairs i < j ("stored"), their FP32 couplings, and per box the list of
-  // partial products (2k: S_k xh_j for i = box, 2k + 1: S_k^T xh_i for
-  // j = box), CSR over boxes
-  bool far_sym = false;
+  // pairs i < j ("stored"; their blocks lie in h2_ctx::S32u_all), and per box
+  // the list of partial products (2k: S_k xh_j for i = box, 2k + 1:
+  // S_k^T xh_i for j = box), CSR over boxes; fs_poff: where the level's
+  // partial products start in h2_ctx::part32c
   int64_t fpu = 0;
-  int64_t fs_goff = 0;  // first index of this level's stored pairs in the all-level batch
-  int32_t *fs_i = nullptr, *fs_j = nullptr, *fs_ent = nullptr;
+  int64_t fs_poff = 0;
+  int32_t* fs_ent = nullptr;
   int64_t* fs_ptr = nullptr;
-  float* S32u = nullptr;
+  // symmetric far list: the pairs i < j (fu_*) and the others with their mirrors
+  bool far_mirrored = false;
+  int64_t n_fu = 0;
+  int32_t *fu_q = nullptr, *fu_i = nullptr, *fu_j = nullptr, *fl_q = nullptr, *fl_m = nullptr;
   void* S16[2] = {nullptr, nullptr};        // couplings scaled into FP16 [0] / BF16 [1]
   float* S16_scale[2] = {nullptr, nullptr};  // their scale and inverse scale (device)
   // symmetric near list (pair (j, i) present for every (i, j)): the pairs
@@ -219,6 +238,7 @@ struct FacLevel {
   T* Vq = nullptr;     // nb * D * K   Householder reflectors (column-major, unit diagonal)
   T* tau = nullptr;    // nb * K
   T* Tw = nullptr;     // nb * K * K   compact-WY triangular factor
+  T* Tp = nullptr;     // nb * Kp * Kp Tm with zero padding (Tm itself without padding)
   T* Qs = nullptr;     // nb * D * K   panel scratch when it does not fit in shared memory
   T* Ain = nullptr;    // NP * D * D   input near blocks of this level (row-major)
   T* Ahat = nullptr;   // NP * D * D   projected blocks (row-major)
@@ -309,6 +329,11 @@ struct h2_ctx {
   h2::KernelFn kfn{};
   h2::HostH2 host;
   std::vector<h2::DevLevel> lv;
+  // The levels as the FP32 arrays hold them: the same lists, with D, K and R
+  // padded to multiples of 4 where no level fits the tensor-core shapes (see
+  // padded_dims); equal to lv otherwise.  hat_off32: as hat_off.
+  std::vector<h2::DevLevel> pv;
+  std::vector<int64_t> hat_off32;
   int L = 0;
   int64_t N = 0;
   int dev = 0;
@@ -342,7 +367,7 @@ struct h2_ctx {
   int32_t *sym_q = nullptr, *sym_i = nullptr, *sym_j = nullptr, *sym_ent = nullptr;
   int64_t* sym_ptr = nullptr;
   float* part32 = nullptr;   // npu * 2 D partial products (FP32 matvec)
-  float* part32c = nullptr;  // cb_n * 2 cb_K coupling partial products (beside the leaf's)
+  float* part32c = nullptr;  // coupling partial products of every level (beside the leaf's)
   // the FP32 matvec's leaf near field runs on leaf_stream beside the passes
   // through the bases (created on first use), forked and joined by events
   cudaStream_t leaf_stream = nullptr;
@@ -352,13 +377,13 @@ struct h2_ctx {
   // basis coefficients xhat, yhat of all levels, as FP32 pairs
   float *xdf_h = nullptr, *xdf_l = nullptr, *hdf_h = nullptr, *hdf_l = nullptr, *ydf_h = nullptr, *ydf_l = nullptr;
   float *xhat32 = nullptr, *yhat32 = nullptr;
-  // the stored coupling pairs of every level as one batch (levels with the
-  // same rank cb_K): the FP32 matvec forms all levels' coupling products in
-  // one launch; cb_i / cb_j index K-slots of xhat32
+  // the stored coupling pairs of every level as one batch: the FP32 matvec
+  // forms all levels' coupling products in one launch (cb: one descriptor per
+  // pair; cb_max the largest rank)
   bool cb_ok = false;
-  int cb_K = 0;
+  int cb_max = 0;
   int64_t cb_n = 0;
-  int32_t *cb_i = nullptr, *cb_j = nullptr;
+  h2::SymPair *sym_desc = nullptr, *cb = nullptr;
   float* S32u_all = nullptr;
   std::vector<double*> X64p, S64p;  // per-level pointers (index l; [0] unused)
   std::vector<float*> X32p, S32p;

@@ -50,8 +50,10 @@ template <typename T>
 void launch_perm_identity(int nb, int D, int K, T* U, cudaStream_t st);
 // U = [Q[:, K:] Q[:, :K]], Q = I - W1 V^T (W1 D x K row-major, V D x K
 // column-major), as column-major U, row-major Ur and 16-bit U16 (NULL: none)
+// (any D, K; with padding, Dp and Kp > their logical sizes, rs: where the
+// logical rows lie; the padding itself is launch_form_u_pads')
 void launch_form_u(int64_t nb, int D, int K, const float* W1, const float* V, float* U, float* Ur, void* u16,
-                   int bf16, cudaStream_t st);
+                   int bf16, int Dp, int Kp, PadSeg rs, cudaStream_t st);
 template <typename T>
 void launch_lu_inverse(int nb, int D, int R, const T* Ablk, const int32_t* diag_idx, double* lu, T* luT,
                        int32_t* piv, T* Ainv, int32_t* status, int level, cudaStream_t st);
@@ -183,13 +185,14 @@ void launch_matvec_leaf_df(const DevLevel& L, const float* Ah, const float* Al, 
 // leaf, symmetric storage: y_i = X_i yhat_i + box i's partial products
 void launch_matvec_sym_sum_df(int nb, int D, int K, const int64_t* ptr, const int32_t* ent, const float* Xh,
                               const float* Xl, const float* yhh, const float* yhl, const float* ph, const float* pl,
-                              double* y, cudaStream_t st);
-void launch_split_lo(const double* a, const float* hi, float* lo, int64_t n, cudaStream_t st);  // lo = fl32(a - hi)
-void launch_split_df(const double* v, float* h, float* l, int64_t n, cudaStream_t st);  // h = fl32(v), l = fl32(v - h)
+                              double* y, int ny, cudaStream_t st);  // ny: rows of a box in y (the rest is padding)
+// h = fl32(v), l = fl32(v - h); v has n entries in segments of p.len, h and l
+// nb segments of p.str (the rest zero)
+void launch_split_df(const double* v, float* h, float* l, int64_t n, PadSeg p, cudaStream_t st);
 // Leaf matvec on the stored (i <= j) halves of symmetric leaf near blocks:
 // per stored pair k = (ui[k], uj[k]) the partial products [A x_j; A^T x_i]
 // into part (2 D per pair), then per box y = X yh + its partial products.
-bool sym_leaf_supported(int D);  // D = 128 or 256
+bool sym_supported(int n);  // n a multiple of 4, at most 256
 // Downward step [yh_2p; yh_2p+1] = X_p yh_p + (the children's coupling
 // products summed over their CSR lists cptr / cent into part, Kc = D / 2
 // entries per product; cptr NULL: none)
@@ -197,18 +200,25 @@ template <typename T>
 void launch_matvec_down_far(const DevLevel& L, const T* X, const T* yh, T* yh_child, const int64_t* cptr,
                             const int32_t* cent, const T* part, cudaStream_t st);
 // (pdl: launched to overlap its predecessor; off where events bracket it)
-void launch_matvec_sym_pairs(int D, int64_t npu, const int32_t* ui, const int32_t* uj, const float* A, const float* x,
-                             float* part, bool pdl, cudaStream_t st);
-void launch_matvec_sym_pairs_df(int D, int64_t npu, const int32_t* ui, const int32_t* uj, const float* Ah,
-                                const float* Al, const float* xh, const float* xl, float* ph, float* pl,
-                                cudaStream_t st);
+// (max_n: the largest block, a multiple of 4 up to 256)
+void launch_matvec_sym_pairs(int max_n, int64_t npu, const SymPair* desc, const float* A, const float* x, float* part,
+                             bool pdl, cudaStream_t st);
+void launch_matvec_sym_pairs_df(int D, int64_t npu, const SymPair* desc, const float* Ah, const float* Al,
+                                const float* xh, const float* xl, float* ph, float* pl, cudaStream_t st);
 template <typename T>
 void launch_matvec_sym_sum(int nb, int D, int K, const int64_t* ptr, const int32_t* ent, const T* X, const T* yh,
                            const T* part, T* y, cudaStream_t st, bool pdl = true);
-// out[k] = fl32(in[idx[k]]), lo[k] = fl32(in[idx[k]] - hi[k]) for blocks of n entries
-void launch_gather_blocks(const double* in, const int32_t* idx, int64_t n, int64_t nblk, float* out, cudaStream_t st);
-void launch_gather_split_lo(const double* in, const int32_t* idx, int64_t n, int64_t nblk, const float* hi, float* lo,
-                            cudaStream_t st);
+// FP32 copies of nblk blocks (block k from in[idx[k]], or in[k]): a block of
+// rows x cols entries whose logical rows and columns lie at rs and cs, zeros
+// elsewhere; hi = fl32(v) and, lo non-NULL, lo = fl32(v - hi).  di / dj
+// non-NULL: blocks with di[k] == dj[k] get 1 on the padding's diagonal.
+template <typename Ti>
+void launch_pad_blocks(const Ti* in, const int32_t* idx, int64_t nblk, int rows, PadSeg rs, int cols, PadSeg cs,
+                       float* hi, float* lo, const int32_t* di, const int32_t* dj, cudaStream_t st);
+// the padding's part of U and Ur (zeros, and one 1 per padding row and
+// column) for D x D blocks with R complement columns, of which Rl and Kl
+// columns and the rows at rs are logical
+void launch_form_u_pads(int64_t nb, int D, int R, int Rl, int Kl, PadSeg rs, float* U, float* Ur, cudaStream_t st);
 
 void launch_gather(const int64_t* slot, const double* src, double* dst, int64_t nslots, cudaStream_t st);
 void launch_scatter(const int64_t* slot, const double* src, double* dst, int64_t nslots, cudaStream_t st);
@@ -217,10 +227,16 @@ template <typename T>
 void launch_norm2(const T* v, int64_t n, double* out, cudaStream_t st);  // out[0] = sum v^2 (FP64), out[1..256] scratch
 template <typename Ti, typename To>
 void launch_scaled_copy(const Ti* in, const double* nrm2, bool inverse, To* out, int64_t n, cudaStream_t st);
+// (the FP32 vectors of the next three have padded boxes: segment p)
+void launch_pad_scaled_copy(const double* in, const double* nrm2, float* out, int64_t n, PadSeg p, cudaStream_t st);
 template <typename T>
-void launch_scale_to(const double* in, const double* norm2, T* out, int64_t n, cudaStream_t st);
+void launch_scale_to(const double* in, const double* norm2, T* out, int64_t n, PadSeg p, cudaStream_t st);
 template <typename T>
-void launch_axpy_from(const T* d, const double* norm2, double* x, int64_t n, cudaStream_t st);
+void launch_axpy_from(const T* d, const double* norm2, double* x, int64_t n, PadSeg p, cudaStream_t st);
+// x += sum_v coef[v] V_v for padded FP32 vectors V_v, ldv apart
+void launch_pad_axpy(const float* V, int64_t ldv, int nv, const double* coef, double* x, int64_t n, PadSeg p,
+                     cudaStream_t st);
+void launch_unpad(const float* in, double* out, int64_t n, PadSeg p, cudaStream_t st);
 // GMRES: out[v] (+)= V_v . w for v < nv (part: nv * 128 scratch); w += sign sum_v coef[v] V_v;
 // w = src / sqrt(nrm2[0])
 template <typename T>

@@ -196,7 +196,11 @@ gemm_batched_kernel(int M, int N, int K, const T* __restrict__ A, int64_t sA, co
 // each holding an 8 x 8 block of C (rows ty*4 + {0..3, 64..67}, columns
 // tx*4 + {0..3, 64..67}) so that every shared-memory read is a 16-byte
 // vector; the next k-slice is fetched into registers while the current one
-// is used, and two shared buffers leave one barrier per slice.
+// is used, and two shared buffers leave one barrier per slice.  Bound by the
+// FP32 pipe's issue: the products go two at a time through fma.rn.f32x2 (the
+// same roundings as two fmaf), 4000 products of 256 x 256 blocks in 2.66
+// instead of 3.18 ms (50 TFLOP/s).  Tiles fitted to the block (104 x 104 for
+// 200 x 200, 169 threads) measured the same as 128 x 128 ones.
 constexpr int G2_BM = 128, G2_BN = 128, G2_BK = 8, G2_LD = 132;
 
 __device__ __forceinline__ void g2_load_a(const float* __restrict__ Ab, int lda, int tA, int M, int K, int m0, int k0,
@@ -275,10 +279,11 @@ __device__ __forceinline__ void g2_mainloop(int M, int N, int K, const float* __
       *reinterpret_cast<float4*>(&Bsb[k][n]) = make_float4(rb[0], rb[1], rb[2], rb[3]);
     }
   };
+  uint64_t c2[8][4];  // pairs of neighbouring columns
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
+    for (int j = 0; j < 4; ++j) c2[i][j] = 0;
   float ra[4], rb[4];
   g2_load_a(Ab, lda, tA, M, K, m0, 0, vecA, ra);
   load_b(0, rb);
@@ -296,14 +301,17 @@ __device__ __forceinline__ void g2_mainloop(int M, int N, int K, const float* __
     for (int kk = 0; kk < G2_BK; ++kk) {
       const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
       const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4 + 64]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4 + 64]);
+      const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][tx * 4]);
+      const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][tx * 4 + 64]);
       const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      const uint64_t bv[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < 8; ++i) {
+        uint64_t aa;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(av[i]));
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c2[i][j]) : "l"(aa), "l"(bv[j]));
+      }
     }
     if (more) {
       g2_store_a(As[buf ^ 1], tA, ra);
@@ -312,6 +320,11 @@ __device__ __forceinline__ void g2_mainloop(int M, int N, int K, const float* __
     __syncthreads();
     buf ^= 1;
   }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[i][2 * j]), "=f"(acc[i][2 * j + 1]) : "l"(c2[i][j]));
 }
 
 template <typename TB>
@@ -362,13 +375,16 @@ gemm_f32_tile_kernel(int M, int N, int K, const float* __restrict__ A, int64_t s
 // row-major; V column-major D x K) and U = [Q[:, K:] Q[:, :K]] written three
 // ways: column-major U, row-major Ur and the 16-bit column-major copy U16
 // (u16 NULL: none).  Tiles and main loop of the tile GEMM; column n of Q is
-// column n - K of U for n >= K and n + R otherwise.  D and K are multiples
-// of 4, so each thread's 4 x 4 groups lie wholly inside or outside the
-// block and on one side of column K.
+// column n - K of U for n >= K and n + R otherwise.  VEC: D and K are
+// multiples of 4 and nothing is padded, so each thread's 4 x 4 groups lie
+// wholly inside or outside the block and on one side of column K and are
+// stored as vectors; otherwise entry by entry, row m at its place of rs and
+// U's columns behind Rp = Dp - Kp complement columns (no 16-bit copy).
+template <bool VEC>
 __global__ void __launch_bounds__(256, 2) form_u_kernel(int D, int K, const float* __restrict__ W1,
                                                         const float* __restrict__ V, float* __restrict__ U,
                                                         float* __restrict__ Ur, void* __restrict__ u16, int bf16,
-                                                        int64_t nb) {
+                                                        int64_t nb, int Dp, int Kp, PadSeg rs, int vecA, int vecB) {
   __shared__ __align__(16) float As[2][G2_BK][G2_LD];
   __shared__ __align__(16) float Bs[2][G2_BK][G2_LD];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -378,7 +394,27 @@ __global__ void __launch_bounds__(256, 2) form_u_kernel(int D, int K, const floa
     const float* Ab = W1 + b * (int64_t)D * K;
     const float* Bb = V + b * (int64_t)D * K;  // V^T row-major K x D
     float acc[8][8];
-    g2_mainloop<float>(D, D, K, Ab, K, 0, Bb, D, 0, m0, n0, 1, 1, As, Bs, acc);
+    g2_mainloop<float>(D, D, K, Ab, K, 0, Bb, D, 0, m0, n0, vecA, vecB, As, Bs, acc);
+    if constexpr (!VEC) {
+      float* Uo = U + b * (int64_t)Dp * Dp;
+      float* Uro = Ur + b * (int64_t)Dp * Dp;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int m = m0 + ty * 4 + (i & 3) + (i >> 2) * 64;
+        if (m >= D) continue;
+        const int mp = m / rs.len * rs.str + m % rs.len;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int n = n0 + tx * 4 + (j & 3) + (j >> 2) * 64;
+          if (n >= D) continue;
+          const int cp = n >= K ? n - K : Dp - Kp + n;
+          const float q = (m == n ? 1.0f : 0.0f) - acc[i][j];
+          Uo[(int64_t)cp * Dp + mp] = q;
+          Uro[(int64_t)mp * Dp + cp] = q;
+        }
+      }
+      continue;
+    }
     float* Ub = U + b * (int64_t)D * D;
     float* Urb = Ur + b * (int64_t)D * D;
     uint16_t* U16b = u16 ? reinterpret_cast<uint16_t*>(u16) + b * (int64_t)D * D : nullptr;
@@ -424,11 +460,14 @@ __global__ void __launch_bounds__(256, 2) form_u_kernel(int D, int K, const floa
   }
 }
 void launch_form_u(int64_t nb, int D, int K, const float* W1, const float* V, float* U, float* Ur, void* u16,
-                   int bf16, cudaStream_t st) {
+                   int bf16, int Dp, int Kp, PadSeg rs, cudaStream_t st) {
   if (nb == 0 || D == 0) return;
   dim3 g((D + G2_BN - 1) / G2_BN, (D + G2_BM - 1) / G2_BM, (unsigned)std::min<int64_t>(nb, 65535));
   ++g_launches;
-  form_u_kernel<<<g, 256, 0, st>>>(D, K, W1, V, U, Ur, u16, bf16, nb);
+  if (D % 4 == 0 && K % 4 == 0 && Dp == D)
+    form_u_kernel<true><<<g, 256, 0, st>>>(D, K, W1, V, U, Ur, u16, bf16, nb, Dp, Kp, rs, 1, 1);
+  else
+    form_u_kernel<false><<<g, 256, 0, st>>>(D, K, W1, V, U, Ur, nullptr, bf16, nb, Dp, Kp, rs, K % 4 == 0, D % 4 == 0);
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }

@@ -1842,17 +1842,35 @@ void launch_matvec_leaf_df(const DevLevel& L, const float* Ah, const float* Al, 
   mv_leaf_df_kernel<<<L.nb, 256, sm, st>>>(L.D, L.K, L.near_ptr, L.near_j, Ah, Al, Xh, Xl, xh, xl, yhh, yhl, y);
 }
 
+// An FP32 vector of padded boxes: entry e of its nb * p.str entries is entry
+// pad_index(p, e) of the logical vector, or padding (-1).
+__device__ __forceinline__ int64_t pad_index(PadSeg p, int64_t e) {
+  if (p.len == p.str) return e;
+  const uint32_t box = (uint32_t)e / (uint32_t)p.str, r = (uint32_t)e - box * (uint32_t)p.str;
+  return r < (uint32_t)p.len ? (int64_t)box * p.len + r : -1;
+}
+// where entry e of the logical vector lies in the padded one
+__device__ __forceinline__ int64_t padded_at(PadSeg p, int64_t e) {
+  return p.len == p.str ? e : e + (int64_t)((uint32_t)e / (uint32_t)p.len) * (p.str - p.len);
+}
+static int64_t padded_size(PadSeg p, int64_t n) { return p.len ? n / p.len * p.str : 0; }
+
 // h = fl32(v), l = fl32(v - h): an FP64 vector as FP32 pairs, once per use
 // of the vector rather than once per block that reads it
-__global__ void split_df_kernel(const double* __restrict__ v, float* __restrict__ h, float* __restrict__ l,
-                                int64_t n) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    df_split(v[e], h[e], l[e]);
+__global__ void split_df_kernel(const double* __restrict__ v, float* __restrict__ h, float* __restrict__ l, int64_t n,
+                                PadSeg p) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t g = pad_index(p, e);
+    float a = 0.0f, b = 0.0f;
+    if (g >= 0) df_split(v[g], a, b);
+    h[e] = a, l[e] = b;
+  }
 }
-void launch_split_df(const double* v, float* h, float* l, int64_t n, cudaStream_t st) {
+void launch_split_df(const double* v, float* h, float* l, int64_t n, PadSeg p, cudaStream_t st) {
   if (n <= 0) return;
+  const int64_t np = padded_size(p, n);
   ++g_launches;
-  split_df_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, st>>>(v, h, l, n);
+  split_df_kernel<<<(unsigned)std::min<int64_t>((np + 255) / 256, 152 * 8), 256, 0, st>>>(v, h, l, np, p);
 }
 
 // The residual's passes through the bases and couplings with every vector
@@ -2016,7 +2034,8 @@ __global__ void __launch_bounds__(256, 2) mv_sym_sum_df_kernel(int D, int K, con
                                                                const float* __restrict__ yhh,
                                                                const float* __restrict__ yhl,
                                                                const float* __restrict__ ph,
-                                                               const float* __restrict__ pl, double* __restrict__ y) {
+                                                               const float* __restrict__ pl, double* __restrict__ y,
+                                                               int ny) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int Kp = (K + 3) & ~3;
   float* shh = reinterpret_cast<float*>(smraw);  // Kp
@@ -2047,39 +2066,28 @@ __global__ void __launch_bounds__(256, 2) mv_sym_sum_df_kernel(int D, int K, con
       float th, tl;
       df_tsum<kRPWdf, 32>(H, L, th, tl);
       const int r = r0 + warp + 8 * tsum_index<kRPWdf, 32>(lane);
-      if (tsum_leader<kRPWdf, 32>(lane) && r < D) {
+      if (tsum_leader<kRPWdf, 32>(lane) && r < ny) {
         df_add(th, tl, sbh[r], sbl[r]);
-        y[(int64_t)i * D + r] = (double)th + (double)tl;
+        y[(int64_t)i * ny + r] = (double)th + (double)tl;
       }
     }
   } else {
-    for (int r = threadIdx.x; r < D; r += blockDim.x) y[(int64_t)i * D + r] = (double)sbh[r] + (double)sbl[r];
+    for (int r = threadIdx.x; r < ny; r += blockDim.x) y[(int64_t)i * ny + r] = (double)sbh[r] + (double)sbl[r];
   }
 }
 void launch_matvec_sym_sum_df(int nb, int D, int K, const int64_t* ptr, const int32_t* ent, const float* Xh,
                               const float* Xl, const float* yhh, const float* yhl, const float* ph, const float* pl,
-                              double* y, cudaStream_t st) {
+                              double* y, int ny, cudaStream_t st) {
   const size_t sm = sizeof(float) * (2 * (size_t)((K + 3) & ~3) + 2 * (size_t)D);
   ++g_launches;
-  mv_sym_sum_df_kernel<<<nb, 256, sm, st>>>(D, K, ptr, ent, Xh, Xl, yhh, yhl, ph, pl, y);
-}
-
-// lo[e] = fl32(a[e] - hi[e]) (hi = fl32(a))
-__global__ void split_lo_kernel(const double* __restrict__ a, const float* __restrict__ hi, float* __restrict__ lo,
-                                int64_t n) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    lo[e] = (float)(a[e] - (double)hi[e]);
-}
-void launch_split_lo(const double* a, const float* hi, float* lo, int64_t n, cudaStream_t st) {
-  if (n <= 0) return;
-  ++g_launches;
-  split_lo_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 32), 256, 0, st>>>(a, hi, lo, n);
+  mv_sym_sum_df_kernel<<<nb, 256, sm, st>>>(D, K, ptr, ent, Xh, Xl, yhh, yhl, ph, pl, y, ny);
 }
 
 // -------------------------------------------- symmetric leaf near blocks ---
-// The leaf near blocks of a symmetric kernel satisfy A_ji = A_ij^T, so the
-// inner solver's matvec keeps only the blocks with i <= j ("stored pairs")
-// and reads each once: the CTA of stored pair k = (a, b) forms
+// The blocks of a symmetric kernel satisfy A_ji = A_ij^T, so the inner
+// solver's matvec keeps only the leaf near blocks with i <= j and the
+// couplings with i < j ("stored pairs", n x n with n a multiple of 4 up to
+// 256) and reads each once: the CTA of stored pair k = (a, b) forms
 // u = A_ab x_b (for box a) and, when a != b, w = A_ab^T x_a (for box b)
 // into part[k] = [u; w]; a per-box kernel then adds y_i = X_i yh_i + the
 // partial products of the box (listed in ent: 2k for a u, 2k + 1 for a w).
@@ -2089,26 +2097,28 @@ void launch_split_lo(const double* a, const float* hi, float* lo, int64_t n, cud
 // memory.
 constexpr int kSymRPW = 8;  // rows per warp in flight
 
-template <int CH>  // 4-column chunks per lane: D = 128 CH
-__global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(int D, int64_t npu, const int32_t* __restrict__ ui,
-                                                             const int32_t* __restrict__ uj,
+template <int CH>  // 4-column chunks per lane: n <= 128 CH
+__global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __restrict__ desc,
                                                              const float* __restrict__ A, const float* __restrict__ x,
                                                              float* __restrict__ part, int pf) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  float* xa = reinterpret_cast<float*>(smraw);  // D
-  float* wp = xa + D;                           // 8 * D
-  const int64_t k = blockIdx.x;
-  const int a = ui[k], b = uj[k], tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool both = a != b;
-  const float* M = A + k * D * D;
-  if (pf) prefetch_l2(M, (int64_t)D * D * sizeof(float));
+  const SymPair ds = desc[blockIdx.x];
+  const int n = ds.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* xa = reinterpret_cast<float*>(smraw);  // n
+  float* wp = xa + n;                           // 8 * n
+  const bool both = ds.xa != ds.xb;
+  const float* M = A + ds.m;
+  if (pf) prefetch_l2(M, (int64_t)n * n * sizeof(float));
   griddep_wait();
   griddep_launch_next();
-  for (int e = tid; e < D; e += blockDim.x) xa[e] = x[(int64_t)a * D + e];
+  for (int e = tid; e < n; e += blockDim.x) xa[e] = x[ds.xa + e];
+  bool in[CH];
   float xb[CH][4];
 #pragma unroll
   for (int h = 0; h < CH; ++h) {
-    const float4 v = *reinterpret_cast<const float4*>(x + (int64_t)b * D + lane * 4 + 128 * h);
+    const int c = lane * 4 + 128 * h;
+    in[h] = c < n;
+    const float4 v = in[h] ? *reinterpret_cast<const float4*>(x + ds.xb + c) : make_float4(0.f, 0.f, 0.f, 0.f);
     xb[h][0] = v.x, xb[h][1] = v.y, xb[h][2] = v.z, xb[h][3] = v.w;
   }
   float wacc[CH][4];
@@ -2117,22 +2127,22 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(int D, int64_t npu,
 #pragma unroll
     for (int e = 0; e < 4; ++e) wacc[h][e] = 0.0f;
   __syncthreads();
-  float* u = part + k * 2 * D;
-  for (int r0 = warp; r0 < D; r0 += 8 * kSymRPW) {
+  float* u = part + ds.p;
+  for (int r0 = warp; r0 < n; r0 += 8 * kSymRPW) {
     float4 v[kSymRPW][CH];
 #pragma unroll
     for (int t = 0; t < kSymRPW; ++t) {
       const int r = r0 + 8 * t;
 #pragma unroll
       for (int h = 0; h < CH; ++h)
-        v[t][h] = (r < D) ? __ldg(reinterpret_cast<const float4*>(M + (int64_t)r * D + lane * 4 + 128 * h))
-                          : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[t][h] = (r < n && in[h]) ? __ldg(reinterpret_cast<const float4*>(M + (int64_t)r * n + lane * 4 + 128 * h))
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     float su[kSymRPW];
 #pragma unroll
     for (int t = 0; t < kSymRPW; ++t) {
       const int r = r0 + 8 * t;
-      const float xr = (r < D) ? xa[r] : 0.0f;
+      const float xr = (r < n) ? xa[r] : 0.0f;
       float s = 0.0f;
 #pragma unroll
       for (int h = 0; h < CH; ++h) {
@@ -2150,20 +2160,21 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(int D, int64_t npu,
     {
       const float sv = tsum<kSymRPW, 32, float>(su);
       const int r = r0 + 8 * tsum_index<kSymRPW, 32>(lane);
-      if (tsum_leader<kSymRPW, 32>(lane) && r < D) u[r] = sv;
+      if (tsum_leader<kSymRPW, 32>(lane) && r < n) u[r] = sv;
     }
   }
   if (!both) return;
 #pragma unroll
   for (int h = 0; h < CH; ++h)
-    *reinterpret_cast<float4*>(wp + warp * D + lane * 4 + 128 * h) =
-        make_float4(wacc[h][0], wacc[h][1], wacc[h][2], wacc[h][3]);
+    if (in[h])
+      *reinterpret_cast<float4*>(wp + warp * n + lane * 4 + 128 * h) =
+          make_float4(wacc[h][0], wacc[h][1], wacc[h][2], wacc[h][3]);
   __syncthreads();
-  for (int c = tid; c < D; c += blockDim.x) {
+  for (int c = tid; c < n; c += blockDim.x) {
     float s = 0.0f;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) s += wp[w * D + c];
-    u[D + c] = s;
+    for (int w = 0; w < 8; ++w) s += wp[w * n + c];
+    u[n + c] = s;
   }
 }
 
@@ -2216,8 +2227,7 @@ __global__ void __launch_bounds__(256) mv_sym_sum_kernel(int D, int K, const int
 // (lane k keeps the row of pass k mod 16 and half k / 16) stores it after
 // the last pass; the column sums of A^T x_i are added over the warps.
 template <int CH>
-__global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(int D, int64_t npu, const int32_t* __restrict__ ui,
-                                                                const int32_t* __restrict__ uj,
+__global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(const SymPair* __restrict__ desc,
                                                                 const float* __restrict__ Ah,
                                                                 const float* __restrict__ Al,
                                                                 const float* __restrict__ xh,
@@ -2225,21 +2235,24 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(int D, int64_t n
                                                                 float* __restrict__ ph, float* __restrict__ pl) {
   constexpr int RPW = 2;
   extern __shared__ __align__(16) unsigned char smraw[];
+  const SymPair ds = desc[blockIdx.x];
+  const int D = ds.n;
   float* xah = reinterpret_cast<float*>(smraw);  // D
   float* xal = xah + D;                          // D
   float* wph = xal + D;                          // 8 * D column partials (high parts)
   float* wpl = wph + 8 * D;                      // 8 * D (low parts)
-  const int64_t k = blockIdx.x;
-  const int a = ui[k], b = uj[k], tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool both = a != b;
-  const float* Mh = Ah + k * D * D;
-  const float* Ml = Al + k * D * D;
-  for (int e = tid; e < D; e += blockDim.x) xah[e] = xh[(int64_t)a * D + e], xal[e] = xl[(int64_t)a * D + e];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool both = ds.xa != ds.xb;
+  const float* Mh = Ah + ds.m;
+  const float* Ml = Al + ds.m;
+  for (int e = tid; e < D; e += blockDim.x) xah[e] = xh[ds.xa + e], xal[e] = xl[ds.xa + e];
+  bool in[CH];
   float xbh[CH][4], xbl[CH][4];
 #pragma unroll
   for (int h = 0; h < CH; ++h) {
-    const float4 vh = *reinterpret_cast<const float4*>(xh + (int64_t)b * D + lane * 4 + 128 * h);
-    const float4 vl = *reinterpret_cast<const float4*>(xl + (int64_t)b * D + lane * 4 + 128 * h);
+    in[h] = lane * 4 + 128 * h < D;
+    const float4 vh = in[h] ? *reinterpret_cast<const float4*>(xh + ds.xb + lane * 4 + 128 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 vl = in[h] ? *reinterpret_cast<const float4*>(xl + ds.xb + lane * 4 + 128 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
     xbh[h][0] = vh.x, xbh[h][1] = vh.y, xbh[h][2] = vh.z, xbh[h][3] = vh.w;
     xbl[h][0] = vl.x, xbl[h][1] = vl.y, xbl[h][2] = vl.z, xbl[h][3] = vl.w;
   }
@@ -2249,8 +2262,8 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(int D, int64_t n
 #pragma unroll
     for (int e = 0; e < 4; ++e) wH[h][e] = 0.0f, wL[h][e] = 0.0f;
   __syncthreads();
-  float* uh = ph + k * 2 * D;
-  float* ul = pl + k * 2 * D;
+  float* uh = ph + ds.p;
+  float* ul = pl + ds.p;
   // rows r0 + 8 t (t < RPW) of this warp; the next group's loads are issued
   // before the current group is used
   auto load_rows = [&](int r0, float4 (&vh)[RPW][CH], float4 (&vl)[RPW][CH]) {
@@ -2260,8 +2273,8 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(int D, int64_t n
 #pragma unroll
       for (int h = 0; h < CH; ++h) {
         const int64_t off = (int64_t)r * D + lane * 4 + 128 * h;
-        vh[t][h] = (r < D) ? __ldg(reinterpret_cast<const float4*>(Mh + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        vl[t][h] = (r < D) ? __ldg(reinterpret_cast<const float4*>(Ml + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        vh[t][h] = (r < D && in[h]) ? __ldg(reinterpret_cast<const float4*>(Mh + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        vl[t][h] = (r < D && in[h]) ? __ldg(reinterpret_cast<const float4*>(Ml + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
   };
@@ -2305,7 +2318,7 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(int D, int64_t n
 #pragma unroll
   for (int h = 0; h < CH; ++h)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
+    for (int e = 0; e < 4 && in[h]; ++e) {
       wph[warp * D + lane * 4 + 128 * h + e] = wH[h][e];
       wpl[warp * D + lane * 4 + 128 * h + e] = wL[h][e];
     }
@@ -2318,48 +2331,33 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(int D, int64_t n
   }
 }
 
-bool sym_leaf_supported(int D) { return D == 128 || D == 256; }
+bool sym_supported(int n) { return n > 0 && n % 4 == 0 && n <= 256; }
 
 template <int CH>
-static void launch_sym_pairs_ch(int D, int64_t npu, const int32_t* ui, const int32_t* uj, const float* A,
-                                const float* x, float* part, bool pdl, cudaStream_t st) {
-  const size_t sm = sizeof(float) * 9 * (size_t)D;
-  set_smem((const void*)mv_sym_pair_kernel<CH>, sm);
+static void launch_sym_pairs_ch(int n, int64_t npu, const SymPair* desc, const float* A, const float* x, float* part,
+                                bool pdl, cudaStream_t st) {
+  const size_t sm = sizeof(float) * 9 * (size_t)n;
   const int pf = small_level(npu) ? 1 : 0;
   if (pdl) {
-    launch_pdl(mv_sym_pair_kernel<CH>, (unsigned)npu, 256, sm, st, D, npu, ui, uj, A, x, part, pf);
+    launch_pdl(mv_sym_pair_kernel<CH>, (unsigned)npu, 256, sm, st, desc, A, x, part, pf);
   } else {
     ++g_launches;
-    mv_sym_pair_kernel<CH><<<(unsigned)npu, 256, sm, st>>>(D, npu, ui, uj, A, x, part, pf);
+    mv_sym_pair_kernel<CH><<<(unsigned)npu, 256, sm, st>>>(desc, A, x, part, pf);
   }
 }
-void launch_matvec_sym_pairs(int D, int64_t npu, const int32_t* ui, const int32_t* uj, const float* A, const float* x,
-                             float* part, bool pdl, cudaStream_t st) {
+void launch_matvec_sym_pairs(int max_n, int64_t npu, const SymPair* desc, const float* A, const float* x, float* part,
+                             bool pdl, cudaStream_t st) {
   if (npu <= 0) return;
-  switch (D / 128) {
-    case 1: launch_sym_pairs_ch<1>(D, npu, ui, uj, A, x, part, pdl, st); break;
-    case 2: launch_sym_pairs_ch<2>(D, npu, ui, uj, A, x, part, pdl, st); break;
-    default: launch_sym_pairs_ch<2>(D, npu, ui, uj, A, x, part, pdl, st); break;
-  }
+  if (max_n <= 128) launch_sym_pairs_ch<1>(max_n, npu, desc, A, x, part, pdl, st);
+  else launch_sym_pairs_ch<2>(max_n, npu, desc, A, x, part, pdl, st);
 }
-template <int CH>
-static void launch_sym_pairs_df_ch(int D, int64_t npu, const int32_t* ui, const int32_t* uj, const float* Ah,
-                                   const float* Al, const float* xh, const float* xl, float* ph, float* pl,
-                                   cudaStream_t st) {
+void launch_matvec_sym_pairs_df(int D, int64_t npu, const SymPair* desc, const float* Ah, const float* Al,
+                                const float* xh, const float* xl, float* ph, float* pl, cudaStream_t st) {
+  if (npu <= 0) return;
   const size_t sm = sizeof(float) * 18 * (size_t)D;
-  set_smem((const void*)mv_sym_pair_df_kernel<CH>, sm);
   ++g_launches;
-  mv_sym_pair_df_kernel<CH><<<(unsigned)npu, 256, sm, st>>>(D, npu, ui, uj, Ah, Al, xh, xl, ph, pl);
-}
-void launch_matvec_sym_pairs_df(int D, int64_t npu, const int32_t* ui, const int32_t* uj, const float* Ah,
-                                const float* Al, const float* xh, const float* xl, float* ph, float* pl,
-                                cudaStream_t st) {
-  if (npu <= 0) return;
-  switch (D / 128) {
-    case 1: launch_sym_pairs_df_ch<1>(D, npu, ui, uj, Ah, Al, xh, xl, ph, pl, st); break;
-    case 2: launch_sym_pairs_df_ch<2>(D, npu, ui, uj, Ah, Al, xh, xl, ph, pl, st); break;
-    default: launch_sym_pairs_df_ch<2>(D, npu, ui, uj, Ah, Al, xh, xl, ph, pl, st); break;
-  }
+  if (D <= 128) mv_sym_pair_df_kernel<1><<<(unsigned)npu, 256, sm, st>>>(desc, Ah, Al, xh, xl, ph, pl);
+  else mv_sym_pair_df_kernel<2><<<(unsigned)npu, 256, sm, st>>>(desc, Ah, Al, xh, xl, ph, pl);
 }
 template <typename T>
 void launch_matvec_sym_sum(int nb, int D, int K, const int64_t* ptr, const int32_t* ent, const T* X, const T* yh,
@@ -2375,37 +2373,74 @@ void launch_matvec_sym_sum(int nb, int D, int K, const int64_t* ptr, const int32
 template void launch_matvec_sym_sum<float>(int, int, int, const int64_t*, const int32_t*, const float*, const float*,
                                            const float*, float*, cudaStream_t, bool);
 
-// out[k] = (To) in[idx[k]] for blocks of n entries
-template <typename Ti, typename To>
-__global__ void gather_blocks_kernel(const Ti* __restrict__ in, const int32_t* __restrict__ idx, int64_t n,
-                                     int64_t nblk, To* __restrict__ out) {
-  const int64_t total = n * nblk;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t k = e / n, r = e - k * n;
-    out[e] = (To)in[(int64_t)idx[k] * n + r];
+// FP32 copies of blocks with their rows and columns at padded places: a warp
+// per padded row (see kernels.h).
+template <typename Ti>
+__global__ void __launch_bounds__(256) pad_blocks_kernel(const Ti* __restrict__ in, const int32_t* __restrict__ idx,
+                                                         int64_t nblk, int rows, PadSeg rs, int cols, PadSeg cs,
+                                                         float* __restrict__ hi, float* __restrict__ lo,
+                                                         const int32_t* __restrict__ di,
+                                                         const int32_t* __restrict__ dj) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int nrl = rows / rs.str * rs.len, ncl = cols / cs.str * cs.len;  // logical rows and columns
+  const int64_t total = nblk * rows;
+  for (int64_t w = blockIdx.x * (int64_t)nw + (threadIdx.x >> 5); w < total; w += (int64_t)gridDim.x * nw) {
+    const int64_t k = w / rows;
+    const int r = (int)(w - k * rows), rseg = r / rs.str, rr = r - rseg * rs.str;
+    const Ti* src = in + ((int64_t)(idx ? idx[k] : k) * nrl + rseg * rs.len + rr) * ncl;
+    const bool row_in = rr < rs.len;
+    const int64_t kk = idx ? idx[k] : k;
+    const bool unit = !row_in && di && di[kk] == dj[kk];
+    for (int c = lane; c < cols; c += 32) {
+      const int cseg = c / cs.str, cc = c - cseg * cs.str;
+      const double v = row_in && cc < cs.len ? (double)src[cseg * cs.len + cc] : (unit && c == r ? 1.0 : 0.0);
+      const float h = (float)v;
+      hi[w * cols + c] = h;
+      if (lo) lo[w * cols + c] = (float)(v - (double)h);
+    }
   }
 }
-void launch_gather_blocks(const double* in, const int32_t* idx, int64_t n, int64_t nblk, float* out, cudaStream_t st) {
-  if (n * nblk <= 0) return;
+template <typename Ti>
+void launch_pad_blocks(const Ti* in, const int32_t* idx, int64_t nblk, int rows, PadSeg rs, int cols, PadSeg cs,
+                       float* hi, float* lo, const int32_t* di, const int32_t* dj, cudaStream_t st) {
+  if (nblk <= 0 || rows <= 0 || cols <= 0) return;
+  const int64_t warps = nblk * rows;
   ++g_launches;
-  gather_blocks_kernel<double, float><<<(unsigned)std::min<int64_t>((n * nblk + 255) / 256, 152 * 32), 256, 0, st>>>(
-      in, idx, n, nblk, out);
+  pad_blocks_kernel<Ti><<<(unsigned)std::min<int64_t>((warps + 7) / 8, 152 * 32), 256, 0, st>>>(
+      in, idx, nblk, rows, rs, cols, cs, hi, lo, di, dj);
 }
-// lo[k] = fl32(in[idx[k]] - hi[k])
-__global__ void gather_split_lo_kernel(const double* __restrict__ in, const int32_t* __restrict__ idx, int64_t n,
-                                       int64_t nblk, const float* __restrict__ hi, float* __restrict__ lo) {
-  const int64_t total = n * nblk;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t k = e / n, r = e - k * n;
-    lo[e] = (float)(in[(int64_t)idx[k] * n + r] - (double)hi[e]);
+template void launch_pad_blocks<double>(const double*, const int32_t*, int64_t, int, PadSeg, int, PadSeg, float*, float*,
+                                        const int32_t*, const int32_t*, cudaStream_t);
+template void launch_pad_blocks<float>(const float*, const int32_t*, int64_t, int, PadSeg, int, PadSeg, float*, float*,
+                                       const int32_t*, const int32_t*, cudaStream_t);
+
+// The padding of U (column-major, U[c D + r]) and Ur (its row-major copy):
+// the t-th padding row meets the t-th padding column (R - Rl of them behind
+// the complement columns, then the rest behind the skeleton columns) in a 1,
+// the other entries of padding rows and columns are 0.  A warp per column.
+__global__ void __launch_bounds__(256) form_u_pads_kernel(int64_t nb, int D, int R, int Rl, int Kl, PadSeg rs,
+                                                          float* __restrict__ U, float* __restrict__ Ur) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5, pad = rs.str - rs.len;
+  for (int64_t w = blockIdx.x * (int64_t)nw + (threadIdx.x >> 5); w < nb * D; w += (int64_t)gridDim.x * nw) {
+    const int64_t b = w / D;
+    const int c = (int)(w - b * D);
+    const bool cpad = c < R ? c >= Rl : c - R >= Kl;
+    const int tc = c < R ? c - Rl : R - Rl + c - R - Kl;  // its number among the padding columns
+    for (int r = lane; r < D; r += 32) {
+      const int seg = r / rs.str, rr = r - seg * rs.str;
+      const bool rpad = rr >= rs.len;
+      if (!cpad && !rpad) continue;
+      const float v = cpad && rpad && seg * pad + rr - rs.len == tc ? 1.0f : 0.0f;
+      U[w * D + r] = v;
+      Ur[(b * D + r) * D + c] = v;
+    }
   }
 }
-void launch_gather_split_lo(const double* in, const int32_t* idx, int64_t n, int64_t nblk, const float* hi, float* lo,
-                            cudaStream_t st) {
-  if (n * nblk <= 0) return;
+void launch_form_u_pads(int64_t nb, int D, int R, int Rl, int Kl, PadSeg rs, float* U, float* Ur, cudaStream_t st) {
+  if (nb <= 0 || D <= 0) return;
   ++g_launches;
-  gather_split_lo_kernel<<<(unsigned)std::min<int64_t>((n * nblk + 255) / 256, 152 * 32), 256, 0, st>>>(in, idx, n,
-                                                                                                        nblk, hi, lo);
+  form_u_pads_kernel<<<(unsigned)std::min<int64_t>((nb * D + 7) / 8, 152 * 32), 256, 0, st>>>(nb, D, R, Rl, Kl, rs, U,
+                                                                                             Ur);
 }
 
 // ------------------------------------------------------------ vectors ---
@@ -2546,40 +2581,67 @@ void launch_scaled_copy(const Ti* in, const double* nrm2, bool inverse, To* out,
   ++g_launches;
   scaled_copy_kernel<Ti, To><<<grid_for(n), 256, 0, st>>>(in, nrm2, inverse ? 1 : 0, out, n);
 }
-template void launch_scaled_copy<double, float>(const double*, const double*, bool, float*, int64_t, cudaStream_t);
-template void launch_scaled_copy<float, double>(const float*, const double*, bool, double*, int64_t, cudaStream_t);
 template void launch_scaled_copy<float, float>(const float*, const double*, bool, float*, int64_t, cudaStream_t);
 template void launch_scaled_copy<double, double>(const double*, const double*, bool, double*, int64_t,
                                                  cudaStream_t);
 template <typename T>
-__global__ void scale_to_kernel(const double* __restrict__ in, const double* __restrict__ nrm2, T* __restrict__ out,
-                                int64_t n) {
+__global__ void scale_to_kernel(const double* __restrict__ in, const double* __restrict__ nrm2, double zero, T* __restrict__ out,
+                                int64_t n, PadSeg p) {
   __shared__ double ss;
-  if (threadIdx.x == 0) ss = nrm2[0] > 0 ? 1.0 / sqrt(nrm2[0]) : 1.0;
+  if (threadIdx.x == 0) ss = nrm2[0] > 0 ? 1.0 / sqrt(nrm2[0]) : zero;
   __syncthreads();
   const double s = ss;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    out[e] = (T)(in[e] * s);
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t g = pad_index(p, e);
+    out[e] = g >= 0 ? (T)(in[g] * s) : T(0);
+  }
 }
 template <typename T>
 __global__ void axpy_from_kernel(const T* __restrict__ d, const double* __restrict__ nrm2, double* __restrict__ x,
-                                 int64_t n) {
+                                 int64_t n, PadSeg p) {
   __shared__ double ss;
   if (threadIdx.x == 0) ss = nrm2[0] > 0 ? sqrt(nrm2[0]) : 1.0;
   __syncthreads();
   const double s = ss;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    x[e] += s * (double)d[e];
+    x[e] += s * (double)d[padded_at(p, e)];
 }
 template <typename T>
-void launch_scale_to(const double* in, const double* norm2, T* out, int64_t n, cudaStream_t st) {
+void launch_scale_to(const double* in, const double* norm2, T* out, int64_t n, PadSeg p, cudaStream_t st) {
   ++g_launches;
-  scale_to_kernel<T><<<grid_for(n), 256, 0, st>>>(in, norm2, out, n);
+  scale_to_kernel<T><<<grid_for(padded_size(p, n)), 256, 0, st>>>(in, norm2, 1.0, out, padded_size(p, n), p);
+}
+void launch_pad_scaled_copy(const double* in, const double* nrm2, float* out, int64_t n, PadSeg p, cudaStream_t st) {
+  ++g_launches;
+  scale_to_kernel<float><<<grid_for(padded_size(p, n)), 256, 0, st>>>(in, nrm2, 0.0, out, padded_size(p, n), p);
 }
 template <typename T>
-void launch_axpy_from(const T* d, const double* norm2, double* x, int64_t n, cudaStream_t st) {
+void launch_axpy_from(const T* d, const double* norm2, double* x, int64_t n, PadSeg p, cudaStream_t st) {
   ++g_launches;
-  axpy_from_kernel<T><<<grid_for(n), 256, 0, st>>>(d, norm2, x, n);
+  axpy_from_kernel<T><<<grid_for(n), 256, 0, st>>>(d, norm2, x, n, p);
+}
+__global__ void pad_axpy_kernel(const float* __restrict__ V, int64_t ldv, int nv, const double* __restrict__ coef,
+                                double* __restrict__ x, int64_t n, PadSeg p) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t g = padded_at(p, e);
+    double s = 0;
+    for (int v = 0; v < nv; ++v) s = fma(coef[v], (double)V[(int64_t)v * ldv + g], s);
+    x[e] += s;
+  }
+}
+void launch_pad_axpy(const float* V, int64_t ldv, int nv, const double* coef, double* x, int64_t n, PadSeg p,
+                     cudaStream_t st) {
+  if (nv == 0) return;
+  ++g_launches;
+  pad_axpy_kernel<<<grid_for(n), 256, 0, st>>>(V, ldv, nv, coef, x, n, p);
+}
+__global__ void unpad_kernel(const float* __restrict__ in, double* __restrict__ out, int64_t n, PadSeg p) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
+    out[e] = (double)in[padded_at(p, e)];
+}
+void launch_unpad(const float* in, double* out, int64_t n, PadSeg p, cudaStream_t st) {
+  ++g_launches;
+  unpad_kernel<<<grid_for(n), 256, 0, st>>>(in, out, n, p);
 }
 // ---------------------------------------------------------- GMRES blocks ---
 // part[v * nblk + blk] = partial sums of V_v . w (FP64); out[v] (+)= the sum
@@ -2686,12 +2748,10 @@ template void launch_multi_axpy<double, double>(const double*, int64_t, int, con
                                                 cudaStream_t);
 template void launch_multi_axpy<float, float>(const float*, int64_t, int, const double*, double, float*, int64_t,
                                               cudaStream_t);
-template void launch_multi_axpy<float, double>(const float*, int64_t, int, const double*, double, double*, int64_t,
-                                               cudaStream_t);
 
-template void launch_scale_to<double>(const double*, const double*, double*, int64_t, cudaStream_t);
-template void launch_scale_to<float>(const double*, const double*, float*, int64_t, cudaStream_t);
-template void launch_axpy_from<double>(const double*, const double*, double*, int64_t, cudaStream_t);
-template void launch_axpy_from<float>(const float*, const double*, double*, int64_t, cudaStream_t);
+template void launch_scale_to<double>(const double*, const double*, double*, int64_t, PadSeg, cudaStream_t);
+template void launch_scale_to<float>(const double*, const double*, float*, int64_t, PadSeg, cudaStream_t);
+template void launch_axpy_from<double>(const double*, const double*, double*, int64_t, PadSeg, cudaStream_t);
+template void launch_axpy_from<float>(const float*, const double*, double*, int64_t, PadSeg, cudaStream_t);
 
 }  // namespace h2
