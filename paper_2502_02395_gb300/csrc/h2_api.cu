@@ -5,6 +5,7 @@
 #include <cstring>
 #include <map>
 #include <sstream>
+#include <thread>
 
 #include "h2_internal.h"
 #include "kernels.h"
@@ -1085,14 +1086,30 @@ void ulv_sweep(h2_ctx* c, Factor<T>& F) {
     }
     return ch;
   };
+  // levels of few boxes: a pair step and the per-box step after it in one
+  // launch (thread-block clusters)
+  std::vector<char> cl(L + 2, 0);
+  for (int l = 1; l <= L; ++l)
+    with_ahat(F.lv[l], F.bf16, [&](auto A, const float*) {
+      using TS = std::remove_const_t<std::remove_pointer_t<decltype(A)>>;
+      cl[l] = subst_clustered<T, TS>(LV[l], A);
+    });
   auto fwd = [&](int l) {
     const DevLevel& d = LV[l];
     FacLevel<T>& f = F.lv[l];
-    launch_fwd1<T>(d, f, child_in(l), st);
+    if (!cl[l + 1]) launch_fwd1<T>(d, f, child_in(l), st);
     with_ahat(f, F.bf16, [&](auto A, const float* isc) {
       using TS = std::remove_const_t<std::remove_pointer_t<decltype(A)>>;
-      launch_fwd2<T, TS>(d, f, A, isc, st);
-      launch_fwd3<T, TS>(d, f, A, isc, l == 1 ? F.root_vec : nullptr, st);
+      if (cl[l]) {
+        launch_cl_fwd2<T, TS>(d, f, A, isc, st);
+        FacLevel<T>& pf = F.lv[l - 1];
+        const int D1 = LV[l - 1].D;
+        if (l > 1) launch_cl_up<T, TS>(d, f, A, isc, D1, LV[l - 1].R, pf.M1, pf.U, pf.u, pf.c, st);
+        else launch_cl_up<T, TS>(d, f, A, isc, D1, D1, F.root_inv, nullptr, F.root_x, nullptr, st);
+      } else {
+        launch_fwd2<T, TS>(d, f, A, isc, st);
+        launch_fwd3<T, TS>(d, f, A, isc, l == 1 ? F.root_vec : nullptr, st);
+      }
     });
   };
   auto bwd = [&](int l) {
@@ -1101,12 +1118,17 @@ void ulv_sweep(h2_ctx* c, Factor<T>& F) {
     const T* px = (l > 1) ? F.lv[l - 1].xs : F.root_x;
     with_ahat(f, F.bf16, [&](auto A, const float* isc) {
       using TS = std::remove_const_t<std::remove_pointer_t<decltype(A)>>;
-      launch_bwd1<T, TS>(d, f, A, isc, px, st);
-      launch_bwd2<T, TS>(d, f, A, isc, px, st);
+      if (cl[l]) {
+        launch_cl_bwd1<T, TS>(d, f, A, isc, px, st);
+        launch_cl_bwd2<T, TS>(d, f, A, isc, px, st);
+      } else {
+        launch_bwd1<T, TS>(d, f, A, isc, px, st);
+        launch_bwd2<T, TS>(d, f, A, isc, px, st);
+      }
     });
   };
   for (int l = L; l >= 1; --l) fwd(l);
-  launch_gemv_rows<T>(LV[0].nb, LV[0].D, F.root_inv, F.root_vec, F.root_x, st);
+  if (!cl[1]) launch_gemv_rows<T>(LV[0].nb, LV[0].D, F.root_inv, F.root_vec, F.root_x, st);
   for (int l = 1; l <= L; ++l) bwd(l);
 }
 template <typename T>
@@ -1134,36 +1156,63 @@ void ulv_apply_impl(h2_ctx* c, Factor<T>& F, const double* r, double* x) {
 }
 
 // Capture fn's work on the context's stream into a CUDA graph (on a private
-// capture stream); nullptr if the capture or instantiation fails, in which
-// case the caller runs fn directly.
+// capture stream); nothing if the capture or instantiation fails.
 template <class Fn>
-cudaGraphExec_t capture_graph(h2_ctx* c, long long& kernels, Fn fn) {
+KernelGraph capture_graph(h2_ctx* c, Fn fn) {
+  KernelGraph out;
   if (!c->cap_stream && cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
-    return nullptr;
+    return out;
   }
   cudaStream_t keep = c->stream;
   c->stream = c->cap_stream;
   cudaGraph_t g = nullptr;
-  cudaGraphExec_t ex = nullptr;
   const long long n0 = g_launches.load();
   if (cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
     fn();
     if (cudaStreamEndCapture(c->cap_stream, &g) == cudaSuccess && g) {
-      if (cudaGraphInstantiate(&ex, g, 0) != cudaSuccess) ex = nullptr;
+      if (cudaGraphInstantiate(&out.ex, g, 0) != cudaSuccess) out.ex = nullptr;
     }
   }
-  kernels = g_launches.load() - n0;
-  g_launches -= kernels;  // counted again per replay
+  out.kernels = g_launches.load() - n0;
+  g_launches -= out.kernels;  // counted again per replay
   if (g) cudaGraphDestroy(g);
   c->stream = keep;
   cudaGetLastError();
-  return ex;
+  return out;
 }
 
 void drop_graphs(h2_ctx* c) {
-  if (c->g_ulv) cudaGraphExecDestroy(c->g_ulv);
-  c->g_ulv = nullptr;
+  for (KernelGraph* g : {&c->g_ulv, &c->g_start, &c->g_iter, &c->g_resid}) {
+    if (g->ex) cudaGraphExecDestroy(g->ex);
+    *g = KernelGraph();
+  }
+}
+
+// Graphs captured under other settings than the present ones are dropped: the
+// operand type of the 16-bit arrays and the process-wide launch options of the
+// substitution (the buffers they read and write are dropped with them).
+void check_graphs(h2_ctx* c) {
+  const long long key = (c->f32.bf16 + 1) + 4 * (g_box_stream.load() + 3 * (g_pair_ctas_per_sm.load() +
+                        4 * (g_box_ctas_per_sm.load() + 16ll * ((c->resid64 ? 1 : 0) + 2 * c->restart))));
+  if (key != c->graph_key) {
+    if (c->graph_key >= 0 && cudaStreamSynchronize(c->stream) != cudaSuccess) cudaGetLastError();
+    drop_graphs(c);
+  }
+  c->graph_key = key;
+}
+
+// fn's launches as a replay of graph g (captured now if it is not there yet),
+// or as plain launches where graphs are off or cannot be captured
+template <class Fn>
+void run_graph(h2_ctx* c, KernelGraph& g, Fn fn) {
+  if (c->use_graphs && !g.ex) g = capture_graph(c, fn);
+  if (c->use_graphs && g.ex) {
+    cudaGraphLaunch(g.ex, c->stream);
+    g_launches += g.kernels;
+  } else {
+    fn();
+  }
 }
 
 // z = ULV^-1 v for FP32 tree vectors (mixed-precision factorization); the
@@ -1171,14 +1220,9 @@ void drop_graphs(h2_ctx* c) {
 void ulv_apply_f32(h2_ctx* c, const float* v, float* z) {
   const int64_t n = nslots32(c);
   Factor<float>& F = c->f32;
+  check_graphs(c);
   cudaMemcpyAsync(ulv_in(c, F), v, n * sizeof(float), cudaMemcpyDeviceToDevice, c->stream);
-  if (c->use_graphs && !c->g_ulv) c->g_ulv = capture_graph(c, c->g_ulv_kernels, [&] { ulv_sweep<float>(c, F); });
-  if (c->use_graphs && c->g_ulv) {
-    cudaGraphLaunch(c->g_ulv, c->stream);
-    g_launches += c->g_ulv_kernels;
-  } else {
-    ulv_sweep<float>(c, F);
-  }
+  run_graph(c, c->g_ulv, [&] { ulv_sweep<float>(c, F); });
   cudaMemcpyAsync(z, ulv_out(c, F), n * sizeof(float), cudaMemcpyDeviceToDevice, c->stream);
 }
 
@@ -1188,11 +1232,22 @@ void ulv_apply_f32(h2_ctx* c, const float* v, float* z) {
 // ---------------------------------------------------------------------------
 using EventPairs = std::vector<std::pair<cudaEvent_t, cudaEvent_t>>;
 
+// the FP32 matvec's second stream and its fork and join events
+void matvec_streams(h2_ctx* c) {
+  if (c->leaf_stream) return;
+  cudaStreamCreateWithFlags(&c->leaf_stream, cudaStreamNonBlocking);
+  cudaEventCreateWithFlags(&c->mv_fork, cudaEventDisableTiming);
+  cudaEventCreateWithFlags(&c->mv_join, cudaEventDisableTiming);
+}
+// whether the FP32 matvec runs on the stored halves (leaf products on the
+// second stream, all couplings in one launch)
+bool matvec32_sym(const h2_ctx* c) { return c->cb_ok && c->sym && c->L >= 1; }
+
 // y = A_H2 x; with leaf_ev set, the leaf-level kernel (near blocks plus the
 // leaf basis) is bracketed by a pair of events appended there.
 template <typename T>
 void matvec_t(h2_ctx* c, const T* A, T* const* X, T* const* S, T* xh, T* yh, const T* x, T* y,
-              EventPairs* leaf_ev = nullptr) {
+              EventPairs* leaf_ev = nullptr, unsigned long long* stamp = nullptr) {
   const int L = c->L;
   const std::vector<DevLevel>& LV = levels<T>(c);
   cudaStream_t st = c->stream;
@@ -1224,22 +1279,18 @@ void matvec_t(h2_ctx* c, const T* A, T* const* X, T* const* S, T* xh, T* yh, con
   }
   const std::vector<int64_t>& off = std::is_same<T, double>::value ? c->hat_off : c->hat_off32;
   if constexpr (std::is_same<T, float>::value) {
-    if (c->cb_ok && c->sym) {
+    if (matvec32_sym(c)) {
       // the leaf near-field products need only x: they run on the leaf
       // stream beside the upward pass, the couplings (every level in one
       // launch) and the downward pass, which adds each level's coupling
       // sums as it goes; the per-box leaf sums follow the join
-      if (!c->leaf_stream) {
-        cudaStreamCreateWithFlags(&c->leaf_stream, cudaStreamNonBlocking);
-        cudaEventCreateWithFlags(&c->mv_fork, cudaEventDisableTiming);
-        cudaEventCreateWithFlags(&c->mv_join, cudaEventDisableTiming);
-      }
+      matvec_streams(c);
       cudaStream_t sl = c->leaf_stream;
       const DevLevel& lf = LV[L];
       cudaEventRecord(c->mv_fork, st);
       cudaStreamWaitEvent(sl, c->mv_fork, 0);
       if (leaf_ev) cudaEventRecord(e0, sl);
-      launch_matvec_sym_pairs(lf.D, c->npu, c->sym_desc, A, x, c->part32, false, sl);
+      launch_matvec_sym_pairs(lf.D, c->npu, c->sym_desc, A, x, c->part32, false, sl, c->gm_state, stamp);
       if (leaf_ev) cudaEventRecord(e1, sl), leaf_ev->push_back({e0, e1});
       cudaEventRecord(c->mv_join, sl);
       launch_matvec_up<T>(LV[L], X[L], x, xh + off[L], st);
@@ -1337,8 +1388,8 @@ void matvec_df(h2_ctx* c, const double* x, double* y) {
                           yhh, yhl, y, st);
   }
 }
-void matvec32(h2_ctx* c, const float* x, float* y, EventPairs* leaf_ev = nullptr) {
-  matvec_t<float>(c, c->A32, c->X32p.data(), c->S32p.data(), c->xhat32, c->yhat32, x, y, leaf_ev);
+void matvec32(h2_ctx* c, const float* x, float* y, EventPairs* leaf_ev = nullptr, unsigned long long* stamp = nullptr) {
+  matvec_t<float>(c, c->A32, c->X32p.data(), c->S32p.data(), c->xhat32, c->yhat32, x, y, leaf_ev, stamp);
 }
 
 // The substitution's TMA-fed kernels set status[3] when a bounded wait
@@ -1458,6 +1509,8 @@ void ulv_apply_any(h2_ctx* c, const double* r, double* x) {
 struct SolveTimer {
   using Pairs = EventPairs;
   Pairs sub, mv, mv32, leaf32;  // leaf32: the leaf kernel inside each FP32 matvec
+  double sub_s = 0, mv32_s = 0, leaf_s = 0;  // the same from device time stamps (inner iterations as graphs)
+  int stamped = 0;                           // iterations they cover
   cudaStream_t st;
   explicit SolveTimer(cudaStream_t s) : st(s) {}
   template <class Fn>
@@ -1520,6 +1573,37 @@ struct GmresWork {
   std::vector<double> Hm, cs, sn, g, y;
 };
 
+// Column j of the Hessenberg matrix (h = a1 + a2 and ||w||^2 = nw2) through
+// the Givens rotations; whether the cycle stops after it.
+bool givens_step(GmresWork& W, int j, const double* a1, const double* a2, double nw2, double tol_abs) {
+  double* col = &W.Hm[(size_t)j * (W.m0 + 1)];
+  for (int i = 0; i <= j; ++i) col[i] = a1[i] + a2[i];
+  col[j + 1] = std::sqrt(nw2);
+  for (int i = 0; i < j; ++i) {
+    double t = W.cs[i] * col[i] + W.sn[i] * col[i + 1];
+    col[i + 1] = -W.sn[i] * col[i] + W.cs[i] * col[i + 1];
+    col[i] = t;
+  }
+  double d = std::hypot(col[j], col[j + 1]);
+  W.cs[j] = d > 0 ? col[j] / d : 1.0;
+  W.sn[j] = d > 0 ? col[j + 1] / d : 0.0;
+  col[j] = d;
+  col[j + 1] = 0.0;
+  W.g[j + 1] = -W.sn[j] * W.g[j];
+  W.g[j] = W.cs[j] * W.g[j];
+  if (!std::isfinite(W.g[j + 1])) return true;
+  if (tol_abs > 0 && std::fabs(W.g[j + 1]) <= tol_abs) return true;
+  return nw2 == 0.0;  // invariant Krylov space: exact solution
+}
+// y of the k-column least-squares problem
+void solve_triangle(GmresWork& W, int k) {
+  for (int i = k - 1; i >= 0; --i) {
+    double t = W.g[i];
+    for (int q = i + 1; q < k; ++q) t -= W.Hm[(size_t)q * (W.m0 + 1) + i] * W.y[q];
+    W.y[i] = t / W.Hm[(size_t)i * (W.m0 + 1) + i];
+  }
+}
+
 template <typename T, class Prec, class Mv>
 h2_status fgmres_cycle(h2_ctx* c, GmresWork& W, int m, double beta, const T* r, double tol_abs, T* V, T* Z, int& k,
                        int& its, Prec prec, Mv mv) {
@@ -1549,49 +1633,41 @@ h2_status fgmres_cycle(h2_ctx* c, GmresWork& W, int m, double beta, const T* r, 
     const double* a1 = W.host;
     const double* a2 = W.host + (m0 + 2);
     const double nw2 = W.host[2 * (m0 + 2)];
-    double* col = &W.Hm[(size_t)j * (m0 + 1)];
-    for (int i = 0; i <= j; ++i) col[i] = a1[i] + a2[i];
-    col[j + 1] = std::sqrt(nw2);
-    for (int i = 0; i < j; ++i) {
-      double t = W.cs[i] * col[i] + W.sn[i] * col[i + 1];
-      col[i + 1] = -W.sn[i] * col[i] + W.cs[i] * col[i + 1];
-      col[i] = t;
-    }
-    double d = std::hypot(col[j], col[j + 1]);
-    W.cs[j] = d > 0 ? col[j] / d : 1.0;
-    W.sn[j] = d > 0 ? col[j + 1] / d : 0.0;
-    col[j] = d;
-    col[j + 1] = 0.0;
-    W.g[j + 1] = -W.sn[j] * W.g[j];
-    W.g[j] = W.cs[j] * W.g[j];
     ++its;
     k = j + 1;
-    if (!std::isfinite(W.g[j + 1])) break;
-    if (tol_abs > 0 && std::fabs(W.g[j + 1]) <= tol_abs) break;
-    if (nw2 == 0.0) break;  // invariant Krylov space: exact solution
+    if (givens_step(W, j, a1, a2, nw2, tol_abs)) break;
   }
-  for (int i = k - 1; i >= 0; --i) {
-    double t = W.g[i];
-    for (int q = i + 1; q < k; ++q) t -= W.Hm[(size_t)q * (m0 + 1) + i] * W.y[q];
-    W.y[i] = t / W.Hm[(size_t)i * (m0 + 1) + i];
-  }
+  solve_triangle(W, k);
   return H2_OK;
 }
 
+// The pinned block (8-byte slots): h1 (m0 + 2), h2 (m0 + 2) and ||w||^2, the
+// residual's norm, k and y of the update, the iteration count, a cycle's times.
+size_t slot_rn(int m0) { return 2 * (size_t)(m0 + 2) + 1; }
+size_t slot_y(int m0) { return slot_rn(m0) + 1; }
+size_t slot_flag(int m0) { return slot_y(m0) + m0 + 8; }
+size_t slot_stamp(int m0) { return slot_flag(m0) + 8; }
+size_t host_slots(int m0) { return slot_stamp(m0) + kGmStamps * (size_t)(m0 + 1); }
+
 h2_status gmres_work(h2_ctx* c, GmresWork& W) {
   const int m0 = std::max(1, c->restart);
-  const int64_t n = nslots(c);
   if (c->gm_cap < m0) {
-    CKC(dalloc(c, &c->gm_V, (size_t)(m0 + 1) * n));
-    CKC(dalloc(c, &c->gm_Z, (size_t)m0 * n));
     const int64_t n32 = nslots32(c);
     CKC(dalloc(c, &c->gm_V32, (size_t)(m0 + 1) * n32));
     CKC(dalloc(c, &c->gm_Z32, (size_t)m0 * n32));
     CKC(dalloc(c, &c->gm_r32, (size_t)n32));
-    CKC(dalloc(c, &c->gm_h, 3 * (size_t)(m0 + 2) + 257));
+    CKC(dalloc(c, &c->gm_h, 3 * (size_t)(m0 + 2) + 258));
+    drop_graphs(c);  // (they hold the old buffers)
     if (c->gm_host) cudaFreeHost(c->gm_host);
-    CKC(cudaMallocHost(&c->gm_host, (2 * (size_t)(m0 + 2) + 1) * sizeof(double)));
-    CKC(dalloc(c, &c->gm_part, (size_t)(m0 + 1) * 128));
+    c->gm_host = nullptr;
+    CKC(cudaMallocHost(&c->gm_host, host_slots(m0) * sizeof(double)));
+    std::memset(c->gm_host, 0, host_slots(m0) * sizeof(double));
+    CKC(dalloc(c, &c->gm_part, (size_t)(2 * (m0 + 1) + 1) * kOrthCtas));
+    CKC(dalloc(c, &c->gm_w32, (size_t)n32));
+    CKC(dalloc(c, &c->gm_state, 1));
+    CKC(dalloc(c, &c->gm_stamp, (size_t)kGmStamps * (m0 + 2)));
+    CKC(cudaMemset(c->gm_state, 0, sizeof(GmState)));
+    c->gm_seq = 0;
     c->gm_cap = m0;
   }
   W.m0 = m0;
@@ -1635,6 +1711,11 @@ h2_status gmres_refine(h2_ctx* c, SolveTimer& tm, double bnorm, double target, i
   GmresWork W;
   CKS(gmres_work(c, W));
   const int64_t n = nslots(c);
+  if (c->gm_cap64 < W.m0) {
+    CKC(dalloc(c, &c->gm_V, (size_t)(W.m0 + 1) * n));
+    CKC(dalloc(c, &c->gm_Z, (size_t)W.m0 * n));
+    c->gm_cap64 = W.m0;
+  }
   double beta = bnorm;
   rel = 1.0;
   auto prec = [&](const double* v, double* z) {
@@ -1658,6 +1739,99 @@ h2_status gmres_refine(h2_ctx* c, SolveTimer& tm, double bnorm, double target, i
   return H2_OK;
 }
 
+// Wait until the device has reported inner iteration seq (it writes the count
+// to pinned memory after the iteration's numbers).  Polling sees it a few
+// microseconds earlier than a stream synchronization would; a stream that has
+// become idle or failed without reporting ends the wait.
+h2_status wait_iteration(h2_ctx* c, int m0, unsigned long long seq) {
+  const unsigned long long* flag = reinterpret_cast<const unsigned long long*>(c->gm_host + slot_flag(m0));
+  for (unsigned n = 1;; ++n) {
+    if (__atomic_load_n(flag, __ATOMIC_ACQUIRE) >= seq) return H2_OK;
+    if (n % 512 == 0) {
+      const cudaError_t e = cudaStreamQuery(c->stream);
+      if (e != cudaErrorNotReady) {
+        if (__atomic_load_n(flag, __ATOMIC_ACQUIRE) >= seq) return H2_OK;
+        c->err = std::string("an inner iteration ended without its result: ") + cudaGetErrorString(e);
+        return H2_ERR_CUDA;
+      }
+      std::this_thread::yield();
+    }
+  }
+}
+
+// One inner FGMRES cycle of the nested refinement on r64 / ||r64||: the same
+// method as fgmres_cycle, each iteration one graph replay (substitution, A z,
+// the vector work; launch gaps of some 4 us between 30 to 100 short kernels
+// were half of an iteration at 16384 points), the iteration's index on the
+// device, its numbers in pinned memory.
+h2_status inner_cycle(h2_ctx* c, GmresWork& W, SolveTimer& tm, int m, double tol_abs, int& k, int& its) {
+  const int m0 = W.m0;
+  Factor<float>& F = c->f32;
+  OrthArgs oa{};
+  oa.V = c->gm_V32, oa.Z = c->gm_Z32, oa.w = c->gm_w32, oa.vin = ulv_in(c, F), oa.xs = ulv_out(c, F);
+  oa.n = nslots32(c), oa.m0 = m0, oa.ctas = orth_ctas(oa.n);
+  oa.part = W.part, oa.h = W.h1, oa.state = c->gm_state, oa.stamp = c->gm_stamp;
+  oa.host = c->gm_host;
+  oa.flag = reinterpret_cast<unsigned long long*>(c->gm_host + slot_flag(m0));
+  run_graph(c, c->g_start, [&] {
+    launch_norm2<double>(c->r64, nslots(c), c->red, c->stream);
+    launch_pad_scaled_copy(c->r64, c->red, c->gm_r32, nslots(c), leaf_seg(c), c->stream);
+    launch_norm2<float>(c->gm_r32, oa.n, W.nrm, c->stream);
+    launch_gm_start(c->gm_r32, W.nrm, oa.V, oa.vin, oa.n, m0, oa.state, oa.stamp, c->stream);
+  });
+  std::fill(W.g.begin(), W.g.end(), 0.0);
+  W.g[0] = 1.0;
+  k = 0;
+  for (int j = 0; j < m; ++j) {
+    run_graph(c, c->g_iter, [&] {
+      ulv_sweep<float>(c, F);
+      matvec32(c, oa.xs, oa.w, nullptr, oa.stamp);
+      launch_orth(oa, c->stream);
+    });
+    CKC(cudaGetLastError());
+    CKS(wait_iteration(c, m0, ++c->gm_seq));
+    ++its;
+    k = j + 1;
+    if (givens_step(W, j, c->gm_host, c->gm_host + m0 + 2, c->gm_host[2 * (m0 + 2)], tol_abs)) break;
+  }
+  solve_triangle(W, k);
+  tm.stamped += k;
+  return H2_OK;
+}
+
+// x64 += beta Z y, the residual r64 = b - A x64 and its norm, and the cycle's
+// times.
+h2_status inner_update(h2_ctx* c, GmresWork& W, SolveTimer& tm, int k, double& beta) {
+  const int m0 = W.m0;
+  const int64_t n = nslots(c);
+  double* y = c->gm_host + slot_y(m0);
+  y[0] = k;
+  for (int i = 0; i < k; ++i) y[1 + i] = W.y[i] * beta;
+  tm.run(tm.mv, [&] {
+    run_graph(c, c->g_resid, [&] {
+      cudaStream_t st = c->stream;
+      cudaMemcpyAsync(W.yv, y, (m0 + 1) * sizeof(double), cudaMemcpyHostToDevice, st);
+      launch_pad_axpy_dev(c->gm_Z32, nslots32(c), W.yv, c->x64, n, leaf_seg(c), st);
+      if (c->resid64) matvec_impl(c, c->x64, c->y64);
+      else matvec_df(c, c->x64, c->y64);
+      launch_residual(c->b64, c->y64, c->r64, n, st);
+      launch_norm2<double>(c->r64, n, c->red + 600, st);
+      cudaMemcpyAsync(c->gm_host + slot_rn(m0), c->red + 600, sizeof(double), cudaMemcpyDeviceToHost, st);
+      cudaMemcpyAsync(c->gm_host + slot_stamp(m0), c->gm_stamp, kGmStamps * (size_t)(m0 + 1) * 8,
+                      cudaMemcpyDeviceToHost, st);
+    });
+  });
+  CKC(cudaStreamSynchronize(c->stream));
+  beta = std::sqrt(c->gm_host[slot_rn(m0)]);
+  const unsigned long long* t = reinterpret_cast<const unsigned long long*>(c->gm_host + slot_stamp(m0));
+  for (int i = 0; i < k; ++i, t += kGmStamps) {
+    tm.sub_s += 1e-9 * (double)(t[1] - t[0]);
+    tm.leaf_s += 1e-9 * (double)(t[3] - t[2]);
+    tm.mv32_s += 1e-9 * (double)(t[4] - t[1]);
+  }
+  return H2_OK;
+}
+
 // Mixed-precision refinement (for the FP32-storage factorizations): the
 // residual r = b - A_H2 x and the update x += d in FP64; each correction d
 // solves A d = r approximately by FGMRES in FP32, with the FP32 copy of
@@ -1671,19 +1845,29 @@ h2_status nested_refine(h2_ctx* c, SolveTimer& tm, double bnorm, double target, 
   cudaStream_t st = c->stream;
   double beta = bnorm;
   rel = 1.0;
+  const bool graphed = matvec32_sym(c);
+  if (graphed) {
+    matvec_streams(c);
+    check_graphs(c);
+  }
   auto prec = [&](const float* v, float* z) { tm.run(tm.sub, [&] { ulv_apply_f32(c, v, z); }); };
   auto mv = [&](const float* z, float* w) { tm.run(tm.mv32, [&] { matvec32(c, z, w, &tm.leaf32); }); };
   while (its < max_iters && (target <= 0 || beta > target * bnorm)) {
-    launch_norm2<double>(c->r64, n, c->red, st);
-    launch_pad_scaled_copy(c->r64, c->red, c->gm_r32, n, leaf_seg(c), st);
     const double tol_in = std::max(c->inner_tol, target > 0 ? 0.5 * target * bnorm / beta : 0.0);
+    const int m = std::min(W.m0, max_iters - its);
     int k = 0;
-    CKS(fgmres_cycle<float>(c, W, std::min(W.m0, max_iters - its), 1.0, c->gm_r32, tol_in, c->gm_V32, c->gm_Z32, k,
-                            its, prec, mv));
-    for (int i = 0; i < k; ++i) W.y[i] *= beta;
-    CKC(cudaMemcpyAsync(W.yv, W.y.data(), k * sizeof(double), cudaMemcpyHostToDevice, st));
-    launch_pad_axpy(c->gm_Z32, nslots32(c), k, W.yv, c->x64, n, leaf_seg(c), st);
-    CKS(fp64_residual(c, tm, beta, !c->resid64));
+    if (graphed) {
+      CKS(inner_cycle(c, W, tm, m, tol_in, k, its));
+      CKS(inner_update(c, W, tm, k, beta));
+    } else {
+      launch_norm2<double>(c->r64, n, c->red, st);
+      launch_pad_scaled_copy(c->r64, c->red, c->gm_r32, n, leaf_seg(c), st);
+      CKS(fgmres_cycle<float>(c, W, m, 1.0, c->gm_r32, tol_in, c->gm_V32, c->gm_Z32, k, its, prec, mv));
+      for (int i = 0; i < k; ++i) W.y[i] *= beta;
+      CKC(cudaMemcpyAsync(W.yv, W.y.data(), k * sizeof(double), cudaMemcpyHostToDevice, st));
+      launch_pad_axpy(c->gm_Z32, nslots32(c), k, W.yv, c->x64, n, leaf_seg(c), st);
+      CKS(fp64_residual(c, tm, beta, !c->resid64));
+    }
     rel = beta / bnorm;
     c->times.history.push_back(rel);
     if (!std::isfinite(rel)) break;
@@ -2003,7 +2187,6 @@ h2_status h2_factor(h2_ctx* c, int32_t prec) {
     return H2_ERR_STATE;
   }
   c->prec = -1;
-  drop_graphs(c);
   const bool fresh = (prec == H2_PREC_FP64) ? c->f64.lv.empty() : c->f32.lv.empty();
   if (fresh) CKS(check_fits(factor_bytes(c, prec == H2_PREC_FP64 ? 8 : 4), "the factorization", c->err));
   h2_status s = (prec == H2_PREC_FP64) ? factor_impl<double>(c, c->f64, prec) : factor_impl<float>(c, c->f32, prec);
@@ -2138,14 +2321,14 @@ h2_status h2_solve(h2_ctx* c, const double* b, double* x, double target, int32_t
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   c->times.solve_total = ms * 1e-3;
-  c->times.n_subst = (int)timer.sub.size();
+  c->times.n_subst = (int)timer.sub.size() + timer.stamped;
   c->times.n_matvec = (int)timer.mv.size();
-  c->times.n_matvec32 = (int)timer.mv32.size();
-  c->times.n_leaf32 = (int)timer.leaf32.size();
-  c->times.leaf32 = SolveTimer::total(timer.leaf32);
-  c->times.subst = SolveTimer::total(timer.sub);
+  c->times.n_matvec32 = (int)timer.mv32.size() + timer.stamped;
+  c->times.n_leaf32 = (int)timer.leaf32.size() + timer.stamped;
+  c->times.leaf32 = SolveTimer::total(timer.leaf32) + timer.leaf_s;
+  c->times.subst = SolveTimer::total(timer.sub) + timer.sub_s;
   c->times.matvec = SolveTimer::total(timer.mv);
-  c->times.matvec32 = SolveTimer::total(timer.mv32);  // the guard then finds the lists empty
+  c->times.matvec32 = SolveTimer::total(timer.mv32) + timer.mv32_s;  // the guard then finds the lists empty
   c->times.iters = it;
   c->times.relres = rel;
   if (relres_out) *relres_out = rel;
@@ -2286,7 +2469,7 @@ h2_status h2_autotune(h2_ctx* c, int32_t prec, char* json, size_t cap) {
   CKS(h2_factor(c, prec));
   o << "{\"tc_kernel\":" << best_form << ",\"factor_s\":[" << tf[0] << "," << tf[1] << "," << tf[2] << "]";
   // (2) the substitution's launch shapes, timed on ULV applications
-  const int64_t n = nslots(c);
+  const int64_t n = nslots32(c);
   float *v = nullptr, *z = nullptr;
   if (cudaMalloc(&v, n * sizeof(float)) != cudaSuccess || cudaMalloc(&z, n * sizeof(float)) != cudaSuccess) {
     cudaGetLastError();

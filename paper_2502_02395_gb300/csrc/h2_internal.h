@@ -170,6 +170,23 @@ struct SymPair {
   int32_t xa, xb, n, pad;
 };
 
+// Device state of an inner FGMRES cycle: the iteration's index, how many CTAs
+// of its last kernel are done, and the number of iterations since the buffers
+// were made (the host waits for it to show up in pinned memory).
+struct GmState {
+  int j;
+  unsigned int done;
+  unsigned long long seq;
+};
+// Device times (globaltimer, ns) of iteration j at t + 5 j: its start, the end
+// of the substitution, the leaf products' first and last, the end of A z.
+constexpr int kGmStamps = 5;
+
+struct KernelGraph {
+  cudaGraphExec_t ex = nullptr;
+  long long kernels = 0;  // in the graph (added to the launch count per replay)
+};
+
 // Where the entries of a logical vector or block lie in its padded form:
 // segments of len entries (a leaf's points, or one child's skeletons) at a
 // stride of str.
@@ -401,8 +418,12 @@ struct h2_ctx {
   // CUDA graph (captured on first use after each h2_factor; H2_OPT_GRAPHS)
   bool use_graphs = true;
   cudaStream_t cap_stream = nullptr;
-  cudaGraphExec_t g_ulv = nullptr;
-  long long g_ulv_kernels = 0;  // kernels in that graph (added to the launch count per replay)
+  // captured sequences (H2_OPT_GRAPHS), kept while the buffers, the operand
+  // type and the launch options they were captured with last (graph_key): the
+  // substitution sweep, and of the nested refinement the start of an inner
+  // cycle, one inner iteration, and the update with its residual
+  h2::KernelGraph g_ulv, g_start, g_iter, g_resid;
+  long long graph_key = -1;
   double inner_tol = 1e-6;       // relative accuracy of the FP32 inner solves
   int restart = 30;              // FGMRES restart length
   double* gm_V = nullptr;        // (restart + 1) * nslot Krylov basis
@@ -414,6 +435,11 @@ struct h2_ctx {
   float* gm_Z32 = nullptr;
   float* gm_r32 = nullptr;
   int gm_cap = 0;                // restart the buffers were sized for
+  int gm_cap64 = 0;              // the same of gm_V and gm_Z
+  float* gm_w32 = nullptr;       // the inner iteration's A z
+  h2::GmState* gm_state = nullptr;
+  unsigned long long* gm_stamp = nullptr;  // 5 (gm_cap + 1) device times of a cycle's iterations
+  unsigned long long gm_seq = 0;  // iterations whose result the host has been told
   h2::Factor<double> f64;
   h2::Factor<float> f32;
   h2::PhaseTimes times;

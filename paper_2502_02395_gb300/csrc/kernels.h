@@ -136,6 +136,23 @@ void launch_bwd1(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const 
 template <typename T, typename TS>
 void launch_bwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
                  cudaStream_t st);
+// The cluster form (a pair step and the per-box step after it in one launch)
+// of levels with few boxes: whether a level takes it, and its four steps.
+// launch_cl_up: level L's SR sums and the parent's first step ([M1; U^S] with
+// dimensions D1, R1 into u and c; at the root M1 = the inverse, R1 = D1).
+template <typename T, typename TS>
+bool subst_clustered(const DevLevel& L, const TS* Ahat);
+template <typename T, typename TS>
+void launch_cl_fwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, cudaStream_t st);
+template <typename T, typename TS>
+void launch_cl_up(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, int D1, int R1,
+                  const T* M1, const T* U, T* u, T* c, cudaStream_t st);
+template <typename T, typename TS>
+void launch_cl_bwd1(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
+                    cudaStream_t st);
+template <typename T, typename TS>
+void launch_cl_bwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
+                    cudaStream_t st);
 template <typename T>
 void launch_gemv_rows(int nb, int n, const T* M, const T* x, T* y, cudaStream_t st);
 template <typename T>
@@ -202,7 +219,8 @@ void launch_matvec_down_far(const DevLevel& L, const T* X, const T* yh, T* yh_ch
 // (pdl: launched to overlap its predecessor; off where events bracket it)
 // (max_n: the largest block, a multiple of 4 up to 256)
 void launch_matvec_sym_pairs(int max_n, int64_t npu, const SymPair* desc, const float* A, const float* x, float* part,
-                             bool pdl, cudaStream_t st);
+                             bool pdl, cudaStream_t st, const GmState* state = nullptr,
+                             unsigned long long* stamp = nullptr);  // (times of iteration state->j)
 void launch_matvec_sym_pairs_df(int D, int64_t npu, const SymPair* desc, const float* Ah, const float* Al,
                                 const float* xh, const float* xl, float* ph, float* pl, cudaStream_t st);
 template <typename T>
@@ -237,6 +255,32 @@ void launch_axpy_from(const T* d, const double* norm2, double* x, int64_t n, Pad
 void launch_pad_axpy(const float* V, int64_t ldv, int nv, const double* coef, double* x, int64_t n, PadSeg p,
                      cudaStream_t st);
 void launch_unpad(const float* in, double* out, int64_t n, PadSeg p, cudaStream_t st);
+// One inner FGMRES iteration's vector work (classical Gram-Schmidt applied
+// twice, FP32 vectors with FP32-pair sums), the iteration's index j read from
+// state->j so that the same launches serve every iteration of a cycle: Z_j =
+// xs; w -= V (V^T w) twice; V_j+1 = vin = w / ||w||; h1, h2, ||w||^2 and the
+// iteration count to pinned host memory.  n entries per vector, m0 the
+// restart; part holds (2 (m0 + 1) + 1) * kOrthCtas doubles.
+constexpr int kOrthCtas = 152;
+struct OrthArgs {
+  float *V, *Z, *w, *vin;
+  const float* xs;
+  int64_t n;
+  int m0, ctas;
+  double *part, *h;  // h: h1 (m0 + 2), h2 (m0 + 2) on the device
+  GmState* state;
+  unsigned long long* stamp;
+  double* host;              // pinned: h1, h2, ||w||^2
+  unsigned long long* flag;  // pinned
+};
+int orth_ctas(int64_t n);
+void launch_orth(const OrthArgs& a, cudaStream_t st);
+// the cycle's start: V_0 = vin = r / sqrt(nrm2), j = 0, times cleared
+void launch_gm_start(const float* r, const double* nrm2, float* V, float* vin, int64_t n, int m0, GmState* state,
+                     unsigned long long* stamp, cudaStream_t st);
+// x += sum_{v < k} y[1 + v] V_v with k = y[0] (device), padded FP32 vectors
+void launch_pad_axpy_dev(const float* V, int64_t ldv, const double* y, double* x, int64_t n, PadSeg p,
+                         cudaStream_t st);
 // GMRES: out[v] (+)= V_v . w for v < nv (part: nv * 128 scratch); w += sign sum_v coef[v] V_v;
 // w = src / sqrt(nrm2[0])
 template <typename T>

@@ -1451,6 +1451,315 @@ void launch_bwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const 
              parent_x, F.part, F.Ur, F.xs);
 }
 
+// ------------------------------------------------------------------------
+// Cluster form of the substitution's steps for levels of few boxes: a
+// thread-block cluster of CS CTAs does a pair step and the per-box step that
+// follows it in one launch.
+//   CL_FWD2: v_i = u_i - Ainv_i s_i,   s_i = sum_{j<i near} Ahat_ij^RR u_j
+//   CL_BWD1: om_i = v_i - Ainv_i s_i,  s_i = sum_{j near} Ahat_ij^RS x_j^S
+//   CL_BWD2: x_i^R = om_i - Ainv_i s_i, s_i = sum_{j>i near} Ahat_ij^RR om_j;
+//            x_i = U_i [x_i^R; x_i^S]
+//   CL_UP:   parent box p: b_p = [c_2p^S - s_2p; c_2p+1^S - s_2p+1],
+//            s_c = sum_{j near c} Ahat_cj^SR v_j; [u_p; c_p^S] = [M1_p;
+//            (U_p^S)^T] b_p, or x = A_root^-1 b at the root
+// The box's pairs go round the CTAs (CL_UP: half of the CTAs per child).  A
+// thread keeps the same rows of every pair's block (16-byte chunks, the rows
+// of cta_gemv), so it accumulates over its CTA's pairs in registers and the
+// rows are reduced once.  The CTAs' partial vectors meet in every CTA's shared
+// memory (distributed shared memory, one cluster barrier), where they are
+// added in rank order; each CTA then applies its slice of the rows of Ainv
+// (and, after a second exchange, of U), which cp.async brought into shared
+// memory before the wait for the previous kernel.
+// Bound by latency: at 64 boxes and fewer a step moves a few MB, and a launch
+// of the pair kernel, one of the per-box kernel and the partial products'
+// round trip through memory cost more than the bytes.
+// ------------------------------------------------------------------------
+enum { CL_FWD2 = 0, CL_BWD1 = 1, CL_BWD2 = 2, CL_UP = 3 };
+
+template <typename T, typename TS>
+struct ClArgs {
+  int D, R, K;            // the pairs' level
+  int CS;                 // CTAs per box
+  const int64_t* ptr;     // near pairs of the boxes
+  const int32_t* cnt;     // CL_FWD2: pairs j < i, CL_BWD2: pairs j > i
+  const int32_t* nj;
+  const TS* Ahat;
+  const float* iscale;
+  const T* xv;            // the pairs' input vector
+  const T* A1;            // Ainv (R x R); CL_UP: M1 (R1 x D1) or the root inverse
+  const T* A2;            // CL_BWD2: Ur (D x D); CL_UP: U (D1 x D1, its columns R1.. are rows here)
+  const T* base;          // u / v / om; CL_UP: the children's c
+  const T* px;            // CL_BWD2: the parent's solution
+  T* out;                 // v / om / xs; CL_UP: u (or the root's x)
+  T* out2;                // CL_UP: c
+  int D1, R1;             // CL_UP: the parent's dimensions (root: R1 = D1)
+};
+
+// rows r0 .. r0 + nr - 1 of a matrix with nc columns lie at rows (shared
+// memory, row stride nc): out(r, sum_c rows[r][c] x[c]); nc a multiple of 4
+template <typename T, typename Out>
+__device__ __forceinline__ void smem_rows(const T* rows, int nr, int nc, const T* x, Out out) {
+  constexpr int VN = 16 / sizeof(T);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int r = warp; r < nr; r += 32) {
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+    for (int c = lane * VN; c < nc; c += 32 * VN) {
+      T xr[VN];
+#pragma unroll
+      for (int e = 0; e < VN; ++e) xr[e] = x[c + e];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r + 8 * u < nr) {
+          T v[VN];
+          Chunk<T>::cvt(*reinterpret_cast<const uint4*>(rows + (size_t)(r + 8 * u) * nc + c), v);
+#pragma unroll
+          for (int e = 0; e < VN; ++e) acc[u] = fma(v[e], xr[e], acc[u]);
+        }
+    }
+    const T v = tsum<4, 32, T>(acc);
+    const int rr = r + 8 * tsum_index<4, 32>(lane);
+    if (tsum_leader<4, 32>(lane) && rr < nr) out(rr, v);
+  }
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+// contiguous bytes (a multiple of 16) into shared memory, by the whole CTA
+__device__ __forceinline__ void cp_async_bytes(void* dst, const void* src, int bytes) {
+  for (int o = threadIdx.x * 16; o < bytes; o += blockDim.x * 16)
+    cp_async16(static_cast<char*>(dst) + o, static_cast<const char*>(src) + o);
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+template <typename T, typename TS, int MODE>
+__global__ void __launch_bounds__(256, sizeof(TS) == 8 ? 1 : 2) box_cluster_kernel(const ClArgs<T, TS> a) {
+  constexpr int VN = Chunk<TS>::VN, UNR = Unr<TS>::v;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int CS = a.CS, rank = (int)(blockIdx.x % CS), i = blockIdx.x / CS;
+  const int D = a.D, R = a.R, K = a.K;
+  cluster_arrive();  // (matched before the first store to another CTA)
+  const int nr = (MODE == CL_UP) ? K : R, nc = (MODE == CL_BWD1) ? K : R;
+  // this CTA's slices of the per-box matrices
+  const int n1 = (MODE == CL_UP) ? a.D1 : R;      // rows of the first matrix
+  const int w1 = (MODE == CL_UP) ? a.D1 : R;      // and its columns
+  const int per1 = (n1 + CS - 1) / CS, a0 = min(rank * per1, n1), m1 = min(per1, n1 - a0);
+  const int per2 = (D + CS - 1) / CS, b0 = min(rank * per2, D), m2 = (MODE == CL_BWD2) ? min(per2, D - b0) : 0;
+  T* rows1 = reinterpret_cast<T*>(sm_raw);                  // per1 x w1
+  T* rows2 = rows1 + (size_t)per1 * w1;                     // per2 x D (CL_BWD2)
+  T* sums = rows2 + (MODE == CL_BWD2 ? (size_t)per2 * D : 0);  // CS x nr partial vectors
+  T* sv = sums + (size_t)CS * nr;                           // input of the per-box step
+  if (MODE == CL_UP) {
+    // rows below R1: M1, above: columns of the column-major U
+    const int e0 = min(a0 + m1, a.R1) - a0;  // rows of M1 in the slice (<= 0: none)
+    if (e0 > 0) cp_async_bytes(rows1, a.A1 + ((size_t)i * a.R1 + a0) * w1, (int)(e0 * w1 * sizeof(T)));
+    const int s0 = max(a0, a.R1);
+    if (a0 + m1 > s0)
+      cp_async_bytes(rows1 + (size_t)(s0 - a0) * w1, a.A2 + ((size_t)i * a.D1 + s0) * w1,
+                     (int)((a0 + m1 - s0) * w1 * sizeof(T)));
+  } else if (m1 > 0) {
+    cp_async_bytes(rows1, a.A1 + ((size_t)i * R + a0) * R, (int)(m1 * R * sizeof(T)));
+  }
+  if (MODE == CL_BWD2 && m2 > 0) cp_async_bytes(rows2, a.A2 + ((size_t)i * D + b0) * D, (int)(m2 * D * sizeof(T)));
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  // the pairs of this CTA: q0 + step * k
+  int64_t q0, q1;
+  int step = CS, first = rank;
+  if (MODE == CL_UP) {
+    const int half = CS / 2, c = 2 * i + (rank >= half);
+    q0 = a.ptr[c], q1 = a.ptr[c + 1];
+    step = half, first = rank % half;
+  } else {
+    q0 = a.ptr[i], q1 = a.ptr[i + 1];
+    if (MODE == CL_FWD2) q1 = q0 + a.cnt[i];
+    if (MODE == CL_BWD2) q0 = q1 - a.cnt[i];
+  }
+  const int nch = (nc + VN - 1) / VN;
+  int cpr = 32;
+  while (cpr > 1 && cpr / 2 >= nch) cpr >>= 1;
+  const int rpi = 32 / cpr, sub = lane / cpr, cl = lane & (cpr - 1);
+  const int nit = (nch + cpr - 1) / cpr;
+  const int64_t off = (MODE == CL_UP ? (int64_t)R * D : (MODE == CL_BWD1 ? R : 0));
+  T acc[UNR];
+#pragma unroll
+  for (int u = 0; u < UNR; ++u) acc[u] = T(0);
+  uint4 raw[UNR];
+  auto load = [&](int64_t p, int it) {
+    const TS* M = a.Ahat + p * D * D + off + (cl + it * cpr) * VN;
+    const bool in = cl + it * cpr < nch;
+#pragma unroll
+    for (int u = 0; u < UNR; ++u) {
+      const int r = (u * nw + warp) * rpi + sub;
+      raw[u] = (in && r < nr) ? __ldg(reinterpret_cast<const uint4*>(M + (int64_t)r * D)) : make_uint4(0, 0, 0, 0);
+    }
+  };
+  int64_t p = q0 + first;
+  if (p < q1) load(p, 0);
+  int j = p < q1 ? a.nj[p] : 0;
+  griddep_wait();
+  griddep_launch_next();
+  while (p < q1) {
+    const int64_t pn = p + step;
+    const int jn = pn < q1 ? a.nj[pn] : 0;
+    const T* x = (MODE == CL_BWD1) ? a.xv + (int64_t)(j >> 1) * 2 * K + (j & 1) * K : a.xv + (int64_t)j * R;
+    for (int it = 0; it < nit; ++it) {
+      const int c = (cl + it * cpr) * VN;
+      T xr[VN];
+#pragma unroll
+      for (int e = 0; e < VN; ++e) xr[e] = (c + e < nc) ? x[c + e] : T(0);
+#pragma unroll
+      for (int u = 0; u < UNR; ++u) {
+        T v[VN];
+        Chunk<TS>::cvt(raw[u], v);
+#pragma unroll
+        for (int e = 0; e < VN; ++e) acc[u] = fma((c + e < nc) ? v[e] : T(0), xr[e], acc[u]);
+      }
+      if (it + 1 < nit) load(p, it + 1);
+      else if (pn < q1) load(pn, 0);
+    }
+    p = pn, j = jn;
+  }
+  // the rows' sums, to every CTA of the cluster
+  cluster_wait();
+#pragma unroll
+  for (int u = 0; u < UNR; ++u) {
+    T t = acc[u];
+    for (int o = cpr >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    const int r = (u * nw + warp) * rpi + sub;
+    if (r < nr)
+      for (int cta = cl; cta < CS; cta += cpr) st_cluster(cluster_map(&sums[(size_t)rank * nr + r], cta), t);
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  cluster_sync();
+  const T isc = a.iscale ? T(a.iscale[0]) : T(1);
+  if (MODE == CL_UP) {
+    for (int e = tid; e < 2 * K; e += blockDim.x) {
+      const int h = e >= K, r = e - h * K;
+      T t = T(0);
+      for (int g = 0; g < CS / 2; ++g) t += sums[(size_t)(h * (CS / 2) + g) * nr + r];
+      sv[e] = a.base[(int64_t)(2 * i + h) * D + R + r] - isc * t;
+    }
+  } else {
+    for (int r = tid; r < R; r += blockDim.x) {
+      T t = T(0);
+      for (int g = 0; g < CS; ++g) t += sums[(size_t)g * nr + r];
+      sv[r] = isc * t;
+    }
+  }
+  __syncthreads();
+  if (MODE == CL_UP) {
+    smem_rows<T>(rows1, m1, w1, sv, [&](int r, T v) {
+      const int g = a0 + r;
+      if (g < a.R1) a.out[(int64_t)i * a.R1 + g] = v;
+      else a.out2[(int64_t)i * a.D1 + g] = v;
+    });
+  } else if (MODE != CL_BWD2) {
+    smem_rows<T>(rows1, m1, w1, sv, [&](int r, T v) {
+      const int64_t g = (int64_t)i * R + a0 + r;
+      a.out[g] = a.base[g] - v;
+    });
+  } else {
+    // z_i = [x_i^R; x_i^S] in every CTA (over sums and sv's successor: z)
+    T* z = sv + R;
+    const T* xi = a.px + (int64_t)(i >> 1) * 2 * K + (i & 1) * K;
+    for (int e = tid; e < K; e += blockDim.x) z[R + e] = xi[e];
+    smem_rows<T>(rows1, m1, w1, sv, [&](int r, T v) {
+      const T t = a.base[(int64_t)i * R + a0 + r] - v;
+      for (int cta = 0; cta < CS; ++cta) st_cluster(cluster_map(&z[a0 + r], cta), t);
+    });
+    cluster_sync();
+    smem_rows<T>(rows2, m2, D, z, [&](int r, T v) { a.out[(int64_t)i * D + b0 + r] = v; });
+  }
+}
+
+// CTAs per box of the cluster form for a level of nb boxes (0: the level
+// takes a pair and a per-box launch): up to two CTAs per SM in all.
+static int cluster_ctas(int nb) {
+  const int room = 2 * num_sms();
+  if (g_box_stream.load() == 2) return 0;  // the streamed form on every level
+  if (nb * 8 <= room) return 8;
+  if (nb * 4 <= room) return 4;
+  return 0;
+}
+// the level's shapes: one register pass over a block's rows, 16-byte rows and
+// quadrants
+template <typename T, typename TS>
+static bool cluster_shape(const DevLevel& L, const TS* Ahat) {
+  auto one_pass = [](int nr, int nc) {
+    const int nch = (nc + Chunk<TS>::VN - 1) / Chunk<TS>::VN;
+    int cpr = 32;
+    while (cpr > 1 && cpr / 2 >= nch) cpr >>= 1;
+    return nr <= 8 * Unr<TS>::v * (32 / cpr);
+  };
+  const int v = 16 / (int)sizeof(TS), w = 16 / (int)sizeof(T);
+  return L.R > 0 && L.K > 0 && L.D % v == 0 && L.R % v == 0 && L.R % w == 0 && L.K % w == 0 && L.D % w == 0 &&
+         (reinterpret_cast<uintptr_t>(Ahat) & 15) == 0 && one_pass(L.R, L.R) && one_pass(L.K, L.R) &&
+         one_pass(L.R, L.K);
+}
+template <typename T, typename TS>
+bool subst_clustered(const DevLevel& L, const TS* Ahat) {
+  return cluster_ctas(L.nb) > 0 && cluster_shape<T, TS>(L, Ahat);
+}
+
+template <typename T, typename TS, int MODE>
+static void launch_cluster(const DevLevel& L, const ClArgs<T, TS>& args, int nbox, cudaStream_t st) {
+  ClArgs<T, TS> a = args;
+  a.D = L.D, a.R = L.R, a.K = L.K, a.ptr = L.near_ptr, a.nj = L.near_j;
+  a.CS = cluster_ctas(MODE == CL_UP ? 2 * nbox : nbox);  // (of the pairs' level)
+  if (MODE == CL_UP) a.CS = std::min(8, 2 * a.CS);
+  const int n1 = MODE == CL_UP ? a.D1 : a.R, per1 = (n1 + a.CS - 1) / a.CS, per2 = (a.D + a.CS - 1) / a.CS;
+  const int nr = MODE == CL_UP ? a.K : a.R;
+  const size_t sm = sizeof(T) * ((size_t)per1 * n1 + (MODE == CL_BWD2 ? (size_t)per2 * a.D : 0) + (size_t)a.CS * nr +
+                                 (MODE == CL_UP ? 2 * a.K : a.R) + (MODE == CL_BWD2 ? a.D : 0));
+  set_smem((const void*)box_cluster_kernel<T, TS, MODE>, sm);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(nbox * a.CS));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)a.CS;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  ++g_launches;
+  cudaLaunchKernelEx(&cfg, box_cluster_kernel<T, TS, MODE>, a);
+}
+
+template <typename T, typename TS>
+void launch_cl_fwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, cudaStream_t st) {
+  ClArgs<T, TS> a{};
+  a.cnt = L.lo_cnt, a.Ahat = Ahat, a.iscale = iscale, a.xv = F.u, a.A1 = F.Ainv, a.base = F.u, a.out = F.v;
+  launch_cluster<T, TS, CL_FWD2>(L, a, L.nb, st);
+}
+template <typename T, typename TS>
+void launch_cl_up(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, int D1, int R1,
+                  const T* M1, const T* U, T* u, T* c, cudaStream_t st) {
+  ClArgs<T, TS> a{};
+  a.Ahat = Ahat, a.iscale = iscale, a.xv = F.v, a.A1 = M1, a.A2 = U, a.base = F.c, a.out = u, a.out2 = c, a.D1 = D1,
+  a.R1 = R1;
+  launch_cluster<T, TS, CL_UP>(L, a, L.nb / 2, st);
+}
+template <typename T, typename TS>
+void launch_cl_bwd1(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
+                    cudaStream_t st) {
+  ClArgs<T, TS> a{};
+  a.Ahat = Ahat, a.iscale = iscale, a.xv = parent_x, a.A1 = F.Ainv, a.base = F.v, a.out = F.om;
+  launch_cluster<T, TS, CL_BWD1>(L, a, L.nb, st);
+}
+template <typename T, typename TS>
+void launch_cl_bwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
+                    cudaStream_t st) {
+  ClArgs<T, TS> a{};
+  a.cnt = L.hi_cnt, a.Ahat = Ahat, a.iscale = iscale, a.xv = F.om, a.A1 = F.Ainv, a.A2 = F.Ur, a.base = F.om,
+  a.px = parent_x, a.out = F.xs;
+  launch_cluster<T, TS, CL_BWD2>(L, a, L.nb, st);
+}
+
 // y_b = M_b x_b for nb n x n row-major matrices, one CTA each (root solves
 // with the explicit inverses: one root, or one per system of a forest)
 template <typename T>
@@ -1489,6 +1798,15 @@ H2_INST_SOLVE(float)
                                    cudaStream_t);                                                              \
   template void launch_bwd1<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, const T*,      \
                                    cudaStream_t);                                                              \
+  template bool subst_clustered<T, TS>(const DevLevel&, const TS*);                                            \
+  template void launch_cl_fwd2<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*,            \
+                                      cudaStream_t);                                                           \
+  template void launch_cl_up<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, int, int,    \
+                                    const T*, const T*, T*, T*, cudaStream_t);                                 \
+  template void launch_cl_bwd1<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, const T*,  \
+                                      cudaStream_t);                                                           \
+  template void launch_cl_bwd2<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, const T*,  \
+                                      cudaStream_t);                                                           \
   template void launch_bwd2<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, const T*,      \
                                    cudaStream_t);
 H2_INST_SUBST(double, double)
@@ -2100,7 +2418,9 @@ constexpr int kSymRPW = 8;  // rows per warp in flight
 template <int CH>  // 4-column chunks per lane: n <= 128 CH
 __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __restrict__ desc,
                                                              const float* __restrict__ A, const float* __restrict__ x,
-                                                             float* __restrict__ part, int pf) {
+                                                             float* __restrict__ part, int pf,
+                                                             const GmState* __restrict__ state,
+                                                             unsigned long long* __restrict__ stamp) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const SymPair ds = desc[blockIdx.x];
   const int n = ds.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -2111,6 +2431,10 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __re
   if (pf) prefetch_l2(M, (int64_t)n * n * sizeof(float));
   griddep_wait();
   griddep_launch_next();
+  if (stamp && blockIdx.x == 0 && tid == 0) {
+    unsigned long long* t = stamp + kGmStamps * state->j;
+    t[1] = t[2] = global_ns();
+  }
   for (int e = tid; e < n; e += blockDim.x) xa[e] = x[ds.xa + e];
   bool in[CH];
   float xb[CH][4];
@@ -2163,6 +2487,7 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __re
       if (tsum_leader<kSymRPW, 32>(lane) && r < n) u[r] = sv;
     }
   }
+  if (stamp && tid == 0) atomicMax(stamp + kGmStamps * state->j + 3, global_ns());
   if (!both) return;
 #pragma unroll
   for (int h = 0; h < CH; ++h)
@@ -2335,21 +2660,21 @@ bool sym_supported(int n) { return n > 0 && n % 4 == 0 && n <= 256; }
 
 template <int CH>
 static void launch_sym_pairs_ch(int n, int64_t npu, const SymPair* desc, const float* A, const float* x, float* part,
-                                bool pdl, cudaStream_t st) {
+                                bool pdl, cudaStream_t st, const GmState* state, unsigned long long* stamp) {
   const size_t sm = sizeof(float) * 9 * (size_t)n;
   const int pf = small_level(npu) ? 1 : 0;
   if (pdl) {
-    launch_pdl(mv_sym_pair_kernel<CH>, (unsigned)npu, 256, sm, st, desc, A, x, part, pf);
+    launch_pdl(mv_sym_pair_kernel<CH>, (unsigned)npu, 256, sm, st, desc, A, x, part, pf, state, stamp);
   } else {
     ++g_launches;
-    mv_sym_pair_kernel<CH><<<(unsigned)npu, 256, sm, st>>>(desc, A, x, part, pf);
+    mv_sym_pair_kernel<CH><<<(unsigned)npu, 256, sm, st>>>(desc, A, x, part, pf, state, stamp);
   }
 }
 void launch_matvec_sym_pairs(int max_n, int64_t npu, const SymPair* desc, const float* A, const float* x, float* part,
-                             bool pdl, cudaStream_t st) {
+                             bool pdl, cudaStream_t st, const GmState* state, unsigned long long* stamp) {
   if (npu <= 0) return;
-  if (max_n <= 128) launch_sym_pairs_ch<1>(max_n, npu, desc, A, x, part, pdl, st);
-  else launch_sym_pairs_ch<2>(max_n, npu, desc, A, x, part, pdl, st);
+  if (max_n <= 128) launch_sym_pairs_ch<1>(max_n, npu, desc, A, x, part, pdl, st, state, stamp);
+  else launch_sym_pairs_ch<2>(max_n, npu, desc, A, x, part, pdl, st, state, stamp);
 }
 void launch_matvec_sym_pairs_df(int D, int64_t npu, const SymPair* desc, const float* Ah, const float* Al,
                                 const float* xh, const float* xl, float* ph, float* pl, cudaStream_t st) {
@@ -2727,6 +3052,197 @@ __global__ void multi_axpy_f32_kernel(const float* __restrict__ V, int64_t ldv, 
     w[e] = wh + wl;
   }
 }
+// ------------------------------------------------------------------------
+// The vector work of one inner FGMRES iteration in four launches (see
+// kernels.h).  Every CTA owns a slice of the vectors; a pass's dot products
+// are finished by the next launch, in which every CTA adds the partial sums of
+// all CTAs itself (FP64, in CTA order), so no launch exists only to add
+// them.  Bound by latency (a few launches in line) up to some 10^5 entries and
+// by the reads of V beyond.  Ten separate launches and a host
+// synchronization took 85 us an iteration at 16384 entries.
+// ------------------------------------------------------------------------
+struct OrthSlice {
+  int64_t b, e;
+};
+__device__ __forceinline__ OrthSlice orth_slice(const OrthArgs& a) {
+  const int64_t ch = ((a.n + a.ctas - 1) / a.ctas + 31) & ~(int64_t)31;
+  const int64_t b = min(a.n, (int64_t)blockIdx.x * ch);
+  return {b, min(a.n, b + ch)};
+}
+// part[v ctas + cta] = this CTA's share of V_v . w, v <= j
+__device__ __forceinline__ void orth_dots(const OrthArgs& a, int j, OrthSlice sl, double* part) {
+  __shared__ float dh[8][8], dl[8][8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int v0 = 0; v0 <= j; v0 += 8) {
+    float H[8], L[8];
+    zero(H);
+    zero(L);
+    const int nv = min(8, j + 1 - v0);
+    for (int64_t e = sl.b + tid; e < sl.e; e += 256) {
+      const float x = a.w[e];
+#pragma unroll
+      for (int g = 0; g < 8; ++g)
+        if (g < nv) df_acc(H[g], L[g], a.V[(int64_t)(v0 + g) * a.n + e], x);
+    }
+    float sh, sl2;
+    df_tsum<8, 32>(H, L, sh, sl2);
+    if (tsum_leader<8, 32>(lane)) dh[warp][tsum_index<8, 32>(lane)] = sh, dl[warp][tsum_index<8, 32>(lane)] = sl2;
+    __syncthreads();
+    if (tid < nv) {
+      float th = dh[0][tid], tl = dl[0][tid];
+      for (int w = 1; w < 8; ++w) df_add(th, tl, dh[w][tid], dl[w][tid]);
+      part[(int64_t)(v0 + tid) * a.ctas + blockIdx.x] = (double)th + (double)tl;
+    }
+    __syncthreads();
+  }
+}
+// w -= V h with h_v = sum of part's row v, by this CTA on its slice; CTA 0
+// keeps h.  ch / cl: j + 1 floats of shared memory each
+__device__ __forceinline__ void orth_update(const OrthArgs& a, int j, OrthSlice sl, const double* part, double* h,
+                                            float* ch, float* cl) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int v = warp; v <= j; v += 8) {
+    double s = 0;
+    for (int k = lane; k < a.ctas; k += 32) s += part[(int64_t)v * a.ctas + k];
+    s = warp_sum(s);
+    if (lane == 0) {
+      df_split(s, ch[v], cl[v]);
+      if (blockIdx.x == 0) h[v] = s;
+    }
+  }
+  __syncthreads();
+  for (int64_t e = sl.b + tid; e < sl.e; e += 256) {
+    float H = 0.0f, L = 0.0f;
+#pragma unroll 4
+    for (int v = 0; v <= j; ++v) {
+      const float x = a.V[(int64_t)v * a.n + e];
+      df_acc(H, L, ch[v], x);
+      L = fmaf(cl[v], x, L);
+    }
+    float wh = a.w[e], wl = 0.0f;
+    df_add(wh, wl, -H, -L);
+    a.w[e] = wh + wl;
+  }
+}
+// STEP 0: Z_j = xs, first dots; 1: first update, second dots; 2: second update,
+// norm; 3: normalization, result to the host
+template <int STEP>
+__global__ void __launch_bounds__(256) orth_kernel(const OrthArgs a) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float* ch = reinterpret_cast<float*>(smraw);
+  float* cl = ch + a.m0 + 1;
+  __shared__ unsigned int last;
+  griddep_wait();
+  griddep_launch_next();
+  const int tid = threadIdx.x, j = a.state->j;
+  const OrthSlice sl = orth_slice(a);
+  double* p1 = a.part;
+  double* p2 = p1 + (int64_t)(a.m0 + 1) * kOrthCtas;
+  double* p3 = p2 + (int64_t)(a.m0 + 1) * kOrthCtas;
+  if constexpr (STEP == 0) {
+    if (blockIdx.x == 0 && tid == 0) a.stamp[kGmStamps * j + 4] = global_ns();
+    float* z = a.Z + (int64_t)j * a.n;
+    for (int64_t e = sl.b + tid; e < sl.e; e += 256) z[e] = a.xs[e];
+    orth_dots(a, j, sl, p1);
+  } else if constexpr (STEP == 1) {
+    orth_update(a, j, sl, p1, a.h, ch, cl);
+    orth_dots(a, j, sl, p2);  // (each thread reads back its own w)
+  } else if constexpr (STEP == 2) {
+    orth_update(a, j, sl, p2, a.h + a.m0 + 2, ch, cl);
+    float H = 0.0f, L = 0.0f;
+    for (int64_t e = sl.b + tid; e < sl.e; e += 256) df_acc(H, L, a.w[e], a.w[e]);
+    const double t = block_df_total(H, L);
+    if (tid == 0) p3[blockIdx.x] = t;
+  } else {
+    __shared__ double ss;
+    if (tid < 32) {
+      double s = 0;
+      for (int k = tid; k < a.ctas; k += 32) s += p3[k];
+      s = warp_sum(s);
+      if (tid == 0) ss = s;
+    }
+    __syncthreads();
+    const double nw2 = ss, r = sqrt(nw2);
+    const float sf = (float)(r > 0 ? 1.0 / r : 0.0);
+    float* vn = a.V + (int64_t)(j + 1) * a.n;
+    for (int64_t e = sl.b + tid; e < sl.e; e += 256) {
+      const float x = a.w[e] * sf;
+      vn[e] = x;
+      a.vin[e] = x;
+    }
+    // the last CTA tells the host and moves to the next iteration
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(&a.state->done, 1u);
+    __syncthreads();
+    if (last + 1 != gridDim.x) return;
+    for (int v = tid; v <= j; v += 256) {
+      a.host[v] = a.h[v];
+      a.host[a.m0 + 2 + v] = a.h[a.m0 + 2 + v];
+    }
+    if (tid == 0) a.host[2 * (a.m0 + 2)] = nw2;
+    __threadfence_system();
+    __syncthreads();
+    if (tid == 0) {
+      const unsigned long long s = a.state->seq + 1;
+      a.state->seq = s;
+      a.state->done = 0;
+      a.state->j = j + 1;
+      a.stamp[kGmStamps * (j + 1)] = global_ns();
+      __threadfence_system();
+      *reinterpret_cast<volatile unsigned long long*>(a.flag) = s;
+    }
+  }
+}
+int orth_ctas(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>(kOrthCtas, n / 512)); }
+void launch_orth(const OrthArgs& a, cudaStream_t st) {
+  const size_t sm = 2 * sizeof(float) * (size_t)(a.m0 + 1);
+  launch_pdl(orth_kernel<0>, (unsigned)a.ctas, 256, sm, st, a);
+  launch_pdl(orth_kernel<1>, (unsigned)a.ctas, 256, sm, st, a);
+  launch_pdl(orth_kernel<2>, (unsigned)a.ctas, 256, sm, st, a);
+  launch_pdl(orth_kernel<3>, (unsigned)a.ctas, 256, sm, st, a);
+}
+__global__ void __launch_bounds__(256) gm_start_kernel(const float* __restrict__ r, const double* __restrict__ nrm2,
+                                                       float* __restrict__ V, float* __restrict__ vin, int64_t n,
+                                                       int nstamp, GmState* __restrict__ state,
+                                                       unsigned long long* __restrict__ stamp) {
+  __shared__ float ss;
+  if (threadIdx.x == 0) {
+    const double s = sqrt(nrm2[0]);
+    ss = (float)(s > 0 ? 1.0 / s : 0.0);
+  }
+  __syncthreads();
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const float x = r[e] * ss;
+    V[e] = x;
+    vin[e] = x;
+  }
+  if (blockIdx.x == 0) {
+    for (int k = threadIdx.x; k < nstamp; k += blockDim.x) stamp[k] = k == 0 ? global_ns() : 0ull;
+    if (threadIdx.x == 0) state->j = 0, state->done = 0;
+  }
+}
+void launch_gm_start(const float* r, const double* nrm2, float* V, float* vin, int64_t n, int m0, GmState* state,
+                     unsigned long long* stamp, cudaStream_t st) {
+  ++g_launches;
+  gm_start_kernel<<<grid_for(n), 256, 0, st>>>(r, nrm2, V, vin, n, kGmStamps * (m0 + 1), state, stamp);
+}
+__global__ void pad_axpy_dev_kernel(const float* __restrict__ V, int64_t ldv, const double* __restrict__ y,
+                                    double* __restrict__ x, int64_t n, PadSeg p) {
+  const int nv = (int)y[0];
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t g = padded_at(p, e);
+    double s = 0;
+    for (int v = 0; v < nv; ++v) s = fma(y[1 + v], (double)V[(int64_t)v * ldv + g], s);
+    x[e] += s;
+  }
+}
+void launch_pad_axpy_dev(const float* V, int64_t ldv, const double* y, double* x, int64_t n, PadSeg p,
+                         cudaStream_t st) {
+  ++g_launches;
+  pad_axpy_dev_kernel<<<grid_for(n), 256, 0, st>>>(V, ldv, y, x, n, p);
+}
+
 template <typename T, typename TW>
 void launch_multi_axpy(const T* V, int64_t ldv, int nv, const double* coef, double sign, TW* w, int64_t n,
                        cudaStream_t st) {

@@ -100,6 +100,9 @@ __device__ __forceinline__ int ld_cluster(uint32_t a, int) {
 __device__ __forceinline__ void st_cluster(uint32_t a, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
+__device__ __forceinline__ void st_cluster(uint32_t a, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
 __device__ __forceinline__ void st_cluster(uint32_t a, long long v) {
   asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
 }
