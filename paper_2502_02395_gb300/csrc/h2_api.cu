@@ -387,11 +387,12 @@ h2_status setup_device(h2_ctx* c) {
   c->Slo.assign(L + 1, nullptr);
   c->Xlo.assign(L + 1, nullptr);
   // the couplings i < j of all levels as one batch
-  c->cb_ok = L >= 1 && far_closed;
+  c->cb_ok = L >= 1 && far_closed && c->sym;
   for (int l = 1; l <= L; ++l)
     if (c->pv[l].FP > 0 && !sym_supported(c->pv[l].K)) c->cb_ok = false;
   std::vector<SymPair> cb;
   std::vector<int32_t*> fsq(L + 1, nullptr);
+  std::vector<int64_t> cb_m0(L + 1, 0);  // each level's first stored coupling
   int64_t cb_m = 0, cb_p = 0;
   for (int l = 1; l <= L && c->cb_ok; ++l) {
     DevLevel& d = c->pv[l];
@@ -406,18 +407,23 @@ h2_status setup_device(h2_ctx* c) {
     cb_m += d.fpu * (int64_t)d.K * d.K;
     cb_p += d.fpu * 2 * (int64_t)d.K;
     c->cb_max = std::max(c->cb_max, d.K);
+    c->cb_min = c->cb_min ? std::min(c->cb_min, d.K) : d.K;
   }
   c->cb_n = (int64_t)cb.size();
   if (c->cb_ok) {
     CKS(upload(c, &c->cb, cb));
     CKC(dalloc(c, &c->S32u_all, (size_t)cb_m));
+    CKC(dalloc(c, &c->Slo_all, (size_t)cb_m));
     CKC(dalloc(c, &c->part32c, (size_t)cb_p));
+    CKC(dalloc(c, &c->part32cd, 2 * (size_t)cb_p));
+    c->cb_part = cb_p;
     int64_t m0 = 0;
     for (int l = 1; l <= L; ++l) {
       const DevLevel& d = c->pv[l];
+      cb_m0[l] = m0;
       if (d.FP == 0) continue;
-      launch_pad_blocks<double>(d.S, fsq[l], d.fpu, d.K, skel_seg(c, l), d.K, skel_seg(c, l), c->S32u_all + m0, nullptr,
-                                nullptr, nullptr, 0);
+      launch_pad_blocks<double>(d.S, fsq[l], d.fpu, d.K, skel_seg(c, l), d.K, skel_seg(c, l), c->S32u_all + m0,
+                                c->Slo_all + m0, nullptr, nullptr, 0);
       m0 += d.fpu * (int64_t)d.K * d.K;
     }
   }
@@ -427,12 +433,15 @@ h2_status setup_device(h2_ctx* c) {
     const size_t nx = (size_t)d.nb * d.D * d.K, ns = (size_t)std::max<int64_t>(d.FP, 1) * d.K * d.K;
     const PadSeg rs = row_seg(c, l), ks = skel_seg(c, l);
     CKC(dalloc(c, &d.X32, nx));
-    CKC(dalloc(c, &d.S32, ns));
     CKC(dalloc(c, &c->Xlo[l], nx));
-    CKC(dalloc(c, &c->Slo[l], ns));
     launch_pad_blocks<double>(d.X, nullptr, d.nb, d.D, rs, d.K, ks, d.X32, c->Xlo[l], nullptr, nullptr, 0);
-    // (the residual's FP32-pair matvec reads the couplings in full)
-    launch_pad_blocks<double>(d.S, nullptr, d.FP, d.K, ks, d.K, ks, d.S32, c->Slo[l], nullptr, nullptr, 0);
+    if (c->cb_ok) {
+      d.S32 = c->S32u_all + cb_m0[l];  // the stored halves
+    } else {
+      CKC(dalloc(c, &d.S32, ns));
+      CKC(dalloc(c, &c->Slo[l], ns));
+      launch_pad_blocks<double>(d.S, nullptr, d.FP, d.K, ks, d.K, ks, d.S32, c->Slo[l], nullptr, nullptr, 0);
+    }
     d.X32q = d.X32;
     if (d.D != g.D || d.K != g.K) {
       CKC(dalloc(c, &d.X32q, (size_t)g.nb * g.D * g.K));
@@ -791,7 +800,9 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       const bool up = d.far_mirrored;
       const int64_t n = up ? d.n_fu : d.FP;
       const int32_t *pq = up ? d.fu_q : nullptr, *pi = up ? d.fu_i : d.far_i, *pj = up ? d.fu_j : d.far_j;
-      gemm<T>(prec, K, K, K, Sc, KK, pq, K, false, f.Tp, KK, pj, K, true, F.Wc, KK, nullptr, K, T(1), T(0), n, sc);
+      // (FP32: the instance's stored halves are in the order of the pairs)
+      const bool halves = up && mixed && c->cb_ok;
+      gemm<T>(prec, K, K, K, Sc, KK, halves ? nullptr : pq, K, false, f.Tp, KK, pj, K, true, F.Wc, KK, nullptr, K, T(1), T(0), n, sc);
       gemm<T>(prec, K, K, K, f.Tp, KK, pi, K, false, F.Wc, KK, nullptr, K, false, f.Shat, KK, pq, K, T(1), T(0), n, sc);
       if (up) launch_transpose_pairs<T>(K, n, d.fl_q, d.fl_m, f.Shat, sc);
     }
@@ -1243,6 +1254,15 @@ void matvec_streams(h2_ctx* c) {
 // second stream, all couplings in one launch)
 bool matvec32_sym(const h2_ctx* c) { return c->cb_ok && c->sym && c->L >= 1; }
 
+// the levels 1 .. L, those with the longest far lists first
+std::vector<int> levels_by_far(const std::vector<DevLevel>& LV, int L) {
+  std::vector<int> order;
+  for (int l = 1; l <= L; ++l) order.push_back(l);
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int u, int v) { return LV[u].FP * (int64_t)LV[v].nb > LV[v].FP * (int64_t)LV[u].nb; });
+  return order;
+}
+
 // y = A_H2 x; with leaf_ev set, the leaf-level kernel (near blocks plus the
 // leaf basis) is bracketed by a pair of events appended there.
 template <typename T>
@@ -1256,72 +1276,77 @@ void matvec_t(h2_ctx* c, const T* A, T* const* X, T* const* S, T* xh, T* yh, con
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
   }
-  // leaf step: y = X_L yh_L + near-field; the FP32 copy may hold only the
-  // i <= j halves of the symmetric near blocks
-  auto leaf = [&](const T* XL, const T* yhL) {
-    if constexpr (std::is_same<T, float>::value) {
-      if (c->sym) {
-        const DevLevel& lf = LV[L];
-        if (leaf_ev) cudaEventRecord(e0, st);
-        launch_matvec_sym_pairs(lf.D, c->npu, c->sym_desc, A, x, c->part32, false, st);
-        if (leaf_ev) cudaEventRecord(e1, st), leaf_ev->push_back({e0, e1});
-        launch_matvec_sym_sum<float>(lf.nb, lf.D, L ? lf.K : 0, c->sym_ptr, c->sym_ent, XL, yhL, c->part32, y, st);
-        return;
-      }
-    }
-    if (leaf_ev) cudaEventRecord(e0, st);
-    launch_matvec_leaf<T>(LV[L], A, XL, x, yhL, y, st);
-    if (leaf_ev) cudaEventRecord(e1, st), leaf_ev->push_back({e0, e1});
-  };
-  if (L == 0) {
-    leaf(nullptr, nullptr);
-    return;
-  }
-  const std::vector<int64_t>& off = std::is_same<T, double>::value ? c->hat_off : c->hat_off32;
+  const DevLevel& lf = LV[L];
   if constexpr (std::is_same<T, float>::value) {
-    if (matvec32_sym(c)) {
+    if (matvec32_sym(c) || (L == 0 && c->sym)) {
       // the leaf near-field products need only x: they run on the leaf
       // stream beside the upward pass, the couplings (every level in one
       // launch) and the downward pass, which adds each level's coupling
       // sums as it goes; the per-box leaf sums follow the join
+      if (L == 0) {
+        if (leaf_ev) cudaEventRecord(e0, st);
+        launch_matvec_sym_pairs(lf.D, lf.D, c->npu, c->sym_desc, A, x, c->part32, false, st);
+        if (leaf_ev) cudaEventRecord(e1, st), leaf_ev->push_back({e0, e1});
+        launch_matvec_rows<float>(lf.nb, lf.D, 0, nullptr, nullptr, nullptr, y, lf.D, c->sym_ptr, c->sym_ent, c->part32,
+                                  true, st);
+        return;
+      }
+      const std::vector<int64_t>& off = c->hat_off32;
       matvec_streams(c);
       cudaStream_t sl = c->leaf_stream;
-      const DevLevel& lf = LV[L];
       cudaEventRecord(c->mv_fork, st);
       cudaStreamWaitEvent(sl, c->mv_fork, 0);
       if (leaf_ev) cudaEventRecord(e0, sl);
-      launch_matvec_sym_pairs(lf.D, c->npu, c->sym_desc, A, x, c->part32, false, sl, c->gm_state, stamp);
+      launch_matvec_sym_pairs(lf.D, lf.D, c->npu, c->sym_desc, A, x, c->part32, false, sl, c->gm_state, stamp);
       if (leaf_ev) cudaEventRecord(e1, sl), leaf_ev->push_back({e0, e1});
       cudaEventRecord(c->mv_join, sl);
-      launch_matvec_up<T>(LV[L], X[L], x, xh + off[L], st);
+      launch_matvec_up<T>(lf, X[L], x, xh + off[L], st);
       for (int l = L - 1; l >= 1; --l) launch_matvec_up<T>(LV[l], X[l], xh + off[l + 1], xh + off[l], st);
-      launch_matvec_sym_pairs(c->cb_max, c->cb_n, c->cb, c->S32u_all, xh, c->part32c, true, st);
+      launch_matvec_sym_pairs(c->cb_min, c->cb_max, c->cb_n, c->cb, c->S32u_all, xh, c->part32c, true, st);
       const DevLevel& d1 = LV[1];
-      if (d1.FP > 0 && d1.K > 0)
-        launch_matvec_sym_sum<float>(d1.nb, d1.K, 0, d1.fs_ptr, d1.fs_ent, nullptr, nullptr,
-                                     c->part32c + d1.fs_poff, yh + off[1], st);
-      else
-        cudaMemsetAsync(yh + off[1], 0, sizeof(T) * (size_t)d1.nb * d1.K, st);
+      const bool far1 = d1.FP > 0 && d1.K > 0;
+      if (far1)
+        launch_matvec_rows<float>(d1.nb, d1.K, 0, nullptr, nullptr, nullptr, yh + off[1], d1.K, d1.fs_ptr, d1.fs_ent,
+                                  c->part32c + d1.fs_poff, true, st);
+      // (without couplings at level 1 its coefficients are zero: no product)
       for (int l = 1; l < L; ++l) {
-        const DevLevel& dc = LV[l + 1];
-        const bool has = dc.FP > 0 && dc.K > 0;
-        launch_matvec_down_far<float>(LV[l], X[l], yh + off[l], yh + off[l + 1], has ? dc.fs_ptr : nullptr,
-                                      has ? dc.fs_ent : nullptr, c->part32c + dc.fs_poff, st);
+        const DevLevel &d = LV[l], &dc = LV[l + 1];
+        const bool has = dc.FP > 0 && dc.K > 0, zero = l == 1 && !far1;
+        launch_matvec_rows<float>(d.nb, d.D, zero ? 0 : d.K, X[l], yh + off[l], nullptr, yh + off[l + 1], d.D / 2,
+                                  has ? dc.fs_ptr : nullptr, has ? dc.fs_ent : nullptr, c->part32c + dc.fs_poff, true, st);
       }
       cudaStreamWaitEvent(st, c->mv_join, 0);
-      launch_matvec_sym_sum<float>(lf.nb, lf.D, lf.K, c->sym_ptr, c->sym_ent, X[L], yh + off[L], c->part32, y, st,
-                                   false);
+      launch_matvec_rows<float>(lf.nb, lf.D, L == 1 && !far1 ? 0 : lf.K, X[L], yh + off[L], nullptr, y, lf.D, c->sym_ptr,
+                                c->sym_ent, c->part32, false, st);
       return;
     }
   }
-  launch_matvec_up<T>(LV[L], X[L], x, xh + off[L], st);
-  for (int l = L - 1; l >= 1; --l) launch_matvec_up<T>(LV[l], X[l], xh + off[l + 1], xh + off[l], st);
-  for (int l = 1; l <= L; ++l) {
-    const DevLevel& d = LV[l];
-    launch_matvec_far<T>(d, S[l], xh + off[l], yh + off[l], st);
+  const std::vector<int64_t>& off = std::is_same<T, double>::value ? c->hat_off : c->hat_off32;
+  BlockRowArgs<T> la{};
+  la.nlev = 1;
+  la.lv[0] = {lf.near_ptr, lf.near_j, A, x, L ? X[L] : nullptr, L ? yh + off[L] : nullptr, y, lf.nb, lf.D, L ? lf.K : 0};
+  if (L >= 1) {
+    launch_matvec_up<T>(lf, X[L], x, xh + off[L], st);
+    for (int l = L - 1; l >= 1; --l) launch_matvec_up<T>(LV[l], X[l], xh + off[l + 1], xh + off[l], st);
+    // couplings, the longest lists first (their CTAs take longest)
+    BlockRowArgs<T> fa{};
+    for (int l : levels_by_far(LV, L)) {
+      const DevLevel& d = LV[l];
+      if (d.K == 0) continue;
+      if (fa.nlev == kMaxRowLevels) {
+        launch_matvec_block_rows<T>(fa, st);
+        fa = BlockRowArgs<T>{};
+      }
+      fa.lv[fa.nlev++] = {d.far_ptr, d.far_j, S[l], xh + off[l], nullptr, nullptr, yh + off[l], d.nb, d.K, 0};
+    }
+    launch_matvec_block_rows<T>(fa, st);
+    for (int l = 1; l < L; ++l)
+      launch_matvec_rows<T>(LV[l].nb, LV[l].D, LV[l].K, X[l], yh + off[l], yh + off[l + 1], yh + off[l + 1], LV[l].D,
+                            nullptr, nullptr, nullptr, true, st);
   }
-  for (int l = 1; l < L; ++l) launch_matvec_down<T>(LV[l], X[l], yh + off[l], yh + off[l + 1], st);
-  leaf(X[L], yh + off[L]);
+  if (leaf_ev) cudaEventRecord(e0, st);
+  launch_matvec_block_rows<T>(la, st);
+  if (leaf_ev) cudaEventRecord(e1, st), leaf_ev->push_back({e0, e1});
 }
 
 void matvec_impl(h2_ctx* c, const double* x, double* y) {
@@ -1336,6 +1361,7 @@ void matvec_df(h2_ctx* c, const double* x, double* y) {
   const std::vector<DevLevel>& LV = c->pv;
   const DevLevel& lf = LV[L];
   const std::vector<int64_t>& off = c->hat_off32;
+  bool far1 = true;  // whether level 1 has coefficients
   launch_split_df(x, c->xdf_h, c->xdf_l, nslots(c), leaf_seg(c), st);
   if (L >= 1) {
     // upward pass, couplings of all levels in one launch, downward pass
@@ -1343,36 +1369,54 @@ void matvec_df(h2_ctx* c, const double* x, double* y) {
     for (int l = L - 1; l >= 1; --l)
       launch_matvec_up_df(LV[l], c->X32p[l], c->Xlo[l], c->hdf_h + off[l + 1], c->hdf_l + off[l + 1],
                           c->hdf_h + off[l], c->hdf_l + off[l], st);
-    // levels with the longest far lists first (their CTAs take longest)
-    std::vector<int> order;
-    for (int l = 1; l <= L; ++l) order.push_back(l);
-    std::stable_sort(order.begin(), order.end(), [&](int u, int v) {
-      return LV[u].FP * (int64_t)LV[v].nb > LV[v].FP * (int64_t)LV[u].nb;
-    });
-    FarDfArgs fa{};
-    int cta = 0;
-    for (int l : order) {
-      const DevLevel& d = LV[l];
-      if (d.FP == 0 || d.K == 0) {
-        // no couplings: yhat starts at zero
-        cudaMemsetAsync(c->ydf_h + off[l], 0, sizeof(float) * d.nb * d.K, st);
-        cudaMemsetAsync(c->ydf_l + off[l], 0, sizeof(float) * d.nb * d.K, st);
-        continue;
+    if (c->cb_ok) {
+      // the stored halves of all levels' couplings in one launch; the downward
+      // pass adds their partial products as it goes
+      float* ch = c->part32cd;
+      float* cl = ch + c->cb_part;
+      launch_matvec_sym_pairs_df(c->cb_min, c->cb_max, c->cb_n, c->cb, c->S32u_all, c->Slo_all, c->hdf_h, c->hdf_l, ch, cl, st);
+      const DevLevel& d1 = LV[1];
+      far1 = d1.FP > 0 && d1.K > 0;
+      if (far1)
+        launch_matvec_rows_df(d1.nb, d1.K, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, d1.K, d1.fs_ptr,
+                              d1.fs_ent, ch + d1.fs_poff, cl + d1.fs_poff, c->ydf_h + off[1], c->ydf_l + off[1], nullptr,
+                              0, st);
+      for (int l = 1; l < L; ++l) {
+        const DevLevel &d = LV[l], &dc = LV[l + 1];
+        const bool has = dc.FP > 0 && dc.K > 0;
+        launch_matvec_rows_df(d.nb, d.D, l == 1 && !far1 ? 0 : d.K, c->X32p[l], c->Xlo[l], c->ydf_h + off[l],
+                              c->ydf_l + off[l], nullptr, nullptr, d.D / 2, has ? dc.fs_ptr : nullptr,
+                              has ? dc.fs_ent : nullptr, ch + dc.fs_poff, cl + dc.fs_poff, c->ydf_h + off[l + 1],
+                              c->ydf_l + off[l + 1], nullptr, 0, st);
       }
-      if (fa.nlev == kMaxFarDfLevels) {
-        launch_matvec_far_df_all(fa, st);
-        fa = FarDfArgs{};
-        cta = 0;
+    } else {
+      // levels with the longest far lists first (their CTAs take longest)
+      FarDfArgs fa{};
+      int cta = 0;
+      for (int l : levels_by_far(LV, L)) {
+        const DevLevel& d = LV[l];
+        if (d.FP == 0 || d.K == 0) {
+          // no couplings: yhat starts at zero
+          cudaMemsetAsync(c->ydf_h + off[l], 0, sizeof(float) * d.nb * d.K, st);
+          cudaMemsetAsync(c->ydf_l + off[l], 0, sizeof(float) * d.nb * d.K, st);
+          continue;
+        }
+        if (fa.nlev == kMaxFarDfLevels) {
+          launch_matvec_far_df_all(fa, st);
+          fa = FarDfArgs{};
+          cta = 0;
+        }
+        FarDfLevel& f = fa.lv[fa.nlev++];
+        f = {d.far_ptr, d.far_j, c->S32p[l], c->Slo[l], c->hdf_h + off[l], c->hdf_l + off[l], c->ydf_h + off[l],
+             c->ydf_l + off[l], d.nb, d.K, (d.K + 63) / 64, cta};
+        cta += d.nb * f.nch;
       }
-      FarDfLevel& f = fa.lv[fa.nlev++];
-      f = {d.far_ptr, d.far_j, c->S32p[l], c->Slo[l], c->hdf_h + off[l], c->hdf_l + off[l], c->ydf_h + off[l],
-           c->ydf_l + off[l], d.nb, d.K, (d.K + 63) / 64, cta};
-      cta += d.nb * f.nch;
+      launch_matvec_far_df_all(fa, st);
+  for (int l = 1; l < L; ++l)
+        launch_matvec_rows_df(LV[l].nb, LV[l].D, LV[l].K, c->X32p[l], c->Xlo[l], c->ydf_h + off[l], c->ydf_l + off[l],
+                              c->ydf_h + off[l + 1], c->ydf_l + off[l + 1], LV[l].D, nullptr, nullptr, nullptr, nullptr,
+                              c->ydf_h + off[l + 1], c->ydf_l + off[l + 1], nullptr, 0, st);
     }
-    launch_matvec_far_df_all(fa, st);
-    for (int l = 1; l < L; ++l)
-      launch_matvec_down_df(LV[l], c->X32p[l], c->Xlo[l], c->ydf_h + off[l], c->ydf_l + off[l],
-                            c->ydf_h + off[l + 1], c->ydf_l + off[l + 1], st);
   }
   const float* yhh = L ? c->ydf_h + off[L] : nullptr;
   const float* yhl = L ? c->ydf_l + off[L] : nullptr;
@@ -1380,9 +1424,10 @@ void matvec_df(h2_ctx* c, const double* x, double* y) {
     // the partial products as FP32 pairs in the space of the FP64 ones
     float* ph = reinterpret_cast<float*>(c->part64);
     float* pl = ph + c->npu * 2 * lf.D;
-    launch_matvec_sym_pairs_df(lf.D, c->npu, c->sym_desc, c->A32, c->Alo, c->xdf_h, c->xdf_l, ph, pl, st);
-    launch_matvec_sym_sum_df(lf.nb, lf.D, L ? lf.K : 0, c->sym_ptr, c->sym_ent, L ? c->X32p[L] : nullptr,
-                             L ? c->Xlo[L] : nullptr, yhh, yhl, ph, pl, y, c->lv[L].D, st);
+    launch_matvec_sym_pairs_df(lf.D, lf.D, c->npu, c->sym_desc, c->A32, c->Alo, c->xdf_h, c->xdf_l, ph, pl, st);
+    launch_matvec_rows_df(lf.nb, lf.D, L == 0 || (L == 1 && !far1) ? 0 : lf.K, L ? c->X32p[L] : nullptr,
+                          L ? c->Xlo[L] : nullptr, yhh, yhl, nullptr, nullptr, lf.D, c->sym_ptr, c->sym_ent, ph, pl,
+                          nullptr, nullptr, y, c->lv[L].D, st);
   } else {
     launch_matvec_leaf_df(lf, c->A32, c->Alo, L ? c->X32p[L] : nullptr, L ? c->Xlo[L] : nullptr, c->xdf_h, c->xdf_l,
                           yhh, yhl, y, st);

@@ -396,12 +396,14 @@ struct h2_ctx {
   float *xhat32 = nullptr, *yhat32 = nullptr;
   // the stored coupling pairs of every level as one batch: the FP32 matvec
   // forms all levels' coupling products in one launch (cb: one descriptor per
-  // pair; cb_max the largest rank)
+  // pair; cb_min and cb_max the smallest and largest rank)
   bool cb_ok = false;
-  int cb_max = 0;
+  int cb_min = 0, cb_max = 0;
   int64_t cb_n = 0;
   h2::SymPair *sym_desc = nullptr, *cb = nullptr;
-  float* S32u_all = nullptr;
+  float *S32u_all = nullptr, *Slo_all = nullptr;  // hi and lo parts
+  float* part32cd = nullptr;  // coupling partial products in FP32 pairs (cb_part each)
+  int64_t cb_part = 0;
   std::vector<double*> X64p, S64p;  // per-level pointers (index l; [0] unused)
   std::vector<float*> X32p, S32p;
   std::vector<int64_t> hat_off;  // per-level offsets into xhat / yhat

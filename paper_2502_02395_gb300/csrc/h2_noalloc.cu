@@ -99,16 +99,26 @@ extern "C" h2_status h2_matvec_noalloc(h2_ctx* c, const double* x, double* y) {
   double* yh = xh + nhat;    // downward skeleton coefficients, per level
   cudaStream_t st = c->stream;
   h2::launch_gather(c->slot_pt, x, xt, (int64_t)nslot, st);
-  if (L == 0) {
-    h2::launch_matvec_leaf<double>(c->lv[0], c->A64, nullptr, xt, nullptr, yt, st);
-  } else {
-    const std::vector<int64_t>& off = c->hat_off;
-    h2::launch_matvec_up<double>(c->lv[L], c->lv[L].X, xt, xh + off[L], st);
+  const std::vector<int64_t>& off = c->hat_off;
+  h2::BlockRowArgs<double> la{}, fa{};
+  la.nlev = 1;
+  la.lv[0] = {lf.near_ptr, lf.near_j, c->A64, xt, L ? lf.X : nullptr, L ? yh + off[L] : nullptr, yt, lf.nb, lf.D,
+              L ? lf.K : 0};
+  if (L >= 1) {
+    h2::launch_matvec_up<double>(lf, lf.X, xt, xh + off[L], st);
     for (int l = L - 1; l >= 1; --l) h2::launch_matvec_up<double>(c->lv[l], c->lv[l].X, xh + off[l + 1], xh + off[l], st);
-    for (int l = 1; l <= L; ++l) h2::launch_matvec_far<double>(c->lv[l], c->lv[l].S, xh + off[l], yh + off[l], st);
-    for (int l = 1; l < L; ++l) h2::launch_matvec_down<double>(c->lv[l], c->lv[l].X, yh + off[l], yh + off[l + 1], st);
-    h2::launch_matvec_leaf<double>(c->lv[L], c->A64, c->lv[L].X, xt, yh + off[L], yt, st);
+    for (int l = L; l >= 1; --l) {
+      const h2::DevLevel& d = c->lv[l];
+      if (d.K > 0) fa.lv[fa.nlev++] = {d.far_ptr, d.far_j, d.S, xh + off[l], nullptr, nullptr, yh + off[l], d.nb, d.K, 0};
+    }
+    h2::launch_matvec_block_rows<double>(fa, st);
+    for (int l = 1; l < L; ++l) {
+      const h2::DevLevel& d = c->lv[l];
+      h2::launch_matvec_rows<double>(d.nb, d.D, d.K, d.X, yh + off[l], yh + off[l + 1], yh + off[l + 1], d.D, nullptr,
+                                     nullptr, nullptr, true, st);
+    }
   }
+  h2::launch_matvec_block_rows<double>(la, st);
   h2::launch_scatter(c->slot_pt, yt, y, (int64_t)nslot, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

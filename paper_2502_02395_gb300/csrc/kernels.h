@@ -162,12 +162,29 @@ void launch_transpose_blocks(int64_t nb, int D, const T* in, T* out, cudaStream_
 
 template <typename T>
 void launch_matvec_up(const DevLevel& L, const T* X, const T* x, T* xh, cudaStream_t st);
+// out rows = base + X yh + sums of partial products (see mv_rows_kernel)
 template <typename T>
-void launch_matvec_far(const DevLevel& L, const T* S, const T* xh, T* yh, cudaStream_t st);
+void launch_matvec_rows(int nb, int D, int K, const T* X, const T* yh, const T* base, T* out, int seg,
+                        const int64_t* ptr, const int32_t* ent, const T* part, bool pdl, cudaStream_t st);
+// Block rows of several levels in one launch (see mv_block_rows_kernel): per
+// level nb boxes of n rows, lists ptr / fj, blocks M, input x, basis X (n x K
+// with coefficients yh, or NULL), output; nch and cta0 are the launcher's.
 template <typename T>
-void launch_matvec_down(const DevLevel& L, const T* X, const T* yh, T* yh_child, cudaStream_t st);
+struct BlockRowLevel {
+  const int64_t* ptr;
+  const int32_t* fj;
+  const T *M, *x, *X, *yh;
+  T* out;
+  int nb, n, K, nch, cta0;
+};
+constexpr int kMaxRowLevels = 32;
 template <typename T>
-void launch_matvec_leaf(const DevLevel& L, const T* A, const T* X, const T* x, const T* yh, T* y, cudaStream_t st);
+struct BlockRowArgs {
+  int nlev;
+  BlockRowLevel<T> lv[kMaxRowLevels];
+};
+template <typename T>
+void launch_matvec_block_rows(BlockRowArgs<T> a, cudaStream_t st);
 // The FP64 matvec with each FP64 matrix held as an FP32 pair (hi = fl32, lo
 // = fl32 of the rest) and FP32-pair arithmetic throughout: the input vector
 // is split once (launch_split_df), the basis coefficients xhat / yhat of
@@ -192,17 +209,15 @@ struct FarDfArgs {
   FarDfLevel lv[kMaxFarDfLevels];
 };
 void launch_matvec_far_df_all(const FarDfArgs& a, cudaStream_t st);
-// down: [yhat_2p; yhat_2p+1] += X_p yhat_p
-void launch_matvec_down_df(const DevLevel& L, const float* Xh, const float* Xl, const float* yh, const float* yl,
-                           float* ych, float* ycl, cudaStream_t st);
+// rows in pairs (see mv_rows_kernel and RowsDf): out = base + X yh + sums of
+// partial products; as pairs into oh / ol, or as FP64 into y (ny rows a box)
+void launch_matvec_rows_df(int nb, int D, int K, const float* Xh, const float* Xl, const float* yhh, const float* yhl,
+                           const float* bh, const float* bl, int seg, const int64_t* ptr, const int32_t* ent,
+                           const float* ph, const float* pl, float* oh, float* ol, double* y, int ny, cudaStream_t st);
 // leaf, general near lists: y_i = X_i yhat_i + sum_{near j} A_ij x_j
 void launch_matvec_leaf_df(const DevLevel& L, const float* Ah, const float* Al, const float* Xh, const float* Xl,
                            const float* xh, const float* xl, const float* yhh, const float* yhl, double* y,
                            cudaStream_t st);
-// leaf, symmetric storage: y_i = X_i yhat_i + box i's partial products
-void launch_matvec_sym_sum_df(int nb, int D, int K, const int64_t* ptr, const int32_t* ent, const float* Xh,
-                              const float* Xl, const float* yhh, const float* yhl, const float* ph, const float* pl,
-                              double* y, int ny, cudaStream_t st);  // ny: rows of a box in y (the rest is padding)
 // h = fl32(v), l = fl32(v - h); v has n entries in segments of p.len, h and l
 // nb segments of p.str (the rest zero)
 void launch_split_df(const double* v, float* h, float* l, int64_t n, PadSeg p, cudaStream_t st);
@@ -210,22 +225,14 @@ void launch_split_df(const double* v, float* h, float* l, int64_t n, PadSeg p, c
 // per stored pair k = (ui[k], uj[k]) the partial products [A x_j; A^T x_i]
 // into part (2 D per pair), then per box y = X yh + its partial products.
 bool sym_supported(int n);  // n a multiple of 4, at most 256
-// Downward step [yh_2p; yh_2p+1] = X_p yh_p + (the children's coupling
-// products summed over their CSR lists cptr / cent into part, Kc = D / 2
-// entries per product; cptr NULL: none)
-template <typename T>
-void launch_matvec_down_far(const DevLevel& L, const T* X, const T* yh, T* yh_child, const int64_t* cptr,
-                            const int32_t* cent, const T* part, cudaStream_t st);
 // (pdl: launched to overlap its predecessor; off where events bracket it)
-// (max_n: the largest block, a multiple of 4 up to 256)
-void launch_matvec_sym_pairs(int max_n, int64_t npu, const SymPair* desc, const float* A, const float* x, float* part,
-                             bool pdl, cudaStream_t st, const GmState* state = nullptr,
+// (min_n, max_n: the smallest and largest block, multiples of 4 up to 256)
+void launch_matvec_sym_pairs(int min_n, int max_n, int64_t npu, const SymPair* desc, const float* A, const float* x,
+                             float* part, bool pdl, cudaStream_t st, const GmState* state = nullptr,
                              unsigned long long* stamp = nullptr);  // (times of iteration state->j)
-void launch_matvec_sym_pairs_df(int D, int64_t npu, const SymPair* desc, const float* Ah, const float* Al,
-                                const float* xh, const float* xl, float* ph, float* pl, cudaStream_t st);
-template <typename T>
-void launch_matvec_sym_sum(int nb, int D, int K, const int64_t* ptr, const int32_t* ent, const T* X, const T* yh,
-                           const T* part, T* y, cudaStream_t st, bool pdl = true);
+void launch_matvec_sym_pairs_df(int min_n, int max_n, int64_t npu, const SymPair* desc, const float* Ah,
+                                const float* Al, const float* xh, const float* xl, float* ph, float* pl,
+                                cudaStream_t st);
 // FP32 copies of nblk blocks (block k from in[idx[k]], or in[k]): a block of
 // rows x cols entries whose logical rows and columns lie at rs and cs, zeros
 // elsewhere; hi = fl32(v) and, lo non-NULL, lo = fl32(v - hi).  di / dj

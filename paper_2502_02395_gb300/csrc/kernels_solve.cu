@@ -1596,6 +1596,13 @@ __global__ void __launch_bounds__(256, sizeof(TS) == 8 ? 1 : 2) box_cluster_kern
   };
   int64_t p = q0 + first;
   if (p < q1) load(p, 0);
+  // the blocks of its later pairs on their way to L2 meanwhile
+  for (int64_t pn = p + step; pn < q1; pn += step) {
+    const char* M = reinterpret_cast<const char*>(a.Ahat + pn * D * D + off);
+    const int lines = (nc * (int)sizeof(TS) + 127) / 128;
+    for (int e = tid; e < nr * lines; e += blockDim.x)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(M + (int64_t)(e / lines) * D * sizeof(TS) + (e % lines) * 128));
+  }
   int j = p < q1 ? a.nj[p] : 0;
   griddep_wait();
   griddep_launch_next();
@@ -1819,175 +1826,278 @@ H2_INST_SUBST(float, __nv_bfloat16)
 // solver of the mixed-precision refinement.  X, S and A are that level's
 // bases, couplings and leaf near blocks in T.
 
-// upward: xh_i[a] = sum_d X_i[d*K + a] x_i[d] (x_i: the box's D inputs):
-// the column form of the CTA GEMV (warps over d, lanes over 16-byte chunks
-// of a, eight rows of X in flight per lane).
+// upward: xh_i[a] = sum_d X_i[d*K + a] x_i[d] (x_i: the box's D inputs).  A
+// box's rows d are split over a cluster of CS CTAs: each brings its rows into
+// shared memory with cp.async before it waits for the previous level, forms
+// the K partial sums (warps over rows, lanes over 16-byte chunks of a), and
+// the CTAs' sums meet in the CTA that owns the output (distributed shared
+// memory, added in rank order).  Bound by latency on small levels: with one
+// CTA per box a level of 64 boxes or fewer took 8 us (128 KB through one SM),
+// and by HBM on large ones.
 template <typename T>
-__global__ void __launch_bounds__(256) mv_up_kernel(int D, int K, const T* __restrict__ X, const T* __restrict__ x,
-                                                    T* __restrict__ xh, int pf) {
+__global__ void __launch_bounds__(256) mv_up_kernel(int D, int K, int CS, const T* __restrict__ X,
+                                                    const T* __restrict__ x, T* __restrict__ xh) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr int VN = 16 / sizeof(T);
+  const int rank = blockIdx.x % CS, i = blockIdx.x / CS, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = (D + CS - 1) / CS, d0 = min(rank * per, D), m = min(per, D - d0), kper = (K + CS - 1) / CS;
+  T* rows = reinterpret_cast<T*>(smraw);  // per x K
+  T* part = rows + (((size_t)per * K + 3) & ~(size_t)3);  // 8 x K
+  T* got = part + 8 * K;                  // CS x kper
+  T* sx = got + CS * kper;                // per
+  if (CS > 1) cluster_arrive();
+  const T* src = X + ((int64_t)i * D + d0) * K;
+  const bool vec = K % VN == 0;
+  if (vec) cp_async_bytes(rows, src, m * K * (int)sizeof(T));
+  else
+    for (int e = tid; e < m * K; e += 256) rows[e] = __ldg(src + e);
+  griddep_wait();
+  griddep_launch_next();
+  for (int e = tid; e < m; e += 256) sx[e] = x[(int64_t)i * D + d0 + e];
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  if (vec) {
+    for (int k0 = lane * VN; k0 < K; k0 += 32 * VN) {
+      T acc[VN];
+#pragma unroll
+      for (int e = 0; e < VN; ++e) acc[e] = T(0);
+#pragma unroll 4
+      for (int n = warp; n < m; n += 8) {
+        T v[VN];
+        Chunk<T>::cvt(*reinterpret_cast<const uint4*>(rows + (size_t)n * K + k0), v);
+        const T xn = sx[n];
+#pragma unroll
+        for (int e = 0; e < VN; ++e) acc[e] = fma(v[e], xn, acc[e]);
+      }
+#pragma unroll
+      for (int e = 0; e < VN; ++e) part[warp * K + k0 + e] = acc[e];
+    }
+  } else {
+    for (int k = lane; k < K; k += 32) {
+      T acc = T(0);
+      for (int n = warp; n < m; n += 8) acc = fma(rows[(size_t)n * K + k], sx[n], acc);
+      part[warp * K + k] = acc;
+    }
+  }
+  __syncthreads();
+  if (CS > 1) cluster_wait();
+  for (int k = tid; k < K; k += 256) {
+    T t = T(0);
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += part[w * K + k];
+    if (CS == 1) xh[(int64_t)i * K + k] = t;
+    else st_cluster(cluster_map(&got[rank * kper + k % kper], k / kper), t);
+  }
+  if (CS == 1) return;
+  cluster_sync();
+  for (int k = tid; k < kper && rank * kper + k < K; k += 256) {
+    T t = T(0);
+    for (int g = 0; g < CS; ++g) t += got[g * kper + k];
+    xh[(int64_t)i * K + rank * kper + k] = t;
+  }
+}
+// the general form (blocks beyond a cluster's shared memory): one CTA a box
+template <typename T>
+__global__ void __launch_bounds__(256) mv_up_big_kernel(int D, int K, const T* __restrict__ X,
+                                                        const T* __restrict__ x, T* __restrict__ xh) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* part = reinterpret_cast<T*>(smraw);  // 8 * K
   T* sx = part + 8 * K;                   // D
   const int i = blockIdx.x, tid = threadIdx.x;
-  if (pf) prefetch_l2(X + (int64_t)i * D * K, (int64_t)D * K * sizeof(T));
   griddep_wait();
   griddep_launch_next();
   for (int e = tid; e < D; e += 256) sx[e] = x[(int64_t)i * D + e];
   __syncthreads();
   cta_gemv_cols<T, T>(X + (int64_t)i * D * K, K, K, D, sx, part, xh + (int64_t)i * K);
 }
+// Launch with clusters of CS CTAs and programmatic stream serialization.
+template <typename... KArgs, typename... Args>
+static void launch_pdl_cluster(void (*kern)(KArgs...), unsigned grid, int CS, size_t smem, cudaStream_t st,
+                               Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)CS;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  set_smem((const void*)kern, smem);
+  ++g_launches;
+  cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+// CTAs per box for a D x K basis of esz-byte entries: slices of at most 32 KB,
+// doubled while the level leaves room for two CTAs per SM; 0: no cluster form
+static int up_ctas(int nb, int D, int K, size_t esz) {
+  int CS = 1;
+  while (CS < 8 && (size_t)((D + CS - 1) / CS) * K * esz > 32 * 1024) CS *= 2;
+  if ((size_t)((D + CS - 1) / CS) * K * esz > 96 * 1024) return 0;
+  while (CS < 8 && nb * CS * 2 <= 2 * num_sms()) CS *= 2;
+  return CS;
+}
 template <typename T>
 void launch_matvec_up(const DevLevel& L, const T* X, const T* x, T* xh, cudaStream_t st) {
-  const size_t sm = sizeof(T) * (8 * (size_t)L.K + L.D);
-  set_smem((const void*)mv_up_kernel<T>, sm);
-  launch_pdl(mv_up_kernel<T>, L.nb, 256, sm, st, L.D, L.K, X, x, xh, small_level(L.nb) ? 1 : 0);
-}
-
-// couplings: yh_i = sum_{far j} S_f xh_j   (overwrites yh_i)
-template <typename T>
-__global__ void __launch_bounds__(256, 2) mv_far_kernel(int K, const int64_t* __restrict__ ptr,
-                                                        const int32_t* __restrict__ fj, const T* __restrict__ S,
-                                                        const T* __restrict__ xh, T* __restrict__ yh) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  T* smv = reinterpret_cast<T*>(smraw);  // nf * K
-  const int i = blockIdx.x, tid = threadIdx.x;
-  const int64_t p0 = ptr[i];
-  const int nf = (int)(ptr[i + 1] - p0);
-  griddep_wait();
-  griddep_launch_next();
-  for (int e = tid; e < nf * K; e += blockDim.x) smv[e] = xh[(int64_t)fj[p0 + e / K] * K + e % K];
-  __syncthreads();
-  T acc[kRPW];
-  for (int r0 = 0; r0 < K; r0 += kChunk) {
-    zero(acc);
-    for (int q = 0; q < nf; ++q) rows_acc<T, kRPW>(r0, S + (p0 + q) * K * K, K, K, K, smv + q * K, acc);
-    rows_finish<T, kRPW>(r0, K, acc, T(1), nullptr, yh + (int64_t)i * K);
+  const int D = L.D, K = L.K, CS = up_ctas(L.nb, D, K, sizeof(T));
+  if (CS == 0) {
+    const size_t sm = sizeof(T) * (8 * (size_t)K + D);
+    set_smem((const void*)mv_up_big_kernel<T>, sm);
+    launch_pdl(mv_up_big_kernel<T>, L.nb, 256, sm, st, D, K, X, x, xh);
+    return;
   }
-}
-template <typename T>
-void launch_matvec_far(const DevLevel& L, const T* S, const T* xh, T* yh, cudaStream_t st) {
-  size_t sm = sizeof(T) * (size_t)L.K * std::max(L.max_far, 1);
-  set_smem((const void*)mv_far_kernel<T>, sm);
-  launch_pdl(mv_far_kernel<T>, L.nb, 256, sm, st, L.K, L.far_ptr, L.far_j, S, xh, yh);
+  const int per = (D + CS - 1) / CS, kper = (K + CS - 1) / CS;
+  const size_t sm = sizeof(T) * ((((size_t)per * K + 3) & ~(size_t)3) + 8 * (size_t)K + (size_t)CS * kper + per);
+  launch_pdl_cluster(mv_up_kernel<T>, (unsigned)(L.nb * CS), CS, sm, st, D, K, CS, X, x, xh);
 }
 
-// downward: [yh_2p; yh_2p+1] += X_p yh_p   (rows d of X_p, D = 2 Kc): a
-// block-row GEMV per parent box
+// The rows of [X_p yh_p] plus sums of partial products: box p's output row r is
+//   base[p D + r] + sum_k X_p[r][k] yh_p[k] + the products of the list of its
+//   part c = p D / seg + r / seg (CSR ptr / ent: product e starts at e seg of
+//   part), entry r % seg.
+// seg = D: a leaf and its near products (every box one list); seg = D / 2: the
+// downward step into the two children and their coupling products.  The rows
+// are split over CTAs (32 or 64 each); a CTA brings its rows of X into shared
+// memory with cp.async before it waits, and adds a row's products with 256 /
+// 32 (or / 64) threads.  One CTA per box took 5 us a level and 11 us for 64
+// leaves.
 template <typename T>
-__global__ void __launch_bounds__(256, 2) mv_down_kernel(int D, int K, const T* __restrict__ X,
-                                                         const T* __restrict__ yh, T* __restrict__ yhc, int pf) {
+__global__ void __launch_bounds__(256) mv_rows_kernel(int D, int K, int ns, int per, const T* __restrict__ X,
+                                                      const T* __restrict__ yh, const T* base, T* out, int seg,
+                                                      const int64_t* __restrict__ ptr, const int32_t* __restrict__ ent,
+                                                      const T* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  T* sy = reinterpret_cast<T*>(smraw);  // K
-  const int p = blockIdx.x;
-  if (pf) prefetch_l2(X + (int64_t)p * D * K, (int64_t)D * K * sizeof(T));
-  griddep_wait();
-  griddep_launch_next();
-  for (int e = threadIdx.x; e < K; e += 256) sy[e] = yh[(int64_t)p * K + e];
-  __syncthreads();
-  T acc[kRPW];
-  T* out = yhc + (int64_t)p * D;
-  for (int r0 = 0; r0 < D; r0 += kChunk) {
-    zero(acc);
-    rows_acc<T, kRPW>(r0, X + (int64_t)p * D * K, K, D, K, sy, acc);
-    rows_finish<T, kRPW>(r0, D, acc, T(1), out, out);
+  constexpr int VN = 16 / sizeof(T);
+  const int p = blockIdx.x / ns, r0 = (blockIdx.x % ns) * per, m = min(per, D - r0), tid = threadIdx.x;
+  T* rows = reinterpret_cast<T*>(smraw);                  // per x K
+  T* sy = rows + (((size_t)per * K + 3) & ~(size_t)3);    // K
+  T* f = sy + ((K + 3) & ~3);                             // 256
+  const bool vec = K % VN == 0;
+  const T* src = X + ((int64_t)p * D + r0) * K;
+  if (vec) cp_async_bytes(rows, src, m * K * (int)sizeof(T));
+  else
+    for (int e = tid; e < m * K; e += 256) rows[e] = __ldg(src + e);
+  const int pr = per <= 32 ? 32 : 64, r = tid & (pr - 1), g = tid / pr, ng = 256 / pr;
+  int64_t e0 = 0, e1 = 0;
+  int rr = 0;
+  if (ptr && r < m) {
+    const int c = p * (D / seg) + (r0 + r) / seg;
+    rr = (r0 + r) % seg;
+    e0 = ptr[c] + g, e1 = ptr[c + 1];
   }
-}
-template <typename T>
-void launch_matvec_down(const DevLevel& L, const T* X, const T* yh, T* yh_child, cudaStream_t st) {
-  launch_pdl(mv_down_kernel<T>, L.nb, 256, sizeof(T) * ((L.K + 3) & ~3), st, L.D, L.K, X, yh, yh_child,
-             small_level(L.nb) ? 1 : 0);
-}
-
-// downward step that also adds the children's coupling products:
-// [yh_2p; yh_2p+1] = X_p yh_p + f, f[h Kc + r] = sum over the partial
-// products of child c = 2p + h (CSR cptr / cent over the child level; entry
-// e = 2k (+1) is part[(2k (+1)) Kc ..]).  cptr NULL: f = 0.  Overwrites the
-// children's yh (the per-level sums of the coupling products are folded in).
-template <typename T>
-__global__ void __launch_bounds__(256, 2) mv_down_far_kernel(int D, int K, const T* __restrict__ X,
-                                                             const T* __restrict__ yh, T* __restrict__ yhc,
-                                                             const int64_t* __restrict__ cptr,
-                                                             const int32_t* __restrict__ cent,
-                                                             const T* __restrict__ part, int pf) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  T* sy = reinterpret_cast<T*>(smraw);  // K
-  T* sf = sy + ((K + 3) & ~3);          // D
-  const int p = blockIdx.x;
-  const int Kc = D / 2;
-  if (pf) prefetch_l2(X + (int64_t)p * D * K, (int64_t)D * K * sizeof(T));
   griddep_wait();
   griddep_launch_next();
-  for (int e = threadIdx.x; e < K; e += 256) sy[e] = yh[(int64_t)p * K + e];
-  for (int r = threadIdx.x; r < D; r += 256) {
-    T s = T(0);
-    if (cptr) {
-      const int c = 2 * p + r / Kc, rr = r % Kc;
-      for (int64_t q = cptr[c]; q < cptr[c + 1]; ++q) s += part[(int64_t)cent[q] * Kc + rr];
+  for (int e = tid; e < K; e += 256) sy[e] = yh[(int64_t)p * K + e];
+  T t = T(0);
+  int64_t q = e0;
+  for (; q + 3 * ng < e1; q += 4 * ng) {
+    T v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = part[(int64_t)ent[q + u * ng] * seg + rr];
+    t += (v[0] + v[1]) + (v[2] + v[3]);
+  }
+  for (; q < e1; q += ng) t += part[(int64_t)ent[q] * seg + rr];
+  if (g == 0 && base && r < m) t += base[(int64_t)p * D + r0 + r];
+  f[tid] = t;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  auto finish = [&](int row, T v) {
+    for (int h = 0; h < ng; ++h) v += f[h * pr + row];
+    out[(int64_t)p * D + r0 + row] = v;
+  };
+  if (K == 0) {
+    if (tid < m) finish(tid, T(0));
+  } else if (vec) {
+    smem_rows<T>(rows, m, K, sy, finish);
+  } else {
+    const int lane = tid & 31;
+    for (int row = tid >> 5; row < m; row += 8) {
+      T v = T(0);
+      for (int k = lane; k < K; k += 32) v = fma(rows[(size_t)row * K + k], sy[k], v);
+      v = warp_sum(v);
+      if (lane == 0) finish(row, v);
     }
-    sf[r] = s;
   }
-  __syncthreads();
-  T acc[kRPW];
-  T* out = yhc + (int64_t)p * D;
-  for (int r0 = 0; r0 < D; r0 += kChunk) {
-    zero(acc);
-    rows_acc<T, kRPW>(r0, X + (int64_t)p * D * K, K, D, K, sy, acc);
-    rows_finish<T, kRPW>(r0, D, acc, T(1), sf, out);
-  }
+}
+// rows per CTA: 32 for 8-byte entries and while that fills at most about four
+// CTAs per SM, else 64;
+// fewer where a slice of X would not fit shared memory
+static int rows_per(int nb, int D, int K, size_t esz) {
+  int per = esz == 8 || (int64_t)nb * ((D + 31) / 32) <= 4 * num_sms() ? 32 : 64;
+  while (per > 8 && (size_t)per * K * esz > 160 * 1024) per /= 2;
+  return std::min(per, std::max(D, 1));
 }
 template <typename T>
-void launch_matvec_down_far(const DevLevel& L, const T* X, const T* yh, T* yh_child, const int64_t* cptr,
-                            const int32_t* cent, const T* part, cudaStream_t st) {
-  const size_t sm = sizeof(T) * ((size_t)((L.K + 3) & ~3) + L.D);
-  launch_pdl(mv_down_far_kernel<T>, L.nb, 256, sm, st, L.D, L.K, X, yh, yh_child, cptr, cent, part,
-             small_level(L.nb) ? 1 : 0);
+void launch_matvec_rows(int nb, int D, int K, const T* X, const T* yh, const T* base, T* out, int seg,
+                        const int64_t* ptr, const int32_t* ent, const T* part, bool pdl, cudaStream_t st) {
+  const int per = rows_per(nb, D, K, sizeof(T)), ns = (D + per - 1) / per;
+  const size_t sm = sizeof(T) * ((((size_t)per * K + 3) & ~(size_t)3) + ((K + 3) & ~3) + 256);
+  set_smem((const void*)mv_rows_kernel<T>, sm);
+  if (pdl) {
+    launch_pdl(mv_rows_kernel<T>, (unsigned)(nb * ns), 256, sm, st, D, K, ns, per, X, yh, base, out, seg, ptr, ent, part);
+  } else {
+    ++g_launches;
+    mv_rows_kernel<T><<<(unsigned)(nb * ns), 256, sm, st>>>(D, K, ns, per, X, yh, base, out, seg, ptr, ent, part);
+  }
 }
-template void launch_matvec_down_far<float>(const DevLevel&, const float*, const float*, float*, const int64_t*,
-                                            const int32_t*, const float*, cudaStream_t);
+template void launch_matvec_rows<float>(int, int, int, const float*, const float*, const float*, float*, int,
+                                        const int64_t*, const int32_t*, const float*, bool, cudaStream_t);
+template void launch_matvec_rows<double>(int, int, int, const double*, const double*, const double*, double*, int,
+                                         const int64_t*, const int32_t*, const double*, bool, cudaStream_t);
 
-// leaf: y_i = X_i yh_i + sum_{near j} A_ij x_j
-template <typename T>
-__global__ void __launch_bounds__(256, 2) mv_leaf_kernel(int D, int K, const int64_t* __restrict__ ptr,
-                                                         const int32_t* __restrict__ nj, const T* __restrict__ A,
-                                                         const T* __restrict__ X, const T* __restrict__ x,
-                                                         const T* __restrict__ yh, T* __restrict__ y) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  T* smv = reinterpret_cast<T*>(smraw);  // K (rounded up to 16 bytes) + nn * D
-  const int i = blockIdx.x, tid = threadIdx.x;
-  const int64_t p0 = ptr[i];
-  const int nn = (int)(ptr[i + 1] - p0);
-  const int kpad = (K + 3) & ~3;
+// Block rows of one or several levels in one launch: CTA (box i of level l,
+// rows 8 RPW c .. 8 RPW (c + 1) - 1) forms those rows of out_i = X_i yh_i (X NULL: 0) +
+// sum_q M_q x_j(q) over the box's list.  The couplings of all levels
+// (M = S, x = xhat), or the leaf near blocks (M = A).  Bound by the FP64 pipe
+// in FP64 (two flops an entry at about 1.75 multiply-adds per clock and SM)
+// and by HBM in FP32; one CTA per box left levels of few boxes to a few SMs
+// (N = 65536: the couplings' eight launches took 1.1 ms a product, 0.96 ms the
+// leaf).  64 rows a CTA, or 16 while that leaves SMs without one.
+template <typename T, int RPW>
+__global__ void __launch_bounds__(256, 2) mv_block_rows_kernel(const __grid_constant__ BlockRowArgs<T> a) {
+  const int b = blockIdx.x;
+  int l = 0;
+  while (l + 1 < a.nlev && b >= a.lv[l + 1].cta0) ++l;
+  const BlockRowLevel<T>& f = a.lv[l];
+  const int loc = b - f.cta0, i = loc / f.nch, r0 = (loc % f.nch) * 8 * RPW;
+  const int64_t p0 = f.ptr[i], p1 = f.ptr[i + 1];
+  const int n = f.n;
+  T acc[RPW];
+  zero(acc);
   griddep_wait();
   griddep_launch_next();
-  T* sh = smv;
-  T* sx = smv + kpad;
-  if (yh)
-    for (int e = tid; e < K; e += blockDim.x) sh[e] = yh[(int64_t)i * K + e];
-  for (int e = tid; e < nn * D; e += blockDim.x) sx[e] = x[(int64_t)nj[p0 + e / D] * D + e % D];
-  __syncthreads();
-  T acc[kRPW];
-  for (int r0 = 0; r0 < D; r0 += kChunk) {
-    zero(acc);
-    if (yh) rows_acc<T, kRPW>(r0, X + (int64_t)i * D * K, K, D, K, sh, acc);
-    for (int q = 0; q < nn; ++q) rows_acc<T, kRPW>(r0, A + (p0 + q) * D * D, D, D, D, sx + q * D, acc);
-    rows_finish<T, kRPW>(r0, D, acc, T(1), nullptr, y + (int64_t)i * D);
-  }
+  if (f.X) rows_acc<T, RPW>(r0, f.X + (int64_t)i * n * f.K, f.K, n, f.K, f.yh + (int64_t)i * f.K, acc);
+  for (int64_t q = p0; q < p1; ++q) rows_acc<T, RPW>(r0, f.M + q * n * n, n, n, n, f.x + (int64_t)f.fj[q] * n, acc);
+  rows_finish<T, RPW>(r0, n, acc, T(1), nullptr, f.out + (int64_t)i * n);
 }
 template <typename T>
-void launch_matvec_leaf(const DevLevel& L, const T* A, const T* X, const T* x, const T* yh, T* y, cudaStream_t st) {
-  const size_t sm = sizeof(T) * ((size_t)((L.K + 3) & ~3) + (size_t)L.D * L.max_near);
-  set_smem((const void*)mv_leaf_kernel<T>, sm);
-  ++g_launches;
-  mv_leaf_kernel<T><<<L.nb, 256, sm, st>>>(L.D, L.K, L.near_ptr, L.near_j, A, X, x, yh, y);
+void launch_matvec_block_rows(BlockRowArgs<T> a, cudaStream_t st) {
+  auto lay = [&](int rows) {
+    int cta = 0;
+    for (int l = 0; l < a.nlev; ++l) {
+      a.lv[l].nch = (a.lv[l].n + rows - 1) / rows;
+      a.lv[l].cta0 = cta;
+      cta += a.lv[l].nb * a.lv[l].nch;
+    }
+    return cta;
+  };
+  int cta = lay(64);
+  if (cta == 0) return;
+  if (cta >= 2 * num_sms()) {
+    launch_pdl(mv_block_rows_kernel<T, 8>, (unsigned)cta, 256, 0, st, a);
+  } else {
+    cta = lay(16);
+    launch_pdl(mv_block_rows_kernel<T, 2>, (unsigned)cta, 256, 0, st, a);
+  }
 }
+template void launch_matvec_block_rows<float>(BlockRowArgs<float>, cudaStream_t);
+template void launch_matvec_block_rows<double>(BlockRowArgs<double>, cudaStream_t);
 
-#define H2_INST_MV(T)                                                                                           \
-  template void launch_matvec_up<T>(const DevLevel&, const T*, const T*, T*, cudaStream_t);                      \
-  template void launch_matvec_far<T>(const DevLevel&, const T*, const T*, T*, cudaStream_t);                     \
-  template void launch_matvec_down<T>(const DevLevel&, const T*, const T*, T*, cudaStream_t);                    \
-  template void launch_matvec_leaf<T>(const DevLevel&, const T*, const T*, const T*, const T*, T*, cudaStream_t);
-H2_INST_MV(double)
-H2_INST_MV(float)
+template void launch_matvec_up<double>(const DevLevel&, const double*, const double*, double*, cudaStream_t);
+template void launch_matvec_up<float>(const DevLevel&, const float*, const float*, float*, cudaStream_t);
 
 // ---------------------------------------------------- FP64 by FP32 pairs ---
 // The FP64 matvec of the mixed refinement's residual, on GB300's FP32 units:
@@ -2278,12 +2388,80 @@ __global__ void __launch_bounds__(256, 2) mv_up_df_kernel(int D, int K, const fl
     ol[(int64_t)i * K + m] = L;
   }
 }
+// The same over a cluster of CS CTAs per box, as mv_up_kernel.
+__global__ void __launch_bounds__(256) mv_up_df_cl_kernel(int D, int K, int CS, const float* __restrict__ Xh,
+                                                          const float* __restrict__ Xl, const float* __restrict__ zh,
+                                                          const float* __restrict__ zl, float* __restrict__ oh,
+                                                          float* __restrict__ ol) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int rank = blockIdx.x % CS, i = blockIdx.x / CS, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = (D + CS - 1) / CS, d0 = min(rank * per, D), m = min(per, D - d0), kper = (K + CS - 1) / CS;
+  float* rh = reinterpret_cast<float*>(smraw);  // per x K (K a multiple of 4)
+  float* rl = rh + (size_t)per * K;
+  float* ph = rl + (size_t)per * K;  // 8 x K
+  float* pl = ph + 8 * K;
+  float* gh = pl + 8 * K;            // CS x kper
+  float* gl = gh + CS * kper;
+  float* sh = gl + CS * kper;        // per
+  float* sl = sh + per;
+  if (CS > 1) cluster_arrive();
+  const int64_t off = ((int64_t)i * D + d0) * K;
+  cp_async_bytes(rh, Xh + off, m * K * 4);
+  cp_async_bytes(rl, Xl + off, m * K * 4);
+  griddep_wait();
+  griddep_launch_next();
+  for (int e = tid; e < m; e += 256) sh[e] = zh[(int64_t)i * D + d0 + e], sl[e] = zl[(int64_t)i * D + d0 + e];
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  for (int k0 = lane * 4; k0 < K; k0 += 128) {
+    float H[4] = {0.f, 0.f, 0.f, 0.f}, L[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int n = warp; n < m; n += 8) {
+      const float4 vh = *reinterpret_cast<const float4*>(rh + (size_t)n * K + k0);
+      const float4 vl = *reinterpret_cast<const float4*>(rl + (size_t)n * K + k0);
+      const float a = sh[n], b = sl[n];
+      df_fma(H[0], L[0], vh.x, vl.x, a, b);
+      df_fma(H[1], L[1], vh.y, vl.y, a, b);
+      df_fma(H[2], L[2], vh.z, vl.z, a, b);
+      df_fma(H[3], L[3], vh.w, vl.w, a, b);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) ph[warp * K + k0 + e] = H[e], pl[warp * K + k0 + e] = L[e];
+  }
+  __syncthreads();
+  if (CS > 1) cluster_wait();
+  for (int k = tid; k < K; k += 256) {
+    float H = ph[k], L = pl[k];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) df_add(H, L, ph[w * K + k], pl[w * K + k]);
+    if (CS == 1) {
+      oh[(int64_t)i * K + k] = H, ol[(int64_t)i * K + k] = L;
+    } else {
+      st_cluster(cluster_map(&gh[rank * kper + k % kper], k / kper), H);
+      st_cluster(cluster_map(&gl[rank * kper + k % kper], k / kper), L);
+    }
+  }
+  if (CS == 1) return;
+  cluster_sync();
+  for (int k = tid; k < kper && rank * kper + k < K; k += 256) {
+    float H = gh[k], L = gl[k];
+    for (int g = 1; g < CS; ++g) df_add(H, L, gh[g * kper + k], gl[g * kper + k]);
+    oh[(int64_t)i * K + rank * kper + k] = H, ol[(int64_t)i * K + rank * kper + k] = L;
+  }
+}
 void launch_matvec_up_df(const DevLevel& L, const float* Xh, const float* Xl, const float* zh, const float* zl,
                          float* oh, float* ol, cudaStream_t st) {
-  const size_t sm = sizeof(float) * (2 * (size_t)L.D + 16 * (size_t)L.K);
-  set_smem((const void*)mv_up_df_kernel, sm);
-  ++g_launches;
-  mv_up_df_kernel<<<L.nb, 256, sm, st>>>(L.D, L.K, Xh, Xl, zh, zl, oh, ol);
+  const int D = L.D, K = L.K, CS = K % 4 == 0 ? up_ctas(L.nb, D, K, 8) : 0;
+  if (CS == 0) {
+    const size_t sm = sizeof(float) * (2 * (size_t)D + 16 * (size_t)K);
+    set_smem((const void*)mv_up_df_kernel, sm);
+    ++g_launches;
+    mv_up_df_kernel<<<L.nb, 256, sm, st>>>(D, K, Xh, Xl, zh, zl, oh, ol);
+    return;
+  }
+  const int per = (D + CS - 1) / CS, kper = (K + CS - 1) / CS;
+  const size_t sm = 2 * sizeof(float) * ((size_t)per * K + 8 * (size_t)K + (size_t)CS * kper + per);
+  launch_pdl_cluster(mv_up_df_cl_kernel, (unsigned)(L.nb * CS), CS, sm, st, D, K, CS, Xh, Xl, zh, zl, oh, ol);
 }
 
 // couplings of every level in one launch: CTA (box i of level l, rows
@@ -2316,89 +2494,116 @@ void launch_matvec_far_df_all(const FarDfArgs& a, cudaStream_t st) {
   mv_far_df_all_kernel<<<grid, 256, 0, st>>>(a);
 }
 
-// downward: [yhat_2p; yhat_2p+1] += X_p yhat_p in pairs
-__global__ void __launch_bounds__(256, 2) mv_down_df_kernel(int D, int K, const float* __restrict__ Xh,
-                                                            const float* __restrict__ Xl, const float* __restrict__ yh,
-                                                            const float* __restrict__ yl, float* __restrict__ ych,
-                                                            float* __restrict__ ycl) {
+// mv_rows_kernel in FP32 pairs: base, X, yh, the partial products and the
+// output are pairs; or, y non-NULL, the output is FP64 with ny rows a box (the
+// others are padding).
+struct RowsDf {
+  const float *Xh, *Xl, *yhh, *yhl, *bh, *bl;
+  const int64_t* ptr;
+  const int32_t* ent;
+  const float *ph, *pl;
+  float *oh, *ol;
+  double* y;
+  int D, K, ns, per, seg, ny;
+};
+__global__ void __launch_bounds__(256) mv_rows_df_kernel(const RowsDf a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int Kp = (K + 3) & ~3;
-  float* sh = reinterpret_cast<float*>(smraw);  // Kp
-  float* sl = sh + Kp;                          // Kp
-  const int p = blockIdx.x;
-  for (int e = threadIdx.x; e < K; e += blockDim.x) sh[e] = yh[(int64_t)p * K + e], sl[e] = yl[(int64_t)p * K + e];
-  __syncthreads();
-  float H[kRPWdf], L[kRPWdf];
-  for (int r0 = 0; r0 < D; r0 += 8 * kRPWdf) {
-    zero(H);
-    zero(L);
-    rows_acc_df<kRPWdf>(r0, Xh + (int64_t)p * D * K, Xl + (int64_t)p * D * K, K, D, K, sh, sl, H, L);
-    rows_finish_pair<kRPWdf>(r0, D, H, L, ych + (int64_t)p * D, ycl + (int64_t)p * D, true);
-  }
-}
-void launch_matvec_down_df(const DevLevel& L, const float* Xh, const float* Xl, const float* yh, const float* yl,
-                           float* ych, float* ycl, cudaStream_t st) {
-  const size_t sm = 2 * sizeof(float) * (size_t)((L.K + 3) & ~3);
-  ++g_launches;
-  mv_down_df_kernel<<<L.nb, 256, sm, st>>>(L.D, L.K, Xh, Xl, yh, yl, ych, ycl);
-}
-
-// leaf output of the symmetric form: y_i = X_i yhat_i + box i's partial
-// products (pairs, in list order), converted to FP64 once per entry
-__global__ void __launch_bounds__(256, 2) mv_sym_sum_df_kernel(int D, int K, const int64_t* __restrict__ ptr,
-                                                               const int32_t* __restrict__ ent,
-                                                               const float* __restrict__ Xh,
-                                                               const float* __restrict__ Xl,
-                                                               const float* __restrict__ yhh,
-                                                               const float* __restrict__ yhl,
-                                                               const float* __restrict__ ph,
-                                                               const float* __restrict__ pl, double* __restrict__ y,
-                                                               int ny) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int Kp = (K + 3) & ~3;
-  float* shh = reinterpret_cast<float*>(smraw);  // Kp
-  float* shl = shh + Kp;                         // Kp
-  float* sbh = shl + Kp;                         // D
-  float* sbl = sbh + D;                          // D
-  const int i = blockIdx.x;
-  const int64_t e0 = ptr[i], e1 = ptr[i + 1];
-  if (Xh)
-    for (int e = threadIdx.x; e < K; e += blockDim.x) shh[e] = yhh[(int64_t)i * K + e], shl[e] = yhl[(int64_t)i * K + e];
-  for (int r = threadIdx.x; r < D; r += blockDim.x) {
-    float H = 0.f, L = 0.f;
-    for (int64_t q = e0; q < e1; ++q) {
-      const int en = ent[q];
-      const int64_t g = (int64_t)(en >> 1) * 2 * D + (en & 1) * D + r;
-      df_add(H, L, ph[g], pl[g]);
-    }
-    sbh[r] = H, sbl[r] = L;
-  }
-  __syncthreads();
-  if (Xh) {
-    float H[kRPWdf], L[kRPWdf];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int r0 = 0; r0 < D; r0 += 8 * kRPWdf) {
-      zero(H);
-      zero(L);
-      rows_acc_df<kRPWdf>(r0, Xh + (int64_t)i * D * K, Xl + (int64_t)i * D * K, K, D, K, shh, shl, H, L);
-      float th, tl;
-      df_tsum<kRPWdf, 32>(H, L, th, tl);
-      const int r = r0 + warp + 8 * tsum_index<kRPWdf, 32>(lane);
-      if (tsum_leader<kRPWdf, 32>(lane) && r < ny) {
-        df_add(th, tl, sbh[r], sbl[r]);
-        y[(int64_t)i * ny + r] = (double)th + (double)tl;
-      }
-    }
+  const int D = a.D, K = a.K, per = a.per, Kp = (K + 3) & ~3;
+  const int p = blockIdx.x / a.ns, r0 = (blockIdx.x % a.ns) * per, m = min(per, D - r0), tid = threadIdx.x;
+  float* rh = reinterpret_cast<float*>(smraw);  // per x K
+  float* rl = rh + (((size_t)per * K + 3) & ~(size_t)3);
+  float* sh = rl + (((size_t)per * K + 3) & ~(size_t)3);  // Kp
+  float* sl = sh + Kp;
+  float* fh = sl + Kp;  // 256
+  float* fl = fh + 256;
+  const int64_t off = ((int64_t)p * D + r0) * K;
+  const bool vec = K % 4 == 0;
+  if (vec) {
+    cp_async_bytes(rh, a.Xh + off, m * K * 4);
+    cp_async_bytes(rl, a.Xl + off, m * K * 4);
   } else {
-    for (int r = threadIdx.x; r < ny; r += blockDim.x) y[(int64_t)i * ny + r] = (double)sbh[r] + (double)sbl[r];
+    for (int e = tid; e < m * K; e += 256) rh[e] = __ldg(a.Xh + off + e), rl[e] = __ldg(a.Xl + off + e);
+  }
+  const int pr = per <= 32 ? 32 : 64, r = tid & (pr - 1), g = tid / pr, ng = 256 / pr;
+  int64_t q = 0, e1 = 0;
+  int rr = 0;
+  if (a.ptr && r < m) {
+    const int c = p * (D / a.seg) + (r0 + r) / a.seg;
+    rr = (r0 + r) % a.seg;
+    q = a.ptr[c] + g, e1 = a.ptr[c + 1];
+  }
+  griddep_wait();
+  griddep_launch_next();
+  for (int e = tid; e < K; e += 256) sh[e] = a.yhh[(int64_t)p * K + e], sl[e] = a.yhl[(int64_t)p * K + e];
+  float H = 0.f, L = 0.f;
+  for (; q + 3 * ng < e1; q += 4 * ng) {
+    float vh[4], vl[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t o = (int64_t)a.ent[q + u * ng] * a.seg + rr;
+      vh[u] = a.ph[o], vl[u] = a.pl[o];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) df_add(H, L, vh[u], vl[u]);
+  }
+  for (; q < e1; q += ng) {
+    const int64_t o = (int64_t)a.ent[q] * a.seg + rr;
+    df_add(H, L, a.ph[o], a.pl[o]);
+  }
+  if (g == 0 && a.bh && r < m) df_add(H, L, a.bh[(int64_t)p * D + r0 + r], a.bl[(int64_t)p * D + r0 + r]);
+  fh[tid] = H, fl[tid] = L;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  auto finish = [&](int row, float th, float tl) {
+    for (int h = 0; h < ng; ++h) df_add(th, tl, fh[h * pr + row], fl[h * pr + row]);
+    if (a.y) {
+      if (r0 + row < a.ny) a.y[(int64_t)p * a.ny + r0 + row] = (double)th + (double)tl;
+    } else {
+      a.oh[(int64_t)p * D + r0 + row] = th, a.ol[(int64_t)p * D + r0 + row] = tl;
+    }
+  };
+  if (K == 0) {
+    if (tid < m) finish(tid, 0.f, 0.f);
+    return;
+  }
+  const int lane = tid & 31;
+  for (int row = tid >> 5; row < m; row += 32) {
+    float ah[4] = {0.f, 0.f, 0.f, 0.f}, al[4] = {0.f, 0.f, 0.f, 0.f};
+    if (vec) {
+      for (int c = lane * 4; c < K; c += 128) {
+        const float4 xh = *reinterpret_cast<const float4*>(sh + c), xl = *reinterpret_cast<const float4*>(sl + c);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (row + 8 * u < m) {
+            const float4 vh = *reinterpret_cast<const float4*>(rh + (size_t)(row + 8 * u) * K + c);
+            const float4 vl = *reinterpret_cast<const float4*>(rl + (size_t)(row + 8 * u) * K + c);
+            df_fma(ah[u], al[u], vh.x, vl.x, xh.x, xl.x);
+            df_fma(ah[u], al[u], vh.y, vl.y, xh.y, xl.y);
+            df_fma(ah[u], al[u], vh.z, vl.z, xh.z, xl.z);
+            df_fma(ah[u], al[u], vh.w, vl.w, xh.w, xl.w);
+          }
+      }
+    } else {
+      for (int c = lane; c < K; c += 32)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (row + 8 * u < m)
+            df_fma(ah[u], al[u], rh[(size_t)(row + 8 * u) * K + c], rl[(size_t)(row + 8 * u) * K + c], sh[c], sl[c]);
+    }
+    float th, tl;
+    df_tsum<4, 32>(ah, al, th, tl);
+    const int ro = row + 8 * tsum_index<4, 32>(lane);
+    if (tsum_leader<4, 32>(lane) && ro < m) finish(ro, th, tl);
   }
 }
-void launch_matvec_sym_sum_df(int nb, int D, int K, const int64_t* ptr, const int32_t* ent, const float* Xh,
-                              const float* Xl, const float* yhh, const float* yhl, const float* ph, const float* pl,
-                              double* y, int ny, cudaStream_t st) {
-  const size_t sm = sizeof(float) * (2 * (size_t)((K + 3) & ~3) + 2 * (size_t)D);
-  ++g_launches;
-  mv_sym_sum_df_kernel<<<nb, 256, sm, st>>>(D, K, ptr, ent, Xh, Xl, yhh, yhl, ph, pl, y, ny);
+void launch_matvec_rows_df(int nb, int D, int K, const float* Xh, const float* Xl, const float* yhh, const float* yhl,
+                           const float* bh, const float* bl, int seg, const int64_t* ptr, const int32_t* ent,
+                           const float* ph, const float* pl, float* oh, float* ol, double* y, int ny, cudaStream_t st) {
+  RowsDf a{Xh, Xl, yhh, yhl, bh, bl, ptr, ent, ph, pl, oh, ol, y, D, K, 0, rows_per(nb, D, K, 8), seg, ny};
+  a.ns = (D + a.per - 1) / a.per;
+  const size_t sm = 2 * sizeof(float) * ((((size_t)a.per * K + 3) & ~(size_t)3) + ((K + 3) & ~3) + 256);
+  set_smem((const void*)mv_rows_df_kernel, sm);
+  launch_pdl(mv_rows_df_kernel, (unsigned)(nb * a.ns), 256, sm, st, a);
 }
 
 // -------------------------------------------- symmetric leaf near blocks ---
@@ -2415,7 +2620,8 @@ void launch_matvec_sym_sum_df(int nb, int D, int K, const int64_t* ptr, const in
 // memory.
 constexpr int kSymRPW = 8;  // rows per warp in flight
 
-template <int CH>  // 4-column chunks per lane: n <= 128 CH
+// (CH 4-column chunks per lane: n <= 128 CH; FULL: n = 128 CH throughout)
+template <int CH, bool FULL>
 __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __restrict__ desc,
                                                              const float* __restrict__ A, const float* __restrict__ x,
                                                              float* __restrict__ part, int pf,
@@ -2423,7 +2629,7 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __re
                                                              unsigned long long* __restrict__ stamp) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const SymPair ds = desc[blockIdx.x];
-  const int n = ds.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = FULL ? 128 * CH : ds.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float* xa = reinterpret_cast<float*>(smraw);  // n
   float* wp = xa + n;                           // 8 * n
   const bool both = ds.xa != ds.xb;
@@ -2441,7 +2647,7 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __re
 #pragma unroll
   for (int h = 0; h < CH; ++h) {
     const int c = lane * 4 + 128 * h;
-    in[h] = c < n;
+    in[h] = FULL || c < n;
     const float4 v = in[h] ? *reinterpret_cast<const float4*>(x + ds.xb + c) : make_float4(0.f, 0.f, 0.f, 0.f);
     xb[h][0] = v.x, xb[h][1] = v.y, xb[h][2] = v.z, xb[h][3] = v.w;
   }
@@ -2459,14 +2665,14 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __re
       const int r = r0 + 8 * t;
 #pragma unroll
       for (int h = 0; h < CH; ++h)
-        v[t][h] = (r < n && in[h]) ? __ldg(reinterpret_cast<const float4*>(M + (int64_t)r * n + lane * 4 + 128 * h))
+        v[t][h] = ((FULL || r < n) && in[h]) ? __ldg(reinterpret_cast<const float4*>(M + (int64_t)r * n + lane * 4 + 128 * h))
                                    : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     float su[kSymRPW];
 #pragma unroll
     for (int t = 0; t < kSymRPW; ++t) {
       const int r = r0 + 8 * t;
-      const float xr = (r < n) ? xa[r] : 0.0f;
+      const float xr = (FULL || r < n) ? xa[r] : 0.0f;
       float s = 0.0f;
 #pragma unroll
       for (int h = 0; h < CH; ++h) {
@@ -2484,7 +2690,7 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __re
     {
       const float sv = tsum<kSymRPW, 32, float>(su);
       const int r = r0 + 8 * tsum_index<kSymRPW, 32>(lane);
-      if (tsum_leader<kSymRPW, 32>(lane) && r < n) u[r] = sv;
+      if (tsum_leader<kSymRPW, 32>(lane) && (FULL || r < n)) u[r] = sv;
     }
   }
   if (stamp && tid == 0) atomicMax(stamp + kGmStamps * state->j + 3, global_ns());
@@ -2503,55 +2709,12 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_kernel(const SymPair* __re
   }
 }
 
-// y_i = X_i yh_i + sum of box i's partial products (in list order)
-template <typename T>
-__global__ void __launch_bounds__(256) mv_sym_sum_kernel(int D, int K, const int64_t* __restrict__ ptr,
-                                                         const int32_t* __restrict__ ent, const T* __restrict__ X,
-                                                         const T* __restrict__ yh, const T* __restrict__ part,
-                                                         T* __restrict__ y) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  T* sh = reinterpret_cast<T*>(smraw);  // K
-  T* sb = sh + ((K + 3) & ~3);          // D
-  const int i = blockIdx.x;
-  const int64_t e0 = ptr[i], e1 = ptr[i + 1];
-  auto hook = [&] {
-    griddep_wait();
-    griddep_launch_next();
-    for (int e = threadIdx.x; e < K; e += blockDim.x) sh[e] = yh[(int64_t)i * K + e];
-    for (int r = threadIdx.x; r < D; r += blockDim.x) {
-      T s = T(0);
-      int64_t q = e0;
-      for (; q + 4 <= e1; q += 4) {
-        T v[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const int en = ent[q + t];
-          v[t] = part[(int64_t)(en >> 1) * 2 * D + (en & 1) * D + r];
-        }
-        s += (v[0] + v[1]) + (v[2] + v[3]);
-      }
-      for (; q < e1; ++q) {
-        const int en = ent[q];
-        s += part[(int64_t)(en >> 1) * 2 * D + (en & 1) * D + r];
-      }
-      sb[r] = s;
-    }
-    __syncthreads();
-  };
-  if (X) {
-    cta_gemv<T, T, Unr<T>::v>(X + (int64_t)i * D * K, K, D, K, sh, T(1), sb, y + (int64_t)i * D, hook);
-  } else {
-    hook();
-    for (int r = threadIdx.x; r < D; r += blockDim.x) y[(int64_t)i * D + r] = sb[r];
-  }
-}
-
 // FP32-pair form for the residual (see df_fma): A as hi + lo, x as FP32
 // pairs xh + xl, partial products as FP32 pairs (ph + pl, 2 D per stored
 // pair).  A row's lanes are added by df_tsum and the lane that keeps the row
 // (lane k keeps the row of pass k mod 16 and half k / 16) stores it after
 // the last pass; the column sums of A^T x_i are added over the warps.
-template <int CH>
+template <int CH, bool FULL>
 __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(const SymPair* __restrict__ desc,
                                                                 const float* __restrict__ Ah,
                                                                 const float* __restrict__ Al,
@@ -2561,7 +2724,7 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(const SymPair* _
   constexpr int RPW = 2;
   extern __shared__ __align__(16) unsigned char smraw[];
   const SymPair ds = desc[blockIdx.x];
-  const int D = ds.n;
+  const int D = FULL ? 128 * CH : ds.n;
   float* xah = reinterpret_cast<float*>(smraw);  // D
   float* xal = xah + D;                          // D
   float* wph = xal + D;                          // 8 * D column partials (high parts)
@@ -2570,12 +2733,14 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(const SymPair* _
   const bool both = ds.xa != ds.xb;
   const float* Mh = Ah + ds.m;
   const float* Ml = Al + ds.m;
+  griddep_wait();
+  griddep_launch_next();
   for (int e = tid; e < D; e += blockDim.x) xah[e] = xh[ds.xa + e], xal[e] = xl[ds.xa + e];
   bool in[CH];
   float xbh[CH][4], xbl[CH][4];
 #pragma unroll
   for (int h = 0; h < CH; ++h) {
-    in[h] = lane * 4 + 128 * h < D;
+    in[h] = FULL || lane * 4 + 128 * h < D;
     const float4 vh = in[h] ? *reinterpret_cast<const float4*>(xh + ds.xb + lane * 4 + 128 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
     const float4 vl = in[h] ? *reinterpret_cast<const float4*>(xl + ds.xb + lane * 4 + 128 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
     xbh[h][0] = vh.x, xbh[h][1] = vh.y, xbh[h][2] = vh.z, xbh[h][3] = vh.w;
@@ -2598,8 +2763,8 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(const SymPair* _
 #pragma unroll
       for (int h = 0; h < CH; ++h) {
         const int64_t off = (int64_t)r * D + lane * 4 + 128 * h;
-        vh[t][h] = (r < D && in[h]) ? __ldg(reinterpret_cast<const float4*>(Mh + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        vl[t][h] = (r < D && in[h]) ? __ldg(reinterpret_cast<const float4*>(Ml + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        vh[t][h] = ((FULL || r < D) && in[h]) ? __ldg(reinterpret_cast<const float4*>(Mh + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        vl[t][h] = ((FULL || r < D) && in[h]) ? __ldg(reinterpret_cast<const float4*>(Ml + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
   };
@@ -2617,7 +2782,7 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(const SymPair* _
 #pragma unroll
     for (int t = 0; t < RPW; ++t) {
       const int r = r0 + 8 * t;
-      const float xrh = (r < D) ? xah[r] : 0.0f, xrl = (r < D) ? xal[r] : 0.0f;
+      const float xrh = (FULL || r < D) ? xah[r] : 0.0f, xrl = (FULL || r < D) ? xal[r] : 0.0f;
       float H = 0.0f, L = 0.0f;
 #pragma unroll
       for (int h = 0; h < CH; ++h) {
@@ -2637,7 +2802,7 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(const SymPair* _
   }
   {
     const int r = warp + 8 * RPW * (lane & 15) + 8 * (lane >> 4);
-    if (r < D) uh[r] = keep_h, ul[r] = keep_l;
+    if (FULL || r < D) uh[r] = keep_h, ul[r] = keep_l;
   }
   if (!both) return;
 #pragma unroll
@@ -2658,46 +2823,39 @@ __global__ void __launch_bounds__(256, 2) mv_sym_pair_df_kernel(const SymPair* _
 
 bool sym_supported(int n) { return n > 0 && n % 4 == 0 && n <= 256; }
 
-template <int CH>
+template <int CH, bool FULL>
 static void launch_sym_pairs_ch(int n, int64_t npu, const SymPair* desc, const float* A, const float* x, float* part,
                                 bool pdl, cudaStream_t st, const GmState* state, unsigned long long* stamp) {
   const size_t sm = sizeof(float) * 9 * (size_t)n;
   const int pf = small_level(npu) ? 1 : 0;
   if (pdl) {
-    launch_pdl(mv_sym_pair_kernel<CH>, (unsigned)npu, 256, sm, st, desc, A, x, part, pf, state, stamp);
+    launch_pdl(mv_sym_pair_kernel<CH, FULL>, (unsigned)npu, 256, sm, st, desc, A, x, part, pf, state, stamp);
   } else {
     ++g_launches;
-    mv_sym_pair_kernel<CH><<<(unsigned)npu, 256, sm, st>>>(desc, A, x, part, pf, state, stamp);
+    mv_sym_pair_kernel<CH, FULL><<<(unsigned)npu, 256, sm, st>>>(desc, A, x, part, pf, state, stamp);
   }
 }
-void launch_matvec_sym_pairs(int max_n, int64_t npu, const SymPair* desc, const float* A, const float* x, float* part,
-                             bool pdl, cudaStream_t st, const GmState* state, unsigned long long* stamp) {
+void launch_matvec_sym_pairs(int min_n, int max_n, int64_t npu, const SymPair* desc, const float* A, const float* x,
+                             float* part, bool pdl, cudaStream_t st, const GmState* state, unsigned long long* stamp) {
   if (npu <= 0) return;
-  if (max_n <= 128) launch_sym_pairs_ch<1>(max_n, npu, desc, A, x, part, pdl, st, state, stamp);
-  else launch_sym_pairs_ch<2>(max_n, npu, desc, A, x, part, pdl, st, state, stamp);
+  const bool full = min_n == max_n && max_n % 128 == 0;
+  if (max_n <= 128 && full) launch_sym_pairs_ch<1, true>(max_n, npu, desc, A, x, part, pdl, st, state, stamp);
+  else if (max_n <= 128) launch_sym_pairs_ch<1, false>(max_n, npu, desc, A, x, part, pdl, st, state, stamp);
+  else if (full) launch_sym_pairs_ch<2, true>(max_n, npu, desc, A, x, part, pdl, st, state, stamp);
+  else launch_sym_pairs_ch<2, false>(max_n, npu, desc, A, x, part, pdl, st, state, stamp);
 }
-void launch_matvec_sym_pairs_df(int D, int64_t npu, const SymPair* desc, const float* Ah, const float* Al,
-                                const float* xh, const float* xl, float* ph, float* pl, cudaStream_t st) {
+void launch_matvec_sym_pairs_df(int min_n, int max_n, int64_t npu, const SymPair* desc, const float* Ah,
+                                const float* Al, const float* xh, const float* xl, float* ph, float* pl,
+                                cudaStream_t st) {
   if (npu <= 0) return;
-  const size_t sm = sizeof(float) * 18 * (size_t)D;
-  ++g_launches;
-  if (D <= 128) mv_sym_pair_df_kernel<1><<<(unsigned)npu, 256, sm, st>>>(desc, Ah, Al, xh, xl, ph, pl);
-  else mv_sym_pair_df_kernel<2><<<(unsigned)npu, 256, sm, st>>>(desc, Ah, Al, xh, xl, ph, pl);
+  const size_t sm = sizeof(float) * 18 * (size_t)max_n;
+  const bool full = min_n == max_n && max_n % 128 == 0;
+  const unsigned g = (unsigned)npu;
+  if (max_n <= 128 && full) launch_pdl(mv_sym_pair_df_kernel<1, true>, g, 256, sm, st, desc, Ah, Al, xh, xl, ph, pl);
+  else if (max_n <= 128) launch_pdl(mv_sym_pair_df_kernel<1, false>, g, 256, sm, st, desc, Ah, Al, xh, xl, ph, pl);
+  else if (full) launch_pdl(mv_sym_pair_df_kernel<2, true>, g, 256, sm, st, desc, Ah, Al, xh, xl, ph, pl);
+  else launch_pdl(mv_sym_pair_df_kernel<2, false>, g, 256, sm, st, desc, Ah, Al, xh, xl, ph, pl);
 }
-template <typename T>
-void launch_matvec_sym_sum(int nb, int D, int K, const int64_t* ptr, const int32_t* ent, const T* X, const T* yh,
-                           const T* part, T* y, cudaStream_t st, bool pdl) {
-  const size_t sm = sizeof(T) * ((size_t)((K + 3) & ~3) + D);
-  if (pdl) {
-    launch_pdl(mv_sym_sum_kernel<T>, nb, 256, sm, st, D, K, ptr, ent, X, yh, part, y);
-  } else {
-    ++g_launches;
-    mv_sym_sum_kernel<T><<<nb, 256, sm, st>>>(D, K, ptr, ent, X, yh, part, y);
-  }
-}
-template void launch_matvec_sym_sum<float>(int, int, int, const int64_t*, const int32_t*, const float*, const float*,
-                                           const float*, float*, cudaStream_t, bool);
-
 // FP32 copies of blocks with their rows and columns at padded places: a warp
 // per padded row (see kernels.h).
 template <typename Ti>
