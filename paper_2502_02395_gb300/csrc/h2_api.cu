@@ -544,7 +544,7 @@ h2_status alloc_factor_arrays(h2_ctx* c, Factor<T>& F) {
       CKC(dalloc(c, &f.luT, nb * R * R));
     }
     CKC(dalloc(c, &f.Ainv, nb * R * R));
-    CKC(dalloc(c, &f.piv, nb * R));
+    CKC(dalloc(c, &f.piv, 2 * nb * R));
     for (T** p : {&f.vin, &f.c, &f.xs}) CKC(dalloc(c, p, nb * D));
     CKC(dalloc(c, &f.M1, std::max<size_t>(nb * R * D, 1)));
     for (T** p : {&f.u, &f.v, &f.om}) CKC(dalloc(c, p, nb * std::max<size_t>(R, 1)));
@@ -577,7 +577,7 @@ h2_status alloc_factor_arrays(h2_ctx* c, Factor<T>& F) {
     CKC(dalloc(c, &F.root_luT, nr * D0 * D0));
   }
   CKC(dalloc(c, &F.root_inv, nr * D0 * D0));
-  CKC(dalloc(c, &F.root_piv, nr * D0));
+  CKC(dalloc(c, &F.root_piv, 2 * nr * D0));
   CKC(dalloc(c, &F.root_vec, nr * D0));
   CKC(dalloc(c, &F.root_x, nr * D0));
   return H2_OK;
@@ -906,11 +906,13 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
     mark();
     // a3: LU of Ahat_ii^RR and its inverse (FP16/BF16 factorizations: in
     // FP64 from the FP32 blocks, or FP32 Gauss-Jordan)
+    bool rows = false;  // piv holds pivot rows
+    if (!mixed) wait_for(st, sp);  // (the FP64 factors are formed beside the chain)
     if (lu64_mixed)
-      launch_lu_inverse_f64_for_f32(d.nb, D, R, reinterpret_cast<const float*>(f.Ahat), d.diag_pair, F.rr_lu,
+      rows = launch_lu_inverse_f64_for_f32(d.nb, D, R, reinterpret_cast<const float*>(f.Ahat), d.diag_pair, F.rr_lu,
                                     F.rr_inv, f.piv, reinterpret_cast<float*>(f.Ainv), c->status, l, st);
     else
-      launch_lu_inverse<T>(d.nb, D, R, f.Ahat, d.diag_pair, f.lu, f.luT, f.piv, f.Ainv, c->status, l, st);
+      rows = launch_lu_inverse<T>(d.nb, D, R, f.Ahat, d.diag_pair, f.lu, f.luT, f.piv, f.Ainv, c->status, l, st, sp);
     mark();
     // the substitution's first product M1 = Ainv (U^R)^T, beside the chain
     // ((U^R)^T: the first R columns of the column-major U, as rows)
@@ -918,6 +920,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       wait_for(st, sp);
       gemm<T>(prec, R, D, R, f.Ainv, (int64_t)R * R, nullptr, R, false, f.U, DD, nullptr, D, false, f.M1,
               (int64_t)R * D, nullptr, D, T(1), T(0), d.nb, sp);
+      if (rows) launch_pivot_sequence(d.nb, R, f.piv, sp);
     }
     // a4 + a5: Z = Ainv Ahat_ii^RS; Ahat_ii^SS -= Ahat_ii^SR Z.  On the
     // tensor cores (16-bit operands, FP32 accumulation) where the level's
@@ -996,16 +999,23 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
     mark();
   }
   if (L >= 1) CKC(cudaStreamWaitEvent(st, evb.back(), 0));
-  wait_for(sp, st);
   // a7: root
   const int D0 = LV[0].D;
   const T* Aroot = (L == 0) ? Aleaf : F.lv[0].Ain;
   const int nr = c->lv[0].nb;  // one root per system (the level-0 blocks are in box order)
+  bool rows = false;
+  if (!mixed) wait_for(st, sp);
   if (lu64_mixed)
-    launch_lu_inverse_f64_for_f32(nr, D0, D0, reinterpret_cast<const float*>(Aroot), nullptr, F.rr_lu, F.rr_inv,
+    rows = launch_lu_inverse_f64_for_f32(nr, D0, D0, reinterpret_cast<const float*>(Aroot), nullptr, F.rr_lu, F.rr_inv,
                                   F.root_piv, reinterpret_cast<float*>(F.root_inv), c->status, 0, st);
   else
-    launch_lu_inverse<T>(nr, D0, D0, Aroot, nullptr, F.root_lu, F.root_luT, F.root_piv, F.root_inv, c->status, 0, st);
+    rows = launch_lu_inverse<T>(nr, D0, D0, Aroot, nullptr, F.root_lu, F.root_luT, F.root_piv, F.root_inv, c->status, 0,
+                                st, sp);
+  if (rows) {
+    wait_for(st, sp);
+    launch_pivot_sequence(nr, D0, F.root_piv, sp);
+  }
+  wait_for(sp, st);
   mark();
   CKC(cudaGetLastError());
   CKC(cudaStreamSynchronize(st));

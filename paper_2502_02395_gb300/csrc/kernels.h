@@ -54,14 +54,18 @@ void launch_perm_identity(int nb, int D, int K, T* U, cudaStream_t st);
 // logical rows lie; the padding itself is launch_form_u_pads')
 void launch_form_u(int64_t nb, int D, int K, const float* W1, const float* V, float* U, float* Ur, void* u16,
                    int bf16, int Dp, int Kp, PadSeg rs, cudaStream_t st);
+// a3: the inverses of the R x R blocks (FP64: their LU factors too, on stream
+// side).  True when piv holds the pivot rows and wants launch_pivot_sequence.
+// (FP64: piv has room for 2 nb R entries.)
 template <typename T>
-void launch_lu_inverse(int nb, int D, int R, const T* Ablk, const int32_t* diag_idx, double* lu, T* luT,
-                       int32_t* piv, T* Ainv, int32_t* status, int level, cudaStream_t st);
-// the FP16/BF16 factorizations' a3 in FP64: FP32 blocks in, FP64 LU and
-// inverse (scratch lu, inv: nb * R * R each), FP32 inverse out
-void launch_lu_inverse_f64_for_f32(int nb, int D, int R, const float* Ablk, const int32_t* diag_idx, double* lu,
+bool launch_lu_inverse(int nb, int D, int R, const T* Ablk, const int32_t* diag_idx, double* lu, T* luT,
+                       int32_t* piv, T* Ainv, int32_t* status, int level, cudaStream_t st, cudaStream_t side);
+// the FP16/BF16 factorizations' a3 in FP64: FP32 blocks in, FP32 inverse out
+// (scratch lu, inv: nb * R * R each)
+bool launch_lu_inverse_f64_for_f32(int nb, int D, int R, const float* Ablk, const int32_t* diag_idx, double* lu,
                                    double* inv, int32_t* piv, float* Ainv, int32_t* status, int level,
                                    cudaStream_t st);
+void launch_pivot_sequence(int nb, int R, int32_t* piv, cudaStream_t st);
 template <typename T>
 void launch_merge(int D, int K, int64_t NP, const T* Ahat, const int32_t* ni, const int32_t* nj,
                   const int32_t* ndst, int64_t FP, const T* Shat, const int32_t* fi, const int32_t* fj,

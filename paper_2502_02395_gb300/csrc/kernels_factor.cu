@@ -1175,274 +1175,255 @@ lu_inverse_kernel(int R, const T* __restrict__ luT, const int32_t* __restrict__ 
 }
 
 // ------------------------------------------------------------------------
-// a3 (cont., FP32 storage): Ainv from the factors with one thread per column
-// b of the inverse.  Column b of P^T is e_{perm^-1(b)}; each thread runs the
-// unit-lower forward and the upper backward substitution on its own column,
-// left-looking in blocks of 32 rows held in registers, reading the factors
-// (row-major in shared memory, identity-padded to Rp = 32 ceil(R/32)) with
-// 16-byte broadcast loads.  No barrier is needed between columns.
+// a3 for R <= 256: (Ahat_ii^RR)^-1 by Gauss-Jordan elimination with partial
+// pivoting (FP32 for the FP16/BF16 factorizations, FP64 for FP64 ones and for
+// H2_OPT_RR_LU_FP64), or the LU factors in getf2's sense (LU), the block in
+// registers.  A cluster of CL CTAs holds a box: CTA q columns 32 CPL q .., its
+// warp w rows RPW w .. RPW w + RPW - 1, lane l columns CPL l .. CPL l + CPL - 1
+// of them.  Step k:
+//   (a) the lanes holding column k publish its entries f_r and each warp its
+//       largest |f_r| among rows not yet used as pivots (the first on ties:
+//       LAPACK's choice), in every CTA of the cluster; barrier (of the cluster);
+//   (b) every warp finds the pivot row p; its warp publishes the row (each CTA
+//       its columns), scaled so that column k becomes 1 / f_p; barrier (CTA);
+//   (c) every other row takes a_r -= f_r (row p), its column k read as 0 (LU:
+//       only rows not used yet, column k becomes the multiplier f_r / f_p).
+// Rows are never moved: with pivot(k) the row of step k,
+//   Ainv[k][pivot(j)] = a[pivot(k)][j];   LU: row k of the factors = a[pivot(k)].
+// Buffers alternate with the step, so two barriers a step suffice.  A zero or
+// non-finite pivot is seen by all threads at the same step, records (level,
+// box) in status[0..1] and leaves the box's output undefined.  The pivot rows
+// go to piv; pivot_sequence_kernel turns them into LAPACK's interchanges.
+// Bound by the latency of a step (two barriers, a shuffle reduction, a
+// reciprocal: about 0.25 us) in FP32 and by the FP64 pipe in FP64.  A panel
+// form in which one warp ran 16 steps at a time took 165 us for 128 x 128;
+// 256 x 256 took 436 us with four CTAs a box and the pivot column read from
+// the owner.
 // ------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) lu_inverse_f32_kernel(int R, int Rp, const float* __restrict__ luT,
-                                                              const int32_t* __restrict__ piv,
-                                                              float* __restrict__ Ainv) {
-  extern __shared__ __align__(16) float smf[];
-  __shared__ int s_perm[1024];
-  float* F = smf;            // Rp x Rp row-major factors
-  float* Y = F + Rp * Rp;    // Rp x Rp row-major; column b belongs to thread b
-  const int box = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-  const float* src = luT + (size_t)box * R * R;
-  for (int e = tid; e < Rp * Rp; e += nt) {
-    const int r = e / Rp, cc = e - r * Rp;
-    F[e] = (r < R && cc < R) ? src[cc * R + r] : (r == cc ? 1.f : 0.f);
+__device__ __forceinline__ float rcp_pivot(float v) { return __frcp_rn(v); }
+__device__ __forceinline__ double rcp_pivot(double v) { return 1.0 / v; }
+
+template <typename T, typename TI, typename TO, int NW, int RPW, int CPL, int CL, bool LU>
+__global__ void __launch_bounds__(32 * NW, (sizeof(T) == 4 && RPW * CPL <= 32) ? 2 : 1)
+    gj_rows_kernel(int D, int R, const TI* __restrict__ Ablk, const int32_t* __restrict__ diag_idx,
+                   TO* __restrict__ out, int32_t* __restrict__ piv, int32_t* __restrict__ status, int level) {
+  constexpr int NR = NW * RPW, NC = 32 * CPL;
+  __shared__ __align__(16) T f[2][NR];
+  __shared__ __align__(16) T prow[2][NC];
+  __shared__ T cv[2][NW];
+  __shared__ int cr[2][NW];
+  __shared__ int pr_of[NR], step_of[NR];  // pivot(k), and its inverse
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int q = CL > 1 ? (int)cluster_rank() : 0, box = blockIdx.x / CL;
+  const int r0 = RPW * warp, c0 = NC * q + CPL * lane;
+  const TI* A = Ablk + (size_t)(diag_idx ? diag_idx[box] : box) * D * D;
+  T a[RPW][CPL];
+  unsigned used = 0;
+#pragma unroll
+  for (int i = 0; i < RPW; ++i) {
+    if (r0 + i >= R) used |= 1u << i;
+#pragma unroll
+    for (int j = 0; j < CPL; ++j)
+      a[i][j] = (r0 + i < R && c0 + j < R) ? static_cast<T>(A[(size_t)(r0 + i) * D + c0 + j]) : T(0);
   }
-  if (tid == 0) {
-    for (int r = 0; r < Rp; ++r) s_perm[r] = r;
-    for (int k = 0; k < R; ++k) {
-      const int p = piv[(size_t)box * R + k];
-      const int t = s_perm[k];
-      s_perm[k] = s_perm[p];
-      s_perm[p] = t;
+  if constexpr (CL > 1) cluster_sync();  // every CTA runs
+  bool ok = true;
+  for (int kc = 0; kc * CPL < R && ok; ++kc) {
+#pragma unroll
+    for (int jk = 0; jk < CPL; ++jk) {
+      const int k = kc * CPL + jk, buf = k & 1;
+      if (k >= R || !ok) break;
+      if (kc / 32 == q) {
+        if (lane == (kc & 31)) {
+          T bv = T(0), best = T(-1);
+          int br = -1;
+#pragma unroll
+          for (int i = 0; i < RPW; ++i) {
+            const T v = a[i][jk];
+            if (!((used >> i) & 1u) && fabs(v) > best) best = fabs(v), bv = v, br = r0 + i;
+            f[buf][r0 + i] = v;
+            if constexpr (!LU) a[i][jk] = T(0);  // (column k is read as 0 by the update)
+          }
+          cv[buf][warp] = bv, cr[buf][warp] = br;
+        }
+        if constexpr (CL > 1) {
+          // to the other CTAs, an entry per lane
+          __syncwarp();
+          if (lane < RPW) {
+            const T v = f[buf][r0 + lane];
+#pragma unroll
+            for (int o = 1; o < CL; ++o) st_cluster(cluster_map(&f[buf][r0 + lane], (q + o) % CL), v);
+          } else if (lane < RPW + CL - 1) {
+            const int cta = (q + 1 + lane - RPW) % CL;
+            st_cluster(cluster_map(&cv[buf][warp], cta), cv[buf][warp]);
+            st_cluster(cluster_map(&cr[buf][warp], cta), cr[buf][warp]);
+          }
+        }
+      }
+      if constexpr (CL > 1) cluster_sync();
+      else __syncthreads();
+      // the pivot: the candidate of largest size, the lowest row on ties
+      const int pc = lane < NW ? cr[buf][lane] : -1;
+      const T vc = lane < NW ? cv[buf][lane] : T(0);
+      int src;
+      if constexpr (sizeof(T) == 4) {
+        // (sizes order as their bits; NaN candidates are never published)
+        const unsigned key = pc >= 0 ? __float_as_uint(fabsf(vc)) : 0u;
+        const unsigned top = __reduce_max_sync(0xffffffffu, key);
+        const unsigned at = __ballot_sync(0xffffffffu, pc >= 0 && key == top);
+        src = at ? __ffs(at) - 1 : 0;  // (warps are in row order)
+      } else {
+        long long key = pc >= 0 ? __double_as_longlong(fabs(vc)) : -1;
+        src = lane;
+#pragma unroll
+        for (int o = NW / 2; o > 0; o >>= 1) {
+          const long long ok2 = __shfl_xor_sync(0xffffffffu, key, o);
+          const int os = __shfl_xor_sync(0xffffffffu, src, o);
+          if (ok2 > key || (ok2 == key && os < src)) key = ok2, src = os;
+        }
+        src = __shfl_sync(0xffffffffu, src, 0);
+      }
+      const int p = __shfl_sync(0xffffffffu, pc, src);
+      const T pv = __shfl_sync(0xffffffffu, vc, src);
+      if (p < 0 || pv == T(0) || !isfinite(pv)) {
+        ok = false;
+        break;
+      }
+      const T inv = rcp_pivot(pv);
+      const int ip = p - r0;  // in 0 .. RPW - 1 in its warp
+      if (ip >= 0 && ip < RPW) {
+#pragma unroll
+        for (int j = 0; j < CPL; ++j) {
+          T v = a[0][j];
+#pragma unroll
+          for (int i = 1; i < RPW; ++i) v = i == ip ? a[i][j] : v;
+          if constexpr (!LU) v = (j == jk && c0 + j == k) ? inv : v * inv;
+          prow[buf][CPL * lane + j] = v;
+        }
+        used |= 1u << ip;
+        if (lane == 0) pr_of[k] = p, step_of[p] = k;
+      }
+      __syncthreads();
+      T pr[CPL];
+#pragma unroll
+      for (int j = 0; j < CPL; ++j) pr[j] = prow[buf][CPL * lane + j];
+      if constexpr (!LU) {
+        T fr[RPW];
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) fr[i] = f[buf][r0 + i];
+        if (ip >= 0 && ip < RPW) {
+#pragma unroll
+          for (int i = 0; i < RPW; ++i)
+#pragma unroll
+            for (int j = 0; j < CPL; ++j) a[i][j] = i == ip ? pr[j] : fma(-fr[i], pr[j], a[i][j]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < RPW; ++i)
+#pragma unroll
+            for (int j = 0; j < CPL; ++j) a[i][j] = fma(-fr[i], pr[j], a[i][j]);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) {
+          if ((used >> i) & 1u) continue;
+          const T l = f[buf][r0 + i] * inv;
+#pragma unroll
+          for (int j = 0; j < CPL; ++j) {
+            const int c = c0 + j;
+            if (c > k) a[i][j] = fma(-l, pr[j], a[i][j]);
+            else if (j == jk && c == k) a[i][j] = l;
+          }
+        }
+      }
     }
+  }
+  if constexpr (CL > 1) cluster_sync();  // no CTA leaves while another may still write to it
+  if (!ok) {
+    if (q == 0) {
+      for (int k = tid; k < R; k += blockDim.x) piv[(size_t)box * R + k] = k;  // (a valid sequence)
+      if (tid == 0 && atomicCAS(status, 0, level + 1) == 0) status[1] = box;
+    }
+    return;
   }
   __syncthreads();
-  const int b = tid;
-  for (int r = 0; r < Rp; ++r) Y[r * Rp + b] = (s_perm[r] == b) ? 1.f : 0.f;
-  float y[32];
-  // forward: L unit lower
-  for (int i0 = 0; i0 < Rp; i0 += 32) {
+  TO* ob = out + (size_t)box * R * R;
 #pragma unroll
-    for (int q = 0; q < 32; ++q) y[q] = Y[(i0 + q) * Rp + b];
-    for (int k = 0; k < i0; k += 4) {
-      const float y0 = Y[k * Rp + b], y1 = Y[(k + 1) * Rp + b], y2 = Y[(k + 2) * Rp + b], y3 = Y[(k + 3) * Rp + b];
+  for (int i = 0; i < RPW; ++i) {
+    if (r0 + i >= R) continue;
+    const int sr = step_of[r0 + i];
 #pragma unroll
-      for (int q = 0; q < 32; ++q) {
-        const float4 l = *reinterpret_cast<const float4*>(F + (i0 + q) * Rp + k);
-        y[q] = fmaf(-l.x, y0, fmaf(-l.y, y1, fmaf(-l.z, y2, fmaf(-l.w, y3, y[q]))));
+    for (int j = 0; j < CPL; ++j)
+      if (c0 + j < R) {
+        if constexpr (LU) ob[(size_t)(c0 + j) * R + sr] = static_cast<TO>(a[i][j]);
+        else ob[(size_t)sr * R + pr_of[c0 + j]] = static_cast<TO>(a[i][j]);
       }
-    }
-#pragma unroll
-    for (int q = 1; q < 32; ++q) {
-#pragma unroll
-      for (int c = 0; c < q; ++c) y[q] = fmaf(-F[(i0 + q) * Rp + i0 + c], y[c], y[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < 32; ++q) Y[(i0 + q) * Rp + b] = y[q];
   }
-  // backward: U upper
-  for (int i0 = Rp - 32; i0 >= 0; i0 -= 32) {
-#pragma unroll
-    for (int q = 0; q < 32; ++q) y[q] = Y[(i0 + q) * Rp + b];
-    for (int k = i0 + 32; k < Rp; k += 4) {
-      const float y0 = Y[k * Rp + b], y1 = Y[(k + 1) * Rp + b], y2 = Y[(k + 2) * Rp + b], y3 = Y[(k + 3) * Rp + b];
-#pragma unroll
-      for (int q = 0; q < 32; ++q) {
-        const float4 u = *reinterpret_cast<const float4*>(F + (i0 + q) * Rp + k);
-        y[q] = fmaf(-u.x, y0, fmaf(-u.y, y1, fmaf(-u.z, y2, fmaf(-u.w, y3, y[q]))));
-      }
-    }
-#pragma unroll
-    for (int q = 31; q >= 0; --q) {
-#pragma unroll
-      for (int c = q + 1; c < 32; ++c) y[q] = fmaf(-F[(i0 + q) * Rp + i0 + c], y[c], y[q]);
-      y[q] = y[q] / F[(i0 + q) * Rp + i0 + q];
-    }
-#pragma unroll
-    for (int q = 0; q < 32; ++q) Y[(i0 + q) * Rp + b] = y[q];
-  }
-  if (b < R) {
-    float* out = Ainv + (size_t)box * R * R;
-    for (int r = 0; r < R; ++r) out[(size_t)r * R + b] = Y[r * Rp + b];
-  }
+  if (q == 0)
+    for (int k = tid; k < R; k += blockDim.x) piv[(size_t)box * R + k] = pr_of[k];
 }
 
-// ------------------------------------------------------------------------
-// a3, mixed precision: (Ahat_ii^RR)^-1 by Gauss-Jordan elimination with
-// partial pivoting, in FP32, with the block held in registers.  Thread
-// (tr, tc) of an (Rp/TR) x (Rp/TC) grid keeps the TR x TC tile at rows
-// TR tr.., columns TC tc.. (Rp = R rounded up to the tile sizes; padding
-// rows never pivot).  Step k: the owners of column k propose their largest
-// |entry| among rows not yet used as pivots (LAPACK's choice: the first
-// largest); the chosen row p is scaled so that its column-k entry becomes
-// 1 / a_pk (the in-place form that stores the inverse where the eliminated
-// column was), and every other row r takes a_r -= a_rk * (scaled row p)
-// with its column-k entry zeroed first.  Rows are never moved, so at the end
-//   Ainv[k][pivot(j)] = a[pivot(k)][j],  pivot(k) = the row chosen at step k.
-// The row-interchange sequence LAPACK's getrf would record (the same pivots:
-// the unused rows of column k are the Schur complement column) is written to
-// piv.  A zero or non-finite pivot column records (level, box) in
-// status[0..1] and leaves the box's output undefined.
-// Tiles: 8 x 8 (256 threads) for R <= 128, 12 x 6 (512 threads) for
-// R <= 192; the register file of one SM sub-partition bounds both.
-// ------------------------------------------------------------------------
-constexpr int kGjMaxR = 192;
+// LAPACK's interchange sequence of the pivot rows in piv, in place (R <= 256):
+// one thread per box, beside the factorization's chain.
+__global__ void __launch_bounds__(32) pivot_sequence_kernel(int R, int32_t* __restrict__ piv) {
+  __shared__ int pos[256], rowat[256], pr[256];
+  int32_t* pv = piv + (size_t)blockIdx.x * R;
+  for (int r = threadIdx.x; r < R; r += 32) pos[r] = r, rowat[r] = r, pr[r] = pv[r];
+  __syncwarp();
+  if (threadIdx.x == 0)
+    for (int k = 0; k < R; ++k) {
+      const int r = pr[k], at = pos[r], rk = rowat[k];
+      pv[k] = at;
+      rowat[k] = r, rowat[at] = rk;
+      pos[r] = k, pos[rk] = at;
+    }
+}
+void launch_pivot_sequence(int nb, int R, int32_t* piv, cudaStream_t st) {
+  if (nb == 0 || R == 0) return;
+  ++g_launches;
+  pivot_sequence_kernel<<<nb, 32, 0, st>>>(R, piv);
+}
 
-struct GjShared {
-  float P[kGjMaxR];
-  float fcol[kGjMaxR];
-  int prow[kGjMaxR], pinv[kGjMaxR], rowat[kGjMaxR];
-  int p;
-  float pv;
-};
-
-// Thread t holds tile (tr, tc) = (t % G, t / G) with G = ntr rounded up to a
-// power of two (G divides 32): the owners of a tile column are one lane
-// group of one warp, so the pivot search is a shuffle reduction in that
-// warp.  One elimination step for column k = TC kc + J (J fixed at compile
-// time so that the tile stays in registers); false on a zero pivot column.
-template <int TR, int TC, int J>
-__device__ __forceinline__ bool gj_step(GjShared& sh, float (&a)[TR][TC], unsigned& used, int kc, int G,
-                                        bool has, int tr, int tc, int r0, int c0) {
-  const int t = threadIdx.x, k = kc * TC + J;
-  // (a) the owner warp of column k finds the pivot: the first largest |a_rk|
-  // over rows not yet used
-  if ((t >> 5) == ((kc * G) >> 5)) {
-    float best = -1.0f, sv = 0.0f;
-    int bi = -1;
-    if (has && tc == kc) {
-#pragma unroll
-      for (int i = 0; i < TR; ++i) {
-        const float v = fabsf(a[i][J]);
-        if (!((used >> i) & 1u) && v > best) best = v, sv = a[i][J], bi = r0 + i;
-      }
-    }
-    for (int o = G >> 1; o > 0; o >>= 1) {
-      const float ob = __shfl_xor_sync(0xffffffffu, best, o), os = __shfl_xor_sync(0xffffffffu, sv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi >= 0 && (bi < 0 || oi < bi))) best = ob, sv = os, bi = oi;
-    }
-    if (tc == kc && tr == 0) {
-      sh.p = bi, sh.pv = sv;
-      if (bi >= 0) sh.prow[k] = bi;
-    }
-  }
-  __syncthreads();
-  const int p = sh.p;
-  const float pv = sh.pv;
-  if (p < 0 || pv == 0.0f || !isfinite(pv)) return false;
-  const float inv = __frcp_rn(pv);
-  // (b) scaled pivot row -> P, column k -> fcol
-  if (has && tr == p / TR) {
-#pragma unroll
-    for (int i = 0; i < TR; ++i)
-      if (r0 + i == p) {
-#pragma unroll
-        for (int jj = 0; jj < TC; ++jj) {
-          const float v = ((jj == J && c0 + jj == k) ? 1.0f : a[i][jj]) * inv;
-          a[i][jj] = v;
-          sh.P[c0 + jj] = v;
-        }
-        used |= 1u << i;
-      }
-  }
-  if (has && tc == kc) {
-#pragma unroll
-    for (int i = 0; i < TR; ++i) sh.fcol[r0 + i] = a[i][J];
-  }
-  __syncthreads();
-  // (c) eliminate column k from every other row
-  if (has) {
-    float pr[TC];
-#pragma unroll
-    for (int jj = 0; jj < TC; ++jj) pr[jj] = sh.P[c0 + jj];
-    const bool own = (tc == kc);
-#pragma unroll
-    for (int i = 0; i < TR; ++i) {
-      const float f = (r0 + i == p) ? 0.0f : sh.fcol[r0 + i];
-      if (own && r0 + i != p) a[i][J] = 0.0f;
-#pragma unroll
-      for (int jj = 0; jj < TC; ++jj) a[i][jj] = fmaf(-f, pr[jj], a[i][jj]);
-    }
+template <typename T, typename TI, typename TO, int NW, int RPW, int CPL, int CL, bool LU>
+static void launch_gj_rows_t(int nb, int D, int R, const TI* A, const int32_t* diag_idx, TO* out, int32_t* piv,
+                             int32_t* status, int level, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(nb * CL));
+  cfg.blockDim = dim3(32 * NW);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CL;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CL > 1 ? 1 : 0;
+  ++g_launches;
+  cudaLaunchKernelEx(&cfg, gj_rows_kernel<T, TI, TO, NW, RPW, CPL, CL, LU>, D, R, A, diag_idx, out, piv, status, level);
+}
+// false for R > 256.  FP64 spreads a box over more CTAs (its time is the FP64
+// pipe's); few rows take fewer warps (a barrier's cost goes with them).
+template <typename T, typename TI, typename TO, bool LU>
+static bool launch_gj_rows(int nb, int D, int R, const TI* A, const int32_t* di, TO* out, int32_t* piv,
+                           int32_t* status, int level, cudaStream_t st) {
+  if (R > 256) return false;
+  if constexpr (sizeof(T) == 4) {
+    if (R <= 32) launch_gj_rows_t<T, TI, TO, 4, 8, 1, 1, LU>(nb, D, R, A, di, out, piv, status, level, st);
+    else if (R <= 64) launch_gj_rows_t<T, TI, TO, 8, 8, 2, 1, LU>(nb, D, R, A, di, out, piv, status, level, st);
+    else if (R <= 128) launch_gj_rows_t<T, TI, TO, 16, 8, 4, 1, LU>(nb, D, R, A, di, out, piv, status, level, st);
+    else launch_gj_rows_t<T, TI, TO, 16, 16, 4, 2, LU>(nb, D, R, A, di, out, piv, status, level, st);
+  } else {
+    if (R <= 32) launch_gj_rows_t<T, TI, TO, 4, 8, 1, 1, LU>(nb, D, R, A, di, out, piv, status, level, st);
+    else if (R <= 64) launch_gj_rows_t<T, TI, TO, 8, 8, 1, 2, LU>(nb, D, R, A, di, out, piv, status, level, st);
+    else if (R <= 128) launch_gj_rows_t<T, TI, TO, 16, 8, 1, 4, LU>(nb, D, R, A, di, out, piv, status, level, st);
+    else launch_gj_rows_t<T, TI, TO, 16, 16, 1, 8, LU>(nb, D, R, A, di, out, piv, status, level, st);
   }
   return true;
 }
 
-template <int TR, int TC, int J>
-__device__ __forceinline__ void gj_steps(bool& ok, GjShared& sh, float (&a)[TR][TC], unsigned& used, int kc, int G,
-                                         int left, bool has, int tr, int tc, int r0, int c0) {
-  if constexpr (J < TC) {
-    if (ok && left > J) ok = gj_step<TR, TC, J>(sh, a, used, kc, G, has, tr, tc, r0, c0);
-    gj_steps<TR, TC, J + 1>(ok, sh, a, used, kc, G, left, has, tr, tc, r0, c0);
-  }
-}
-
-// group size of the kernel's thread mapping (a power of two >= ntr, <= 32)
-__host__ __device__ inline int gj_group(int ntr) {
-  int g = 1;
-  while (g < ntr) g <<= 1;
-  return g;
-}
-
-template <int TR, int TC, int NT>
-__global__ void __launch_bounds__(NT) gj_inverse_kernel(int D, int R, const float* __restrict__ Ablk,
-                                                        const int32_t* __restrict__ diag_idx,
-                                                        float* __restrict__ Ainv, int32_t* __restrict__ piv,
-                                                        int32_t* __restrict__ status, int level) {
-  __shared__ GjShared sh;
-  constexpr int TL = (TR > TC ? TR : TC);  // Rp is a multiple of both tile edges
-  static_assert(TL % TR == 0 && TL % TC == 0, "tile edges must divide the larger one");
-  const int box = blockIdx.x, t = threadIdx.x;
-  const int Rp = (R + TL - 1) / TL * TL, ntr = Rp / TR, ntc = Rp / TC, G = gj_group(ntr);
-  const int tr = t % G, tc = t / G;
-  const bool has = tr < ntr && tc < ntc;
-  const int r0 = tr * TR, c0 = tc * TC;
-  const float* A = Ablk + (size_t)(diag_idx ? diag_idx[box] : box) * D * D;
-  float a[TR][TC];
-  unsigned used = 0;
-#pragma unroll
-  for (int i = 0; i < TR; ++i) {
-    const int r = r0 + i;
-    if (!has || r >= R) used |= 1u << i;
-#pragma unroll
-    for (int j = 0; j < TC; ++j) {
-      const int c = c0 + j;
-      a[i][j] = (has && r < R && c < R) ? A[(size_t)r * D + c] : 0.0f;
-    }
-  }
-  bool ok = true;
-  for (int kc = 0; kc < ntc && ok; ++kc)
-    gj_steps<TR, TC, 0>(ok, sh, a, used, kc, G, R - kc * TC, has, tr, tc, r0, c0);
-  if (!ok) {
-    if (t == 0 && atomicCAS(status, 0, level + 1) == 0) status[1] = box;
-    return;
-  }
-  // unscramble: Ainv[k][prow[j]] = a[prow[k]][j]
-  for (int k = t; k < R; k += blockDim.x) sh.pinv[sh.prow[k]] = k;
-  __syncthreads();
-  if (has) {
-    float* out = Ainv + (size_t)box * R * R;
-#pragma unroll
-    for (int i = 0; i < TR; ++i) {
-      const int r = r0 + i;
-      if (r >= R) continue;
-      const size_t row = (size_t)sh.pinv[r] * R;
-#pragma unroll
-      for (int jj = 0; jj < TC; ++jj)
-        if (c0 + jj < R) out[row + sh.prow[c0 + jj]] = a[i][jj];
-    }
-  }
-  // LAPACK-style interchange sequence of the same pivots: pos[r] is the
-  // current position of original row r, rowat[q] the row at position q
-  __syncthreads();
-  if (t == 0) {
-    int* pos = sh.pinv;
-    for (int q = 0; q < R; ++q) pos[q] = q, sh.rowat[q] = q;
-    int32_t* pv_out = piv + (size_t)box * R;
-    for (int k = 0; k < R; ++k) {
-      const int r = sh.prow[k], q = pos[r], rk = sh.rowat[k];
-      pv_out[k] = q;
-      sh.rowat[k] = r, sh.rowat[q] = rk;
-      pos[r] = k, pos[rk] = q;
-    }
-  }
-}
-
 // ------------------------------------------------------------------------
-// The same in-place elimination for blocks too large for the registers of
-// one CTA (FP32 192 < R <= 512, FP64 128 < R <= 256): the columns are split
-// over a cluster of CL CTAs (thread-block cluster, distributed shared
+// The same in-place elimination in FP32 for 256 < R <= 512: the columns are
+// split over a cluster of CL CTAs (thread-block cluster, distributed shared
 // memory).  CTA q of a box holds the columns [q W, (q + 1) W), W = Rp / CL,
-// as TR x TC register tiles, thread t at tile (t % G, q W / TC + t / G)
-// (16 x 4 tiles of FP32 or 16 x 2 of FP64: 64 registers of data).
+// as TR x TC register tiles, thread t at tile (t % G, q W / TC + t / G).
 // Step k: the CTA owning column k picks the pivot row among the unused rows
 // and publishes (p, a_pk) and column k in its shared memory, in the buffer
 // of the step's parity; one cluster barrier; every CTA reads them from the
@@ -1463,8 +1444,11 @@ struct __align__(16) GjcShared {
   int prow[512], pinv[512], rowat[512];
 };
 
-__device__ __forceinline__ float rcp_pivot(float v) { return __frcp_rn(v); }
-__device__ __forceinline__ double rcp_pivot(double v) { return 1.0 / v; }
+__host__ __device__ inline int gj_group(int ntr) {
+  int g = 1;
+  while (g < ntr) g <<= 1;
+  return g;
+}
 
 template <typename T, int TR, int TC, int J>
 __device__ __forceinline__ bool gjc_step(GjcShared<T>& sh, T (&a)[TR][TC], unsigned& used, int kc, int oq, int kcl,
@@ -1619,456 +1603,54 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1)
 
 // Inverses of nb blocks by the cluster kernel: FP32 elimination (fp64 = 0)
 // for 192 < R <= 512, FP64 for 128 < R <= 256.  False: R not covered.
-static bool launch_gj_cluster(bool fp64, int nb, int D, int R, const float* Ablk, const int32_t* diag_idx,
-                              float* Ainv, int32_t* piv, int32_t* status, int level, cudaStream_t st) {
-  if (!fp64 && R > 192 && R <= 256) {
-    ++g_launches;
-    gj_cluster_kernel<float, 16, 4, 4, 256><<<nb * 4, 256, 0, st>>>(D, R, (R + 15) / 16 * 16, Ablk, diag_idx, Ainv,
-                                                                     piv, status, level);
-    return true;
-  }
-  if (!fp64 && R > 256 && R <= 512) {
-    ++g_launches;
-    gj_cluster_kernel<float, 16, 4, 8, 512><<<nb * 8, 512, 0, st>>>(D, R, (R + 31) / 32 * 32, Ablk, diag_idx, Ainv,
-                                                                     piv, status, level);
-    return true;
-  }
-  if (fp64 && R > 128 && R <= 256) {
-    ++g_launches;
-    gj_cluster_kernel<double, 16, 2, 8, 256><<<nb * 8, 256, 0, st>>>(D, R, (R + 15) / 16 * 16, Ablk, diag_idx,
-                                                                      Ainv, piv, status, level);
-    return true;
-  }
-  return false;
-}
-
-// The same elimination for R <= 128 in 16-column panels.  Thread t of warp
-// w holds the 8 x 8 tile at rows 8 (lane % 16), columns 16 w + 8 (lane / 16),
-// so warp w holds panel w (columns 16 w .. 16 w + 15) for every row.  Per
-// panel: (1) its warp runs the 16 in-place steps on the panel columns only
-// (pivot search, pivot row and column multipliers by shuffles and a
-// warp-private shared row), leaving in column 16 w + a the column p_a of
-// the combined elimination E of the 16 steps (p_a: pivot row of step a);
-// (2) the rows p_a of every other column are published; (3) every other
-// column takes E's effect at once, a_c += (E - I)[:, P] a_old[P, c]: a rank-16
-// update.  The pivots are those of the one-column form (the same row order
-// of choice); the sums are grouped differently.
-constexpr int kGbP = 16;  // panel width
-
-struct GbShared {
-  float WmT[2][kGbP][128];   // (E - I)[:, p_a], transposed: WmT[a][r]
-  float Prow[2][kGbP][128];  // rows p_a of the matrix before the panel
-  float pan[128][kGbP + 1];   // the panel warp's columns, moved between its tile and row layouts
-  int pidx[2][128];          // panel slot a of row r, -1 for rows that are no pivot of the panel
-  unsigned char used[128];   // rows already chosen as pivots
-  int prow[128], pinv[128], rowat[128];
-  int bad;
-};
-
-__global__ void __launch_bounds__(256, 2) gj_blocked_kernel(int D, int R, const float* __restrict__ Ablk,
-                                                            const int32_t* __restrict__ diag_idx,
-                                                            float* __restrict__ Ainv, int32_t* __restrict__ piv,
-                                                            int32_t* __restrict__ status, int level) {
-  __shared__ __align__(16) GbShared sh;
-  const int box = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int tr = lane & 15, h = lane >> 4;
-  const int r0 = 8 * tr, c0 = 16 * warp + 8 * h;
-  const int npan = (R + kGbP - 1) / kGbP;
-  const float* A = Ablk + (size_t)(diag_idx ? diag_idx[box] : box) * D * D;
-  float x[8][8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = r0 + i;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int c = c0 + j;
-      x[i][j] = (r < R && c < R) ? A[(size_t)r * D + c] : 0.0f;
-    }
-  }
-  for (int e = t; e < 128; e += blockDim.x) sh.used[e] = (e >= R);
-  if (t == 0) sh.bad = 0;
-  __syncthreads();
-  for (int pn = 0; pn < npan; ++pn) {
-    const int b = pn & 1;
-    if (warp == pn) {
-      // (1) the panel's 16 steps, in a row layout: lane l holds rows
-      // l + 32 k (k < 4) of the 16 panel columns
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) sh.pan[r0 + i][8 * h + j] = x[i][j], x[i][j] = 0.0f;  // (x reloaded below)
-      for (int e = lane; e < 128; e += 32) sh.pidx[b][e] = -1;
-      __syncwarp();
-      float y[4][kGbP];
-      unsigned used = 0;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        used |= (unsigned)sh.used[lane + 32 * k] << k;
-#pragma unroll
-        for (int c = 0; c < kGbP; ++c) y[k][c] = sh.pan[lane + 32 * k][c];
-      }
-      bool bad = false;
-#pragma unroll
-      for (int a = 0; a < kGbP; ++a) {
-        const int kcol = kGbP * pn + a;
-        if (kcol >= R || bad) break;
-        // pivot: the first largest |y| of column a over unused rows
-        float best = -1.0f, sv = 0.0f;
-        int bi = -1;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float v = fabsf(y[k][a]);
-          if (!((used >> k) & 1u) && v > best) best = v, sv = y[k][a], bi = lane + 32 * k;
-        }
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const float ob = __shfl_xor_sync(0xffffffffu, best, o), os = __shfl_xor_sync(0xffffffffu, sv, o);
-          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-          if (ob > best || (ob == best && oi >= 0 && (bi < 0 || oi < bi))) best = ob, sv = os, bi = oi;
-        }
-        const int p = bi;
-        if (p < 0 || sv == 0.0f || !isfinite(sv)) {
-          bad = true;
-          break;
-        }
-        const float inv = __frcp_rn(sv);
-        const int owner = p & 31, slot = p >> 5;
-        float f[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) f[k] = y[k][a];
-        // eight columns at a time: the pivot row's entries from its owner lane
-        // (slot p / 32 picked by selects), scaled (its column-a entry
-        // becomes 1 / pv), then every row updated
-#pragma unroll
-        for (int hc = 0; hc < kGbP / 8; ++hc) {
-          float pr[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int cc = 8 * hc + q;
-            const float t01 = (slot & 1) ? y[1][cc] : y[0][cc], t23 = (slot & 1) ? y[3][cc] : y[2][cc];
-            const float v = __shfl_sync(0xffffffffu, (slot & 2) ? t23 : t01, owner);
-            pr[q] = (cc == a) ? inv : v * inv;
-          }
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const bool piv = (lane + 32 * k == p);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const int cc = 8 * hc + q;
-              y[k][cc] = piv ? pr[q] : fmaf(-f[k], pr[q], cc == a ? 0.0f : y[k][cc]);
-            }
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (lane + 32 * k == p) used |= 1u << k;
-        if (lane == 0) {
-          sh.prow[kcol] = p;
-          sh.used[p] = 1;
-          sh.pidx[b][p] = a;
-        }
-      }
-      if (bad && lane == 0) sh.bad = 1;
-      __syncwarp();
-      // (E - I)[:, p_a] = the panel columns minus 1 at the pivot rows; the
-      // panel back to the tile layout
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int r = lane + 32 * k;
-        const int pa = sh.pidx[b][r];
-#pragma unroll
-        for (int c = 0; c < kGbP; ++c) {
-          sh.WmT[b][c][r] = y[k][c] - (pa == c ? 1.0f : 0.0f);
-          sh.pan[r][c] = y[k][c];
-        }
-      }
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) x[i][j] = sh.pan[r0 + i][8 * h + j];
-    }
-    __syncthreads();
-    if (sh.bad) break;
-    const int kn = min(kGbP, R - kGbP * pn);  // steps of this panel
-    // (2) rows p_a of the other columns, before the update
-    if (warp != pn) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int a = sh.pidx[b][r0 + i];
-        if (a >= 0) {
-          float4* dst = reinterpret_cast<float4*>(&sh.Prow[b][a][c0]);
-          dst[0] = make_float4(x[i][0], x[i][1], x[i][2], x[i][3]);
-          dst[1] = make_float4(x[i][4], x[i][5], x[i][6], x[i][7]);
-        }
-      }
-    }
-    __syncthreads();
-    // (3) rank-kn update of the other columns
-    if (warp != pn) {
-#pragma unroll 1
-      for (int a = 0; a < kn; ++a) {
-        const float4 w0 = *reinterpret_cast<const float4*>(&sh.WmT[b][a][r0]);
-        const float4 w1 = *reinterpret_cast<const float4*>(&sh.WmT[b][a][r0 + 4]);
-        const float4 p0 = *reinterpret_cast<const float4*>(&sh.Prow[b][a][c0]);
-        const float4 p1 = *reinterpret_cast<const float4*>(&sh.Prow[b][a][c0 + 4]);
-        const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-        const float q[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) x[i][j] = fmaf(w[i], q[j], x[i][j]);
-      }
-    }
-  }
-  if (sh.bad) {
-    if (t == 0 && atomicCAS(status, 0, level + 1) == 0) status[1] = box;
-    return;
-  }
-  // unscramble: Ainv[k][prow[j]] = a[prow[k]][j]
-  for (int k = t; k < R; k += blockDim.x) sh.pinv[sh.prow[k]] = k;
-  __syncthreads();
-  float* out = Ainv + (size_t)box * R * R;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = r0 + i;
-    if (r >= R) continue;
-    const size_t row = (size_t)sh.pinv[r] * R;
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (c0 + j < R) out[row + sh.prow[c0 + j]] = x[i][j];
-  }
-  // LAPACK-style interchange sequence of the same pivots
-  __syncthreads();
-  if (t == 0) {
-    int* pos = sh.pinv;
-    for (int q = 0; q < R; ++q) pos[q] = q, sh.rowat[q] = q;
-    int32_t* pv_out = piv + (size_t)box * R;
-    for (int k = 0; k < R; ++k) {
-      const int r = sh.prow[k], q = pos[r], rk = sh.rowat[k];
-      pv_out[k] = q;
-      sh.rowat[k] = r, sh.rowat[q] = rk;
-      pos[r] = k, pos[rk] = q;
-    }
-  }
+static bool launch_gj_cluster(int nb, int D, int R, const float* Ablk, const int32_t* diag_idx, float* Ainv,
+                              int32_t* piv, int32_t* status, int level, cudaStream_t st) {
+  if (R <= 256 || R > 512) return false;
+  ++g_launches;
+  gj_cluster_kernel<float, 16, 4, 8, 512><<<nb * 8, 512, 0, st>>>(D, R, (R + 31) / 32 * 32, Ablk, diag_idx, Ainv, piv,
+                                                                   status, level);
+  return true;
 }
 
 template <typename T>
-void launch_lu_inverse(int nb, int D, int R, const T* Ablk, const int32_t* diag_idx, double* lu, T* luT,
-                       int32_t* piv, T* Ainv, int32_t* status, int level, cudaStream_t st) {
-  if (nb == 0 || R == 0) return;
+bool launch_lu_inverse(int nb, int D, int R, const T* Ablk, const int32_t* diag_idx, double* lu, T* luT,
+                       int32_t* piv, T* Ainv, int32_t* status, int level, cudaStream_t st, cudaStream_t side) {
+  if (nb == 0 || R == 0) return false;
   (void)lu;  // for T = double, luT is the lu array
-  if (std::is_same<T, float>::value && R <= kGjMaxR) {
+  if constexpr (std::is_same<T, float>::value) {
     // mixed precision: the inverse directly, no LU factors kept
-    const float* Af = reinterpret_cast<const float*>(Ablk);
-    float* Af_inv = reinterpret_cast<float*>(Ainv);
-    ++g_launches;
-    if (R <= 128) {
-      const int warps = (R + kGbP - 1) / kGbP;
-      gj_blocked_kernel<<<nb, 32 * warps, 0, st>>>(D, R, Af, diag_idx, Af_inv, piv, status, level);
-    } else {
-      const int Rp = (R + 11) / 12 * 12, threads = gj_group(Rp / 12) * (Rp / 6);
-      gj_inverse_kernel<12, 6, 512><<<nb, (threads + 31) / 32 * 32, 0, st>>>(D, R, Af, diag_idx, Af_inv, piv, status,
-                                                                               level);
+    if (launch_gj_rows<float, float, float, false>(nb, D, R, Ablk, diag_idx, Ainv, piv, status, level, st)) return true;
+    if (launch_gj_cluster(nb, D, R, Ablk, diag_idx, Ainv, piv, status, level, st)) return false;
+  } else {
+    // the inverse on the chain, the factors (kept for inspection) beside it;
+    // both pick the same pivots
+    if (launch_gj_rows<double, double, double, true>(nb, D, R, Ablk, diag_idx, luT, piv, status, level, side)) {
+      launch_pivot_sequence(nb, R, piv, side);
+      launch_gj_rows<double, double, double, false>(nb, D, R, Ablk, diag_idx, Ainv, piv + (size_t)nb * R, status, level,
+                                                    st);
+      return false;
     }
-    return;
   }
-  if (std::is_same<T, float>::value &&
-      launch_gj_cluster(false, nb, D, R, reinterpret_cast<const float*>(Ablk), diag_idx, reinterpret_cast<float*>(Ainv),
-                        piv, status, level, st))
-    return;
   const size_t cap = 220 * 1024;
   size_t sm1 = sizeof(T) * (size_t)R * (R + 1);
   int use = sm1 <= cap;
   allow_smem((const void*)lu_factor_kernel<T>);
   ++g_launches;
   lu_factor_kernel<T><<<nb, 256, use ? sm1 : 0, st>>>(D, R, Ablk, diag_idx, luT, piv, status, level, use);
-  if (R > 1024) return;  // the permutation table holds 1024 rows; larger blocks are rejected by the caller
-  if (std::is_same<T, float>::value) {
-    const int Rp = (R + 31) / 32 * 32;
-    const size_t smf = sizeof(float) * 2 * (size_t)Rp * Rp;
-    if (smf <= 200 * 1024 && Rp <= 256) {
-      allow_smem((const void*)lu_inverse_f32_kernel);
-      ++g_launches;
-      lu_inverse_f32_kernel<<<nb, Rp, smf, st>>>(R, Rp, reinterpret_cast<const float*>(luT), piv,
-                                                  reinterpret_cast<float*>(Ainv));
-      return;
-    }
-  }
+  if (R > 1024) return false;  // the permutation table holds 1024 rows; larger blocks are rejected by the caller
   size_t f = sizeof(T) * (size_t)R * (R + 1), y = sizeof(T) * (size_t)R * R;
   int mode = (f + y <= cap) ? 2 : (f <= cap ? 1 : 0);
   size_t sm = mode == 2 ? f + y : (mode == 1 ? f : 0);
   allow_smem((const void*)lu_inverse_kernel<T>);
   ++g_launches;
   lu_inverse_kernel<T><<<nb, 256, sm, st>>>(R, luT, piv, Ainv, mode);
+  return false;
 }
-// ------------------------------------------------------------------------
-// a3 in FP64 for R <= 128: in-place Gauss-Jordan inversion with partial
-// pivoting, the matrix in registers.  The R x R block (identity-padded to
-// 128 x 128) is spread over 16 x 16 threads; thread (ty, tx) owns rows
-// 8 ty .. 8 ty + 7 and columns 8 tx .. 8 tx + 7.  Step k:
-//   (a) the owners of column k publish it (f_i = a_ik) and the owners of
-//       row k publish that row; barrier;
-//   (b) warp 0 picks the pivot row p >= k of largest |a_pk| (the first on
-//       ties: LAPACK's choice, which Gauss-Jordan shares with LU because the
-//       entries below the diagonal are those of the Schur complement);
-//       barrier;
-//   (c) the owners of row p publish the scaled pivot row
-//       w_j = a_pj / a_pk (j != k), w_k = 1 / a_pk; barrier;
-//   (d) rows k and p trade places and every row i != k becomes
-//       a_ij - f_i w_j (with a_ik read as 0); row k becomes w.
-// After step R-1 the array holds (P A)^-1 = A^-1 P^T; the interchanges
-// applied to the columns in reverse order give A^-1, which is written in
-// FP32 (one rounding).  Work: R^3 FP64 multiply-adds, bound by the FP64
-// pipe; three barriers per step.
-// ------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 1) gj64_reg_kernel(int D, int R, const float* __restrict__ Ablk,
-                                                          const int32_t* __restrict__ diag_idx,
-                                                          float* __restrict__ Ainv, int32_t* __restrict__ piv,
-                                                          int32_t* __restrict__ status, int level) {
-  __shared__ double colk[2][128], oldk[2][128], rowk[2][128];
-  __shared__ int s_p[2], s_bad;
-  __shared__ int src[128], dst[128], pv[128];
-  const int box = blockIdx.x, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const float* A = Ablk + (size_t)(diag_idx ? diag_idx[box] : box) * D * D;
-  double a[8][8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int i = ty * 8 + r;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int j = tx * 8 + c;
-      a[r][c] = (i < R && j < R) ? (double)__ldg(A + (size_t)i * D + j) : (i == j ? 1.0 : 0.0);
-    }
-  }
-  if (tid == 0) s_bad = 0;
-  for (int k = 0; k < R; ++k) {
-    const int b = k & 1;
-    const int kt = k >> 3, kc = k & 7;
-    // (a) column k and row k
-    if (tx == kt) {
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        double v = 0.0;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) v = (c == kc) ? a[r][c] : v;
-        colk[b][ty * 8 + r] = v;
-      }
-    }
-    if (ty == kt) {
-#pragma unroll
-      for (int r = 0; r < 8; ++r)
-        if (r == kc) {
-#pragma unroll
-          for (int c = 0; c < 8; ++c) oldk[b][tx * 8 + c] = a[r][c];
-        }
-    }
-    __syncthreads();
-    // (b) pivot row
-    if (tid < 32) {
-      double best = -1.0;
-      int bi = k;
-      for (int i = k + tid; i < R; i += 32) {
-        const double v = fabs(colk[b][i]);
-        if (v > best) { best = v; bi = i; }
-      }
-      for (int o = 16; o; o >>= 1) {
-        const double ob = __shfl_down_sync(0xffffffffu, best, o);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (tid == 0) {
-        s_p[b] = bi;
-        pv[k] = bi;
-        if (!(best > 0.0)) s_bad = 1;
-      }
-    }
-    __syncthreads();
-    if (s_bad) break;
-    const int p = s_p[b];
-    const double dinv = 1.0 / colk[b][p];
-    // (c) scaled pivot row
-    if (ty == (p >> 3)) {
-      const int pr = p & 7;
-#pragma unroll
-      for (int r = 0; r < 8; ++r)
-        if (r == pr) {
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const int j = tx * 8 + c;
-            rowk[b][j] = (j == k) ? dinv : a[r][c] * dinv;
-          }
-        }
-    }
-    __syncthreads();
-    // (d) swap rows k and p, eliminate column k from every other row
-    double w[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) w[c] = rowk[b][tx * 8 + c];
-    const double fk = colk[b][k];  // row k's entry, which moves to row p
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int i = ty * 8 + r;
-      if (i == k) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) a[r][c] = w[c];
-      } else {
-        const bool isp = (i == p);
-        const double f = isp ? fk : colk[b][i];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const int j = tx * 8 + c;
-          const double base = isp ? oldk[b][j] : a[r][c];
-          a[r][c] = fma(-f, w[c], (j == k) ? 0.0 : base);
-        }
-      }
-    }
-  }
-  __syncthreads();
-  if (s_bad) {
-    if (tid == 0 && atomicCAS(status, 0, level + 1) == 0) status[1] = box;
-    return;
-  }
-  // column unscramble: A^-1[:, j] = X[:, src[j]] after the swaps k = R-1 .. 0
-  if (tid == 0) {
-    for (int j = 0; j < R; ++j) src[j] = j;
-    for (int k = R - 1; k >= 0; --k) {
-      const int t = src[k];
-      src[k] = src[pv[k]];
-      src[pv[k]] = t;
-    }
-    for (int j = 0; j < R; ++j) dst[src[j]] = j;
-  }
-  __syncthreads();
-  for (int k = tid; k < R; k += 256) piv[(size_t)box * R + k] = pv[k];
-  float* Y = Ainv + (size_t)box * R * R;
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int i = ty * 8 + r;
-    if (i >= R) continue;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int j = tx * 8 + c;
-      if (j < R) Y[(size_t)i * R + dst[j]] = (float)a[r][c];
-    }
-  }
-}
-
-// a3 for the FP16/BF16 factorizations with FP64 arithmetic: the FP32
-// Ahat_ii^RR are widened as they are read and inverted in FP64, and the
-// inverse is rounded once to FP32 (Ainv); the pivots are LAPACK's.  R <= 128:
-// the register Gauss-Jordan kernel above; larger R: the FP64 getf2 kernel
-// (lu, nb * R * R FP64 scratch) and the FP64 inverse (inv, the same size).
-void launch_lu_inverse_f64_for_f32(int nb, int D, int R, const float* Ablk, const int32_t* diag_idx, double* lu,
+bool launch_lu_inverse_f64_for_f32(int nb, int D, int R, const float* Ablk, const int32_t* diag_idx, double* lu,
                                    double* inv, int32_t* piv, float* Ainv, int32_t* status, int level,
                                    cudaStream_t st) {
-  if (nb == 0 || R == 0 || R > 1024) return;
-  if (R <= 128) {
-    ++g_launches;
-    gj64_reg_kernel<<<nb, 256, 0, st>>>(D, R, Ablk, diag_idx, Ainv, piv, status, level);
-    return;
-  }
-  if (launch_gj_cluster(true, nb, D, R, Ablk, diag_idx, Ainv, piv, status, level, st)) return;
+  if (nb == 0 || R == 0 || R > 1024) return false;
+  if (launch_gj_rows<double, float, float, false>(nb, D, R, Ablk, diag_idx, Ainv, piv, status, level, st)) return true;
   const size_t cap = 220 * 1024;
   const size_t sm1 = sizeof(double) * (size_t)R * (R + 1);
   const int use = sm1 <= cap;
@@ -2082,12 +1664,13 @@ void launch_lu_inverse_f64_for_f32(int nb, int D, int R, const float* Ablk, cons
   ++g_launches;
   lu_inverse_kernel<double><<<nb, 256, sm, st>>>(R, lu, piv, inv, mode);
   launch_convert<double, float>(inv, Ainv, (int64_t)nb * R * R, st);
+  return false;
 }
 
-template void launch_lu_inverse<double>(int, int, int, const double*, const int32_t*, double*, double*, int32_t*,
-                                        double*, int32_t*, int, cudaStream_t);
-template void launch_lu_inverse<float>(int, int, int, const float*, const int32_t*, double*, float*, int32_t*,
-                                       float*, int32_t*, int, cudaStream_t);
+template bool launch_lu_inverse<double>(int, int, int, const double*, const int32_t*, double*, double*, int32_t*,
+                                        double*, int32_t*, int, cudaStream_t, cudaStream_t);
+template bool launch_lu_inverse<float>(int, int, int, const float*, const int32_t*, double*, float*, int32_t*,
+                                       float*, int32_t*, int, cudaStream_t, cudaStream_t);
 
 // ------------------------------------------------------------------------
 // a6: merge.  Child pair q of level l (near: its SS part of Ahat; far: Shat)
