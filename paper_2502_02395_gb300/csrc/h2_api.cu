@@ -597,10 +597,13 @@ h2_status alloc_factor(h2_ctx* c, Factor<T>& F) {
 }
 
 template <typename T>
-void gemm(int prec, int M, int N, int K, const T* A, int64_t sA, const int32_t* ia, int lda, bool tA, const T* B,
+void gemm(int32_t* err, int M, int N, int K, const T* A, int64_t sA, const int32_t* ia, int lda, bool tA, const T* B,
           int64_t sB, const int32_t* ib, int ldb, bool tB, T* C, int64_t sC, const int32_t* ic, int ldc, T alpha,
           T beta, int64_t batch, cudaStream_t st) {
-  (void)prec;
+  if constexpr (std::is_same<T, double>::value)
+    if (batch > 0 && M > 0 && N > 0 &&
+        gemm_split(M, N, K, A, sA, ia, lda, tA, B, sB, ib, ldb, tB, C, sC, ic, ldc, alpha, beta, batch, err, st))
+      return;
   gemm_simt<T, T>(M, N, K, A, sA, ia, lda, tA, B, sB, ib, ldb, tB, C, sC, ic, ldc, alpha, beta, batch, st);
 }
 
@@ -722,9 +725,9 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
         const int Kc = c->lv[l + 1].K;
         const T* Tc = F.lv[l + 1].Tm;
         const int64_t KcKc = (int64_t)Kc * Kc;
-        gemm<T>(prec, Kc, K, Kc, Tc, 2 * KcKc, nullptr, Kc, false, Xc, DK, nullptr, K, false, f.Xo, DK, nullptr, K,
+        gemm<T>(c->status + 2, Kc, K, Kc, Tc, 2 * KcKc, nullptr, Kc, false, Xc, DK, nullptr, K, false, f.Xo, DK, nullptr, K,
                 T(1), T(0), nb, sb);
-        gemm<T>(prec, Kc, K, Kc, Tc + KcKc, 2 * KcKc, nullptr, Kc, false, Xc + (int64_t)Kc * K, DK, nullptr, K,
+        gemm<T>(c->status + 2, Kc, K, Kc, Tc + KcKc, 2 * KcKc, nullptr, Kc, false, Xc + (int64_t)Kc * K, DK, nullptr, K,
                 false, f.Xo + (int64_t)Kc * K, DK, nullptr, K, T(1), T(0), nb, sb);
         Xin = f.Xo;
       }
@@ -734,11 +737,11 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       T* W1 = F.Wq + (int64_t)nb * KK;
       if (K > 0) {
         if (!tw_done) {
-          gemm<T>(prec, K, K, D, f.Vq, DK, nullptr, D, false, f.Vq, DK, nullptr, D, true, Sb, KK, nullptr, K, T(1),
+          gemm<T>(c->status + 2, K, K, D, f.Vq, DK, nullptr, D, false, f.Vq, DK, nullptr, D, true, Sb, KK, nullptr, K, T(1),
                   T(0), nb, sb);
           launch_wy_tfactor<T>(nb, K, Sb, f.tau, f.Tw, sb);
         }
-        gemm<T>(prec, D, K, K, f.Vq, DK, nullptr, D, true, f.Tw, KK, nullptr, K, false, W1, DK, nullptr, K, T(1), T(0),
+        gemm<T>(c->status + 2, D, K, K, f.Vq, DK, nullptr, D, true, f.Tw, KK, nullptr, K, false, W1, DK, nullptr, K, T(1), T(0),
                 nb, sb);
       }
       bool formed = false;
@@ -759,9 +762,9 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
         launch_perm_identity<T>(nb, D, K, f.U, sb);
         if (K > 0) {
           if (R > 0)
-            gemm<T>(prec, R, D, K, f.Vq + K, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U, DD, nullptr, D,
+            gemm<T>(c->status + 2, R, D, K, f.Vq + K, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U, DD, nullptr, D,
                     T(-1), T(1), nb, sb);
-          gemm<T>(prec, K, D, K, f.Vq, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U + (int64_t)R * D, DD,
+          gemm<T>(c->status + 2, K, D, K, f.Vq, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U + (int64_t)R * D, DD,
                   nullptr, D, T(-1), T(1), nb, sb);
         }
         launch_transpose_blocks<T>(nb, D, f.U, f.Ur, sb);
@@ -802,8 +805,8 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       const int32_t *pq = up ? d.fu_q : nullptr, *pi = up ? d.fu_i : d.far_i, *pj = up ? d.fu_j : d.far_j;
       // (FP32: the instance's stored halves are in the order of the pairs)
       const bool halves = up && mixed && c->cb_ok;
-      gemm<T>(prec, K, K, K, Sc, KK, halves ? nullptr : pq, K, false, f.Tp, KK, pj, K, true, F.Wc, KK, nullptr, K, T(1), T(0), n, sc);
-      gemm<T>(prec, K, K, K, f.Tp, KK, pi, K, false, F.Wc, KK, nullptr, K, false, f.Shat, KK, pq, K, T(1), T(0), n, sc);
+      gemm<T>(c->status + 2, K, K, K, Sc, KK, halves ? nullptr : pq, K, false, f.Tp, KK, pj, K, true, F.Wc, KK, nullptr, K, T(1), T(0), n, sc);
+      gemm<T>(c->status + 2, K, K, K, f.Tp, KK, pi, K, false, F.Wc, KK, nullptr, K, false, f.Shat, KK, pq, K, T(1), T(0), n, sc);
       if (up) launch_transpose_pairs<T>(K, n, d.fl_q, d.fl_m, f.Shat, sc);
     }
     // max |Shat| for the 16-bit merge's scale, beside the main chain
@@ -891,16 +894,16 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       // symmetric near list: project the upper pairs i <= j, then
       // Ahat_ji = Ahat_ij^T for the lower ones (the kernels are symmetric)
       const T* Ain = (l == L) ? Aleaf : f.Ain;
-      gemm<T>(prec, D, D, D, Ain, DD, l == L && leaf_halves ? nullptr : d.su_q, D, false, f.U, DD, d.su_j, D, true, F.Wk, DD, nullptr, D, T(1), T(0),
+      gemm<T>(c->status + 2, D, D, D, Ain, DD, l == L && leaf_halves ? nullptr : d.su_q, D, false, f.U, DD, d.su_j, D, true, F.Wk, DD, nullptr, D, T(1), T(0),
               d.n_up, st);
-      gemm<T>(prec, D, D, D, f.U, DD, d.su_i, D, false, F.Wk, DD, nullptr, D, false, f.Ahat, DD, d.su_q, D, T(1),
+      gemm<T>(c->status + 2, D, D, D, f.U, DD, d.su_i, D, false, F.Wk, DD, nullptr, D, false, f.Ahat, DD, d.su_q, D, T(1),
               T(0), d.n_up, st);
       launch_transpose_pairs<T>(D, d.n_lw, d.lw_q, d.lw_m, f.Ahat, st);
     } else {
       const T* Ain = (l == L) ? Aleaf : f.Ain;
-      gemm<T>(prec, D, D, D, Ain, DD, nullptr, D, false, f.U, DD, d.near_j, D, true, F.Wk, DD, nullptr, D, T(1),
+      gemm<T>(c->status + 2, D, D, D, Ain, DD, nullptr, D, false, f.U, DD, d.near_j, D, true, F.Wk, DD, nullptr, D, T(1),
               T(0), d.NP, st);
-      gemm<T>(prec, D, D, D, f.U, DD, d.near_i, D, false, F.Wk, DD, nullptr, D, false, f.Ahat, DD, nullptr, D, T(1),
+      gemm<T>(c->status + 2, D, D, D, f.U, DD, d.near_i, D, false, F.Wk, DD, nullptr, D, false, f.Ahat, DD, nullptr, D, T(1),
               T(0), d.NP, st);
     }
     mark();
@@ -918,7 +921,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
     // ((U^R)^T: the first R columns of the column-major U, as rows)
     if (R > 0) {
       wait_for(st, sp);
-      gemm<T>(prec, R, D, R, f.Ainv, (int64_t)R * R, nullptr, R, false, f.U, DD, nullptr, D, false, f.M1,
+      gemm<T>(c->status + 2, R, D, R, f.Ainv, (int64_t)R * R, nullptr, R, false, f.U, DD, nullptr, D, false, f.M1,
               (int64_t)R * D, nullptr, D, T(1), T(0), d.nb, sp);
       if (rows) launch_pivot_sequence(d.nb, R, f.piv, sp);
     }
@@ -958,9 +961,9 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       if (!ok) return fail(H2_ERR_CUDA, "tensor-core Schur update setup failed at level " + std::to_string(l));
       F.schur_tc = true;
     } else if (R > 0 && K > 0) {
-      gemm<T>(prec, R, K, R, f.Ainv, (int64_t)R * R, nullptr, R, false, f.Ahat + R, DD, d.diag_pair, D, false, f.Z,
+      gemm<T>(c->status + 2, R, K, R, f.Ainv, (int64_t)R * R, nullptr, R, false, f.Ahat + R, DD, d.diag_pair, D, false, f.Z,
               (int64_t)R * K, nullptr, K, T(1), T(0), d.nb, st);
-      gemm<T>(prec, K, K, R, f.Ahat + (int64_t)R * D, DD, d.diag_pair, D, false, f.Z, (int64_t)R * K, nullptr, K,
+      gemm<T>(c->status + 2, K, K, R, f.Ahat + (int64_t)R * D, DD, d.diag_pair, D, false, f.Z, (int64_t)R * K, nullptr, K,
               false, f.Ahat + (int64_t)R * D + R, DD, d.diag_pair, D, T(-1), T(1), d.nb, st);
     }
     mark();
