@@ -980,6 +980,150 @@ __global__ void __launch_bounds__(512) qr_reg_kernel(int D, int K, int Kp, const
   }
 }
 
+// The same factorization in FP64, a thread-block cluster of C CTAs per box and
+// the panel in registers: column j belongs to warp j mod G (G = 16 C), lane l
+// holds rows l, l + 32, ... (D <= 256, K <= CW G).  Step k: the warp of column k
+// + 1 updates that column first, forms its reflector and writes it to every
+// CTA of the cluster (distributed shared memory, two buffers) while the others
+// still update; one cluster barrier a step.  Bound by the FP64 pipe (2
+// multiply-adds per clock and SM: 5 M per 256 x 128 box) where a level has many
+// boxes, by the chain of the steps (two reductions, a square root and a
+// division in FP64) where it has few; C is the largest that leaves one CTA an
+// SM.  256 x 128: 1.06 ms for 32 boxes, 1.1 ms for 16 to 2; with one CTA per box
+// and the panel in global memory 3.4 - 3.9 ms.
+template <int CW>
+__global__ void __launch_bounds__(512, 1) qr_cluster_kernel(int D, int K, int C, const double* __restrict__ Xin,
+                                                            double* __restrict__ Vout, double* __restrict__ tau_out,
+                                                            double* __restrict__ Tm) {
+  constexpr int NR = 8;
+  __shared__ __align__(16) double vb[2][32 * NR];
+  __shared__ double tb[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rank = (int)cluster_rank(), box = blockIdx.x / C, g = rank * 16 + warp, G = 16 * C;
+  const double* src = Xin + (size_t)box * D * K;  // row-major D x K
+  double x[CW][NR];
+#pragma unroll
+  for (int c = 0; c < CW; ++c)
+#pragma unroll
+    for (int s = 0; s < NR; ++s) {
+      const int r = lane + 32 * s, j = g + G * c;
+      x[c][s] = (r < D && j < K) ? src[(size_t)r * K + j] : 0.0;
+    }
+  // reflector of this warp's column k = g + G * kc, to buffer k & 1 of every CTA
+  auto reflect = [&](int k) {
+    const int kc = k / G, s0 = k >> 5;
+    double xc[NR];
+#pragma unroll
+    for (int s = 0; s < NR; ++s) {
+      xc[s] = x[0][s];
+#pragma unroll
+      for (int c = 1; c < CW; ++c) xc[s] = kc == c ? x[c][s] : xc[s];
+    }
+    double alpha = 0.0, p0 = 0.0, p1 = 0.0;
+#pragma unroll
+    for (int s = 0; s < NR; ++s) {
+      const int r = lane + 32 * s;
+      if (s == s0) alpha = xc[s];
+      const double v = r > k ? xc[s] : 0.0;
+      if (s >= s0) (s & 1 ? p1 : p0) = fma(v, v, s & 1 ? p1 : p0);
+    }
+    alpha = __shfl_sync(0xffffffffu, alpha, k & 31);
+    double part = p0 + p1;
+    for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    double tau = 0.0, beta = alpha, scal = 0.0;
+    if (part != 0.0) {
+      beta = -copysign(sqrt(fma(alpha, alpha, part)), alpha);
+      tau = (beta - alpha) / beta;
+      scal = 1.0 / (alpha - beta);
+    }
+#pragma unroll
+    for (int s = 0; s < NR; ++s) {
+      const int r = lane + 32 * s;
+      double v = r == k ? 1.0 : 0.0;
+      if (r == k) {
+        xc[s] = beta;
+      } else if (r > k && tau != 0.0) {
+        xc[s] *= scal;
+        v = xc[s];
+      }
+      for (int q = 0; q < C; ++q) st_cluster(cluster_map(&vb[k & 1][r], q), v);
+#pragma unroll
+      for (int c = 0; c < CW; ++c)
+        if (kc == c) x[c][s] = xc[s];
+    }
+    if (lane < C) st_cluster(cluster_map(&tb[k & 1], lane), tau);
+    if (lane == 0) tau_out[(size_t)box * K + k] = tau;
+  };
+  cluster_sync();  // every CTA runs (its shared memory may be written)
+  if (g == 0) reflect(0);
+  for (int k = 0; k < K; ++k) {
+    cluster_sync();
+    const double tk = tb[k & 1];
+    double v[NR];
+#pragma unroll
+    for (int s = 0; s < NR; ++s) v[s] = vb[k & 1][lane + 32 * s];
+    const int s0 = k >> 5;
+    const bool next = k + 1 < K && (k + 1) % G == g;
+    const int nc = next ? (k + 1) / G : -1;
+    // column c's update with reflector k
+    auto update = [&](int c) {
+      double d0 = 0.0, d1 = 0.0;
+#pragma unroll
+      for (int s = 0; s < NR; ++s)
+        if (s >= s0) (s & 1 ? d1 : d0) = fma(v[s], x[c][s], s & 1 ? d1 : d0);
+      double d = d0 + d1;
+      for (int o = 16; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+      d *= -tk;
+#pragma unroll
+      for (int s = 0; s < NR; ++s)
+        if (s >= s0) x[c][s] = fma(d, v[s], x[c][s]);
+    };
+    if (next) {
+      if (tk != 0.0) {
+#pragma unroll
+        for (int c = 0; c < CW; ++c)
+          if (c == nc) update(c);
+      }
+      reflect(k + 1);
+    }
+    if (tk != 0.0) {
+#pragma unroll
+      for (int c = 0; c < CW; ++c)
+        if (c != nc && g + G * c > k && g + G * c < K) update(c);
+    }
+  }
+  cluster_sync();  // no CTA leaves while its buffers may be written
+  double* Rb = Tm + (size_t)box * K * K;
+  double* Vb = Vout + (size_t)box * D * K;
+#pragma unroll
+  for (int c = 0; c < CW; ++c) {
+    const int j = g + G * c;
+    if (j >= K) continue;
+#pragma unroll
+    for (int s = 0; s < NR; ++s) {
+      const int r = lane + 32 * s;
+      if (r < K) Rb[(size_t)r * K + j] = (r <= j) ? x[c][s] : 0.0;
+      if (r < D) Vb[(size_t)j * D + r] = (r > j) ? x[c][s] : (r == j ? 1.0 : 0.0);
+    }
+  }
+}
+template <int CW>
+static void launch_qr_cluster(int nb, int D, int K, int C, const double* Xin, double* Vout, double* tau, double* Tm,
+                              cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(nb * C));
+  cfg.blockDim = dim3(512);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  ++g_launches;
+  cudaLaunchKernelEx(&cfg, qr_cluster_kernel<CW>, D, K, C, Xin, Vout, tau, Tm);
+}
+
 template <typename T>
 bool launch_qr_panel(int nb, int D, int K, const T* Xin, T* Vout, T* tau, T* Tm, T* gscr, cudaStream_t st, T* Tw) {
   if (nb == 0 || K == 0) return false;
@@ -995,6 +1139,16 @@ bool launch_qr_panel(int nb, int D, int K, const T* Xin, T* Vout, T* tau, T* Tm,
                                           reinterpret_cast<float*>(Tm), reinterpret_cast<float*>(Tw));
     return Tw != nullptr;
   }
+  if constexpr (std::is_same<T, double>::value)
+    if (D <= 256 && K <= 128) {
+      // C = 2, 4 or 8 CTAs a box with 64 / C or fewer doubles of the panel a thread
+      int C = 8;
+      while (C > 2 && nb * C > 152) C /= 2;
+      const int cw = (K + 16 * C - 1) / (16 * C);
+      auto go = cw <= 1 ? launch_qr_cluster<1> : cw <= 2 ? launch_qr_cluster<2> : launch_qr_cluster<4>;
+      go(nb, D, K, C, Xin, Vout, tau, Tm, st);
+      return false;
+    }
   const size_t sm = sizeof(T) * (size_t)D * K;
   const int use = sm <= 200 * 1024;
   allow_smem((const void*)qr_panel_kernel<T>);
