@@ -80,8 +80,7 @@ h2_status make_leaf_lowp(h2_ctx* c, int bf16) {
   CKC(dalloc(c, reinterpret_cast<uint16_t**>(&c->A16[bf16]), n));
   CKC(cudaMemsetAsync(amax, 0, sizeof(unsigned int), c->stream));
   launch_amax_blocks<double>(c->A64, lf.NP, (int64_t)lf.D * lf.D, lf.D, lf.D, lf.D, amax, c->stream);
-  launch_pow2_scale(amax, 128.0f, c->A16_scale[bf16], c->stream);
-  launch_to_lowp<double>(bf16, c->A64, c->A16[bf16], n, c->A16_scale[bf16], c->stream);
+  launch_to_lowp<double>(bf16, c->A64, c->A16[bf16], n, {amax, 128.0f, c->A16_scale[bf16]}, c->stream);
   // couplings, per level, with max |S| scaled to sqrt(32768 / K): the
   // tensor-core coupling products then stay inside FP16 (|S T^T| <= 32768)
   for (int l = 1; l <= c->L; ++l) {
@@ -92,8 +91,7 @@ h2_status make_leaf_lowp(h2_ctx* c, int bf16) {
     CKC(dalloc(c, reinterpret_cast<uint16_t**>(&d.S16[bf16]), ns));
     CKC(cudaMemsetAsync(amax, 0, sizeof(unsigned int), c->stream));
     launch_amax_blocks<double>(d.S, d.FP, (int64_t)d.K * d.K, d.K, d.K, d.K, amax, c->stream);
-    launch_pow2_scale(amax, std::sqrt(32768.0f / d.K), d.S16_scale[bf16], c->stream);
-    launch_to_lowp<double>(bf16, d.S, d.S16[bf16], ns, d.S16_scale[bf16], c->stream);
+    launch_to_lowp<double>(bf16, d.S, d.S16[bf16], ns, {amax, std::sqrt(32768.0f / d.K), d.S16_scale[bf16]}, c->stream);
   }
   CKC(cudaGetLastError());
   CKC(cudaStreamSynchronize(c->stream));
@@ -565,9 +563,8 @@ h2_status alloc_factor_arrays(h2_ctx* c, Factor<T>& F) {
   CKC(dalloc(c, &F.scales, 2 * (size_t)(L + 1)));
   CKC(dalloc(c, &F.tscale, 2 * (size_t)(L + 1)));
   CKC(dalloc(c, &F.cscale, (size_t)(L + 1)));
-  CKC(dalloc(c, &F.amax, 3 * (size_t)(L + 1)));
+  CKC(dalloc(c, &F.amax, 5 * (size_t)(L + 1)));
   CKC(dalloc(c, &F.sch, 8));
-  CKC(dalloc(c, &F.sch_amax, 2));
   // one root block per system (a forest has several)
   const size_t nr = (size_t)c->lv[0].nb;
   if (std::is_same<T, double>::value) {
@@ -630,6 +627,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
   }
   cudaStream_t sb = c->basis_stream, sc = c->coupling_stream, sp = c->product_stream;
   CKC(cudaMemsetAsync(c->status, 0, 4 * sizeof(int32_t), st));
+  if (F.amax) CKC(cudaMemsetAsync(F.amax, 0, 5 * (size_t)(c->L + 1) * sizeof(unsigned int), st));
   // timing marks: ev on the context's stream, evb on the basis stream
   std::vector<cudaEvent_t> ev, evb, sync;
   auto mark_on = [&](std::vector<cudaEvent_t>& v, cudaStream_t s) {
@@ -751,7 +749,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
           const bool u16 = f.tc && D % 4 == 0 && K % 4 == 0;
           launch_form_u(nb, D, K, W1, f.Vq, f.U, f.Ur, u16 ? f.U16 : nullptr, bf16, d.D, d.K, row_seg(c, l), sb);
           if (d.D != D) launch_form_u_pads(nb, d.D, d.R, R, K, row_seg(c, l), f.U, f.Ur, sb);
-          if (f.tc && !u16) launch_to_lowp<T>(bf16, f.U, f.U16, (int64_t)d.nb * DD, nullptr, sb);
+          if (f.tc && !u16) launch_to_lowp<T>(bf16, f.U, f.U16, (int64_t)d.nb * DD, {}, sb);
           if (d.K != K)
             launch_pad_blocks<float>(f.Tm, nullptr, nb, d.K, skel_seg(c, l), d.K, skel_seg(c, l), f.Tp, nullptr, nullptr,
                                      nullptr, sb);
@@ -768,7 +766,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
                   nullptr, D, T(-1), T(1), nb, sb);
         }
         launch_transpose_blocks<T>(nb, D, f.U, f.Ur, sb);
-        if (f.tc) launch_to_lowp<T>(bf16, f.U, f.U16, (int64_t)d.nb * DD, nullptr, sb);
+        if (f.tc) launch_to_lowp<T>(bf16, f.U, f.U16, (int64_t)d.nb * DD, {}, sb);
       }
     }
     const int K = d.K;
@@ -781,11 +779,9 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       // tensor cores: V^T = (S_s T_j,s^T)^T in 16 bits, then Shat = T_i,s V / (s_S s_T^2)
       const int64_t KK = (int64_t)K * K;
       unsigned int* am = F.amax + (L + 1) + l;
-      CKC(cudaMemsetAsync(am, 0, sizeof(unsigned int), sc));
       launch_amax_blocks<T>(f.Tp, d.nb, KK, K, K, K, am, sc);
-      launch_pow2_scale(am, std::sqrt(32768.0f / K), F.tscale + 2 * l, sc);
-      launch_to_lowp<T>(bf16, f.Tp, f.T16, d.nb * KK, F.tscale + 2 * l, sc);
-      launch_inv_scale_product(d.S16_scale[bf16], F.tscale + 2 * l, F.cscale + l, sc);
+      launch_to_lowp<T>(bf16, f.Tp, f.T16, d.nb * KK,
+                        {am, std::sqrt(32768.0f / K), F.tscale + 2 * l, d.S16_scale[bf16], F.cscale + l, true}, sc);
       bool ok = gemm_tc(bf16, K, K, K, d.S16[bf16], d.FP, K, K, nullptr, f.T16, d.nb, K, K, d.far_j, F.W16c, KK,
                         nullptr, K, 1, bf16, 1.0f, nullptr, d.FP, c->status + 2, sc, nullptr, -1, nullptr, nullptr,
                         nullptr, 0, 0) &&
@@ -812,7 +808,6 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
     // max |Shat| for the 16-bit merge's scale, beside the main chain
     if (mixed && F.lv[l - 1].tc && std::is_same<T, float>::value) {
       unsigned int* am = F.amax + 2 * (L + 1) + l;
-      CKC(cudaMemsetAsync(am, 0, sizeof(unsigned int), sc));
       launch_amax_blocks<float>(reinterpret_cast<const float*>(f.Shat), d.FP, (int64_t)K * K, K, K, K, am, sc);
     }
     mark_on(evb, sc);
@@ -842,6 +837,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
     CKC(cudaStreamWaitEvent(st, evb_at(l, 1), 0));
     mark();
     // a2: Ahat_ij = U_i^T A_ij U_j
+    unsigned int* am_ss = nullptr;  // max |SS| (the projection's and the Schur update's epilogues)
     if (f.tc) {
       // tensor cores: W^T = (s A_ij) U_j in 16 bits, then Ahat_ij = U_i^T W / s in FP32
       const void* A16 = (l == L) ? c->A16[bf16] : f.Ain16;
@@ -875,10 +871,8 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       // GEMM's epilogue also takes max |SS| of those pairs for the 16-bit
       // merge's scale.
       f.ahat_ss_only = sub16 && R % 16 == 0;
-      unsigned int* am_ss = nullptr;
       if (f.ahat_ss_only && F.lv[l - 1].tc) {
         am_ss = F.amax + (l - 1);
-        CKC(cudaMemsetAsync(am_ss, 0, sizeof(unsigned int), st));
       }
       bool ok = gemm_tc(bf16, D, D, D, A16, d.NP, D, D, pq, f.U16, d.nb, D, D, pj, F.W16, DD, nullptr, D, 1, bf16,
                         1.0f, nullptr, np_proj, c->status + 2, st) &&
@@ -933,6 +927,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
     //   SS -= Ahat_ii^SR (Z^T)^T       (GEMM 2: A = s SR, B = s_z Z^T)
     // with power-of-two scales s_i, s_z from max |Ainv|, max |Z^T|.
     const float* sc_l = (l == L) ? c->A16_scale[bf16] : F.scales + 2 * l;
+    bool ss_max_done = false;  // max |SS| of the diagonal pairs is in am_ss
     const bool schur_tc = mixed && f.tc && f.ahat_isc && d.near_sym && R > 0 && K > 0 && R % 64 == 0 &&
                           gemm_tc_supported(K, R, R, D, R, R) && gemm_tc_supported(K, K, R, D, R, D);
     if (schur_tc) {
@@ -940,23 +935,22 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       float* Zt = reinterpret_cast<float*>(F.Wk);
       uint16_t* Ai16 = reinterpret_cast<uint16_t*>(F.W16);
       uint16_t* Z16 = Ai16 + nb * RR;
-      CKC(cudaMemsetAsync(F.sch_amax, 0, 2 * sizeof(unsigned int), st));
-      launch_amax_blocks<float>(reinterpret_cast<const float*>(f.Ainv), nb, RR, R, R, R, F.sch_amax, st);
-      launch_pow2_scale(F.sch_amax, 16384.0f, F.sch, st);
-      launch_to_lowp<float>(bf16, reinterpret_cast<const float*>(f.Ainv), Ai16, nb * RR, F.sch, st);
-      launch_inv_scale_pair(sc_l, F.sch, F.sch + 4, st);
+      unsigned int* am = F.amax + 3 * (L + 1) + 2 * l;  // max |Ainv|, max |Z^T|
+      launch_amax_blocks<float>(reinterpret_cast<const float*>(f.Ainv), nb, RR, R, R, R, am, st);
+      launch_to_lowp<float>(bf16, reinterpret_cast<const float*>(f.Ainv), Ai16, nb * RR,
+                            {am, 16384.0f, F.sch, sc_l, F.sch + 4}, st);
       const void* SR16 = static_cast<const uint16_t*>(f.Ahat16) + (int64_t)R * D;
       bool ok = gemm_tc(bf16, K, R, R, SR16, d.NP, D, D, d.diag_pair, Ai16, nb, R, R, nullptr, Zt, KR, nullptr, R, 0,
-                        0, 1.0f, F.sch + 4, nb, c->status + 2, st, nullptr, -1, nullptr, nullptr, nullptr,
+                        0, 1.0f, F.sch + 4, nb, c->status + 2, st, nullptr, -1, nullptr, nullptr, am + 1,
                         d.NP * (int64_t)D - R);
       if (ok) {
-        launch_amax_blocks<float>(Zt, nb, KR, K, R, R, F.sch_amax + 1, st);
-        launch_pow2_scale(F.sch_amax + 1, 16384.0f, F.sch + 2, st);
-        launch_to_lowp<float>(bf16, Zt, Z16, nb * KR, F.sch + 2, st);
-        launch_inv_scale_pair(sc_l, F.sch + 2, F.sch + 5, st);
+        launch_to_lowp<float>(bf16, Zt, Z16, nb * KR, {am + 1, 16384.0f, F.sch + 2, sc_l, F.sch + 5}, st);
+        // (the epilogue takes max |SS| of the diagonal pairs for the merge)
         ok = gemm_tc(bf16, K, K, R, SR16, d.NP, D, D, d.diag_pair, Z16, nb, K, R, nullptr,
                      reinterpret_cast<float*>(f.Ahat) + (int64_t)R * D + R, DD, d.diag_pair, D, 3, 0, -1.0f,
-                     F.sch + 5, nb, c->status + 2, st, nullptr, -1, nullptr, nullptr, nullptr, d.NP * (int64_t)D - R);
+                     F.sch + 5, nb, c->status + 2, st, nullptr, -1, nullptr, nullptr, am_ss,
+                     d.NP * (int64_t)D - R);
+        ss_max_done = am_ss != nullptr;
       }
       if (!ok) return fail(H2_ERR_CUDA, "tensor-core Schur update setup failed at level " + std::to_string(l));
       F.schur_tc = true;
@@ -980,19 +974,18 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
         const float* Ah = reinterpret_cast<const float*>(f.Ahat);
         const float* Sh = reinterpret_cast<const float*>(f.Shat);
         if (f.tc && f.ahat_ss_only) {
-          launch_amax_blocks<float>(Ah + (int64_t)R * D + R, d.nb, DD, K, K, D, am, st, d.diag_pair);
+          if (!ss_max_done) launch_amax_blocks<float>(Ah + (int64_t)R * D + R, d.nb, DD, K, K, D, am, st, d.diag_pair);
         } else {
           // (the lower pairs' SS are their mirrors' transposed: the upper
           // ones cover every value)
-          CKC(cudaMemsetAsync(am, 0, sizeof(unsigned int), st));
           launch_amax_blocks<float>(Ah + (int64_t)R * D + R, f.proj_sym ? d.n_up : d.NP, DD, K, K, D, am, st,
                                     f.proj_sym ? d.su_q : nullptr);
         }
-        launch_pow2_scale(am, 128.0f, F.scales + 2 * (l - 1), st, d.FP > 0 && K > 0 ? F.amax + 2 * (L + 1) + l : nullptr);
         // (pairs bound for a lower parent pair are skipped when the parent
         // projects its upper pairs only)
         launch_merge_lowp(D, K, d.NP, Ah, d.near_i, d.near_j, d.near_dst, d.FP, Sh, d.far_i, d.far_j, d.far_dst,
-                          pf.Ain16, F.scales + 2 * (l - 1), bf16, st, f.proj_sym ? d.mirror : nullptr,
+                          pf.Ain16, am, d.FP > 0 && K > 0 ? F.amax + 2 * (L + 1) + l : nullptr,
+                          F.scales + 2 * (l - 1), bf16, st, f.proj_sym ? d.mirror : nullptr,
                           pf.proj_sym ? 1 : 0);
       }
     } else {

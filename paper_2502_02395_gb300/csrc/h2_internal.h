@@ -322,7 +322,6 @@ struct Factor {
   // (Ahat_ii^RR)^-1 [0, 1] and Z^T [2, 3], the two GEMMs' output scales
   // [4, 5]; max-abs accumulators [0, 1]
   float* sch = nullptr;
-  unsigned int* sch_amax = nullptr;
   bool schur_tc = false;  // the last factorization ran a4/a5 on the tensor cores at some level
   int bf16 = -1;              // operand type the 16-bit buffers hold
   std::vector<void*> allocs;  // this factorization's device arrays (h2_release_factorization)

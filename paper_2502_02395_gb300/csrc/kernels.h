@@ -89,7 +89,6 @@ bool gemm_tc(int ab_bf16, int M, int N, int K, const void* A, int64_t nA, int ro
              const int32_t* qi = nullptr, const int32_t* qj = nullptr, unsigned int* amax_ss = nullptr,
              int64_t rowsA_total = 0,  // rowsA_total > 0: the rows A's tensor map spans (else nA * rowsA)
              int form = -1);           // kernel form 0 / 1 / 2 (g_tc_kernel's meaning); -1: g_tc_kernel
-void launch_inv_scale_pair(const float* a, const float* b, float* out, cudaStream_t st);  // out = 1 / (a b)
 // 2-D tensor map over a rows x cols 16-bit array (row stride ld elements)
 // with box_rows x box_cols tiles, no swizzle (dense row-major tiles in
 // shared memory).  False if the driver or the shape does not allow it.
@@ -101,15 +100,23 @@ void launch_wait_selftest(unsigned long long timeout_ns, int32_t* flag, cudaStre
 template <typename S>
 void launch_amax_blocks(const S* base, int64_t nblk, int64_t stride, int rows, int cols, int ld, unsigned int* out,
                         cudaStream_t st, const int32_t* idx = nullptr);  // idx: block q is base + idx[q] stride
-void launch_pow2_scale(const unsigned int* amax_bits, float target, float* scale, cudaStream_t st,
-                       const unsigned int* amax2 = nullptr);
-void launch_inv_scale_product(const float* a, const float* b, float* out, cudaStream_t st);
+// Scale of a 16-bit copy: the largest power of two s with max |in| s <= target,
+// to scale[0] (1 / s to scale[1]); inv (optional) = 1 / (other s) or, squared,
+// 1 / (other s s).  amax NULL: s = 1, nothing is written.
+struct LowpScale {
+  const unsigned int* amax = nullptr;
+  float target = 1.0f;
+  float* scale = nullptr;
+  const float* other = nullptr;
+  float* inv = nullptr;
+  bool squared = false;
+};
 template <typename S>
-void launch_to_lowp(int bf16, const S* in, void* out, int64_t n, const float* scale, cudaStream_t st);
+void launch_to_lowp(int bf16, const S* in, void* out, int64_t n, const LowpScale& sc, cudaStream_t st);
 void launch_merge_lowp(int D, int K, int64_t NP, const float* Ahat, const int32_t* ni, const int32_t* nj,
                        const int32_t* ndst, int64_t FP, const float* Shat, const int32_t* fi, const int32_t* fj,
-                       const int32_t* fdst, void* Apar, const float* scale, int bf16, cudaStream_t st,
-                       const int32_t* mirror = nullptr, int skip_lower = 0);
+                       const int32_t* fdst, void* Apar, const unsigned int* am, const unsigned int* am2, float* scale,
+                       int bf16, cudaStream_t st, const int32_t* mirror = nullptr, int skip_lower = 0);
 // 16-bit D x D blocks dst[k] = (block src[k])^T outside the SS quadrant
 void launch_transpose16_blocks(int D, int R, int64_t n, const int32_t* dst, const int32_t* src, void* A,
                                cudaStream_t st);

@@ -89,7 +89,8 @@ struct TcArgs {
   const int32_t* qi;
   const int32_t* qj;
   // optional: max |FP32 output| over the SS quadrants of the off-diagonal
-  // entries, accumulated by atomicMax on the float bits (the merge's scale)
+  // entries (no split: over everything), accumulated by atomicMax on the float
+  // bits (the scale of the next 16-bit copy)
   unsigned int* amax_ss;
 };
 
@@ -100,8 +101,9 @@ struct TcArgs {
 // row (8 rows per store) or 2 lanes per 16-bit row (16 rows per store),
 // instead of one 16-byte piece of 32 different rows per store.  add: C +=
 // (read-modify-write).  Warp-collective.
-__device__ __forceinline__ void tc_rows_store_f32(float* stg, const float (&v)[16], float* C, int64_t ldc, bool add) {
+__device__ __forceinline__ float tc_rows_store_f32(float* stg, const float (&v)[16], float* C, int64_t ldc, bool add) {
   const int lane = threadIdx.x & 31;
+  float mx = 0.0f;  // max |stored value| of this lane
 #pragma unroll
   for (int j = 0; j < 16; ++j) stg[lane * 17 + j] = v[j];
   __syncwarp();
@@ -116,8 +118,10 @@ __device__ __forceinline__ void tc_rows_store_f32(float* stg, const float (&v)[1
       w.x += old.x, w.y += old.y, w.z += old.z, w.w += old.w;
     }
     *o = w;
+    mx = fmaxf(mx, fmaxf(fmaxf(fabsf(w.x), fabsf(w.y)), fmaxf(fabsf(w.z), fabsf(w.w))));
   }
   __syncwarp();
+  return mx;
 }
 __device__ __forceinline__ void tc_rows_store_u16(float* stg, const uint32_t (&h)[8], uint16_t* C, int64_t ldc) {
   const int lane = threadIdx.x & 31;
@@ -138,8 +142,8 @@ __device__ __forceinline__ void tc_rows_store_u16(float* stg, const uint32_t (&h
 // accumulator columns from TMEM (lane_addr: this warp's lane quarter) in
 // 16-column chunks and stores them in the output mode of p.  Every lane of
 // the warp must call it (tcgen05.ld is warp-collective); rows m >= M and
-// failed tiles (ok false) store nothing.  Returns max |FP32 output| over the
-// SS quadrant of an off-diagonal split entry (0 otherwise).  With stg (this
+// failed tiles (ok false) store nothing.  Returns max |stored FP32 output| of
+// this lane.  With stg (this
 // warp's 32 x 17 words of shared memory), the warp's rows are m - lane ..
 // m - lane + 31, and the row-major outputs (modes 0 and 3) go through
 // tc_rows_store_*.
@@ -168,18 +172,16 @@ __device__ __forceinline__ float tc_epilogue_row(const TcArgs& p, int64_t b, int
         float v[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]) * alpha;
-        tc_rows_store_f32(stg, v, reinterpret_cast<float*>(Cb) + cbase + row0, p.ldc, true);
+        ss_max = fmaxf(ss_max, tc_rows_store_f32(stg, v, reinterpret_cast<float*>(Cb) + cbase + row0, p.ldc, true));
         continue;
       }
       const bool ss = (m >= p.qsplit) && (n0 >= p.qsplit);
       if (!split || ss) {
         float v[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          v[j] = __uint_as_float(r[j]) * alpha;
-          if (split) ss_max = fmaxf(ss_max, fabsf(v[j]));
-        }
-        tc_rows_store_f32(stg, v, reinterpret_cast<float*>(Cb) + cbase + row0, p.ldc, false);
+        for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]) * alpha;
+        ss_max =
+            fmaxf(ss_max, tc_rows_store_f32(stg, v, reinterpret_cast<float*>(Cb) + cbase + row0, p.ldc, false));
       }
       if (p.C2 && !(p.qsplit >= 0 && ss)) {
         uint32_t h[8];
@@ -207,8 +209,7 @@ __device__ __forceinline__ float tc_epilogue_row(const TcArgs& p, int64_t b, int
           float4 v = make_float4(__uint_as_float(r[j]) * alpha, __uint_as_float(r[j + 1]) * alpha,
                                  __uint_as_float(r[j + 2]) * alpha, __uint_as_float(r[j + 3]) * alpha);
           *reinterpret_cast<float4*>(out + j) = v;
-          if (split)
-            ss_max = fmaxf(ss_max, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+          ss_max = fmaxf(ss_max, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
         }
       }
       if (p.C2 && !(p.qsplit >= 0 && ss)) {
@@ -238,6 +239,7 @@ __device__ __forceinline__ float tc_epilogue_row(const TcArgs& p, int64_t b, int
         v.z = fmaf(__uint_as_float(r[j + 2]), alpha, v.z);
         v.w = fmaf(__uint_as_float(r[j + 3]), alpha, v.w);
         *reinterpret_cast<float4*>(out + j) = v;
+        ss_max = fmaxf(ss_max, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
       }
     } else if (p.out_bf16) {
       __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(Cb) + cbase;
@@ -352,7 +354,7 @@ __global__ void __launch_bounds__(128) tc_gemm_kernel(const __grid_constant__ CU
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
     const bool split = p.qsplit >= 0 && p.qi[b] != p.qj[b];
     float ss_max = tc_epilogue_row(p, b, m, lane_addr, ok, stg_sh[warp]);
-    if (p.amax_ss && split) {
+    if (p.amax_ss && (split || p.qsplit < 0)) {
       for (int o = 16; o; o >>= 1) ss_max = fmaxf(ss_max, __shfl_xor_sync(0xffffffffu, ss_max, o));
       if (lane == 0 && ss_max > 0.0f) atomicMax(p.amax_ss, __float_as_uint(ss_max));
     }
@@ -523,7 +525,7 @@ __global__ void __launch_bounds__(192, 1) tc_gemm_ws_kernel(const __grid_constan
       const int64_t b = t / mtiles;
       const int m = (int)(t % mtiles) * TC_BM + row;
       float ss_max = tc_epilogue_row(p, b, m, tmem + buf * cols + lane_off, ok, stg_sh[q]);
-      if (p.amax_ss && p.qsplit >= 0 && p.qi[b] != p.qj[b]) {
+      if (p.amax_ss && (p.qsplit < 0 || p.qi[b] != p.qj[b])) {
         for (int o = 16; o; o >>= 1) ss_max = fmaxf(ss_max, __shfl_xor_sync(0xffffffffu, ss_max, o));
         if (lane == 0 && ss_max > 0.0f) atomicMax(p.amax_ss, __float_as_uint(ss_max));
       }
@@ -652,7 +654,7 @@ bool gemm_tc(int ab_bf16, int M, int N, int K, const void* A, int64_t nA, int ro
   p.qsplit = split ? qsplit : -1;
   p.qi = split ? qi : nullptr;
   p.qj = split ? qj : nullptr;
-  p.amax_ss = split ? amax_ss : nullptr;
+  p.amax_ss = split || qsplit < 0 ? amax_ss : nullptr;
   uint32_t cols = 32;
   while (cols < (uint32_t)N) cols <<= 1;
   p.tmem_cols = cols;
@@ -1022,9 +1024,11 @@ void launch_wait_selftest(unsigned long long timeout_ns, int32_t* flag, cudaStre
 // operand preparation
 // ------------------------------------------------------------------------
 // amax[0] = max |x| over nblk strided sub-blocks: block q holds rows x cols
-// entries at base + q*stride + r*ld + c.  One CTA per block; warps over
-// rows, lanes over columns.
-template <typename S>
+// entries at base + q*stride + r*ld + c.  gridDim.y CTAs share a block's rows;
+// warps over rows, lanes over columns (VEC: four columns a lane, 16-byte
+// aligned rows).  Latency-bound on the levels of few boxes (128 blocks of 128 x
+// 128: 7 us with one CTA a block).
+template <typename S, bool VEC>
 __global__ void __launch_bounds__(256) amax_blocks_kernel(const S* __restrict__ base, int64_t nblk, int64_t stride,
                                                           int rows, int cols, int ld, const int32_t* __restrict__ idx,
                                                           unsigned int* __restrict__ out) {
@@ -1032,8 +1036,17 @@ __global__ void __launch_bounds__(256) amax_blocks_kernel(const S* __restrict__ 
   float m = 0.0f;
   for (int64_t q = blockIdx.x; q < nblk; q += gridDim.x) {
     const S* B = base + (idx ? (int64_t)idx[q] : q) * stride;
-    for (int r = warp; r < rows; r += 8)
-      for (int c = lane; c < cols; c += 32) m = fmaxf(m, fabsf((float)__ldg(B + (int64_t)r * ld + c)));
+#pragma unroll 4
+    for (int r = blockIdx.y * 8 + warp; r < rows; r += 8 * gridDim.y) {
+      if constexpr (VEC) {
+        for (int c = 4 * lane; c < cols; c += 128) {
+          const float4 v = __ldg(reinterpret_cast<const float4*>(B + (int64_t)r * ld + c));
+          m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+        }
+      } else {
+        for (int c = lane; c < cols; c += 32) m = fmaxf(m, fabsf((float)__ldg(B + (int64_t)r * ld + c)));
+      }
+    }
   }
   for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (lane == 0) atomicMax(out, __float_as_uint(m));  // non-negative floats order as uints
@@ -1043,19 +1056,23 @@ void launch_amax_blocks(const S* base, int64_t nblk, int64_t stride, int rows, i
                         cudaStream_t st, const int32_t* idx) {
   if (nblk == 0 || rows == 0 || cols == 0) return;
   const int blocks = (int)std::min<int64_t>(nblk, 152 * 16);
+  const int bands = std::max(1, std::min((rows + 15) / 16, 152 * 8 / blocks));
   ++g_launches;
-  amax_blocks_kernel<S><<<blocks, 256, 0, st>>>(base, nblk, stride, rows, cols, ld, idx, out);
+  if constexpr (std::is_same<S, float>::value)
+    if (cols % 4 == 0 && ld % 4 == 0 && stride % 4 == 0 && (reinterpret_cast<uintptr_t>(base) & 15) == 0) {
+      amax_blocks_kernel<S, true><<<dim3(blocks, bands), 256, 0, st>>>(base, nblk, stride, rows, cols, ld, idx, out);
+      return;
+    }
+  amax_blocks_kernel<S, false><<<dim3(blocks, bands), 256, 0, st>>>(base, nblk, stride, rows, cols, ld, idx, out);
 }
 template void launch_amax_blocks<float>(const float*, int64_t, int64_t, int, int, int, unsigned int*, cudaStream_t,
                                         const int32_t*);
 template void launch_amax_blocks<double>(const double*, int64_t, int64_t, int, int, int, unsigned int*, cudaStream_t,
                                          const int32_t*);
 
-// scale[0] = 2^e with amax * 2^e <= target (largest such power of two),
-// scale[1] = 2^-e.  amax = 0 gives scale 1.  amax is the larger of the two
-// accumulators (the second optional).
-__global__ void pow2_scale_kernel(const unsigned int* __restrict__ amax_bits, const unsigned int* __restrict__ amax2,
-                                  float target, float* __restrict__ scale) {
+// The largest power of two s with amax * s <= target (1 for amax = 0).  amax is
+// the larger of the two accumulators (the second optional).
+__device__ __forceinline__ float pow2_scale(const unsigned int* amax_bits, const unsigned int* amax2, float target) {
   float a = __uint_as_float(amax_bits[0]);
   if (amax2) a = fmaxf(a, __uint_as_float(amax2[0]));
   float s = 1.0f;
@@ -1065,60 +1082,66 @@ __global__ void pow2_scale_kernel(const unsigned int* __restrict__ amax_bits, co
     s = ldexpf(1.0f, e);
     while (a * s > target) s *= 0.5f;
   }
-  scale[0] = s;
-  scale[1] = 1.0f / s;
-}
-void launch_pow2_scale(const unsigned int* amax_bits, float target, float* scale, cudaStream_t st,
-                       const unsigned int* amax2) {
-  ++g_launches;
-  pow2_scale_kernel<<<1, 1, 0, st>>>(amax_bits, amax2, target, scale);
+  return s;
 }
 
-// out[0] = 1 / (a[0] * b[0] * b[0])  (the inverse scale of a product A B B^T)
-__global__ void inv_scale_product_kernel(const float* __restrict__ a, const float* __restrict__ b,
-                                         float* __restrict__ out) {
-  out[0] = 1.0f / (a[0] * b[0] * b[0]);
-}
-void launch_inv_scale_product(const float* a, const float* b, float* out, cudaStream_t st) {
-  ++g_launches;
-  inv_scale_product_kernel<<<1, 1, 0, st>>>(a, b, out);
-}
-
-// out[0] = 1 / (a[0] * b[0])  (the inverse scale of a product of two scaled operands)
-__global__ void inv_scale_pair_kernel(const float* __restrict__ a, const float* __restrict__ b,
-                                      float* __restrict__ out) {
-  out[0] = 1.0f / (a[0] * b[0]);
-}
-void launch_inv_scale_pair(const float* a, const float* b, float* out, cudaStream_t st) {
-  ++g_launches;
-  inv_scale_pair_kernel<<<1, 1, 0, st>>>(a, b, out);
+__device__ __forceinline__ uint32_t pack2_lowp(float a, float b, int bf16) {
+  if (bf16) {
+    __nv_bfloat162 t = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t*>(&t);
+  }
+  __half2 t = __floats2half2_rn(a, b);
+  return *reinterpret_cast<uint32_t*>(&t);
 }
 
-// out16[e] = (16-bit) (in[e] * scale[0])
-template <typename S>
-__global__ void to_lowp_kernel(const S* __restrict__ in, void* __restrict__ out, int64_t n, const float* __restrict__ scale,
-                               int bf16) {
-  const float s = scale ? scale[0] : 1.0f;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    float v = (float)in[e] * s;
-    if (bf16) reinterpret_cast<__nv_bfloat16*>(out)[e] = __float2bfloat16_rn(v);
-    else reinterpret_cast<__half*>(out)[e] = __float2half_rn(v);
+// out16[e] = (16-bit) (in[e] * s), s from max |in| (sc.amax NULL: 1).  The scale,
+// its inverse and the inverse scale of a product with this operand are left
+// for the kernels that follow (one launch instead of three in a chain where
+// each costs more to start than to run).
+template <typename S, bool VEC>
+__global__ void to_lowp_kernel(const S* __restrict__ in, void* __restrict__ out, int64_t n, LowpScale sc, int bf16) {
+  const float s = sc.amax ? pow2_scale(sc.amax, nullptr, sc.target) : 1.0f;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  if (t == 0 && sc.amax) {
+    sc.scale[0] = s;
+    sc.scale[1] = 1.0f / s;
+    if (sc.inv) sc.inv[0] = 1.0f / (sc.squared ? sc.other[0] * s * s : sc.other[0] * s);
+  }
+  if constexpr (VEC) {
+    for (int64_t e = t; e < n / 4; e += step) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(in) + e);
+      reinterpret_cast<uint2*>(out)[e] =
+          make_uint2(pack2_lowp(v.x * s, v.y * s, bf16), pack2_lowp(v.z * s, v.w * s, bf16));
+    }
+  } else {
+    for (int64_t e = t; e < n; e += step) {
+      const float v = (float)in[e] * s;
+      if (bf16) reinterpret_cast<__nv_bfloat16*>(out)[e] = __float2bfloat16_rn(v);
+      else reinterpret_cast<__half*>(out)[e] = __float2half_rn(v);
+    }
   }
 }
 template <typename S>
-void launch_to_lowp(int bf16, const S* in, void* out, int64_t n, const float* scale, cudaStream_t st) {
+void launch_to_lowp(int bf16, const S* in, void* out, int64_t n, const LowpScale& sc, cudaStream_t st) {
   if (n == 0) return;
-  int blocks = (int)std::min<int64_t>((n + 255) / 256, 152 * 32);
   ++g_launches;
-  to_lowp_kernel<S><<<blocks, 256, 0, st>>>(in, out, n, scale, bf16);
+  if constexpr (std::is_same<S, float>::value)
+    if (n % 4 == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0) {
+      const int blocks = (int)std::min<int64_t>((n / 4 + 255) / 256, 152 * 16);
+      to_lowp_kernel<S, true><<<blocks, 256, 0, st>>>(in, out, n, sc, bf16);
+      return;
+    }
+  const int blocks = (int)std::min<int64_t>((n + 255) / 256, 152 * 32);
+  to_lowp_kernel<S, false><<<blocks, 256, 0, st>>>(in, out, n, sc, bf16);
 }
-template void launch_to_lowp<float>(int, const float*, void*, int64_t, const float*, cudaStream_t);
-template void launch_to_lowp<double>(int, const double*, void*, int64_t, const float*, cudaStream_t);
+template void launch_to_lowp<float>(int, const float*, void*, int64_t, const LowpScale&, cudaStream_t);
+template void launch_to_lowp<double>(int, const double*, void*, int64_t, const LowpScale&, cudaStream_t);
 
 // 16-bit merge (the merge of Algorithm 2 in the scaled low-precision layout):
 // child SS blocks (FP32 Ahat, rows/cols R..D) and couplings (FP32 Shat) go
-// to the parent's 16-bit near blocks, multiplied by scale[0].  One CTA per
-// child pair; warps over rows, lanes over columns.  mirror (non-NULL when
+// to the parent's 16-bit near blocks, multiplied by a power of two from am and
+// am2 (left in scale[0], its inverse in scale[1]).  One CTA per child pair (gridDim.y: per
+// band of 32 rows); warps over rows, lanes over columns.  mirror (non-NULL when
 // only the upper pairs were projected): a lower near pair (i > j) takes its
 // mirror's SS transposed.  skip_lower: the parent level projects its upper
 // pairs only, so pairs bound for a lower parent pair are skipped.
@@ -1127,11 +1150,12 @@ __global__ void __launch_bounds__(256) merge_lowp_kernel(int D, int K, int64_t N
                                                          const int32_t* __restrict__ ndst, int64_t FP,
                                                          const float* __restrict__ Shat, const int32_t* __restrict__ fi,
                                                          const int32_t* __restrict__ fj, const int32_t* __restrict__ fdst,
-                                                         void* __restrict__ Apar, const float* __restrict__ scale,
-                                                         int bf16, const int32_t* __restrict__ mirror, int skip_lower) {
+                                                         void* __restrict__ Apar, const unsigned int* __restrict__ am,
+                                                         const unsigned int* __restrict__ am2, float* __restrict__ scale, int bf16, const int32_t* __restrict__ mirror, int skip_lower) {
   const int R = D - K, Dp = 2 * K;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float s = scale[0];
+  const float s = pow2_scale(am, am2, 128.0f);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) scale[0] = s, scale[1] = 1.0f / s;
   for (int64_t q = blockIdx.x; q < NP + FP; q += gridDim.x) {
     const bool nr = q < NP;
     const int64_t qq = nr ? q : q - NP;
@@ -1161,15 +1185,6 @@ __global__ void __launch_bounds__(256) merge_lowp_kernel(int D, int K, int64_t N
 // pairs and written as 8 packed 16-bit entries per thread; a lower pair's
 // quadrant (its mirror's SS transposed) goes through 32 x 32 shared-memory
 // tiles so that both its reads and its writes stay coalesced.
-__device__ __forceinline__ uint32_t pack2_lowp(float a, float b, int bf16) {
-  if (bf16) {
-    __nv_bfloat162 t = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&t);
-  }
-  __half2 t = __floats2half2_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&t);
-}
-
 __global__ void __launch_bounds__(256) merge_lowp_vec_kernel(int D, int K, int64_t NP, const float* __restrict__ Ahat,
                                                              const int32_t* __restrict__ ni,
                                                              const int32_t* __restrict__ nj,
@@ -1178,11 +1193,14 @@ __global__ void __launch_bounds__(256) merge_lowp_vec_kernel(int D, int K, int64
                                                              const int32_t* __restrict__ fi,
                                                              const int32_t* __restrict__ fj,
                                                              const int32_t* __restrict__ fdst, void* __restrict__ Apar,
-                                                             const float* __restrict__ scale, int bf16,
+                                                             const unsigned int* __restrict__ am,
+                                                             const unsigned int* __restrict__ am2,
+                                                             float* __restrict__ scale, int bf16,
                                                              const int32_t* __restrict__ mirror, int skip_lower) {
   __shared__ float t[32][33];
   const int R = D - K, Dp = 2 * K;
-  const float s = scale[0];
+  const float s = pow2_scale(am, am2, 128.0f);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) scale[0] = s, scale[1] = 1.0f / s;
   uint16_t* out16 = reinterpret_cast<uint16_t*>(Apar);
   for (int64_t q = blockIdx.x; q < NP + FP; q += gridDim.x) {
     const bool nr = q < NP;
@@ -1197,8 +1215,8 @@ __global__ void __launch_bounds__(256) merge_lowp_vec_kernel(int D, int K, int64
     const int64_t obase = dst * Dp * Dp + (int64_t)(i & 1) * K * Dp + (j & 1) * K;
     if (!tr) {
       const int groups = K / 8;
-      for (int e = threadIdx.x; e < K * groups; e += blockDim.x) {
-        const int a = e / groups, g = e - a * groups;
+      for (int e = threadIdx.x; e < 32 * groups; e += blockDim.x) {
+        const int a = 32 * blockIdx.y + e / groups, g = e % groups;
         const float4 v0 = __ldg(reinterpret_cast<const float4*>(src + (int64_t)a * lds + g * 8));
         const float4 v1 = __ldg(reinterpret_cast<const float4*>(src + (int64_t)a * lds + g * 8 + 4));
         const uint4 w = make_uint4(pack2_lowp(v0.x * s, v0.y * s, bf16), pack2_lowp(v0.z * s, v0.w * s, bf16),
@@ -1206,9 +1224,8 @@ __global__ void __launch_bounds__(256) merge_lowp_vec_kernel(int D, int K, int64
         *reinterpret_cast<uint4*>(out16 + obase + (int64_t)a * Dp + g * 8) = w;
       }
     } else {
-      const int nt = K / 32, x = threadIdx.x & 31, y0 = threadIdx.x >> 5;
-      for (int tile = 0; tile < nt * nt; ++tile) {
-        const int ta = tile / nt, tb = tile - ta * nt;  // output rows ta*32.., columns tb*32..
+      const int nt = K / 32, x = threadIdx.x & 31, y0 = threadIdx.x >> 5, ta = blockIdx.y;
+      for (int tb = 0; tb < nt; ++tb) {  // output rows ta*32.., columns tb*32..
         __syncthreads();
         for (int y = y0; y < 32; y += 8) t[y][x] = __ldg(src + (int64_t)(tb * 32 + y) * lds + ta * 32 + x);
         __syncthreads();
@@ -1295,20 +1312,20 @@ static bool R_aligned(int D, int K) { return D % 4 == 0 && (D - K) % 4 == 0; }
 
 void launch_merge_lowp(int D, int K, int64_t NP, const float* Ahat, const int32_t* ni, const int32_t* nj,
                        const int32_t* ndst, int64_t FP, const float* Shat, const int32_t* fi, const int32_t* fj,
-                       const int32_t* fdst, void* Apar, const float* scale, int bf16, cudaStream_t st,
-                       const int32_t* mirror, int skip_lower) {
+                       const int32_t* fdst, void* Apar, const unsigned int* am, const unsigned int* am2, float* scale,
+                       int bf16, cudaStream_t st, const int32_t* mirror, int skip_lower) {
   const int64_t n = NP + FP;
   if (n == 0 || K == 0) return;
   const int blocks = (int)std::min<int64_t>(n, 152 * 16);
   ++g_launches;
   if (K % 32 == 0 && R_aligned(D, K) && (reinterpret_cast<uintptr_t>(Apar) & 15) == 0 &&
       (reinterpret_cast<uintptr_t>(Ahat) & 15) == 0 && (reinterpret_cast<uintptr_t>(Shat) & 15) == 0) {
-    merge_lowp_vec_kernel<<<blocks, 256, 0, st>>>(D, K, NP, Ahat, ni, nj, ndst, FP, Shat, fi, fj, fdst, Apar, scale,
-                                                  bf16, mirror, skip_lower);
+    merge_lowp_vec_kernel<<<dim3(blocks, K / 32), 256, 0, st>>>(D, K, NP, Ahat, ni, nj, ndst, FP, Shat, fi, fj, fdst,
+                                                                Apar, am, am2, scale, bf16, mirror, skip_lower);
     return;
   }
-  merge_lowp_kernel<<<blocks, 256, 0, st>>>(D, K, NP, Ahat, ni, nj, ndst, FP, Shat, fi, fj, fdst, Apar, scale, bf16,
-                                            mirror, skip_lower);
+  merge_lowp_kernel<<<blocks, 256, 0, st>>>(D, K, NP, Ahat, ni, nj, ndst, FP, Shat, fi, fj, fdst, Apar, am, am2, scale,
+                                            bf16, mirror, skip_lower);
 }
 
 }  // namespace h2
