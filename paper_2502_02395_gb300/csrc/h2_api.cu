@@ -723,10 +723,9 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
         const int Kc = c->lv[l + 1].K;
         const T* Tc = F.lv[l + 1].Tm;
         const int64_t KcKc = (int64_t)Kc * Kc;
-        gemm<T>(c->status + 2, Kc, K, Kc, Tc, 2 * KcKc, nullptr, Kc, false, Xc, DK, nullptr, K, false, f.Xo, DK, nullptr, K,
-                T(1), T(0), nb, sb);
-        gemm<T>(c->status + 2, Kc, K, Kc, Tc + KcKc, 2 * KcKc, nullptr, Kc, false, Xc + (int64_t)Kc * K, DK, nullptr, K,
-                false, f.Xo + (int64_t)Kc * K, DK, nullptr, K, T(1), T(0), nb, sb);
+        // (box i's halves are the children 2 i and 2 i + 1: D = 2 Kc)
+        gemm<T>(c->status + 2, Kc, K, Kc, Tc, KcKc, nullptr, Kc, false, Xc, (int64_t)Kc * K, nullptr, K, false, f.Xo,
+                (int64_t)Kc * K, nullptr, K, T(1), T(0), 2 * (int64_t)nb, sb);
         Xin = f.Xo;
       }
       // (the FP32 register form also forms the compact-WY factor Tw)

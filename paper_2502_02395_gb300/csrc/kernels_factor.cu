@@ -201,13 +201,22 @@ gemm_batched_kernel(int M, int N, int K, const T* __restrict__ A, int64_t sA, co
 // same roundings as two fmaf), 4000 products of 256 x 256 blocks in 2.66
 // instead of 3.18 ms (50 TFLOP/s).  Tiles fitted to the block (104 x 104 for
 // 200 x 200, 169 threads) measured the same as 128 x 128 ones.
-constexpr int G2_BM = 128, G2_BN = 128, G2_BK = 8, G2_LD = 132;
+// H = 1: 64 x 64 tiles, BK = 16, a 4 x 4 block a thread, the same sums, for
+// batches whose 128 x 128 tiles leave SMs idle (there a tile's chain of slices
+// is the time: 16 products 128 x 128 x 128 in 10 instead of 17 us, U of 16 boxes
+// of 256 in 9 instead of 22).
+template <int H>
+struct G2 {
+  static constexpr int BM = 64 * H, BN = BM, BK = H == 2 ? 8 : 16, LD = BM + 4;
+  static constexpr int KQ = BK / 4, MQ = BM / 4;  // float4 pieces of a slice's row (k contiguous), of its column
+};
 
+template <int H>
 __device__ __forceinline__ void g2_load_a(const float* __restrict__ Ab, int lda, int tA, int M, int K, int m0, int k0,
                                           bool vec, float (&ra)[4]) {
   const int t = threadIdx.x;
   if (!tA) {  // A[m * lda + k]: 4 consecutive k of row m
-    const int m = m0 + (t >> 1), k = k0 + (t & 1) * 4;
+    const int m = m0 + t / G2<H>::KQ, k = k0 + (t % G2<H>::KQ) * 4;
     if (vec && m < M && k + 3 < K) {
       const float4 v = *reinterpret_cast<const float4*>(Ab + (int64_t)m * lda + k);
       ra[0] = v.x, ra[1] = v.y, ra[2] = v.z, ra[3] = v.w;
@@ -216,7 +225,7 @@ __device__ __forceinline__ void g2_load_a(const float* __restrict__ Ab, int lda,
       for (int e = 0; e < 4; ++e) ra[e] = (m < M && k + e < K) ? Ab[(int64_t)m * lda + k + e] : 0.0f;
     }
   } else {  // A[k * lda + m]: 4 consecutive m of row k
-    const int k = k0 + (t >> 5), m = m0 + (t & 31) * 4;
+    const int k = k0 + t / G2<H>::MQ, m = m0 + (t % G2<H>::MQ) * 4;
     if (vec && k < K && m + 3 < M) {
       const float4 v = *reinterpret_cast<const float4*>(Ab + (int64_t)k * lda + m);
       ra[0] = v.x, ra[1] = v.y, ra[2] = v.z, ra[3] = v.w;
@@ -226,129 +235,133 @@ __device__ __forceinline__ void g2_load_a(const float* __restrict__ Ab, int lda,
     }
   }
 }
-__device__ __forceinline__ void g2_store_a(float (*As)[G2_LD], int tA, const float (&ra)[4]) {
+template <int H>
+__device__ __forceinline__ void g2_store_a(float (*As)[G2<H>::LD], int tA, const float (&ra)[4]) {
   const int t = threadIdx.x;
   if (!tA) {
-    const int m = t >> 1, k = (t & 1) * 4;
+    const int m = t / G2<H>::KQ, k = (t % G2<H>::KQ) * 4;
 #pragma unroll
     for (int e = 0; e < 4; ++e) As[k + e][m] = ra[e];
   } else {
-    const int k = t >> 5, m = (t & 31) * 4;
+    const int k = t / G2<H>::MQ, m = (t % G2<H>::MQ) * 4;
     *reinterpret_cast<float4*>(&As[k][m]) = make_float4(ra[0], ra[1], ra[2], ra[3]);
   }
 }
 
-// acc = op(A)[m0.., :] op(B)[:, n0..] for one 128 x 128 tile (thread layout
+// acc = op(A)[m0.., :] op(B)[:, n0..] for one 64 H x 64 H tile (thread layout
 // of the tile kernel below); As / Bs are the CTA's two shared buffers.
-template <typename TB>
+template <int H>
 __device__ __forceinline__ void g2_mainloop(int M, int N, int K, const float* __restrict__ Ab, int lda, int tA,
-                                            const TB* __restrict__ Bb, int ldb, int tB, int m0, int n0, int vecA,
-                                            int vecB, float (*As)[G2_BK][G2_LD], float (*Bs)[G2_BK][G2_LD],
-                                            float (&acc)[8][8]) {
+                                            const float* __restrict__ Bb, int ldb, int tB, int m0, int n0, int vecA,
+                                            int vecB, float (*As)[G2<H>::BK][G2<H>::LD], float (*Bs)[G2<H>::BK][G2<H>::LD],
+                                            float (&acc)[4 * H][4 * H]) {
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
   // op(B)(k, n) tile: B[k * ldb + n] (!tB) or B[n * ldb + k] (tB), stored as
   // Bs[k][n]; the same code as A with the roles of m and n exchanged
   auto load_b = [&](int k0, float (&rb)[4]) {
     if (tB) {  // B[n * ldb + k]: 4 consecutive k of row n
-      const int n = n0 + (t >> 1), k = k0 + (t & 1) * 4;
+      const int n = n0 + t / G2<H>::KQ, k = k0 + (t % G2<H>::KQ) * 4;
       if (vecB && n < N && k + 3 < K) {
         const float4 v = *reinterpret_cast<const float4*>(Bb + (int64_t)n * ldb + k);
         rb[0] = v.x, rb[1] = v.y, rb[2] = v.z, rb[3] = v.w;
       } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) rb[e] = (n < N && k + e < K) ? (float)Bb[(int64_t)n * ldb + k + e] : 0.0f;
+        for (int e = 0; e < 4; ++e) rb[e] = (n < N && k + e < K) ? Bb[(int64_t)n * ldb + k + e] : 0.0f;
       }
     } else {  // B[k * ldb + n]: 4 consecutive n of row k
-      const int k = k0 + (t >> 5), n = n0 + (t & 31) * 4;
+      const int k = k0 + t / G2<H>::MQ, n = n0 + (t % G2<H>::MQ) * 4;
       if (vecB && k < K && n + 3 < N) {
         const float4 v = *reinterpret_cast<const float4*>(Bb + (int64_t)k * ldb + n);
         rb[0] = v.x, rb[1] = v.y, rb[2] = v.z, rb[3] = v.w;
       } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) rb[e] = (k < K && n + e < N) ? (float)Bb[(int64_t)k * ldb + n + e] : 0.0f;
+        for (int e = 0; e < 4; ++e) rb[e] = (k < K && n + e < N) ? Bb[(int64_t)k * ldb + n + e] : 0.0f;
       }
     }
   };
-  auto store_b = [&](float (*Bsb)[G2_LD], const float (&rb)[4]) {
+  auto store_b = [&](float (*Bsb)[G2<H>::LD], const float (&rb)[4]) {
     if (tB) {
-      const int n = t >> 1, k = (t & 1) * 4;
+      const int n = t / G2<H>::KQ, k = (t % G2<H>::KQ) * 4;
 #pragma unroll
       for (int e = 0; e < 4; ++e) Bsb[k + e][n] = rb[e];
     } else {
-      const int k = t >> 5, n = (t & 31) * 4;
+      const int k = t / G2<H>::MQ, n = (t % G2<H>::MQ) * 4;
       *reinterpret_cast<float4*>(&Bsb[k][n]) = make_float4(rb[0], rb[1], rb[2], rb[3]);
     }
   };
-  uint64_t c2[8][4];  // pairs of neighbouring columns
+  uint64_t c2[4 * H][2 * H];  // pairs of neighbouring columns
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < 4 * H; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) c2[i][j] = 0;
+    for (int j = 0; j < 2 * H; ++j) c2[i][j] = 0;
   float ra[4], rb[4];
-  g2_load_a(Ab, lda, tA, M, K, m0, 0, vecA, ra);
+  g2_load_a<H>(Ab, lda, tA, M, K, m0, 0, vecA, ra);
   load_b(0, rb);
-  g2_store_a(As[0], tA, ra);
+  g2_store_a<H>(As[0], tA, ra);
   store_b(Bs[0], rb);
   __syncthreads();
   int buf = 0;
-  for (int k0 = 0; k0 < K; k0 += G2_BK) {
-    const bool more = k0 + G2_BK < K;
+  for (int k0 = 0; k0 < K; k0 += G2<H>::BK) {
+    const bool more = k0 + G2<H>::BK < K;
     if (more) {
-      g2_load_a(Ab, lda, tA, M, K, m0, k0 + G2_BK, vecA, ra);
-      load_b(k0 + G2_BK, rb);
+      g2_load_a<H>(Ab, lda, tA, M, K, m0, k0 + G2<H>::BK, vecA, ra);
+      load_b(k0 + G2<H>::BK, rb);
     }
 #pragma unroll
-    for (int kk = 0; kk < G2_BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4 + 64]);
-      const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][tx * 4]);
-      const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][tx * 4 + 64]);
-      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const uint64_t bv[4] = {b0.x, b0.y, b1.x, b1.y};
+    for (int kk = 0; kk < G2<H>::BK; ++kk) {
+      float av[4 * H];
+      uint64_t bv[2 * H];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int h = 0; h < H; ++h) {
+        const float4 a = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4 + 64 * h]);
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][tx * 4 + 64 * h]);
+        av[4 * h] = a.x, av[4 * h + 1] = a.y, av[4 * h + 2] = a.z, av[4 * h + 3] = a.w;
+        bv[2 * h] = b.x, bv[2 * h + 1] = b.y;
+      }
+#pragma unroll
+      for (int i = 0; i < 4 * H; ++i) {
         uint64_t aa;
         asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(av[i]));
 #pragma unroll
-        for (int j = 0; j < 4; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c2[i][j]) : "l"(aa), "l"(bv[j]));
+        for (int j = 0; j < 2 * H; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c2[i][j]) : "l"(aa), "l"(bv[j]));
       }
     }
     if (more) {
-      g2_store_a(As[buf ^ 1], tA, ra);
+      g2_store_a<H>(As[buf ^ 1], tA, ra);
       store_b(Bs[buf ^ 1], rb);
     }
     __syncthreads();
     buf ^= 1;
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < 4 * H; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < 2 * H; ++j)
       asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[i][2 * j]), "=f"(acc[i][2 * j + 1]) : "l"(c2[i][j]));
 }
 
-template <typename TB>
-__global__ void __launch_bounds__(256, 2)
+template <int H>
+__global__ void __launch_bounds__(256, H == 2 ? 2 : 4)
 gemm_f32_tile_kernel(int M, int N, int K, const float* __restrict__ A, int64_t sA, const int32_t* __restrict__ ia,
-                     int lda, int tA, const TB* __restrict__ B, int64_t sB, const int32_t* __restrict__ ib, int ldb,
+                     int lda, int tA, const float* __restrict__ B, int64_t sB, const int32_t* __restrict__ ib, int ldb,
                      int tB, float* __restrict__ C, int64_t sC, const int32_t* __restrict__ ic, int ldc, float alpha,
                      float beta, int64_t batch, int vecA, int vecB, int vecC) {
-  __shared__ __align__(16) float As[2][G2_BK][G2_LD];
-  __shared__ __align__(16) float Bs[2][G2_BK][G2_LD];
+  __shared__ __align__(16) float As[2][G2<H>::BK][G2<H>::LD];
+  __shared__ __align__(16) float Bs[2][G2<H>::BK][G2<H>::LD];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int m0 = blockIdx.y * G2_BM, n0 = blockIdx.x * G2_BN;
+  const int m0 = blockIdx.y * G2<H>::BM, n0 = blockIdx.x * G2<H>::BN;
   for (int64_t b = blockIdx.z; b < batch; b += gridDim.z) {
     const float* Ab = A + (ia ? (int64_t)ia[b] : b) * sA;
-    const TB* Bb = B + (ib ? (int64_t)ib[b] : b) * sB;
+    const float* Bb = B + (ib ? (int64_t)ib[b] : b) * sB;
     float* Cb = C + (ic ? (int64_t)ic[b] : b) * sC;
-    float acc[8][8];
-    g2_mainloop<TB>(M, N, K, Ab, lda, tA, Bb, ldb, tB, m0, n0, vecA, vecB, As, Bs, acc);
+    float acc[4 * H][4 * H];
+    g2_mainloop<H>(M, N, K, Ab, lda, tA, Bb, ldb, tB, m0, n0, vecA, vecB, As, Bs, acc);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < 4 * H; ++i) {
       const int m = m0 + ty * 4 + (i & 3) + (i >> 2) * 64;
       if (m >= M) continue;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < H; ++h) {
         const int n = n0 + tx * 4 + h * 64;
         float* cp = Cb + (int64_t)m * ldc + n;
         float v[4];
@@ -380,31 +393,31 @@ gemm_f32_tile_kernel(int M, int N, int K, const float* __restrict__ A, int64_t s
 // wholly inside or outside the block and on one side of column K and are
 // stored as vectors; otherwise entry by entry, row m at its place of rs and
 // U's columns behind Rp = Dp - Kp complement columns (no 16-bit copy).
-template <bool VEC>
-__global__ void __launch_bounds__(256, 2) form_u_kernel(int D, int K, const float* __restrict__ W1,
+template <bool VEC, int H>
+__global__ void __launch_bounds__(256, H == 2 ? 2 : 4) form_u_kernel(int D, int K, const float* __restrict__ W1,
                                                         const float* __restrict__ V, float* __restrict__ U,
                                                         float* __restrict__ Ur, void* __restrict__ u16, int bf16,
                                                         int64_t nb, int Dp, int Kp, PadSeg rs, int vecA, int vecB) {
-  __shared__ __align__(16) float As[2][G2_BK][G2_LD];
-  __shared__ __align__(16) float Bs[2][G2_BK][G2_LD];
+  __shared__ __align__(16) float As[2][G2<H>::BK][G2<H>::LD];
+  __shared__ __align__(16) float Bs[2][G2<H>::BK][G2<H>::LD];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int m0 = blockIdx.y * G2_BM, n0 = blockIdx.x * G2_BN;
+  const int m0 = blockIdx.y * G2<H>::BM, n0 = blockIdx.x * G2<H>::BN;
   const int R = D - K;
   for (int64_t b = blockIdx.z; b < nb; b += gridDim.z) {
     const float* Ab = W1 + b * (int64_t)D * K;
     const float* Bb = V + b * (int64_t)D * K;  // V^T row-major K x D
-    float acc[8][8];
-    g2_mainloop<float>(D, D, K, Ab, K, 0, Bb, D, 0, m0, n0, vecA, vecB, As, Bs, acc);
+    float acc[4 * H][4 * H];
+    g2_mainloop<H>(D, D, K, Ab, K, 0, Bb, D, 0, m0, n0, vecA, vecB, As, Bs, acc);
     if constexpr (!VEC) {
       float* Uo = U + b * (int64_t)Dp * Dp;
       float* Uro = Ur + b * (int64_t)Dp * Dp;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < 4 * H; ++i) {
         const int m = m0 + ty * 4 + (i & 3) + (i >> 2) * 64;
         if (m >= D) continue;
         const int mp = m / rs.len * rs.str + m % rs.len;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 4 * H; ++j) {
           const int n = n0 + tx * 4 + (j & 3) + (j >> 2) * 64;
           if (n >= D) continue;
           const int cp = n >= K ? n - K : Dp - Kp + n;
@@ -424,8 +437,8 @@ __global__ void __launch_bounds__(256, 2) form_u_kernel(int D, int K, const floa
     for (int pass = 0; pass < 3; ++pass) {
       if (pass == 2 && !U16b) break;
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const int q4 = g >> 1, h = g & 1;
+      for (int g = 0; g < H * H; ++g) {
+        const int q4 = g / H, h = g % H;
         const int mb = m0 + ty * 4 + q4 * 64, nbase = n0 + tx * 4 + h * 64;
         if (mb >= D || nbase >= D) continue;
         const int cb = nbase >= K ? nbase - K : nbase + R;  // U column of Q column nbase
@@ -462,12 +475,16 @@ __global__ void __launch_bounds__(256, 2) form_u_kernel(int D, int K, const floa
 void launch_form_u(int64_t nb, int D, int K, const float* W1, const float* V, float* U, float* Ur, void* u16,
                    int bf16, int Dp, int Kp, PadSeg rs, cudaStream_t st) {
   if (nb == 0 || D == 0) return;
-  dim3 g((D + G2_BN - 1) / G2_BN, (D + G2_BM - 1) / G2_BM, (unsigned)std::min<int64_t>(nb, 65535));
+  // (64 x 64 tiles while 128 x 128 ones leave SMs idle)
+  const int64_t big = nb * ((D + 127) / 128) * ((D + 127) / 128);
+  const int bm = big < 152 ? 64 : 128;
+  const dim3 g((D + bm - 1) / bm, (D + bm - 1) / bm, (unsigned)std::min<int64_t>(nb, 65535));
+  const bool vec = D % 4 == 0 && K % 4 == 0 && Dp == D;
+  auto go = vec ? (bm == 64 ? form_u_kernel<true, 1> : form_u_kernel<true, 2>)
+                : (bm == 64 ? form_u_kernel<false, 1> : form_u_kernel<false, 2>);
   ++g_launches;
-  if (D % 4 == 0 && K % 4 == 0 && Dp == D)
-    form_u_kernel<true><<<g, 256, 0, st>>>(D, K, W1, V, U, Ur, u16, bf16, nb, Dp, Kp, rs, 1, 1);
-  else
-    form_u_kernel<false><<<g, 256, 0, st>>>(D, K, W1, V, U, Ur, nullptr, bf16, nb, Dp, Kp, rs, K % 4 == 0, D % 4 == 0);
+  go<<<g, 256, 0, st>>>(D, K, W1, V, U, Ur, vec ? u16 : nullptr, bf16, nb, Dp, Kp, rs, vec || K % 4 == 0,
+                        vec || D % 4 == 0);
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
@@ -482,10 +499,14 @@ void gemm_simt(int M, int N, int K, const T* A, int64_t sA, const int32_t* ia, i
     const int vecA = (lda % 4 == 0) && (sA % 4 == 0) && aligned16(A);
     const int vecB = (ldb % 4 == 0) && (sB % 4 == 0) && aligned16(B);
     const int vecC = (ldc % 4 == 0) && (sC % 4 == 0) && aligned16(C);
-    dim3 g2((N + G2_BN - 1) / G2_BN, (M + G2_BM - 1) / G2_BM, (unsigned)std::min<int64_t>(batch, 65535));
+    // (64 x 64 tiles while 128 x 128 ones leave SMs idle)
+    const int64_t big = batch * ((M + 127) / 128) * ((N + 127) / 128);
+    const int bm = big < 152 ? 64 : 128;
+    const dim3 g2((N + bm - 1) / bm, (M + bm - 1) / bm, (unsigned)std::min<int64_t>(batch, 65535));
+    auto go = bm == 64 ? gemm_f32_tile_kernel<1> : gemm_f32_tile_kernel<2>;
     ++g_launches;
-    gemm_f32_tile_kernel<float><<<g2, 256, 0, st>>>(M, N, K, A, sA, ia, lda, tA, B, sB, ib, ldb, tB, C, sC, ic, ldc,
-                                                    alpha, beta, batch, vecA, vecB, vecC);
+    go<<<g2, 256, 0, st>>>(M, N, K, A, sA, ia, lda, tA, B, sB, ib, ldb, tB, C, sC, ic, ldc, alpha, beta, batch, vecA,
+                           vecB, vecC);
     return;
   }
   dim3 grid((N + 63) / 64, (M + 63) / 64, (unsigned)std::min<int64_t>(batch, 65535));
@@ -499,9 +520,6 @@ template void gemm_simt<double, double>(int, int, int, const double*, int64_t, c
 template void gemm_simt<float, float>(int, int, int, const float*, int64_t, const int32_t*, int, bool,
                                       const float*, int64_t, const int32_t*, int, bool, float*, int64_t,
                                       const int32_t*, int, float, float, int64_t, cudaStream_t);
-template void gemm_simt<float, double>(int, int, int, const float*, int64_t, const int32_t*, int, bool,
-                                       const double*, int64_t, const int32_t*, int, bool, float*, int64_t,
-                                       const int32_t*, int, float, float, int64_t, cudaStream_t);
 
 // ------------------------------------------------------------------------
 // block-wide sum
