@@ -830,7 +830,8 @@ __device__ __forceinline__ void qr_reduce_cols(float (&d)[CPW]) {
 
 // Householder reflector of one register-held column (rows lane + 32 s) at
 // pivot row k, by the warp that owns it: the column becomes beta at row k and
-// v below it (v_k = 1 implied); v (zeros above k) goes to vb, tau to *stau.
+// v below it (v_k = 1 implied); v (zeros above k) goes to vb (this lane's rows
+// together), tau to *stau.
 template <int RPL>
 __device__ __forceinline__ void qr_reflector(float (&xc)[RPL], int k, int lane, float* vb, float* stau) {
   float alpha = 0.0f, part = 0.0f;
@@ -838,46 +839,66 @@ __device__ __forceinline__ void qr_reflector(float (&xc)[RPL], int k, int lane, 
   for (int s = 0; s < RPL; ++s) {
     const int r = lane + 32 * s;
     if (r == k) alpha = xc[s];
-    if (r > k) part += xc[s] * xc[s];
+    if (r > k) part = fmaf(xc[s], xc[s], part);
   }
-  for (int o = 16; o; o >>= 1) {
-    part += __shfl_xor_sync(0xffffffffu, part, o);
-    alpha += __shfl_xor_sync(0xffffffffu, alpha, o);
-  }
+  alpha = __shfl_sync(0xffffffffu, alpha, k & 31);
+  for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   float tau = 0.0f, beta = alpha, scal = 0.0f;
   if (part != 0.0f) {
-    beta = -copysignf(sqrtf(alpha * alpha + part), alpha);
+    beta = -copysignf(sqrtf(fmaf(alpha, alpha, part)), alpha);
     tau = (beta - alpha) / beta;
     scal = 1.0f / (alpha - beta);
   }
+  float v[RPL];
 #pragma unroll
   for (int s = 0; s < RPL; ++s) {
     const int r = lane + 32 * s;
-    float vv = 0.0f;
+    v[s] = 0.0f;
     if (r == k) {
-      vv = 1.0f;
+      v[s] = 1.0f;
       xc[s] = beta;
     } else if (r > k && tau != 0.0f) {
-      vv = xc[s] * scal;
-      xc[s] = vv;
+      xc[s] *= scal;
+      v[s] = xc[s];
     }
-    vb[r] = vv;
   }
+#pragma unroll
+  for (int s = 0; s < RPL; s += 4)
+    *reinterpret_cast<float4*>(vb + lane * RPL + s) = make_float4(v[s], v[s + 1], v[s + 2], v[s + 3]);
   if (lane == 0) *stau = tau;
 }
+// Barriers 1 and 2 of 512 threads: arrive without waiting, or wait.
+__device__ __forceinline__ void qr_arrive(int id) { asm volatile("barrier.cta.arrive %0, 512;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void qr_wait(int id) { asm volatile("barrier.cta.sync %0, 512;" ::"r"(id) : "memory"); }
 
-// The same factorization in FP32 with the panel in registers: warp w owns
-// the contiguous columns 8 w .. 8 w + 7 and lane l rows l, l + 32, ...
-// (D <= 32 RPL, K <= 128).  Step k: the owner warp of column k forms the
-// reflector (warp reductions only) and publishes v and tau through a
-// double-buffered shared vector; after one barrier the warps that still
-// hold columns j > k update them: w = tau v^T x_j (lane-local products, one
-// warp reduction), x_j -= w v.  The warps whose columns are finished
-// reflectors (j < k) form the Gram entries v_j^T v_k instead, so that after
-// the last step the compact-WY factor Tw = (striu(V^T V) + diag(1 / tau))^-1
-// (zero-tau rows and columns masked, as in wy_tinv_kernel) is inverted in
-// shared memory by the same CTA (Tw NULL: no factor).  The rank-1 updates
-// stay in registers; shared memory carries v, the Gram matrix and Tw.
+// two floats in one register pair
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t p, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
+}
+
+// The same factorization in FP32 with the panel in registers: column j belongs to
+// warp j mod 16 and lane l holds rows l, l + 32, ... (D <= 32 RPL, K <= 128).
+// Step k: v_k and tau lie in shared memory (two buffers).  The warp of column k
+// + 1 updates that column first, forms its reflector, publishes it and arrives
+// at step k + 1's barrier without waiting, then catches up with its other
+// columns; the other warps update theirs (w = tau v^T x_j, lane-local
+// products, one warp reduction for eight columns, x_j -= w v) and wait
+// there.  A warp's finished columns (j < k) give the Gram entries v_j^T v_k
+// instead, so that after the last step the compact-WY factor Tw = (striu(V^T V) +
+// diag(1 / tau))^-1 (zero-tau rows and columns masked, as in wy_tinv_kernel) is
+// inverted in shared memory by the same CTA (Tw NULL: no factor).  Two barriers
+// alternate: the next publisher has passed the barrier at which everybody
+// else had read the buffer it overwrites (the last publisher read it before it arrived).
+// Bound by the chain of the reflectors (update of one column, two reductions, a
+// square root, a division) and the issue of the updates.  Ten levels of 262144
+// points (1024 to 2 boxes of 256 x 128) 3.87 ms; with a barrier between every
+// reflector and its updates, columns contiguous and scalar products 5.07 ms; a
+// cluster of 2 to 8 CTAs a box was slower (0.27 - 0.42 ms a level against 0.19).
 template <int RPL>
 __global__ void __launch_bounds__(512) qr_reg_kernel(int D, int K, int Kp, const float* __restrict__ Xin,
                                                      float* __restrict__ Vout, float* __restrict__ tau_out,
@@ -894,7 +915,7 @@ __global__ void __launch_bounds__(512) qr_reg_kernel(int D, int K, int Kp, const
   float(*tile)[NW * CPW + 1] = reinterpret_cast<float(*)[NW * CPW + 1]>(scr);
   const int box = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float* src = Xin + (size_t)box * D * K;  // row-major D x K
-  float x[CPW][RPL];
+  uint64_t x2[CPW / 2][RPL];  // columns 2 q and 2 q + 1 of this warp (fma.rn.f32x2: the roundings of two fmaf)
   // load through shared memory, 32 rows at a time (coalesced reads)
 #pragma unroll
   for (int s = 0; s < RPL; ++s) {
@@ -904,60 +925,99 @@ __global__ void __launch_bounds__(512) qr_reg_kernel(int D, int K, int Kp, const
     }
     __syncthreads();
 #pragma unroll
-    for (int c = 0; c < CPW; ++c) {
-      const int j = CPW * warp + c;
-      x[c][s] = (j < K) ? tile[lane][j] : 0.0f;
+    for (int q = 0; q < CPW / 2; ++q) {
+      const int j = warp + 2 * NW * q;
+      x2[q][s] = pack2((j < K) ? tile[lane][j] : 0.0f, (j + NW < K) ? tile[lane][j + NW] : 0.0f);
     }
     __syncthreads();
   }
-  // columns c >= c_lo of this warp take the update with reflector (vb, tk);
-  // columns c < c_gram (finished reflectors j < k) give G[j][k] = v_j^T v_k
-  auto update = [&](int c_lo, int c_gram, const float* vb, float tk, int k) {
-    float v[RPL];
+  const bool gram = Tw != nullptr;
+  // column c (a constant) as a copy, and back
+  auto get = [&](int c, float(&xc)[RPL]) {
 #pragma unroll
-    for (int s = 0; s < RPL; ++s) v[s] = vb[lane + 32 * s];
-    float d[CPW];
-#pragma unroll
-    for (int c = 0; c < CPW; ++c) {
-      d[c] = 0.0f;
-      if ((c >= c_lo || c < c_gram) && CPW * warp + c < K) {
-#pragma unroll
-        for (int s = 0; s < RPL; ++s) d[c] = fmaf(v[s], x[c][s], d[c]);
-      }
-    }
-    qr_reduce_cols<CPW>(d);
-#pragma unroll
-    for (int c = 0; c < CPW; ++c) {
-      if (c >= c_lo && CPW * warp + c < K) {
-        const float dj = d[c] * tk;
-#pragma unroll
-        for (int s = 0; s < RPL; ++s) x[c][s] = fmaf(-dj, v[s], x[c][s]);
-      }
-    }
-    if (lane == 0) {
-#pragma unroll
-      for (int c = 0; c < CPW; ++c)
-        if (c < c_gram && CPW * warp + c < K) Gm[(CPW * warp + c) * ldg + k] = d[c];
+    for (int s = 0; s < RPL; ++s) {
+      float lo, hi;
+      unpack2(x2[c / 2][s], lo, hi);
+      xc[s] = c % 2 ? hi : lo;
     }
   };
-  const bool gram = Tw != nullptr;
-  int buf = 0;
-  for (int cw = 0; cw < NW; ++cw) {
+  auto put = [&](int c, const float(&xc)[RPL]) {
 #pragma unroll
-    for (int cc = 0; cc < CPW; ++cc) {
-      const int k = CPW * cw + cc;
+    for (int s = 0; s < RPL; ++s) {
+      float lo, hi;
+      unpack2(x2[c / 2][s], lo, hi);
+      x2[c / 2][s] = c % 2 ? pack2(lo, xc[s]) : pack2(xc[s], hi);
+    }
+  };
+  if (warp == 0) {
+    float xc[RPL];
+    get(0, xc);
+    qr_reflector<RPL>(xc, 0, lane, vsb, s_tau);
+    put(0, xc);
+    qr_arrive(1);
+  }
+#pragma unroll
+  for (int kc = 0; kc < CPW; ++kc) {
+    for (int w = 0; w < NW; ++w) {
+      const int k = NW * kc + w, buf = k & 1;
       if (k >= K) break;
-      float* vb = vsb + buf * RPL * 32;
-      if (warp == cw) qr_reflector<RPL>(x[cc], k, lane, vb, &s_tau[buf]);
-      __syncthreads();
+      if (warp == w) __syncwarp();  // (published v_k and arrived itself)
+      else qr_wait(buf + 1);
       const float tk = s_tau[buf];
-      if (tk != 0.0f) {
-        if (warp > cw) update(0, 0, vb, tk, k);
-        else if (warp == cw) update(cc + 1, gram ? cc : 0, vb, tk, k);
-        else if (gram) update(CPW, CPW, vb, tk, k);
+      float v[RPL];
+#pragma unroll
+      for (int s = 0; s < RPL; s += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(vsb + buf * RPL * 32 + lane * RPL + s);
+        v[s] = t.x, v[s + 1] = t.y, v[s + 2] = t.z, v[s + 3] = t.w;
       }
       if (threadIdx.x == 0) tau_out[(size_t)box * K + k] = tk, tau_s[k] = tk;
-      buf ^= 1;
+      // the next column first
+      auto ahead = [&](int c) {
+        float xc[RPL], d = 0.0f;
+        get(c, xc);
+#pragma unroll
+        for (int s = 0; s < RPL; ++s) d = fmaf(v[s], xc[s], d);
+        for (int o = 16; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        const float dj = d * tk;
+        if (tk != 0.0f)
+#pragma unroll
+          for (int s = 0; s < RPL; ++s) xc[s] = fmaf(-dj, v[s], xc[s]);
+        qr_reflector<RPL>(xc, k + 1, lane, vsb + (buf ^ 1) * RPL * 32, &s_tau[buf ^ 1]);
+        qr_arrive((buf ^ 1) + 1);
+        put(c, xc);
+      };
+      const bool next0 = k + 1 < K && w + 1 < NW && warp == w + 1;
+      const bool next1 = kc + 1 < CPW && k + 1 < K && w + 1 == NW && warp == 0;
+      if (next0) ahead(kc);
+      if (kc + 1 < CPW)
+        if (next1) ahead(kc + 1);
+      if (tk == 0.0f) continue;
+      uint64_t vv[RPL], d2[CPW / 2];
+#pragma unroll
+      for (int s = 0; s < RPL; ++s) vv[s] = pack2(v[s], v[s]);
+      float d[CPW];
+#pragma unroll
+      for (int q = 0; q < CPW / 2; ++q) {
+        d2[q] = 0;
+#pragma unroll
+        for (int s = 0; s < RPL; ++s) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d2[q]) : "l"(vv[s]), "l"(x2[q][s]));
+        unpack2(d2[q], d[2 * q], d[2 * q + 1]);
+      }
+      qr_reduce_cols<CPW>(d);
+      float u[CPW];  // -tau w, 0 for the columns that are finished or ahead
+#pragma unroll
+      for (int c = 0; c < CPW; ++c) {
+        const bool after = c > kc ? !(c == kc + 1 && next1) : (c == kc && warp > w && !next0);
+        u[c] = after ? -(d[c] * tk) : 0.0f;
+        if (gram && lane == 0 && (c < kc || (c == kc && warp < w))) Gm[(warp + NW * c) * ldg + k] = d[c];
+      }
+#pragma unroll
+      for (int q = 0; q < CPW / 2; ++q) {
+        if (2 * q + 1 < kc) continue;
+        const uint64_t uu = pack2(u[2 * q], u[2 * q + 1]);
+#pragma unroll
+        for (int s = 0; s < RPL; ++s) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(x2[q][s]) : "l"(uu), "l"(vv[s]));
+      }
     }
   }
   // R (row-major, upper) and V (column-major, unit diagonal, zeros above)
@@ -965,13 +1025,15 @@ __global__ void __launch_bounds__(512) qr_reg_kernel(int D, int K, int Kp, const
   float* Vb = Vout + (size_t)box * D * K;
 #pragma unroll
   for (int c = 0; c < CPW; ++c) {
-    const int j = CPW * warp + c;
+    const int j = warp + NW * c;
     if (j >= K) continue;
+    float xc[RPL];
+    get(c, xc);
 #pragma unroll
     for (int s = 0; s < RPL; ++s) {
       const int r = lane + 32 * s;
-      if (r < K) Rb[(size_t)r * K + j] = (r <= j) ? x[c][s] : 0.0f;
-      if (r < D) Vb[(size_t)j * D + r] = (r > j) ? x[c][s] : (r == j ? 1.0f : 0.0f);
+      if (r < K) Rb[(size_t)r * K + j] = (r <= j) ? xc[s] : 0.0f;
+      if (r < D) Vb[(size_t)j * D + r] = (r > j) ? xc[s] : (r == j ? 1.0f : 0.0f);
     }
   }
   if (!gram) return;
