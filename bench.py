@@ -237,7 +237,7 @@ LEAF_TRAFFIC = {"digest": "1381b342a0b471df", "bytes_per_launch": (347.004160e6 
 def leaf_kernel_digest() -> str:
     src = open(os.path.join(ROOT, "paper_2502_02395_gb300", "csrc", "kernels_solve.cu")).read()
     a = src.index("// -------------------------------------------- symmetric leaf near blocks ---")
-    b = src.index("// y_i = X_i yh_i + sum of box i's partial products")
+    b = src.index("// FP32-pair form for the residual (see df_fma)")
     return hashlib.sha256(src[a:b].encode()).hexdigest()[:16]
 
 
@@ -254,7 +254,7 @@ def kernel_roofline(stats, t_leaf, n_leaf, peaks):
     if LEAF_TRAFFIC and LEAF_TRAFFIC.get("digest") == leaf_kernel_digest():
         traffic = LEAF_TRAFFIC["bytes_per_launch"]
     return {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak, "traffic": traffic,
-            "kernel": stats.get("leaf_kernel", "mv_leaf_kernel<float>"), "launches_per_step": n_leaf,
+            "kernel": stats.get("leaf_kernel", "mv_sym_pair_kernel<float>"), "launches_per_step": n_leaf,
             "bytes_per_launch": by,
             "ms_per_launch": per * 1e3,
             "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if "hbm_gbs" in peaks else "fallback 6800 GB/s"}

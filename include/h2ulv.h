@@ -301,12 +301,14 @@ h2_status h2_matvec_noalloc(h2_ctx* c, const double* x, double* y);
  *   H2_OPT_RESIDUAL_FP64  refinement scheme 2: 0 (default) forms
  *                         b - A_H2 x in FP32-pair arithmetic, 1 with FP64
  *                         instructions (the h2_matvec operator).
- *   H2_OPT_GRAPHS         1 (default): the FP32 substitution of FP16/BF16
- *                         factorizations is captured once per factorization
- *                         as a CUDA graph (on a private stream) and replayed
- *                         for every preconditioner application; 0: plain
- *                         launches.  A capture that fails falls back to
- *                         plain launches.
+ *   H2_OPT_GRAPHS         1 (default): the refinement of FP16/BF16
+ *                         factorizations is captured as CUDA graphs (the
+ *                         inner iteration: substitution, matvec and
+ *                         orthogonalization; the residual; one ULV
+ *                         application), on a private stream, the first time
+ *                         each is needed after a factorization or a change
+ *                         of an option, and replayed; 0: plain launches.  A
+ *                         capture that fails falls back to plain launches.
  *   H2_OPT_TC_KERNEL      the kernel form of the factorization's main-chain
  *                         tensor-core GEMMs (projection, Schur update;
  *                         process-wide, all contexts): 0 one CTA per batch

@@ -2841,7 +2841,7 @@ h2_status h2_stats(const h2_ctx* c, char* json, size_t cap) {
   }
   o << "],\"bytes_proj\":" << by_proj << ",\"bytes_subst\":" << by_sub << ",\"bytes_matvec\":" << by_mv << ",\"flops_matvec\":" << fl_mv
     << ",\"bytes_matvec32\":" << by_mv / 2 << ",\"bytes_matvec32_leaf\":" << by_leaf32 << ",\"leaf_kernel\":\""
-    << ((c->sym && c->prec != H2_PREC_FP64) ? "mv_sym_pair_kernel<float>" : "mv_leaf_kernel<float>") << "\"";
+    << ((c->sym && c->prec != H2_PREC_FP64) ? "mv_sym_pair_kernel<float>" : "mv_block_rows_kernel<float>") << "\"";
   o << ",\"flops\":{\"a1_qr\":" << fl_qr << ",\"a2_proj\":" << fl_proj << ",\"a3_lu\":" << fl_lu
     << ",\"a45_schur\":" << fl_schur << ",\"a2c_coupling\":" << fl_coup << "}";
   o << ",\"times\":{\"a1_qr\":" << t.a1_qr << ",\"a2_proj\":" << t.a2_proj << ",\"a3_lu\":" << t.a3_lu

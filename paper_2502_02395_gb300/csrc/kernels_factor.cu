@@ -3,15 +3,16 @@
 //   eval_blocks_kernel     dense kernel blocks G(B_i, B_j) of the leaf near
 //                          pairs and couplings G(SK_i, SK_j) (Algorithm 1),
 //                          evaluated from the points
-//   gemm_batched_kernel    SIMT batched GEMM C = alpha op(A) op(B) + beta C
-//                          (FP64 path: the projection and Schur update
-//                          of Algorithm 4, couplings)
-//   qr_panel_kernel,       Householder QR of X^orth, its compact WY factor
-//   wy_tfactor_kernel      and the explicit U = [U^R U^S] (Eq. 6-7)
-//   lu_inverse_kernel      partial-pivot LU of Ahat_ii^RR in FP64 (Algorithm
-//                          2, with LU in place of Cholesky) and the
-//                          explicit inverse (Ahat_ii^RR)^-1 used by the
-//                          Schur update and by the substitution of Eq. 31
+//   gemm_f32_tile_kernel,  SIMT batched GEMM C = alpha op(A) op(B) + beta C in
+//   gemm_batched_kernel    FP32, and in FP64 where the digit form on the tensor
+//                          cores does not apply
+//   qr_reg_kernel,         Householder QR of X^orth (FP32; FP64; any size), its
+//   qr_cluster_kernel,     compact WY factor and the explicit U = [U^R U^S]
+//   qr_panel_kernel        (Eq. 6-7)
+//   gj_rows_kernel,        partial-pivot elimination of Ahat_ii^RR (Algorithm
+//   gj_cluster_kernel,     2, with LU in place of Cholesky) and the explicit
+//   lu_inverse_kernel      inverse (Ahat_ii^RR)^-1 used by the Schur update and by
+//                          the substitution of Eq. 31
 //   merge_kernel           children's SS blocks / couplings into the parent
 //                          near blocks (the merge of Algorithm 2)
 #include <type_traits>

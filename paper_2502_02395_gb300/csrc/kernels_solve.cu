@@ -4,7 +4,8 @@
 // backward pass.  With Ainv_i = (Ahat_ii^RR)^-1 = U'_ii^-1 (P_i L_ii)^-1, the
 // product form of L^-1 in Eq. 31 needs only whole-block inverses and
 // matrix-vector products, so every step below is a batched GEMV over all
-// boxes of a level (one CTA per box), with no serial triangular solve:
+// boxes of a level (one CTA per box, or a cluster on levels of few boxes), with
+// no serial triangular solve:
 //   fwd1  c_i = U_i^T b_i;                  u_i = Ainv_i c_i^R
 //   fwd2  v_i = Ainv_i (c_i^R - sum_{j<i near} Ahat_ij^RR u_j)
 //   fwd3  s_i = c_i^S - sum_{j near} Ahat_ij^SR v_j   -> parent input
@@ -232,8 +233,6 @@ __device__ __forceinline__ void zero(T (&acc)[RPW]) {
   for (int t = 0; t < RPW; ++t) acc[t] = T(0);
 }
 
-constexpr int kRPW = 16;  // rows per warp per pass: 128-row chunks with 8 warps
-constexpr int kChunk = 8 * kRPW;
 
 // ------------------------------------------------------------------------
 // CTA-wide GEMV on 16-byte chunks.
