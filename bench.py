@@ -226,11 +226,11 @@ def fp64_peak_tflops() -> float:
 # DRAM traffic of one launch of the FP32 matvec's leaf kernel (the step's
 # largest kernel: the symmetric-storage pair kernel), valid while the
 # kernel's source is the one captured (digest of its text below).  Captured
-# on the small case cube32768_yukawa (1323 stored pairs: 347.00 MB read +
-# 4.45 MB written in one launch) and scaled to the 12875 stored pairs of
+# on a small case (32768 points of the cube, Yukawa, 1304 stored pairs: 342.07 MB read +
+# 4.72 MB written in one launch) and scaled to the 12875 stored pairs of
 # cube262144_yukawa: the kernel reads each stored 256 x 256 block once, so
 # its traffic grows with the stored pairs.
-LEAF_TRAFFIC = {"digest": "1381b342a0b471df", "bytes_per_launch": (347.004160e6 + 4.454144e6) * 12875 / 1323,
+LEAF_TRAFFIC = {"digest": "debcdaa0c5696a32", "bytes_per_launch": (342.071040e6 + 4.721408e6) * 12875 / 1304,
                 "profile": "profiles/mv_sym_pair_kernel_cube262144_yukawa.md"}
 
 

@@ -1430,10 +1430,12 @@ lu_inverse_kernel(int R, const T* __restrict__ luT, const int32_t* __restrict__ 
 // box) in status[0..1] and leaves the box's output undefined.  The pivot rows
 // go to piv; pivot_sequence_kernel turns them into LAPACK's interchanges.
 // Bound by the latency of a step (two barriers, a shuffle reduction, a
-// reciprocal: about 0.25 us) in FP32 and by the FP64 pipe in FP64.  A panel
-// form in which one warp ran 16 steps at a time took 165 us for 128 x 128;
-// 256 x 256 took 436 us with four CTAs a box and the pivot column read from
-// the owner.
+// reciprocal: 0.7 us at R = 128) in FP32 and by the FP64 pipe in FP64.  FP32:
+// 128 x 128 in 92 us, 256 x 256 in 346 us; a panel form in which one warp ran 16
+// steps at a time took 165 us, and 256 x 256 with four CTAs a box and the pivot
+// column read from the owner 436 us.  FP64: 128 x 128 in 0.6 ms (inverse) and 0.8
+// ms (LU), 256 x 256 in 2.0 and 2.1 ms; the LU of one 256 x 256 root by one CTA in
+// global memory and its inverse took 20.6 ms.
 // ------------------------------------------------------------------------
 __device__ __forceinline__ float rcp_pivot(float v) { return __frcp_rn(v); }
 __device__ __forceinline__ double rcp_pivot(double v) { return 1.0 / v; }
