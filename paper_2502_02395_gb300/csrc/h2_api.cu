@@ -1350,6 +1350,18 @@ void matvec_t(h2_ctx* c, const T* A, T* const* X, T* const* S, T* xh, T* yh, con
                             nullptr, nullptr, nullptr, true, st);
   }
   if (leaf_ev) cudaEventRecord(e0, st);
+  if constexpr (std::is_same<T, float>::value) {
+    if (c->sym) {
+      // A holds the pairs i <= j only, also where the couplings do not
+      // qualify for the form above (a rank that is no multiple of 4 beside a
+      // leaf of tensor-core shape, a far list that is not closed)
+      launch_matvec_sym_pairs(lf.D, lf.D, c->npu, c->sym_desc, A, x, c->part32, false, st);
+      if (leaf_ev) cudaEventRecord(e1, st), leaf_ev->push_back({e0, e1});
+      launch_matvec_rows<float>(lf.nb, lf.D, lf.K, X[L], yh + off[L], nullptr, y, lf.D, c->sym_ptr, c->sym_ent,
+                                c->part32, true, st);
+      return;
+    }
+  }
   launch_matvec_block_rows<T>(la, st);
   if (leaf_ev) cudaEventRecord(e1, st), leaf_ev->push_back({e0, e1});
 }

@@ -1,0 +1,59 @@
+"""Instances whose leaf blocks are kept as symmetric halves while their
+couplings are not: ranks that are no multiple of 4 beside leaves of a
+tensor-core shape, and an imported far list that is not closed under (i, j) ->
+(j, i).  The FP32 operator of the mixed refinement then takes the general form
+of the couplings with the halves of the leaf blocks."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2502_02395_gb300 import build as bld
+    bld.build()
+    from paper_2502_02395_gb300 import binding
+    return binding
+
+
+def check_arithmetics(S, n):
+    """FP32 sums of at most some thousand terms: 1e-6; FP32 pairs: 2^-44 (the
+    bounds of the other shapes)."""
+    x = W.uniform_rhs(n, 4)
+    y = S.matvec(x)
+    assert np.linalg.norm(S.matvec_arith(x, "fp32") - y) <= 1e-6 * np.linalg.norm(y)
+    assert np.linalg.norm(S.matvec_arith(x, "fp32_pair") - y) <= 2.0 ** -44 * np.linalg.norm(y)
+
+
+@pytest.mark.parametrize("n,leaf,rank", [(2048, 256, 77), (4096, 256, 98), (2048, 128, 50), (2048, 128, 33)])
+def test_halves_with_odd_ranks(B, n, leaf, rank):
+    S = B.H2Solver.build(W.cube_points(n, 3), kernel="yukawa_eps", diag_shift=1.0, leaf=leaf, eta=1.0, tol=1e-12,
+                         max_rank=rank, far_samples=512, near_samples=32)
+    lv = S.stats()["levels"]
+    assert lv[-1]["D"] % 128 == 0 and lv[-1]["K"] == rank and any(d["FP"] > 0 for d in lv)
+    check_arithmetics(S, n)
+    b = W.uniform_rhs(n, 5)
+    for prec in ("fp16", "bf16"):
+        S.factor(prec)
+        x, rel, _ = S.solve(b, target=1e-10, max_iters=300)
+        assert rel <= 1e-10 and np.linalg.norm(b - S.matvec(x)) <= 2e-10 * np.linalg.norm(b)
+
+
+def test_halves_with_an_open_far_list(B):
+    from oracle.construct import construct
+    from oracle.instance import flatten
+    from oracle.kernels import Kernel
+    n = 1024
+    H = construct(W.cube_points(n, 3), Kernel("yukawa_eps", diag_shift=1.0), 128, 1.0, 1e-8, 64, 256, 32)
+    flat = flatten(H)
+    l = max(k for k in range(flat["L"] + 1) if len(flat["far"][k]))
+    flat["far"][l] = np.ascontiguousarray(flat["far"][l][:-1])  # (j, i) stays, (i, j) goes
+    S = B.H2Solver.from_instance(flat, kernel="yukawa_eps", leaf=128, eta=1.0, tol=1e-8, max_rank=64, far_samples=256,
+                                 near_samples=32, diag_shift=1.0)
+    check_arithmetics(S, n)
