@@ -1704,11 +1704,15 @@ h2_status fgmres_cycle(h2_ctx* c, GmresWork& W, int m, double beta, const T* r, 
 }
 
 // The pinned block (8-byte slots): h1 (m0 + 2), h2 (m0 + 2) and ||w||^2, the
-// residual's norm, k and y of the update, the iteration count, a cycle's times.
+// residual's norm, k and y of the update, a cycle's times.  The places go with
+// the restart m0 in force; every slot is written before it is read within a
+// cycle.  The iteration count that wait_iteration polls lies behind all of
+// them, at a place that does not move while the block lives (host_slots of
+// the restart it was made for): elsewhere the numbers of an earlier cycle
+// under another restart would pass for a count.
 size_t slot_rn(int m0) { return 2 * (size_t)(m0 + 2) + 1; }
 size_t slot_y(int m0) { return slot_rn(m0) + 1; }
-size_t slot_flag(int m0) { return slot_y(m0) + m0 + 8; }
-size_t slot_stamp(int m0) { return slot_flag(m0) + 8; }
+size_t slot_stamp(int m0) { return slot_y(m0) + m0 + 8; }
 size_t host_slots(int m0) { return slot_stamp(m0) + kGmStamps * (size_t)(m0 + 1); }
 
 h2_status gmres_work(h2_ctx* c, GmresWork& W) {
@@ -1722,8 +1726,9 @@ h2_status gmres_work(h2_ctx* c, GmresWork& W) {
     drop_graphs(c);  // (they hold the old buffers)
     if (c->gm_host) cudaFreeHost(c->gm_host);
     c->gm_host = nullptr;
-    CKC(cudaMallocHost(&c->gm_host, host_slots(m0) * sizeof(double)));
-    std::memset(c->gm_host, 0, host_slots(m0) * sizeof(double));
+    CKC(cudaMallocHost(&c->gm_host, (host_slots(m0) + 8) * sizeof(double)));
+    std::memset(c->gm_host, 0, (host_slots(m0) + 8) * sizeof(double));
+    c->gm_flag = reinterpret_cast<unsigned long long*>(c->gm_host + host_slots(m0));
     CKC(dalloc(c, &c->gm_part, (size_t)(2 * (m0 + 1) + 1) * kOrthCtas));
     CKC(dalloc(c, &c->gm_w32, (size_t)n32));
     CKC(dalloc(c, &c->gm_state, 1));
@@ -1805,8 +1810,8 @@ h2_status gmres_refine(h2_ctx* c, SolveTimer& tm, double bnorm, double target, i
 // to pinned memory after the iteration's numbers).  Polling sees it a few
 // microseconds earlier than a stream synchronization would; a stream that has
 // become idle or failed without reporting ends the wait.
-h2_status wait_iteration(h2_ctx* c, int m0, unsigned long long seq) {
-  const unsigned long long* flag = reinterpret_cast<const unsigned long long*>(c->gm_host + slot_flag(m0));
+h2_status wait_iteration(h2_ctx* c, unsigned long long seq) {
+  const unsigned long long* flag = c->gm_flag;
   for (unsigned n = 1;; ++n) {
     if (__atomic_load_n(flag, __ATOMIC_ACQUIRE) >= seq) return H2_OK;
     if (n % 512 == 0) {
@@ -1834,7 +1839,7 @@ h2_status inner_cycle(h2_ctx* c, GmresWork& W, SolveTimer& tm, int m, double tol
   oa.n = nslots32(c), oa.m0 = m0, oa.ctas = orth_ctas(oa.n);
   oa.part = W.part, oa.h = W.h1, oa.state = c->gm_state, oa.stamp = c->gm_stamp;
   oa.host = c->gm_host;
-  oa.flag = reinterpret_cast<unsigned long long*>(c->gm_host + slot_flag(m0));
+  oa.flag = c->gm_flag;
   run_graph(c, c->g_start, [&] {
     launch_norm2<double>(c->r64, nslots(c), c->red, c->stream);
     launch_pad_scaled_copy(c->r64, c->red, c->gm_r32, nslots(c), leaf_seg(c), c->stream);
@@ -1851,7 +1856,7 @@ h2_status inner_cycle(h2_ctx* c, GmresWork& W, SolveTimer& tm, int m, double tol
       launch_orth(oa, c->stream);
     });
     CKC(cudaGetLastError());
-    CKS(wait_iteration(c, m0, ++c->gm_seq));
+    CKS(wait_iteration(c, ++c->gm_seq));
     ++its;
     k = j + 1;
     if (givens_step(W, j, c->gm_host, c->gm_host + m0 + 2, c->gm_host[2 * (m0 + 2)], tol_abs)) break;

@@ -430,8 +430,8 @@ struct h2_ctx {
   double* gm_V = nullptr;        // (restart + 1) * nslot Krylov basis
   double* gm_Z = nullptr;        // restart * nslot preconditioned directions
   double* gm_h = nullptr;        // h1, h2 (restart + 2 each), the norm slot (257), y (restart + 2)
-  double* gm_host = nullptr;     // pinned copy of h1, h2 and the norm (one read per FGMRES step)
-  double* gm_part = nullptr;     // (restart + 1) * 128 dot-product partials
+  double* gm_host = nullptr;     // pinned: h1, h2, norms, y, times and the iteration count (host_slots)
+  double* gm_part = nullptr;     // (2 (restart + 1) + 1) * kOrthCtas dot-product partials
   float* gm_V32 = nullptr;       // FP32 Krylov basis / directions of the inner solver
   float* gm_Z32 = nullptr;
   float* gm_r32 = nullptr;
@@ -440,6 +440,7 @@ struct h2_ctx {
   float* gm_w32 = nullptr;       // the inner iteration's A z
   h2::GmState* gm_state = nullptr;
   unsigned long long* gm_stamp = nullptr;  // 5 (gm_cap + 1) device times of a cycle's iterations
+  unsigned long long* gm_flag = nullptr;  // in gm_host: inner iterations that the device has reported
   unsigned long long gm_seq = 0;  // iterations whose result the host has been told
   h2::Factor<double> f64;
   h2::Factor<float> f32;
