@@ -1718,6 +1718,7 @@ size_t host_slots(int m0) { return slot_stamp(m0) + kGmStamps * (size_t)(m0 + 1)
 h2_status gmres_work(h2_ctx* c, GmresWork& W) {
   const int m0 = std::max(1, c->restart);
   if (c->gm_cap < m0) {
+    c->gm_cap = 0;  // (a failure below leaves nothing that a later solve would use)
     const int64_t n32 = nslots32(c);
     CKC(dalloc(c, &c->gm_V32, (size_t)(m0 + 1) * n32));
     CKC(dalloc(c, &c->gm_Z32, (size_t)m0 * n32));
@@ -1733,8 +1734,6 @@ h2_status gmres_work(h2_ctx* c, GmresWork& W) {
     CKC(dalloc(c, &c->gm_w32, (size_t)n32));
     CKC(dalloc(c, &c->gm_state, 1));
     CKC(dalloc(c, &c->gm_stamp, (size_t)kGmStamps * (m0 + 2)));
-    CKC(cudaMemset(c->gm_state, 0, sizeof(GmState)));
-    c->gm_seq = 0;
     c->gm_cap = m0;
   }
   W.m0 = m0;
@@ -1806,10 +1805,11 @@ h2_status gmres_refine(h2_ctx* c, SolveTimer& tm, double bnorm, double target, i
   return H2_OK;
 }
 
-// Wait until the device has reported inner iteration seq (it writes the count
-// to pinned memory after the iteration's numbers).  Polling sees it a few
-// microseconds earlier than a stream synchronization would; a stream that has
-// become idle or failed without reporting ends the wait.
+// Wait until the device has reported inner iteration seq of the cycle, counted
+// from 1 (it writes the count to pinned memory after the iteration's numbers).
+// Polling sees it a few microseconds earlier than a stream synchronization
+// would; a stream that has become idle or failed without reporting ends the
+// wait.
 h2_status wait_iteration(h2_ctx* c, unsigned long long seq) {
   const unsigned long long* flag = c->gm_flag;
   for (unsigned n = 1;; ++n) {
@@ -1840,6 +1840,11 @@ h2_status inner_cycle(h2_ctx* c, GmresWork& W, SolveTimer& tm, int m, double tol
   oa.part = W.part, oa.h = W.h1, oa.state = c->gm_state, oa.stamp = c->gm_stamp;
   oa.host = c->gm_host;
   oa.flag = c->gm_flag;
+  // Both sides count from 0 in every cycle (the device's count is set by
+  // launch_gm_start), so that a solve which ended between a launch and its
+  // result leaves nothing behind.  The stream is idle here: h2_solve and
+  // inner_update synchronize it.
+  __atomic_store_n(c->gm_flag, 0ull, __ATOMIC_RELEASE);
   run_graph(c, c->g_start, [&] {
     launch_norm2<double>(c->r64, nslots(c), c->red, c->stream);
     launch_pad_scaled_copy(c->r64, c->red, c->gm_r32, nslots(c), leaf_seg(c), c->stream);
@@ -1856,7 +1861,7 @@ h2_status inner_cycle(h2_ctx* c, GmresWork& W, SolveTimer& tm, int m, double tol
       launch_orth(oa, c->stream);
     });
     CKC(cudaGetLastError());
-    CKS(wait_iteration(c, ++c->gm_seq));
+    CKS(wait_iteration(c, (unsigned long long)j + 1));
     ++its;
     k = j + 1;
     if (givens_step(W, j, c->gm_host, c->gm_host + m0 + 2, c->gm_host[2 * (m0 + 2)], tol_abs)) break;

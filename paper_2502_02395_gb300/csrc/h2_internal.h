@@ -170,13 +170,11 @@ struct SymPair {
   int32_t xa, xb, n, pad;
 };
 
-// Device state of an inner FGMRES cycle: the iteration's index, how many CTAs
-// of its last kernel are done, and the number of iterations since the buffers
-// were made (the host waits for it to show up in pinned memory).
+// Device state of an inner FGMRES cycle, set at its start: the iteration's
+// index and how many CTAs of its last kernel are done.
 struct GmState {
   int j;
   unsigned int done;
-  unsigned long long seq;
 };
 // Device times (globaltimer, ns) of iteration j at t + 5 j: its start, the end
 // of the substitution, the leaf products' first and last, the end of A z.
@@ -440,8 +438,7 @@ struct h2_ctx {
   float* gm_w32 = nullptr;       // the inner iteration's A z
   h2::GmState* gm_state = nullptr;
   unsigned long long* gm_stamp = nullptr;  // 5 (gm_cap + 1) device times of a cycle's iterations
-  unsigned long long* gm_flag = nullptr;  // in gm_host: inner iterations that the device has reported
-  unsigned long long gm_seq = 0;  // iterations whose result the host has been told
+  unsigned long long* gm_flag = nullptr;  // in gm_host: the cycle's iterations that the device has reported
   h2::Factor<double> f64;
   h2::Factor<float> f32;
   h2::PhaseTimes times;

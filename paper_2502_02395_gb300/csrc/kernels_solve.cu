@@ -3344,13 +3344,11 @@ __global__ void __launch_bounds__(256) orth_kernel(const OrthArgs a) {
     __threadfence_system();
     __syncthreads();
     if (tid == 0) {
-      const unsigned long long s = a.state->seq + 1;
-      a.state->seq = s;
       a.state->done = 0;
       a.state->j = j + 1;
       a.stamp[kGmStamps * (j + 1)] = global_ns();
       __threadfence_system();
-      *reinterpret_cast<volatile unsigned long long*>(a.flag) = s;
+      *reinterpret_cast<volatile unsigned long long*>(a.flag) = (unsigned long long)j + 1;
     }
   }
 }
