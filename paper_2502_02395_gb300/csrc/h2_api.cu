@@ -1104,7 +1104,7 @@ void ulv_sweep(h2_ctx* c, Factor<T>& F) {
   };
   // levels of few boxes: a pair step and the per-box step after it in one
   // launch (thread-block clusters)
-  std::vector<char> cl(L + 2, 0);
+  std::vector<int> cl(L + 2, 0);  // CTAs per box
   for (int l = 1; l <= L; ++l)
     with_ahat(F.lv[l], F.bf16, [&](auto A, const float*) {
       using TS = std::remove_const_t<std::remove_pointer_t<decltype(A)>>;
@@ -1117,11 +1117,11 @@ void ulv_sweep(h2_ctx* c, Factor<T>& F) {
     with_ahat(f, F.bf16, [&](auto A, const float* isc) {
       using TS = std::remove_const_t<std::remove_pointer_t<decltype(A)>>;
       if (cl[l]) {
-        launch_cl_fwd2<T, TS>(d, f, A, isc, st);
+        launch_cl_fwd2<T, TS>(d, cl[l], f, A, isc, st);
         FacLevel<T>& pf = F.lv[l - 1];
         const int D1 = LV[l - 1].D;
-        if (l > 1) launch_cl_up<T, TS>(d, f, A, isc, D1, LV[l - 1].R, pf.M1, pf.U, pf.u, pf.c, st);
-        else launch_cl_up<T, TS>(d, f, A, isc, D1, D1, F.root_inv, nullptr, F.root_x, nullptr, st);
+        if (l > 1) launch_cl_up<T, TS>(d, cl[l], f, A, isc, D1, LV[l - 1].R, pf.M1, pf.U, pf.u, pf.c, st);
+        else launch_cl_up<T, TS>(d, cl[l], f, A, isc, D1, D1, F.root_inv, nullptr, F.root_x, nullptr, st);
       } else {
         launch_fwd2<T, TS>(d, f, A, isc, st);
         launch_fwd3<T, TS>(d, f, A, isc, l == 1 ? F.root_vec : nullptr, st);
@@ -1135,8 +1135,8 @@ void ulv_sweep(h2_ctx* c, Factor<T>& F) {
     with_ahat(f, F.bf16, [&](auto A, const float* isc) {
       using TS = std::remove_const_t<std::remove_pointer_t<decltype(A)>>;
       if (cl[l]) {
-        launch_cl_bwd1<T, TS>(d, f, A, isc, px, st);
-        launch_cl_bwd2<T, TS>(d, f, A, isc, px, st);
+        launch_cl_bwd1<T, TS>(d, cl[l], f, A, isc, px, st);
+        launch_cl_bwd2<T, TS>(d, cl[l], f, A, isc, px, st);
       } else {
         launch_bwd1<T, TS>(d, f, A, isc, px, st);
         launch_bwd2<T, TS>(d, f, A, isc, px, st);

@@ -152,21 +152,22 @@ template <typename T, typename TS>
 void launch_bwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
                  cudaStream_t st);
 // The cluster form (a pair step and the per-box step after it in one launch)
-// of levels with few boxes: whether a level takes it, and its four steps.
+// of levels with few boxes: the CTAs per box a level takes it with (0: not at
+// all), and its four steps.
 // launch_cl_up: level L's SR sums and the parent's first step ([M1; U^S] with
 // dimensions D1, R1 into u and c; at the root M1 = the inverse, R1 = D1).
 template <typename T, typename TS>
-bool subst_clustered(const DevLevel& L, const TS* Ahat);
+int subst_clustered(const DevLevel& L, const TS* Ahat);
 template <typename T, typename TS>
-void launch_cl_fwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, cudaStream_t st);
+void launch_cl_fwd2(const DevLevel& L, int CS, const FacLevel<T>& F, const TS* Ahat, const float* iscale, cudaStream_t st);
 template <typename T, typename TS>
-void launch_cl_up(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, int D1, int R1,
+void launch_cl_up(const DevLevel& L, int CS, const FacLevel<T>& F, const TS* Ahat, const float* iscale, int D1, int R1,
                   const T* M1, const T* U, T* u, T* c, cudaStream_t st);
 template <typename T, typename TS>
-void launch_cl_bwd1(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
+void launch_cl_bwd1(const DevLevel& L, int CS, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
                     cudaStream_t st);
 template <typename T, typename TS>
-void launch_cl_bwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
+void launch_cl_bwd2(const DevLevel& L, int CS, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
                     cudaStream_t st);
 template <typename T>
 void launch_gemv_rows(int nb, int n, const T* M, const T* x, T* y, cudaStream_t st);

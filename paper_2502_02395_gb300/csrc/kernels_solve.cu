@@ -1047,6 +1047,13 @@ void allow_smem(const void* f) {
     return;
   done.insert({dev, f});
 }
+// (of a kernel without static shared memory)
+static size_t max_smem() {
+  int dev = 0, optin = 48 * 1024;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return (size_t)optin;
+}
 static void set_smem(const void* f, size_t sm) {
   if (sm > 32 * 1024) allow_smem(f);
 }
@@ -1706,21 +1713,34 @@ static bool cluster_shape(const DevLevel& L, const TS* Ahat) {
          (reinterpret_cast<uintptr_t>(Ahat) & 15) == 0 && one_pass(L.R, L.R) && one_pass(L.K, L.R) &&
          one_pass(L.R, L.K);
 }
+// CTAs per box of one of the steps (CL_UP has half as many boxes), and the
+// shared memory of one CTA: its slices of the per-box matrices, the CTAs'
+// partial vectors and the step's input.
+static int cluster_step_ctas(int CS, int mode) { return mode == CL_UP ? std::min(8, 2 * CS) : CS; }
+static size_t cluster_smem(int CS, int mode, int D, int R, int K, size_t esz) {
+  const size_t n1 = mode == CL_UP ? 2 * K : R, per1 = (n1 + CS - 1) / CS, per2 = (D + CS - 1) / CS;
+  const size_t nr = mode == CL_UP ? K : R;
+  return esz * (per1 * n1 + (mode == CL_BWD2 ? per2 * D : 0) + CS * nr + (mode == CL_UP ? 2 * K : R) +
+                (mode == CL_BWD2 ? D : 0));
+}
+// The level's CTAs per box, 0 where a step's shapes or shared memory do not
+// allow the form (few complement rows beside a high rank: FP64 from K = 232 on
+// at R <= 32; such levels keep the pair and the per-box launches).
 template <typename T, typename TS>
-bool subst_clustered(const DevLevel& L, const TS* Ahat) {
-  return cluster_ctas(L.nb) > 0 && cluster_shape<T, TS>(L, Ahat);
+int subst_clustered(const DevLevel& L, const TS* Ahat) {
+  const int CS = cluster_ctas(L.nb);
+  if (CS == 0 || !cluster_shape<T, TS>(L, Ahat)) return 0;
+  for (int mode : {CL_FWD2, CL_BWD1, CL_BWD2, CL_UP})
+    if (cluster_smem(cluster_step_ctas(CS, mode), mode, L.D, L.R, L.K, sizeof(T)) > max_smem()) return 0;
+  return CS;
 }
 
 template <typename T, typename TS, int MODE>
-static void launch_cluster(const DevLevel& L, const ClArgs<T, TS>& args, int nbox, cudaStream_t st) {
+static void launch_cluster(const DevLevel& L, int CS, const ClArgs<T, TS>& args, int nbox, cudaStream_t st) {
   ClArgs<T, TS> a = args;
   a.D = L.D, a.R = L.R, a.K = L.K, a.ptr = L.near_ptr, a.nj = L.near_j;
-  a.CS = cluster_ctas(MODE == CL_UP ? 2 * nbox : nbox);  // (of the pairs' level)
-  if (MODE == CL_UP) a.CS = std::min(8, 2 * a.CS);
-  const int n1 = MODE == CL_UP ? a.D1 : a.R, per1 = (n1 + a.CS - 1) / a.CS, per2 = (a.D + a.CS - 1) / a.CS;
-  const int nr = MODE == CL_UP ? a.K : a.R;
-  const size_t sm = sizeof(T) * ((size_t)per1 * n1 + (MODE == CL_BWD2 ? (size_t)per2 * a.D : 0) + (size_t)a.CS * nr +
-                                 (MODE == CL_UP ? 2 * a.K : a.R) + (MODE == CL_BWD2 ? a.D : 0));
+  a.CS = cluster_step_ctas(CS, MODE);
+  const size_t sm = cluster_smem(a.CS, MODE, a.D, a.R, a.K, sizeof(T));
   set_smem((const void*)box_cluster_kernel<T, TS, MODE>, sm);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(nbox * a.CS));
@@ -1740,33 +1760,33 @@ static void launch_cluster(const DevLevel& L, const ClArgs<T, TS>& args, int nbo
 }
 
 template <typename T, typename TS>
-void launch_cl_fwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, cudaStream_t st) {
+void launch_cl_fwd2(const DevLevel& L, int CS, const FacLevel<T>& F, const TS* Ahat, const float* iscale, cudaStream_t st) {
   ClArgs<T, TS> a{};
   a.cnt = L.lo_cnt, a.Ahat = Ahat, a.iscale = iscale, a.xv = F.u, a.A1 = F.Ainv, a.base = F.u, a.out = F.v;
-  launch_cluster<T, TS, CL_FWD2>(L, a, L.nb, st);
+  launch_cluster<T, TS, CL_FWD2>(L, CS, a, L.nb, st);
 }
 template <typename T, typename TS>
-void launch_cl_up(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, int D1, int R1,
+void launch_cl_up(const DevLevel& L, int CS, const FacLevel<T>& F, const TS* Ahat, const float* iscale, int D1, int R1,
                   const T* M1, const T* U, T* u, T* c, cudaStream_t st) {
   ClArgs<T, TS> a{};
   a.Ahat = Ahat, a.iscale = iscale, a.xv = F.v, a.A1 = M1, a.A2 = U, a.base = F.c, a.out = u, a.out2 = c, a.D1 = D1,
   a.R1 = R1;
-  launch_cluster<T, TS, CL_UP>(L, a, L.nb / 2, st);
+  launch_cluster<T, TS, CL_UP>(L, CS, a, L.nb / 2, st);
 }
 template <typename T, typename TS>
-void launch_cl_bwd1(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
+void launch_cl_bwd1(const DevLevel& L, int CS, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
                     cudaStream_t st) {
   ClArgs<T, TS> a{};
   a.Ahat = Ahat, a.iscale = iscale, a.xv = parent_x, a.A1 = F.Ainv, a.base = F.v, a.out = F.om;
-  launch_cluster<T, TS, CL_BWD1>(L, a, L.nb, st);
+  launch_cluster<T, TS, CL_BWD1>(L, CS, a, L.nb, st);
 }
 template <typename T, typename TS>
-void launch_cl_bwd2(const DevLevel& L, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
+void launch_cl_bwd2(const DevLevel& L, int CS, const FacLevel<T>& F, const TS* Ahat, const float* iscale, const T* parent_x,
                     cudaStream_t st) {
   ClArgs<T, TS> a{};
   a.cnt = L.hi_cnt, a.Ahat = Ahat, a.iscale = iscale, a.xv = F.om, a.A1 = F.Ainv, a.A2 = F.Ur, a.base = F.om,
   a.px = parent_x, a.out = F.xs;
-  launch_cluster<T, TS, CL_BWD2>(L, a, L.nb, st);
+  launch_cluster<T, TS, CL_BWD2>(L, CS, a, L.nb, st);
 }
 
 // y_b = M_b x_b for nb n x n row-major matrices, one CTA each (root solves
@@ -1807,14 +1827,14 @@ H2_INST_SOLVE(float)
                                    cudaStream_t);                                                              \
   template void launch_bwd1<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, const T*,      \
                                    cudaStream_t);                                                              \
-  template bool subst_clustered<T, TS>(const DevLevel&, const TS*);                                            \
-  template void launch_cl_fwd2<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*,            \
+  template int subst_clustered<T, TS>(const DevLevel&, const TS*);                                            \
+  template void launch_cl_fwd2<T, TS>(const DevLevel&, int, const FacLevel<T>&, const TS*, const float*,            \
                                       cudaStream_t);                                                           \
-  template void launch_cl_up<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, int, int,    \
+  template void launch_cl_up<T, TS>(const DevLevel&, int, const FacLevel<T>&, const TS*, const float*, int, int,    \
                                     const T*, const T*, T*, T*, cudaStream_t);                                 \
-  template void launch_cl_bwd1<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, const T*,  \
+  template void launch_cl_bwd1<T, TS>(const DevLevel&, int, const FacLevel<T>&, const TS*, const float*, const T*,  \
                                       cudaStream_t);                                                           \
-  template void launch_cl_bwd2<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, const T*,  \
+  template void launch_cl_bwd2<T, TS>(const DevLevel&, int, const FacLevel<T>&, const TS*, const float*, const T*,  \
                                       cudaStream_t);                                                           \
   template void launch_bwd2<T, TS>(const DevLevel&, const FacLevel<T>&, const TS*, const float*, const T*,      \
                                    cudaStream_t);

@@ -57,3 +57,27 @@ def test_halves_with_an_open_far_list(B):
     S = B.H2Solver.from_instance(flat, kernel="yukawa_eps", leaf=128, eta=1.0, tol=1e-8, max_rank=64, far_samples=256,
                                  near_samples=32, diag_shift=1.0)
     check_arithmetics(S, n)
+
+
+@pytest.mark.parametrize("n,leaf,rank,precs", [(2048, 256, 232, ("fp64",)), (2048, 256, 240, ("fp64", "fp16")),
+                                               (2912, 364, 332, ("fp16",))])
+def test_few_complement_rows_beside_a_high_rank(B, n, leaf, rank, precs):
+    """Per-box matrices of [x^R; x^S] too large for the slices that the cluster
+    form of the substitution keeps in shared memory (K = 232 and above in FP64,
+    332 in FP32, at 32 complement rows and fewer), against plain launches."""
+    S = B.H2Solver.build(W.cube_points(n, 3), kernel="yukawa_eps", diag_shift=1.0, leaf=leaf, eta=1.0, tol=1e-14,
+                         max_rank=rank, far_samples=512, near_samples=0)
+    assert S.stats()["levels"][-1]["K"] == rank
+    b = W.uniform_rhs(n, 5)
+    for prec in precs:
+        S.factor(prec)
+        z = [S.ulv_apply(b)]
+        S.set_option("box_stream", 2)  # (process-wide)
+        try:
+            z.append(S.ulv_apply(b))
+        finally:
+            S.set_option("box_stream", 0)
+        u = 2.0 ** -53 if prec == "fp64" else 2.0 ** -24
+        assert np.linalg.norm(z[0] - z[1]) <= 1e3 * u * np.linalg.norm(z[1]), prec
+        x, rel, _ = S.solve(b, target=1e-10, max_iters=100)
+        assert rel <= 1e-10 and np.linalg.norm(b - S.matvec(x)) <= 2e-10 * np.linalg.norm(b)
