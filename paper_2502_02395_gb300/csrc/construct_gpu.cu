@@ -711,7 +711,7 @@ struct DeviceGpuCompressor : GpuCompressor {
     launch_sketch(G, pts, j.nb, j.D, j.m, nz, d_nbox, d_bpts, d_fptr, d_fidx, d_nptr, d_nidx, d_cptr, d_cidx, d_W,
                   j.seed, d_Y, 0);
     GC_TRY(launch_pivqr_id(j.nb, j.D, j.m, j.ms, j.q, j.K, nz, d_nbox, d_bpts, d_Y, d_X, d_SK, d_rho, d_err, 0));
-    GC_TRY(cudaGetLastError());
+    GC_TRY(take_launch_error());
     j.X.resize(nb * D * K);
     j.SK.resize(nb * K);
     j.rho.resize(nb);

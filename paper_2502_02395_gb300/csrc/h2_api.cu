@@ -93,7 +93,7 @@ h2_status make_leaf_lowp(h2_ctx* c, int bf16) {
     launch_amax_blocks<double>(d.S, d.FP, (int64_t)d.K * d.K, d.K, d.K, d.K, amax, c->stream);
     launch_to_lowp<double>(bf16, d.S, d.S16[bf16], ns, {amax, std::sqrt(32768.0f / d.K), d.S16_scale[bf16]}, c->stream);
   }
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
   CKC(cudaStreamSynchronize(c->stream));
   return H2_OK;
 }
@@ -286,12 +286,12 @@ h2_status setup_device(h2_ctx* c) {
   CKS(upload(c, &c->slot_pt, slot));
   CKC(dalloc(c, &c->A64, (size_t)lf.NP * lf.D * lf.D));
   launch_eval_blocks(c->kfn, c->pts, lf.NP, lf.near_ptr, lf.near_i, lf.near_j, c->slot_pt, lf.D, c->A64, 0);
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
   for (int l = 1; l <= L; ++l) {
     DevLevel& d = c->lv[l];
     CKC(dalloc(c, &d.S, (size_t)std::max<int64_t>(d.FP, 1) * d.K * d.K));
     launch_eval_blocks(c->kfn, c->pts, d.FP, d.far_ptr, d.far_i, d.far_j, d.SK, d.K, d.S, 0);
-    CKC(cudaGetLastError());
+    CKC(take_launch_error());
   }
   // vectors and scratch
   const int64_t nslot = (int64_t)lf.nb * lf.D;
@@ -454,7 +454,7 @@ h2_status setup_device(h2_ctx* c) {
     CKC(dalloc(c, &c->part32, npart));
     CKC(dalloc(c, &c->part64, npart));
   }
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
 
   CKC(dalloc(c, &c->red, 1024));  // three norm slots of 257 doubles: 0, 300, 600
   CKC(dalloc(c, &c->status, 4));
@@ -1012,7 +1012,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
   }
   wait_for(sp, st);
   mark();
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
   CKC(cudaStreamSynchronize(st));
   // phase times
   PhaseTimes& t = c->times;
@@ -1172,10 +1172,13 @@ void ulv_apply_impl(h2_ctx* c, Factor<T>& F, const double* r, double* x) {
 }
 
 // Capture fn's work on the context's stream into a CUDA graph (on a private
-// capture stream); nothing if the capture or instantiation fails.
+// capture stream); nothing if the capture, a launch in it or the instantiation
+// fails, or if an error of earlier work is pending, which stays so.  The caller
+// then runs fn directly and reports what that leaves.
 template <class Fn>
 KernelGraph capture_graph(h2_ctx* c, Fn fn) {
   KernelGraph out;
+  if (launch_error_pending()) return out;
   if (!c->cap_stream && cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
     return out;
@@ -1186,7 +1189,8 @@ KernelGraph capture_graph(h2_ctx* c, Fn fn) {
   const long long n0 = g_launches.load();
   if (cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
     fn();
-    if (cudaStreamEndCapture(c->cap_stream, &g) == cudaSuccess && g) {
+    const bool launched = take_launch_error() == cudaSuccess;
+    if (cudaStreamEndCapture(c->cap_stream, &g) == cudaSuccess && g && launched) {
       if (cudaGraphInstantiate(&out.ex, g, 0) != cudaSuccess) out.ex = nullptr;
     }
   }
@@ -1860,7 +1864,7 @@ h2_status inner_cycle(h2_ctx* c, GmresWork& W, SolveTimer& tm, int m, double tol
       matvec32(c, oa.xs, oa.w, nullptr, oa.stamp);
       launch_orth(oa, c->stream);
     });
-    CKC(cudaGetLastError());
+    CKC(take_launch_error());
     CKS(wait_iteration(c, (unsigned long long)j + 1));
     ++its;
     k = j + 1;
@@ -1893,6 +1897,7 @@ h2_status inner_update(h2_ctx* c, GmresWork& W, SolveTimer& tm, int k, double& b
                       cudaMemcpyDeviceToHost, st);
     });
   });
+  CKC(take_launch_error());
   CKC(cudaStreamSynchronize(c->stream));
   beta = std::sqrt(c->gm_host[slot_rn(m0)]);
   const unsigned long long* t = reinterpret_cast<const unsigned long long*>(c->gm_host + slot_stamp(m0));
@@ -2272,7 +2277,7 @@ h2_status h2_release_factorization(h2_ctx* c) {
   release_factor(c, c->f64);
   release_factor(c, c->f32);
   c->prec = -1;
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
   return H2_OK;
 }
 
@@ -2286,7 +2291,7 @@ h2_status h2_ulv_apply(h2_ctx* c, const double* b, double* x) {
   CKC(cudaMemsetAsync(c->x64, 0, nslot * sizeof(double), c->stream));
   CKS(subst_clear(c));
   ulv_apply_any(c, c->r64, c->x64);
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
   CKS(vec_out(c, c->x64, x));
   CKC(cudaStreamSynchronize(c->stream));
   return subst_check(c);
@@ -2298,7 +2303,7 @@ h2_status h2_matvec(h2_ctx* c, const double* x, double* y) {
   if (!c->A64) { c->err = "the FP64 leaf blocks were released (H2_OPT_FP64_LEAF)"; return H2_ERR_STATE; }
   CKS(vec_in(c, x, c->x64));
   matvec_impl(c, c->x64, c->y64);
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
   CKS(vec_out(c, c->y64, y));
   CKC(cudaStreamSynchronize(c->stream));
   return H2_OK;
@@ -2384,7 +2389,7 @@ h2_status h2_solve(h2_ctx* c, const double* b, double* x, double target, int32_t
       if (!std::isfinite(rel)) break;
     }
   }
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
   CKS(vec_out(c, c->x64, x));
   cudaEventRecord(e1, st);
   CKC(cudaEventSynchronize(e1));
@@ -2514,7 +2519,7 @@ h2_status h2_matvec_arith(h2_ctx* c, const double* x, double* y, int32_t arith) 
     matvec32(c, c->mv32_x, c->mv32_y);
     launch_unpad(c->mv32_y, c->y64, n, leaf_seg(c), c->stream);
   }
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
   CKS(vec_out(c, c->y64, y));
   CKC(cudaStreamSynchronize(c->stream));
   return H2_OK;
@@ -2623,7 +2628,7 @@ h2_status h2_wait_selftest(h2_ctx* c, int64_t timeout_ns) {
   // kernel when it gives up, read back
   CKS(subst_clear(c));
   launch_wait_selftest((unsigned long long)timeout_ns, c->status + 3, c->stream);
-  CKC(cudaGetLastError());
+  CKC(take_launch_error());
   const h2_status s = subst_check(c);
   if (s == H2_ERR_TIMEOUT) {
     c->err = "self-test: the bounded wait gave up after " + std::to_string(timeout_ns) + " ns as designed";

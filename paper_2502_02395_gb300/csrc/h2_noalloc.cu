@@ -120,7 +120,7 @@ extern "C" h2_status h2_matvec_noalloc(h2_ctx* c, const double* x, double* y) {
   }
   h2::launch_matvec_block_rows<double>(la, st);
   h2::launch_scatter(c->slot_pt, yt, y, (int64_t)nslot, st);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = h2::take_launch_error();
   if (e != cudaSuccess) {
     c->err = std::string("h2_matvec_noalloc: ") + cudaGetErrorString(e);
     return H2_ERR_CUDA;

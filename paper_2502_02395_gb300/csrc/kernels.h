@@ -31,6 +31,14 @@ extern std::atomic<int> g_pair_ctas_per_sm;
 // allows (once per kernel and device; safe from several threads).
 void allow_smem(const void* f);
 
+// The first failed launch of this thread since the last look, and none from
+// then on.  (cudaGetLastError alone does not do: a cudaFuncSetAttribute that
+// succeeds resets the runtime's record.)
+cudaError_t take_launch_error();
+// whether there is one
+bool launch_error_pending();
+void note_launch(cudaError_t e);
+
 // kernels_factor.cu
 void launch_eval_blocks(const KernelFn& G, const double* pts, int64_t npairs, const int64_t* ptr, const int32_t* pi,
                         const int32_t* pj, const int64_t* idx, int n, double* out, cudaStream_t st);

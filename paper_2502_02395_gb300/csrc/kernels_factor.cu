@@ -1202,7 +1202,7 @@ static void launch_qr_cluster(int nb, int D, int K, int C, const double* Xin, do
   cfg.attrs = at;
   cfg.numAttrs = 1;
   ++g_launches;
-  cudaLaunchKernelEx(&cfg, qr_cluster_kernel<CW>, D, K, C, Xin, Vout, tau, Tm);
+  note_launch(cudaLaunchKernelEx(&cfg, qr_cluster_kernel<CW>, D, K, C, Xin, Vout, tau, Tm));
 }
 
 template <typename T>
@@ -1634,7 +1634,8 @@ static void launch_gj_rows_t(int nb, int D, int R, const TI* A, const int32_t* d
   cfg.attrs = attr;
   cfg.numAttrs = CL > 1 ? 1 : 0;
   ++g_launches;
-  cudaLaunchKernelEx(&cfg, gj_rows_kernel<T, TI, TO, NW, RPW, CPL, CL, LU>, D, R, A, diag_idx, out, piv, status, level);
+  note_launch(cudaLaunchKernelEx(&cfg, gj_rows_kernel<T, TI, TO, NW, RPW, CPL, CL, LU>, D, R, A, diag_idx, out, piv,
+                                 status, level));
 }
 // false for R > 256.  FP64 spreads a box over more CTAs (its time is the FP64
 // pipe's); few rows take fewer warps (a barrier's cost goes with them).

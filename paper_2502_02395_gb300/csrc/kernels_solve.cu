@@ -1028,6 +1028,18 @@ void launch_transpose_pairs(int D, int64_t n, const int32_t* dst, const int32_t*
   transpose_pairs_kernel<T><<<grid, dim3(32, 8), 0, st>>>(D, n, dst, src, A);
 }
 
+static thread_local cudaError_t t_launch_error = cudaSuccess;
+void note_launch(cudaError_t e) {
+  if (t_launch_error == cudaSuccess) t_launch_error = e;
+}
+cudaError_t take_launch_error() {
+  note_launch(cudaGetLastError());
+  const cudaError_t e = t_launch_error;
+  t_launch_error = cudaSuccess;
+  return e;
+}
+bool launch_error_pending() { return t_launch_error != cudaSuccess || cudaPeekAtLastError() != cudaSuccess; }
+
 // The largest dynamic shared memory a kernel may be launched with, raised to
 // what the device allows, once per kernel and device.  (Set to each launch's
 // own size it was a race: with two contexts in two threads, one could lower
@@ -1039,6 +1051,7 @@ void allow_smem(const void* f) {
   cudaGetDevice(&dev);
   std::lock_guard<std::mutex> lock(mu);
   if (done.count({dev, f})) return;
+  note_launch(cudaPeekAtLastError());
   int optin = 0;
   cudaFuncAttributes a{};
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
@@ -1073,7 +1086,7 @@ static void launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, si
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   ++g_launches;
-  cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+  note_launch(cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...));
 }
 
 static int num_sms() {
@@ -1756,7 +1769,7 @@ static void launch_cluster(const DevLevel& L, int CS, const ClArgs<T, TS>& args,
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   ++g_launches;
-  cudaLaunchKernelEx(&cfg, box_cluster_kernel<T, TS, MODE>, a);
+  note_launch(cudaLaunchKernelEx(&cfg, box_cluster_kernel<T, TS, MODE>, a));
 }
 
 template <typename T, typename TS>
@@ -1951,7 +1964,7 @@ static void launch_pdl_cluster(void (*kern)(KArgs...), unsigned grid, int CS, si
   cfg.numAttrs = 2;
   set_smem((const void*)kern, smem);
   ++g_launches;
-  cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+  note_launch(cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...));
 }
 // CTAs per box for a D x K basis of esz-byte entries: slices of at most 32 KB,
 // doubled while the level leaves room for two CTAs per SM; 0: no cluster form
