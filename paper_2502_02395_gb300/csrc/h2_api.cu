@@ -85,7 +85,8 @@ h2_status make_leaf_lowp(h2_ctx* c, int bf16) {
   // tensor-core coupling products then stay inside FP16 (|S T^T| <= 32768)
   for (int l = 1; l <= c->L; ++l) {
     DevLevel& d = c->pv[l];
-    if (d.FP == 0 || d.K == 0) continue;
+    // (a padded level's couplings stay in FP32: S has the logical rank)
+    if (d.FP == 0 || d.K == 0 || d.K != c->lv[l].K) continue;
     const int64_t ns = d.FP * (int64_t)d.K * d.K;
     CKC(dalloc(c, &d.S16_scale[bf16], 2));
     CKC(dalloc(c, reinterpret_cast<uint16_t**>(&d.S16[bf16]), ns));

@@ -81,3 +81,41 @@ def test_few_complement_rows_beside_a_high_rank(B, n, leaf, rank, precs):
         assert np.linalg.norm(z[0] - z[1]) <= 1e3 * u * np.linalg.norm(z[1]), prec
         x, rel, _ = S.solve(b, target=1e-10, max_iters=100)
         assert rel <= 1e-10 and np.linalg.norm(b - S.matvec(x)) <= 2e-10 * np.linalg.norm(b)
+
+
+def test_tensor_core_rank_above_a_padded_level(B):
+    """A rank of 128 (16-bit couplings) over a level whose rank of 125 is padded
+    in the FP32 arrays: three more skeletons at level 1 of an instance whose
+    ranks the construction left at 125."""
+    from oracle.construct import construct
+    from oracle.instance import flatten
+    from oracle.kernels import Kernel
+    n = 800
+    H = construct(W.cube_points(n, 3), Kernel("yukawa_eps", diag_shift=1.0), 200, 0.0, 1e-13, 125, 0, 0)
+    flat = flatten(H)
+    assert list(flat["K"]) == [0, 125, 125] and len(flat["far"][1]) and len(flat["far"][2])
+    X, SK = np.zeros((2, 250, 128)), np.zeros((2, 128), dtype=np.int64)
+    for i in range(2):
+        rows = np.concatenate([flat["SK"][2][2 * i], flat["SK"][2][2 * i + 1]])  # the box's points
+        X[i, :, :125], SK[i, :125] = flat["X"][1][i], flat["SK"][1][i]
+        more = np.flatnonzero(~np.isin(rows, SK[i, :125]))[:3]
+        X[i, more, :] = 0.0
+        X[i, more, 125 + np.arange(3)] = 1.0
+        SK[i, 125:] = rows[more]
+    flat["X"][1], flat["SK"][1] = X, SK
+    flat["K"] = np.array([0, 128, 125], dtype=np.int32)
+    flat["D"] = np.array([256, 250, 200], dtype=np.int32)
+    S = B.H2Solver.from_instance(flat, kernel="yukawa_eps", leaf=200, eta=0.0, tol=1e-13, max_rank=128, far_samples=0,
+                                 near_samples=0, diag_shift=1.0)
+    check_arithmetics(S, n)
+    S.factor("fp64")
+    sh64 = S.export("Shat", 2)
+    b = W.uniform_rhs(n, 5)
+    for prec in ("fp16", "bf16"):
+        S.factor(prec)
+        # (T in FP32 is within 1e-3 of the FP64 one; it stands on both sides)
+        sh = S.export("Shat", 2).astype(np.float64)
+        assert sh.shape == sh64.shape
+        assert np.linalg.norm(sh - sh64) <= 2e-3 * np.linalg.norm(sh64)
+        x, rel, _ = S.solve(b, target=1e-10, max_iters=100)
+        assert rel <= 1e-10 and np.linalg.norm(b - S.matvec(x)) <= 2e-10 * np.linalg.norm(b)
