@@ -2068,6 +2068,7 @@ static int rows_per(int nb, int D, int K, size_t esz) {
 template <typename T>
 void launch_matvec_rows(int nb, int D, int K, const T* X, const T* yh, const T* base, T* out, int seg,
                         const int64_t* ptr, const int32_t* ent, const T* part, bool pdl, cudaStream_t st) {
+  if (nb == 0 || D == 0) return;  // (above a level of rank 0)
   const int per = rows_per(nb, D, K, sizeof(T)), ns = (D + per - 1) / per;
   const size_t sm = sizeof(T) * ((((size_t)per * K + 3) & ~(size_t)3) + ((K + 3) & ~3) + 256);
   set_smem((const void*)mv_rows_kernel<T>, sm);
@@ -2634,6 +2635,7 @@ __global__ void __launch_bounds__(256) mv_rows_df_kernel(const RowsDf a) {
 void launch_matvec_rows_df(int nb, int D, int K, const float* Xh, const float* Xl, const float* yhh, const float* yhl,
                            const float* bh, const float* bl, int seg, const int64_t* ptr, const int32_t* ent,
                            const float* ph, const float* pl, float* oh, float* ol, double* y, int ny, cudaStream_t st) {
+  if (nb == 0 || D == 0) return;
   RowsDf a{Xh, Xl, yhh, yhl, bh, bl, ptr, ent, ph, pl, oh, ol, y, D, K, 0, rows_per(nb, D, K, 8), seg, ny};
   a.ns = (D + a.per - 1) / a.per;
   const size_t sm = 2 * sizeof(float) * ((((size_t)a.per * K + 3) & ~(size_t)3) + ((K + 3) & ~3) + 256);

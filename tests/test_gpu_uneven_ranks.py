@@ -119,3 +119,34 @@ def test_tensor_core_rank_above_a_padded_level(B):
         assert np.linalg.norm(sh - sh64) <= 2e-3 * np.linalg.norm(sh64)
         x, rel, _ = S.solve(b, target=1e-10, max_iters=100)
         assert rel <= 1e-10 and np.linalg.norm(b - S.matvec(x)) <= 2e-10 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n,leaf", [(130, 33), (1000, 128)])
+def test_rank_zero(B, n, leaf):
+    """An imported instance of rank 0 on every level: boxes of dimension 0 above
+    the leaves, and the near blocks alone (products against the blocks)."""
+    from oracle.construct import construct
+    from oracle.instance import flatten
+    from oracle.kernels import Kernel
+    flat = flatten(construct(W.cube_points(n, 3), Kernel("yukawa_eps", diag_shift=1.0), leaf, 1.0, 1e-6, 0, 64, 8))
+    L, D = flat["L"], int(flat["D"][-1])
+    flat["K"] = np.zeros(L + 1, dtype=np.int32)
+    flat["D"] = np.array([0] * L + [D], dtype=np.int32)
+    flat["far"] = [np.zeros((0, 2), dtype=np.int32) for _ in range(L + 1)]
+    flat["X"] = [None] + [np.zeros((2 ** l, flat["D"][l], 0)) for l in range(1, L + 1)]
+    flat["SK"] = [None] + [np.zeros((2 ** l, 0), dtype=np.int64) for l in range(1, L + 1)]
+    S = B.H2Solver.from_instance(flat, kernel="yukawa_eps", leaf=leaf, eta=1.0, tol=1e-6, far_samples=64,
+                                 near_samples=8, diag_shift=1.0)
+    A = S.export("A", L).reshape(-1, D, D)
+    off, perm = flat["leaf_offsets"], flat["perm"]
+    x = W.uniform_rhs(n, 4)
+    y = np.zeros(n)
+    for q, (i, j) in enumerate(flat["near"][L]):
+        pi, pj = perm[off[i]:off[i + 1]], perm[off[j]:off[j + 1]]
+        y[pi] += A[q][:len(pi), :len(pj)] @ x[pj]
+    assert np.linalg.norm(S.matvec(x) - y) <= 1e-13 * np.linalg.norm(y)
+    check_arithmetics(S, n)
+    for prec in ("fp64", "fp16"):
+        S.factor(prec)
+        xs, rel, _ = S.solve(x, target=1e-10, max_iters=200)
+        assert rel <= 1e-10 and np.linalg.norm(x - S.matvec(xs)) <= 2e-10 * np.linalg.norm(x)
