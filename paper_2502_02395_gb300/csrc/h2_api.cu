@@ -595,13 +595,9 @@ h2_status alloc_factor(h2_ctx* c, Factor<T>& F) {
 }
 
 template <typename T>
-void gemm(int32_t* err, int M, int N, int K, const T* A, int64_t sA, const int32_t* ia, int lda, bool tA, const T* B,
-          int64_t sB, const int32_t* ib, int ldb, bool tB, T* C, int64_t sC, const int32_t* ic, int ldc, T alpha,
-          T beta, int64_t batch, cudaStream_t st) {
-  if constexpr (std::is_same<T, double>::value)
-    if (batch > 0 && M > 0 && N > 0 &&
-        gemm_split(M, N, K, A, sA, ia, lda, tA, B, sB, ib, ldb, tB, C, sC, ic, ldc, alpha, beta, batch, err, st))
-      return;
+void gemm(int M, int N, int K, const T* A, int64_t sA, const int32_t* ia, int lda, bool tA, const T* B, int64_t sB,
+          const int32_t* ib, int ldb, bool tB, T* C, int64_t sC, const int32_t* ic, int ldc, T alpha, T beta,
+          int64_t batch, cudaStream_t st) {
   gemm_simt<T, T>(M, N, K, A, sA, ia, lda, tA, B, sB, ib, ldb, tB, C, sC, ic, ldc, alpha, beta, batch, st);
 }
 
@@ -725,7 +721,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
         const T* Tc = F.lv[l + 1].Tm;
         const int64_t KcKc = (int64_t)Kc * Kc;
         // (box i's halves are the children 2 i and 2 i + 1: D = 2 Kc)
-        gemm<T>(c->status + 2, Kc, K, Kc, Tc, KcKc, nullptr, Kc, false, Xc, (int64_t)Kc * K, nullptr, K, false, f.Xo,
+        gemm<T>(Kc, K, Kc, Tc, KcKc, nullptr, Kc, false, Xc, (int64_t)Kc * K, nullptr, K, false, f.Xo,
                 (int64_t)Kc * K, nullptr, K, T(1), T(0), 2 * (int64_t)nb, sb);
         Xin = f.Xo;
       }
@@ -735,11 +731,11 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       T* W1 = F.Wq + (int64_t)nb * KK;
       if (K > 0) {
         if (!tw_done) {
-          gemm<T>(c->status + 2, K, K, D, f.Vq, DK, nullptr, D, false, f.Vq, DK, nullptr, D, true, Sb, KK, nullptr, K, T(1),
+          gemm<T>(K, K, D, f.Vq, DK, nullptr, D, false, f.Vq, DK, nullptr, D, true, Sb, KK, nullptr, K, T(1),
                   T(0), nb, sb);
           launch_wy_tfactor<T>(nb, K, Sb, f.tau, f.Tw, sb);
         }
-        gemm<T>(c->status + 2, D, K, K, f.Vq, DK, nullptr, D, true, f.Tw, KK, nullptr, K, false, W1, DK, nullptr, K, T(1), T(0),
+        gemm<T>(D, K, K, f.Vq, DK, nullptr, D, true, f.Tw, KK, nullptr, K, false, W1, DK, nullptr, K, T(1), T(0),
                 nb, sb);
       }
       bool formed = false;
@@ -760,9 +756,9 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
         launch_perm_identity<T>(nb, D, K, f.U, sb);
         if (K > 0) {
           if (R > 0)
-            gemm<T>(c->status + 2, R, D, K, f.Vq + K, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U, DD, nullptr, D,
+            gemm<T>(R, D, K, f.Vq + K, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U, DD, nullptr, D,
                     T(-1), T(1), nb, sb);
-          gemm<T>(c->status + 2, K, D, K, f.Vq, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U + (int64_t)R * D, DD,
+          gemm<T>(K, D, K, f.Vq, DK, nullptr, D, true, W1, DK, nullptr, K, true, f.U + (int64_t)R * D, DD,
                   nullptr, D, T(-1), T(1), nb, sb);
         }
         launch_transpose_blocks<T>(nb, D, f.U, f.Ur, sb);
@@ -801,8 +797,8 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       const int32_t *pq = up ? d.fu_q : nullptr, *pi = up ? d.fu_i : d.far_i, *pj = up ? d.fu_j : d.far_j;
       // (FP32: the instance's stored halves are in the order of the pairs)
       const bool halves = up && mixed && c->cb_ok;
-      gemm<T>(c->status + 2, K, K, K, Sc, KK, halves ? nullptr : pq, K, false, f.Tp, KK, pj, K, true, F.Wc, KK, nullptr, K, T(1), T(0), n, sc);
-      gemm<T>(c->status + 2, K, K, K, f.Tp, KK, pi, K, false, F.Wc, KK, nullptr, K, false, f.Shat, KK, pq, K, T(1), T(0), n, sc);
+      gemm<T>(K, K, K, Sc, KK, halves ? nullptr : pq, K, false, f.Tp, KK, pj, K, true, F.Wc, KK, nullptr, K, T(1), T(0), n, sc);
+      gemm<T>(K, K, K, f.Tp, KK, pi, K, false, F.Wc, KK, nullptr, K, false, f.Shat, KK, pq, K, T(1), T(0), n, sc);
       if (up) launch_transpose_pairs<T>(K, n, d.fl_q, d.fl_m, f.Shat, sc);
     }
     // max |Shat| for the 16-bit merge's scale, beside the main chain
@@ -888,16 +884,16 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       // symmetric near list: project the upper pairs i <= j, then
       // Ahat_ji = Ahat_ij^T for the lower ones (the kernels are symmetric)
       const T* Ain = (l == L) ? Aleaf : f.Ain;
-      gemm<T>(c->status + 2, D, D, D, Ain, DD, l == L && leaf_halves ? nullptr : d.su_q, D, false, f.U, DD, d.su_j, D, true, F.Wk, DD, nullptr, D, T(1), T(0),
+      gemm<T>(D, D, D, Ain, DD, l == L && leaf_halves ? nullptr : d.su_q, D, false, f.U, DD, d.su_j, D, true, F.Wk, DD, nullptr, D, T(1), T(0),
               d.n_up, st);
-      gemm<T>(c->status + 2, D, D, D, f.U, DD, d.su_i, D, false, F.Wk, DD, nullptr, D, false, f.Ahat, DD, d.su_q, D, T(1),
+      gemm<T>(D, D, D, f.U, DD, d.su_i, D, false, F.Wk, DD, nullptr, D, false, f.Ahat, DD, d.su_q, D, T(1),
               T(0), d.n_up, st);
       launch_transpose_pairs<T>(D, d.n_lw, d.lw_q, d.lw_m, f.Ahat, st);
     } else {
       const T* Ain = (l == L) ? Aleaf : f.Ain;
-      gemm<T>(c->status + 2, D, D, D, Ain, DD, nullptr, D, false, f.U, DD, d.near_j, D, true, F.Wk, DD, nullptr, D, T(1),
+      gemm<T>(D, D, D, Ain, DD, nullptr, D, false, f.U, DD, d.near_j, D, true, F.Wk, DD, nullptr, D, T(1),
               T(0), d.NP, st);
-      gemm<T>(c->status + 2, D, D, D, f.U, DD, d.near_i, D, false, F.Wk, DD, nullptr, D, false, f.Ahat, DD, nullptr, D, T(1),
+      gemm<T>(D, D, D, f.U, DD, d.near_i, D, false, F.Wk, DD, nullptr, D, false, f.Ahat, DD, nullptr, D, T(1),
               T(0), d.NP, st);
     }
     mark();
@@ -915,7 +911,7 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
     // ((U^R)^T: the first R columns of the column-major U, as rows)
     if (R > 0) {
       wait_for(st, sp);
-      gemm<T>(c->status + 2, R, D, R, f.Ainv, (int64_t)R * R, nullptr, R, false, f.U, DD, nullptr, D, false, f.M1,
+      gemm<T>(R, D, R, f.Ainv, (int64_t)R * R, nullptr, R, false, f.U, DD, nullptr, D, false, f.M1,
               (int64_t)R * D, nullptr, D, T(1), T(0), d.nb, sp);
       if (rows) launch_pivot_sequence(d.nb, R, f.piv, sp);
     }
@@ -955,9 +951,9 @@ h2_status factor_impl(h2_ctx* c, Factor<T>& F, int prec) {
       if (!ok) return fail(H2_ERR_CUDA, "tensor-core Schur update setup failed at level " + std::to_string(l));
       F.schur_tc = true;
     } else if (R > 0 && K > 0) {
-      gemm<T>(c->status + 2, R, K, R, f.Ainv, (int64_t)R * R, nullptr, R, false, f.Ahat + R, DD, d.diag_pair, D, false, f.Z,
+      gemm<T>(R, K, R, f.Ainv, (int64_t)R * R, nullptr, R, false, f.Ahat + R, DD, d.diag_pair, D, false, f.Z,
               (int64_t)R * K, nullptr, K, T(1), T(0), d.nb, st);
-      gemm<T>(c->status + 2, K, K, R, f.Ahat + (int64_t)R * D, DD, d.diag_pair, D, false, f.Z, (int64_t)R * K, nullptr, K,
+      gemm<T>(K, K, R, f.Ahat + (int64_t)R * D, DD, d.diag_pair, D, false, f.Z, (int64_t)R * K, nullptr, K,
               false, f.Ahat + (int64_t)R * D + R, DD, d.diag_pair, D, T(-1), T(1), d.nb, st);
     }
     mark();

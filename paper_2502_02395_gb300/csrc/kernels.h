@@ -48,10 +48,6 @@ template <typename T, typename TB>
 void gemm_simt(int M, int N, int K, const T* A, int64_t sA, const int32_t* ia, int lda, bool tA, const TB* B,
                int64_t sB, const int32_t* ib, int ldb, bool tB, T* C, int64_t sC, const int32_t* ic, int ldc,
                T alpha, T beta, int64_t batch, cudaStream_t st);
-// the same in FP64 on the tensor cores, from exact digit products (false: not for this K)
-bool gemm_split(int M, int N, int K, const double* A, int64_t sA, const int32_t* ia, int lda, bool tA, const double* B,
-                int64_t sB, const int32_t* ib, int ldb, bool tB, double* C, int64_t sC, const int32_t* ic, int ldc,
-                double alpha, double beta, int64_t batch, int32_t* err, cudaStream_t st);
 template <typename T>
 // true when the compact-WY factor Tw was formed too (Tw non-NULL, FP32 register form)
 bool launch_qr_panel(int nb, int D, int K, const T* Xin, T* Vout, T* tau, T* Tm, T* gscr, cudaStream_t st,

@@ -4,8 +4,7 @@
 //                          pairs and couplings G(SK_i, SK_j) (Algorithm 1),
 //                          evaluated from the points
 //   gemm_f32_tile_kernel,  SIMT batched GEMM C = alpha op(A) op(B) + beta C in
-//   gemm_batched_kernel    FP32, and in FP64 where the digit form on the tensor
-//                          cores does not apply
+//   gemm_batched_kernel    FP32 and in FP64
 //   qr_reg_kernel,         Householder QR of X^orth (FP32; FP64; any size), its
 //   qr_cluster_kernel,     compact WY factor and the explicit U = [U^R U^S]
 //   qr_panel_kernel        (Eq. 6-7)

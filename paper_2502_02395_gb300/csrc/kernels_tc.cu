@@ -690,314 +690,6 @@ bool gemm_tc(int ab_bf16, int M, int N, int K, const void* A, int64_t nA, int ro
 }
 
 // ------------------------------------------------------------------------
-// FP64 batched GEMM from exact 16-bit tensor-core products.
-//   op(A)(m,k) = tA ? A[k*lda+m] : A[m*lda+k]
-//   op(B)(k,n) = tB ? B[n*ldb+k] : B[k*ldb+n]
-//   C = alpha op(A) op(B) + beta C   (batch entries through ia / ib / ic)
-// Every row of op(A) and column of op(B) is scaled by a power of two above
-// its largest entry and cut into S = 8 signed digits of 7 bits (the splitting
-// of Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix
-// multiplication", 2012): x = 2^E sum_s d_s 2^(-6 - 7 s), |d_s| <= 64, 56
-// bits.  A digit is exact in BF16, a product of two at most 2^12 and a sum
-// of up to S products over K <= 512 at most 2^24, so the FP32 accumulators
-// hold the sums of digits i + j = g exactly and no order of summation matters.
-// The digits are stored with their weights 2^(-7 s), so that the products of
-// i + j = 8 can join accumulator 7 (there the lowest bits round); those
-// below are left out.  The epilogue adds the accumulators (64-bit integers,
-// one FP64 rounding) and scales back.  Error: about 2^-56 of (row maximum x
-// column maximum) per product, below the rounding of a 53-bit running sum
-// of that size.  A row or column holding a NaN or an infinity gives NaN.
-//
-// One CTA per 128 x 64 tile, all 512 columns of TMEM.  All threads cut a
-// 64-wide slice of K into swizzled digit tiles in shared memory (integer work:
-// the FP64 pipe, 2 per clock and SM, is not used for it), one thread issues
-// the 43 tcgen05.mma chains, and the next slice is fetched into registers
-// meanwhile.  Bound by the phases of one CTA following each other (58 us a tile of
-// K = 256: maxima, cutting, MMAs, epilogue).  300 products of 256^3: 0.96 ms,
-// 196^3 x 600: 1.65 ms; in FP64 multiply-adds (gemm_batched_kernel) 8.2 and 13.3
-// ms.  Error in the Frobenius norm against 113-bit sums, random, graded and
-// diagonally dominant operands: 0.5 - 1.4e-16, there 3.3 - 7.4e-16.
-// K < 16 and K > 512 stay there.  The wait is bounded (2 s); on expiry err is set.
-// ------------------------------------------------------------------------
-struct SplitArgs {
-  int M, N, K;
-  const double* A;
-  int64_t sA;
-  const int32_t* ia;
-  int lda, tA;
-  const double* B;
-  int64_t sB;
-  const int32_t* ib;
-  int ldb, tB;
-  double* C;
-  int64_t sC;
-  const int32_t* ic;
-  int ldc;
-  double alpha, beta;
-  int vecA, vecB, vecC;  // 16-byte accesses allowed
-  int32_t* err;
-};
-
-__device__ __forceinline__ int split_expo(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-// round(x 2^(55 - E)) + the digits' offsets, E = ef - 1022
-__device__ __forceinline__ unsigned long long split_fix(double x, int ef) {
-  const long long b = __double_as_longlong(x);
-  const int e = (int)(b >> 52) & 0x7ff, sh = min(ef - max(e, 1), 62);
-  const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0ull);
-  const unsigned long long r = ((m << 2) + (sh ? 1ull << (sh - 1) : 0ull)) >> sh;
-  constexpr unsigned long long off = 64ull * (((1ull << 56) - 1) / 127);
-  return (b < 0 ? 0ull - r : r) + off;
-}
-// A row's and a column's scale multiply to 2^(EA + EB - 61); NaN for a row that is not finite.
-__device__ __forceinline__ double split_scale(int ef, int col) {
-  return ef == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(1.0, ef - 1022 - 30 - col);
-}
-
-constexpr int SP_S = 8, SP_NT = 512;
-constexpr int SP_BM = 128, SP_BN = 64, SP_BK = 64;
-
-// Eight entries of an operand row (k0 .. k0 + 7): rs / ks strides of row and k.
-__device__ __forceinline__ void split_load(const double* P, int64_t rs, int64_t ks, int row, int rows, int k, int K, bool vec,
-                                           double (&x)[8]) {
-  const double* q = P + row * rs + k * ks;
-  if (row < rows && k + 8 <= K) {
-    if (vec) {
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const double2 w = __ldg(reinterpret_cast<const double2*>(q) + v);
-        x[2 * v] = w.x, x[2 * v + 1] = w.y;
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) x[j] = q[j * ks];
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) x[j] = (row < rows && k + j < K) ? q[j * ks] : 0.0;
-  }
-}
-
-__global__ void __launch_bounds__(SP_NT, 1) gemm_split_kernel(SplitArgs p, int64_t batch) {
-  constexpr int S = SP_S, NT = SP_NT, TA = SP_BM * 8 / NT, TB = SP_BN * 8 / NT, TK = TA + TB;
-  constexpr uint32_t A_BYTES = SP_BM * 128, B_BYTES = SP_BN * 128;  // one digit's tile
-  extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t done_bar;
-  __shared__ uint32_t tmem_base_sh;
-  __shared__ int emax[SP_BM + SP_BN];
-  __shared__ double scl[SP_BM + SP_BN];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  uint8_t* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  if (tid == 0) {
-    mbar_init(&done_bar, 1);
-    mbar_init_fence();
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_sh)),
-                 "r"((uint32_t)(S * SP_BN))
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = tmem_base_sh;
-  const int m0 = blockIdx.y * SP_BM, n0 = blockIdx.x * SP_BN;
-  const int64_t rsA = p.tA ? 1 : p.lda, ksA = p.tA ? p.lda : 1, rsB = p.tB ? p.ldb : 1, ksB = p.tB ? 1 : p.ldb;
-  // this thread's (row, chunk of 8 k) pieces: chunks fastest where k is
-  // contiguous, rows fastest otherwise (coalesced either way)
-  int row[TK], ch[TK];
-#pragma unroll
-  for (int i = 0; i < TK; ++i) {
-    const bool a = i < TA;
-    const int t = tid + NT * (a ? i : i - TA), rows = a ? SP_BM : SP_BN;
-    const bool kc = (a ? ksA : ksB) == 1;
-    row[i] = kc ? t >> 3 : t % rows;
-    ch[i] = kc ? t & 7 : t / rows;
-  }
-  uint32_t ph = 0;
-  bool failed = false;
-  for (int64_t b = blockIdx.z; b < batch && !failed; b += gridDim.z) {
-    const double* Ab = p.A + (p.ia ? (int64_t)p.ia[b] : b) * p.sA + m0 * rsA;
-    const double* Bb = p.B + (p.ib ? (int64_t)p.ib[b] : b) * p.sB + n0 * rsB;
-    const int mrows = min(p.M - m0, SP_BM), nrows = min(p.N - n0, SP_BN);
-    double x[TK][8];
-    auto load = [&](int k0) {
-#pragma unroll
-      for (int i = 0; i < TK; ++i) {
-        const bool a = i < TA;
-        split_load(a ? Ab : Bb, a ? rsA : rsB, a ? ksA : ksB, row[i], a ? mrows : nrows, k0 + 8 * ch[i], p.K,
-                      a ? p.vecA : p.vecB, x[i]);
-      }
-    };
-    // row maxima (exponents only)
-    for (int r = tid; r < SP_BM + SP_BN; r += NT) emax[r] = 1;
-    __syncthreads();
-    int mx[TK];
-#pragma unroll
-    for (int i = 0; i < TK; ++i) mx[i] = 1;
-    for (int k0 = 0; k0 < p.K; k0 += SP_BK) {
-      load(k0);
-#pragma unroll
-      for (int i = 0; i < TK; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) mx[i] = max(mx[i], split_expo(x[i][j]));
-    }
-#pragma unroll
-    for (int i = 0; i < TK; ++i) atomicMax(&emax[(i < TA ? 0 : SP_BM) + row[i]], mx[i]);
-    if (p.K > SP_BK) load(0);
-    __syncthreads();
-    for (int r = tid; r < SP_BM + SP_BN; r += NT) scl[r] = split_scale(emax[r], r < SP_BM ? 0 : 1);
-    int ef[TK];
-#pragma unroll
-    for (int i = 0; i < TK; ++i) ef[i] = emax[(i < TA ? 0 : SP_BM) + row[i]];
-    for (int k0 = 0; k0 < p.K; k0 += SP_BK) {
-#pragma unroll
-      for (int i = 0; i < TK; ++i) {
-        unsigned long long q[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) q[j] = split_fix(x[i][j], ef[i]);
-        const uint32_t bytes = i < TA ? A_BYTES : B_BYTES;
-        uint8_t* dst = base + (i < TA ? 0u : S * A_BYTES) + row[i] * 128 + ((ch[i] ^ (row[i] & 7)) << 4);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const int sh = 7 * (S - 1 - s);
-          uint32_t w[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            // BF16 (128 + u) 2^(-7 s) is 0x4300 - 896 s + u exactly (u <= 128);
-            // minus 192 2^(-7 s) gives the weighted digit
-            const uint32_t u0 = (uint32_t)(q[2 * j] >> sh), u1 = (uint32_t)(q[2 * j + 1] >> sh);
-            const uint32_t v = s == 0 ? u0 + (u1 << 16) : (u0 & 127u) | ((u1 & 127u) << 16);
-            const uint32_t h = v + (0x4300u - 896u * s) * 0x10001u;
-            const float c = 192.0f / (float)(1ull << (7 * s));
-            const __nv_bfloat162 d =
-                __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&h), __floats2bfloat162_rn(c, c));
-            w[j] = *reinterpret_cast<const uint32_t*>(&d);
-          }
-          *reinterpret_cast<uint4*>(dst + s * bytes) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      tc_fence_before();
-      __syncthreads();
-      if (tid == 0) {
-        tc_fence_after();
-        const uint32_t sa = smem_u32(base), sb = sa + S * A_BYTES;
-        const uint32_t idesc = idesc_f16(1, SP_BM, SP_BN);
-        const int ks = min(SP_BK, p.K - k0);
-        for (int k = 0; k < ks; k += 16) {
-          const uint64_t off = (uint64_t)((k * 2) >> 4);
-#pragma unroll
-          for (int i = 0; i < S; ++i) {
-            const uint64_t da = smem_desc_sw128(sa + i * A_BYTES) + off;
-            const uint32_t acc = (k0 > 0 || k > 0 || i > 0) ? 1u : 0u;
-#pragma unroll
-            for (int j = 0; j < min(S, S + 1 - i); ++j) {
-              const uint64_t db = smem_desc_sw128(sb + j * B_BYTES) + off;
-              asm volatile(
-                  "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem + min(i + j, S - 1) * SP_BN),
-                  "l"(da), "l"(db), "r"(idesc), "r"(acc)
-                  : "memory");
-            }
-          }
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         smem_u32(&done_bar))
-                     : "memory");
-      }
-      __syncwarp();
-      if (k0 + SP_BK < p.K) load(k0 + SP_BK);
-      const bool ok = mbar_wait(&done_bar, ph & 1);
-      ++ph;
-      failed = __syncthreads_or(!ok);
-      if (failed) break;
-    }
-    if (failed) break;
-    tc_fence_after();
-    // epilogue: TMEM lane quarter warp % 4, the warps of a quarter share the columns
-    constexpr int CW = SP_BN / (NT / 128);
-    const int m = (warp & 3) * 32 + lane, c0 = (warp >> 2) * CW;
-    double* Cb = p.C + (p.ic ? (int64_t)p.ic[b] : b) * p.sC + (int64_t)(m0 + m) * p.ldc + n0;
-    const double am = scl[m];
-    for (int c = c0; c < c0 + CW; c += 8) {
-      uint32_t r[S][8];
-#pragma unroll
-      for (int g = 0; g < S; ++g)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]), "=r"(r[g][4]), "=r"(r[g][5]),
-                       "=r"(r[g][6]), "=r"(r[g][7])
-                     : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * SP_BN + c)));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (m >= mrows || c >= nrows) continue;
-      double v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const double bn = scl[SP_BM + c + j] * p.alpha;
-        long long hi = 0, lo = 0;  // accumulators 0 - 3 and 4 - 7, in units of 2^(-7 3) and 2^(-7 7)
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          hi += (long long)__float2int_rn(__uint_as_float(r[g][j]) * (float)(1ull << (7 * g))) * (1ll << (7 * (3 - g)));
-          lo += (long long)__float2int_rn(__uint_as_float(r[4 + g][j]) * (float)(1ull << (7 * (4 + g)))) *
-                (1ll << (7 * (3 - g)));
-        }
-        // integers below 2^51 as doubles: 1.5 2^52 + i by its bits
-        const double mg = 6755399441055744.0;
-        const double dh = __longlong_as_double(__double_as_longlong(mg) + hi) - mg;
-        const double dl = __longlong_as_double(__double_as_longlong(mg) + lo) - mg;
-        v[j] = fma(dh, 268435456.0, dl) * am * bn;
-      }
-      if (p.vecC && c + 8 <= nrows) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          double2* o = reinterpret_cast<double2*>(Cb + c) + q;
-          double2 w = make_double2(v[2 * q], v[2 * q + 1]);
-          if (p.beta != 0.0) {
-            const double2 t = *o;
-            w.x = fma(p.beta, t.x, w.x), w.y = fma(p.beta, t.y, w.y);
-          }
-          *o = w;
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (c + j < nrows) Cb[c + j] = p.beta != 0.0 ? fma(p.beta, Cb[c + j], v[j]) : v[j];
-      }
-    }
-    tc_fence_before();
-    __syncthreads();
-  }
-  if (failed && tid == 0) {
-    atomicExch(p.err, 1);
-    mbar_wait(&done_bar, (ph - 1) & 1);  // the MMAs in flight
-  }
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(S * SP_BN))
-                 : "memory");
-  }
-}
-
-bool gemm_split(int M, int N, int K, const double* A, int64_t sA, const int32_t* ia, int lda, bool tA, const double* B,
-                int64_t sB, const int32_t* ib, int ldb, bool tB, double* C, int64_t sC, const int32_t* ic, int ldc,
-                double alpha, double beta, int64_t batch, int32_t* err, cudaStream_t st) {
-  if (K < 16 || K > 512) return false;
-  auto vec = [](const void* q, int64_t s, int ld) {
-    return ld % 2 == 0 && s % 2 == 0 && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
-  };
-  const SplitArgs p{M,  N,  K,   A,  sA, ia, lda, tA,    B,    sB,
-                    ib, ldb, tB, C,  sC, ic, ldc, alpha, beta, !tA && vec(A, sA, lda),
-                    tB && vec(B, sB, ldb), vec(C, sC, ldc), err};
-  const size_t sm = (size_t)SP_S * (SP_BM + SP_BN) * 128 + 1024;
-  allow_smem((const void*)gemm_split_kernel);
-  dim3 grid((N + SP_BN - 1) / SP_BN, (M + SP_BM - 1) / SP_BM, (unsigned)std::min<int64_t>(batch, 65535));
-  ++g_launches;
-  gemm_split_kernel<<<grid, SP_NT, sm, st>>>(p, batch);
-  return true;
-}
-
-// ------------------------------------------------------------------------
 // self-test of the bounded waits: an mbarrier that expects one arrival which
 // never comes.  Thread 0 waits with the same helper the TMA kernels use; when
 // the wait gives up it records the failure in *flag (as those kernels record
