@@ -12,7 +12,7 @@
 
 using namespace h2;
 
-std::atomic<long long> h2::g_launches{0};
+LaunchCount h2::g_launches;
 
 namespace {
 
@@ -1183,7 +1183,7 @@ KernelGraph capture_graph(h2_ctx* c, Fn fn) {
   cudaStream_t keep = c->stream;
   c->stream = c->cap_stream;
   cudaGraph_t g = nullptr;
-  const long long n0 = g_launches.load();
+  const long long n0 = LaunchCount::mine;
   if (cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
     fn();
     const bool launched = take_launch_error() == cudaSuccess;
@@ -1191,8 +1191,8 @@ KernelGraph capture_graph(h2_ctx* c, Fn fn) {
       if (cudaGraphInstantiate(&out.ex, g, 0) != cudaSuccess) out.ex = nullptr;
     }
   }
-  out.kernels = g_launches.load() - n0;
-  g_launches -= out.kernels;  // counted again per replay
+  out.kernels = LaunchCount::mine - n0;
+  g_launches += -out.kernels;  // counted again per replay
   if (g) cudaGraphDestroy(g);
   c->stream = keep;
   cudaGetLastError();
@@ -2876,7 +2876,7 @@ h2_status h2_stats(const h2_ctx* c, char* json, size_t cap) {
     << "},\"calls\":{\"subst\":" << t.n_subst << ",\"matvec\":" << t.n_matvec << ",\"matvec32\":" << t.n_matvec32 << ",\"matvec32_leaf\":" << t.n_leaf32
     << "},\"method\":" << t.method
     << ",\"iters\":" << t.iters << ",\"relres\":" << t.relres
-    << ",\"kernel_launches\":" << g_launches.load() << ",\"refine_method\":" << c->refine_method
+    << ",\"kernel_launches\":" << g_launches.all.load() << ",\"refine_method\":" << c->refine_method
     << ",\"restart\":" << c->restart << ",\"tensor_cores\":" << (c->used_tc ? "true" : "false")
     << ",\"schur_tensor_cores\":" << ((c->prec > 0 && c->f32.schur_tc) ? "true" : "false")
     << ",\"rr_lu_fp64\":" << (c->rr_lu64 ? "true" : "false")

@@ -7,8 +7,15 @@
 
 namespace h2 {
 
-// Number of kernels this library has launched (reported by h2_stats).
-extern std::atomic<long long> g_launches;
+// Number of kernels this library has launched (reported by h2_stats), and of
+// those this thread launched (what a capture holds: other threads go on).
+struct LaunchCount {
+  std::atomic<long long> all{0};
+  inline static thread_local long long mine = 0;
+  void operator++() { *this += 1; }
+  void operator+=(long long n) { all += n, mine += n; }
+};
+extern LaunchCount g_launches;
 // Tensor-core GEMM kernel form of the factorization's main chain
 // (projection, Schur update), process-wide (H2_OPT_TC_KERNEL): 0 one CTA per
 // batch entry, 1 a persistent grid of two CTAs per SM, 2 (default) the

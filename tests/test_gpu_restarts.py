@@ -48,3 +48,35 @@ def test_restarts_on_one_context(B, graphs):
         assert np.allclose(hist, F.stats()["history"], rtol=1e-6, atol=0), restart
         assert np.linalg.norm(x - xf) <= 1e-9 * np.linalg.norm(xf)
         F.close()
+
+
+def test_launch_count_with_threads(B):
+    """Contexts whose solves are captured and replayed in four threads at a time
+    count as many launches as one after another."""
+    import threading
+    sizes = [1024, 1500, 2048, 3000]
+    ctx = lambda n: context(B, n)
+
+    def work(S, n):
+        S.factor("fp16")
+        for k in range(3):
+            S.solve(W.uniform_rhs(n, k), target=1e-10, max_iters=300)
+
+    def count(threads):
+        solvers = [(ctx(n), n) for n in sizes]
+        n0 = solvers[0][0].stats()["kernel_launches"]
+        ts = [threading.Thread(target=work, args=s) for s in solvers]
+        for t in ts:
+            t.start()
+            if not threads:
+                t.join()
+        for t in ts:
+            t.join()
+        n1 = solvers[0][0].stats()["kernel_launches"]
+        for S, _ in solvers:
+            S.close()
+        return n1 - n0
+
+    one = count(False)
+    for _ in range(5):
+        assert count(True) == one
