@@ -701,12 +701,17 @@ struct DeviceGpuCompressor : GpuCompressor {
     GC_TRY(put(&d_cptr, j.cptr));
     GC_TRY(put(&d_cidx, j.cidx));
     GC_TRY(make(&d_W, j.cidx.size() * m));
-    const int nz = sketch_splits(j.nb, (j.D + GC_ROWS - 1) / GC_ROWS);
-    GC_TRY(make(&d_Y, nz * nb * D * m));
     GC_TRY(make(&d_X, nb * D * K));
     GC_TRY(make(&d_SK, nb * K));
     GC_TRY(make(&d_rho, nb));
     GC_TRY(make(&d_err, nb));
+    // (the splits' partial sums last: fewer splits where they do not fit)
+    int nz = sketch_splits(j.nb, (j.D + GC_ROWS - 1) / GC_ROWS);
+    while ((e = make(&d_Y, nz * nb * D * m)) == cudaErrorMemoryAllocation && nz > 1) {
+      cudaGetLastError();
+      nz /= 2;
+    }
+    if (e != cudaSuccess) return std::string("the sketch's sums: ") + cudaGetErrorString(e);
     launch_cc_weights(G, pts, j.nb, d_cptr, d_cidx, j.m, j.seed, j.gs, d_W, 0);
     launch_sketch(G, pts, j.nb, j.D, j.m, nz, d_nbox, d_bpts, d_fptr, d_fidx, d_nptr, d_nidx, d_cptr, d_cidx, d_W,
                   j.seed, d_Y, 0);

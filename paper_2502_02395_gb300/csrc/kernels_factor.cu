@@ -522,21 +522,6 @@ template void gemm_simt<float, float>(int, int, int, const float*, int64_t, cons
                                       const int32_t*, int, float, float, int64_t, cudaStream_t);
 
 // ------------------------------------------------------------------------
-// block-wide sum
-// ------------------------------------------------------------------------
-template <typename T>
-__device__ T block_sum(T v, T* sbuf) {
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (lane == 0) sbuf[warp] = v;
-  __syncthreads();
-  T t = T(0);
-  for (int w = 0; w < nw; ++w) t += sbuf[w];
-  return t;
-}
-
-// ------------------------------------------------------------------------
 // a1: complement bases (Eq. 6-7) in three steps:
 //   qr_panel_kernel   Householder QR of X^orth (LAPACK geqr2 conventions:
 //                     beta = -sign(alpha) |x|), one CTA per box, the panel in
