@@ -566,13 +566,6 @@ __global__ void __launch_bounds__(512, 1)
 }  // namespace
 
 namespace {
-int num_sms() {
-  int dev = 0, nsm = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  return nsm;
-}
-
 void launch_cc_weights(const KernelFn& G, const double* pts, int nb, const int64_t* cptr, const int64_t* cidx, int m,
                        uint64_t seed, int gs, double* W, cudaStream_t st) {
   ++g_launches;

@@ -34,6 +34,8 @@ extern std::atomic<int> g_box_stream;
 extern std::atomic<int> g_box_ctas_per_sm;
 extern std::atomic<int> g_pair_ctas_per_sm;
 
+int num_sms();  // of the current device
+
 // Lets kernel f be launched with as much dynamic shared memory as the device
 // allows (once per kernel and device; safe from several threads).
 void allow_smem(const void* f);

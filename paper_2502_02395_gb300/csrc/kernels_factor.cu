@@ -477,7 +477,7 @@ void launch_form_u(int64_t nb, int D, int K, const float* W1, const float* V, fl
   if (nb == 0 || D == 0) return;
   // (64 x 64 tiles while 128 x 128 ones leave SMs idle)
   const int64_t big = nb * ((D + 127) / 128) * ((D + 127) / 128);
-  const int bm = big < 152 ? 64 : 128;
+  const int bm = big < num_sms() ? 64 : 128;
   const dim3 g((D + bm - 1) / bm, (D + bm - 1) / bm, (unsigned)std::min<int64_t>(nb, 65535));
   const bool vec = D % 4 == 0 && K % 4 == 0 && Dp == D;
   auto go = vec ? (bm == 64 ? form_u_kernel<true, 1> : form_u_kernel<true, 2>)
@@ -501,7 +501,7 @@ void gemm_simt(int M, int N, int K, const T* A, int64_t sA, const int32_t* ia, i
     const int vecC = (ldc % 4 == 0) && (sC % 4 == 0) && aligned16(C);
     // (64 x 64 tiles while 128 x 128 ones leave SMs idle)
     const int64_t big = batch * ((M + 127) / 128) * ((N + 127) / 128);
-    const int bm = big < 152 ? 64 : 128;
+    const int bm = big < num_sms() ? 64 : 128;
     const dim3 g2((N + bm - 1) / bm, (M + bm - 1) / bm, (unsigned)std::min<int64_t>(batch, 65535));
     auto go = bm == 64 ? gemm_f32_tile_kernel<1> : gemm_f32_tile_kernel<2>;
     ++g_launches;
@@ -1208,7 +1208,7 @@ bool launch_qr_panel(int nb, int D, int K, const T* Xin, T* Vout, T* tau, T* Tm,
     if (D <= 256 && K <= 128) {
       // C = 2, 4 or 8 CTAs a box with 64 / C or fewer doubles of the panel a thread
       int C = 8;
-      while (C > 2 && nb * C > 152) C /= 2;
+      while (C > 2 && nb * C > num_sms()) C /= 2;
       const int cw = (K + 16 * C - 1) / (16 * C);
       auto go = cw <= 1 ? launch_qr_cluster<1> : cw <= 2 ? launch_qr_cluster<2> : launch_qr_cluster<4>;
       go(nb, D, K, C, Xin, Vout, tau, Tm, st);

@@ -1089,13 +1089,12 @@ static void launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, si
   note_launch(cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...));
 }
 
-static int num_sms() {
-  static int nsm = 0;
-  if (!nsm) {
-    int dev = 0;
+int num_sms() {
+  static const int nsm = [] {
+    int dev = 0, n = 0;
     cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 152;
-  }
+    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 152;
+  }();
   return nsm;
 }
 

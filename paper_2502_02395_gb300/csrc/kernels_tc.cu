@@ -665,9 +665,7 @@ bool gemm_tc(int ab_bf16, int M, int N, int K, const void* A, int64_t nA, int ro
   const size_t max_ctas = 512 / cols;
   smem = std::max(smem, per_sm / (max_ctas + 1) + 1024);
   allow_smem((const void*)tc_gemm_kernel);
-  int dev = 0, nsm = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int nsm = num_sms();
   const int mode = form >= 0 ? form : g_tc_kernel.load();
   if (mode == 2 && 2 * cols <= 512) {
     // persistent warp-specialized kernel: one CTA per SM (TMEM holds two
@@ -748,7 +746,7 @@ void launch_amax_blocks(const S* base, int64_t nblk, int64_t stride, int rows, i
                         cudaStream_t st, const int32_t* idx) {
   if (nblk == 0 || rows == 0 || cols == 0) return;
   const int blocks = (int)std::min<int64_t>(nblk, 152 * 16);
-  const int bands = std::max(1, std::min((rows + 15) / 16, 152 * 8 / blocks));
+  const int bands = std::max(1, std::min((rows + 15) / 16, 8 * num_sms() / blocks));
   ++g_launches;
   if constexpr (std::is_same<S, float>::value)
     if (cols % 4 == 0 && ld % 4 == 0 && stride % 4 == 0 && (reinterpret_cast<uintptr_t>(base) & 15) == 0) {
