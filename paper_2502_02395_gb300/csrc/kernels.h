@@ -297,7 +297,7 @@ void launch_unpad(const float* in, double* out, int64_t n, PadSeg p, cudaStream_
 // xs; w -= V (V^T w) twice; V_j+1 = vin = w / ||w||; h1, h2, ||w||^2 and the
 // iteration count to pinned host memory.  n entries per vector, m0 the
 // restart; part holds (2 (m0 + 1) + 1) * kOrthCtas doubles.
-constexpr int kOrthCtas = 152;
+constexpr int kOrthCtas = 2 * 152;
 struct OrthArgs {
   float *V, *Z, *w, *vin;
   const float* xs;

@@ -3251,9 +3251,14 @@ __global__ void multi_axpy_f32_kernel(const float* __restrict__ V, int64_t ldv, 
 // kernels.h).  Every CTA owns a slice of the vectors; a pass's dot products
 // are finished by the next launch, in which every CTA adds the partial sums of
 // all CTAs itself (FP64, in CTA order), so no launch exists only to add
-// them.  Bound by latency (a few launches in line) up to some 10^5 entries and
-// by the reads of V beyond.  Ten separate launches and a host
-// synchronization took 85 us an iteration at 16384 entries.
+// them.  Entries are read four at a time (n is a multiple of 4: the symmetric
+// storage of the inner iterations wants boxes of multiples of 4).  Bound by
+// latency (a few launches in line) up to some 10^5 entries and by the reads of
+// V beyond, which want two CTAs an SM (kOrthCtas) and, in the last step, the
+// FP64 root and quotient of the scale in one thread of a CTA: the four steps of
+// 19 iterations at 262144 entries took 2.25 ms with one CTA an SM, scalar loads
+// and the root in every thread, 1.18 ms now (2048 entries, 5 iterations: 0.14
+// and 0.12 ms).
 // ------------------------------------------------------------------------
 struct OrthSlice {
   int64_t b, e;
@@ -3272,11 +3277,15 @@ __device__ __forceinline__ void orth_dots(const OrthArgs& a, int j, OrthSlice sl
     zero(H);
     zero(L);
     const int nv = min(8, j + 1 - v0);
-    for (int64_t e = sl.b + tid; e < sl.e; e += 256) {
-      const float x = a.w[e];
+    for (int64_t e = sl.b + 4 * tid; e < sl.e; e += 1024) {
+      const float4 x = *reinterpret_cast<const float4*>(a.w + e);
 #pragma unroll
       for (int g = 0; g < 8; ++g)
-        if (g < nv) df_acc(H[g], L[g], a.V[(int64_t)(v0 + g) * a.n + e], x);
+        if (g < nv) {
+          const float4 v = *reinterpret_cast<const float4*>(a.V + (int64_t)(v0 + g) * a.n + e);
+          df_acc(H[g], L[g], v.x, x.x), df_acc(H[g], L[g], v.y, x.y);
+          df_acc(H[g], L[g], v.z, x.z), df_acc(H[g], L[g], v.w, x.w);
+        }
     }
     float sh, sl2;
     df_tsum<8, 32>(H, L, sh, sl2);
@@ -3305,27 +3314,39 @@ __device__ __forceinline__ void orth_update(const OrthArgs& a, int j, OrthSlice 
     }
   }
   __syncthreads();
-  for (int64_t e = sl.b + tid; e < sl.e; e += 256) {
-    float H = 0.0f, L = 0.0f;
+  for (int64_t e = sl.b + 4 * tid; e < sl.e; e += 1024) {
+    float H[4], L[4];
+    zero(H);
+    zero(L);
 #pragma unroll 4
     for (int v = 0; v <= j; ++v) {
-      const float x = a.V[(int64_t)v * a.n + e];
-      df_acc(H, L, ch[v], x);
-      L = fmaf(cl[v], x, L);
+      const float4 x = *reinterpret_cast<const float4*>(a.V + (int64_t)v * a.n + e);
+      const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        df_acc(H[q], L[q], ch[v], xs[q]);
+        L[q] = fmaf(cl[v], xs[q], L[q]);
+      }
     }
-    float wh = a.w[e], wl = 0.0f;
-    df_add(wh, wl, -H, -L);
-    a.w[e] = wh + wl;
+    const float4 w = *reinterpret_cast<const float4*>(a.w + e);
+    float wh[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float wl = 0.0f;
+      df_add(wh[q], wl, -H[q], -L[q]);
+      wh[q] += wl;
+    }
+    *reinterpret_cast<float4*>(a.w + e) = make_float4(wh[0], wh[1], wh[2], wh[3]);
   }
 }
 // STEP 0: Z_j = xs, first dots; 1: first update, second dots; 2: second update,
-// norm; 3: normalization, result to the host
+// norm; 3: result to the host (by CTA 0 as it starts: everything it reports is
+// complete then, and the host works while the vectors are written), normalization
 template <int STEP>
 __global__ void __launch_bounds__(256) orth_kernel(const OrthArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   float* ch = reinterpret_cast<float*>(smraw);
   float* cl = ch + a.m0 + 1;
-  __shared__ unsigned int last;
   griddep_wait();
   griddep_launch_next();
   const int tid = threadIdx.x, j = a.state->j;
@@ -3336,7 +3357,8 @@ __global__ void __launch_bounds__(256) orth_kernel(const OrthArgs a) {
   if constexpr (STEP == 0) {
     if (blockIdx.x == 0 && tid == 0) a.stamp[kGmStamps * j + 4] = global_ns();
     float* z = a.Z + (int64_t)j * a.n;
-    for (int64_t e = sl.b + tid; e < sl.e; e += 256) z[e] = a.xs[e];
+    for (int64_t e = sl.b + 4 * tid; e < sl.e; e += 1024)
+      *reinterpret_cast<float4*>(z + e) = *reinterpret_cast<const float4*>(a.xs + e);
     orth_dots(a, j, sl, p1);
   } else if constexpr (STEP == 1) {
     orth_update(a, j, sl, p1, a.h, ch, cl);
@@ -3344,45 +3366,49 @@ __global__ void __launch_bounds__(256) orth_kernel(const OrthArgs a) {
   } else if constexpr (STEP == 2) {
     orth_update(a, j, sl, p2, a.h + a.m0 + 2, ch, cl);
     float H = 0.0f, L = 0.0f;
-    for (int64_t e = sl.b + tid; e < sl.e; e += 256) df_acc(H, L, a.w[e], a.w[e]);
+    for (int64_t e = sl.b + 4 * tid; e < sl.e; e += 1024) {
+      const float4 x = *reinterpret_cast<const float4*>(a.w + e);
+      df_acc(H, L, x.x, x.x), df_acc(H, L, x.y, x.y), df_acc(H, L, x.z, x.z), df_acc(H, L, x.w, x.w);
+    }
     const double t = block_df_total(H, L);
     if (tid == 0) p3[blockIdx.x] = t;
   } else {
-    __shared__ double ss;
+    __shared__ float ss;
     if (tid < 32) {
       double s = 0;
       for (int k = tid; k < a.ctas; k += 32) s += p3[k];
       s = warp_sum(s);
-      if (tid == 0) ss = s;
+      if (tid == 0) {
+        const double r = sqrt(s);
+        ss = (float)(r > 0 ? 1.0 / r : 0.0);
+        if (blockIdx.x == 0) a.host[2 * (a.m0 + 2)] = s;
+      }
+    }
+    if (blockIdx.x == 0) {
+      for (int v = tid; v <= j; v += 256) {
+        a.host[v] = a.h[v];
+        a.host[a.m0 + 2 + v] = a.h[a.m0 + 2 + v];
+      }
+      __threadfence_system();
     }
     __syncthreads();
-    const double nw2 = ss, r = sqrt(nw2);
-    const float sf = (float)(r > 0 ? 1.0 / r : 0.0);
+    if (blockIdx.x == 0 && tid == 0) {
+      __threadfence_system();
+      *reinterpret_cast<volatile unsigned long long*>(a.flag) = (unsigned long long)j + 1;
+    }
+    const float sf = ss;
     float* vn = a.V + (int64_t)(j + 1) * a.n;
-    for (int64_t e = sl.b + tid; e < sl.e; e += 256) {
-      const float x = a.w[e] * sf;
-      vn[e] = x;
-      a.vin[e] = x;
+    for (int64_t e = sl.b + 4 * tid; e < sl.e; e += 1024) {
+      float4 x = *reinterpret_cast<const float4*>(a.w + e);
+      x.x *= sf, x.y *= sf, x.z *= sf, x.w *= sf;
+      *reinterpret_cast<float4*>(vn + e) = x;
+      *reinterpret_cast<float4*>(a.vin + e) = x;
     }
-    // the last CTA tells the host and moves to the next iteration
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(&a.state->done, 1u);
-    __syncthreads();
-    if (last + 1 != gridDim.x) return;
-    for (int v = tid; v <= j; v += 256) {
-      a.host[v] = a.h[v];
-      a.host[a.m0 + 2 + v] = a.h[a.m0 + 2 + v];
-    }
-    if (tid == 0) a.host[2 * (a.m0 + 2)] = nw2;
-    __threadfence_system();
-    __syncthreads();
-    if (tid == 0) {
+    // the last CTA to have read the index moves it to the next iteration
+    if (tid == 0 && atomicAdd(&a.state->done, 1u) + 1 == gridDim.x) {
       a.state->done = 0;
       a.state->j = j + 1;
       a.stamp[kGmStamps * (j + 1)] = global_ns();
-      __threadfence_system();
-      *reinterpret_cast<volatile unsigned long long*>(a.flag) = (unsigned long long)j + 1;
     }
   }
 }
