@@ -1448,7 +1448,7 @@ void matvec_df(h2_ctx* c, const double* x, double* y) {
                           nullptr, nullptr, y, c->lv[L].D, st);
   } else {
     launch_matvec_leaf_df(lf, c->A32, c->Alo, L ? c->X32p[L] : nullptr, L ? c->Xlo[L] : nullptr, c->xdf_h, c->xdf_l,
-                          yhh, yhl, y, st);
+                          yhh, yhl, y, c->lv[L].D, st);
   }
 }
 void matvec32(h2_ctx* c, const float* x, float* y, EventPairs* leaf_ev = nullptr, unsigned long long* stamp = nullptr) {

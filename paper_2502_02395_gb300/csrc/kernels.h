@@ -243,9 +243,10 @@ void launch_matvec_far_df_all(const FarDfArgs& a, cudaStream_t st);
 void launch_matvec_rows_df(int nb, int D, int K, const float* Xh, const float* Xl, const float* yhh, const float* yhl,
                            const float* bh, const float* bl, int seg, const int64_t* ptr, const int32_t* ent,
                            const float* ph, const float* pl, float* oh, float* ol, double* y, int ny, cudaStream_t st);
-// leaf, general near lists: y_i = X_i yhat_i + sum_{near j} A_ij x_j
+// leaf, general near lists: y_i = X_i yhat_i + sum_{near j} A_ij x_j, ny rows a
+// box in y
 void launch_matvec_leaf_df(const DevLevel& L, const float* Ah, const float* Al, const float* Xh, const float* Xl,
-                           const float* xh, const float* xl, const float* yhh, const float* yhl, double* y,
+                           const float* xh, const float* xl, const float* yhh, const float* yhl, double* y, int ny,
                            cudaStream_t st);
 // h = fl32(v), l = fl32(v - h); v has n entries in segments of p.len, h and l
 // nb segments of p.str (the rest zero)

@@ -2259,8 +2259,9 @@ __device__ __forceinline__ void df_split(double v, float& h, float& l) {
   l = (float)(v - (double)h);
 }
 
-// leaf: y_i = X_i yh_i + sum_{near j} A_ij x_j
-__global__ void __launch_bounds__(256, 2) mv_leaf_df_kernel(int D, int K, const int64_t* __restrict__ ptr,
+// leaf: y_i = X_i yh_i + sum_{near j} A_ij x_j, ny rows a box in y (the boxes'
+// points; rows ny .. D - 1 are padding)
+__global__ void __launch_bounds__(256, 2) mv_leaf_df_kernel(int D, int ny, int K, const int64_t* __restrict__ ptr,
                                                             const int32_t* __restrict__ nj, const float* __restrict__ Ah,
                                                             const float* __restrict__ Al, const float* __restrict__ Xh,
                                                             const float* __restrict__ Xl, const float* __restrict__ xh,
@@ -2292,17 +2293,17 @@ __global__ void __launch_bounds__(256, 2) mv_leaf_df_kernel(int D, int K, const 
     for (int q = 0; q < nn; ++q)
       rows_acc_df<kRPWdf>(r0, Ah + (p0 + q) * D * D, Al + (p0 + q) * D * D, D, D, D, xsh + q * Dp, xsl + q * Dp, H,
                           L);
-    rows_finish_df<kRPWdf>(r0, D, H, L, nullptr, y + (int64_t)i * D);
+    rows_finish_df<kRPWdf>(r0, ny, H, L, nullptr, y + (int64_t)i * ny);
   }
 }
 void launch_matvec_leaf_df(const DevLevel& L, const float* Ah, const float* Al, const float* Xh, const float* Xl,
-                           const float* xh, const float* xl, const float* yhh, const float* yhl, double* y,
+                           const float* xh, const float* xl, const float* yhh, const float* yhl, double* y, int ny,
                            cudaStream_t st) {
   const size_t Kp = (L.K + 3) & ~3, Dp = (L.D + 3) & ~3;
   const size_t sm = 2 * sizeof(float) * (Kp + Dp * (size_t)L.max_near);
   set_smem((const void*)mv_leaf_df_kernel, sm);
   ++g_launches;
-  mv_leaf_df_kernel<<<L.nb, 256, sm, st>>>(L.D, L.K, L.near_ptr, L.near_j, Ah, Al, Xh, Xl, xh, xl, yhh, yhl, y);
+  mv_leaf_df_kernel<<<L.nb, 256, sm, st>>>(L.D, ny, L.K, L.near_ptr, L.near_j, Ah, Al, Xh, Xl, xh, xl, yhh, yhl, y);
 }
 
 // An FP32 vector of padded boxes: entry e of its nb * p.str entries is entry

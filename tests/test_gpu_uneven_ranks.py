@@ -45,16 +45,21 @@ def test_halves_with_odd_ranks(B, n, leaf, rank):
         assert rel <= 1e-10 and np.linalg.norm(b - S.matvec(x)) <= 2e-10 * np.linalg.norm(b)
 
 
-def test_halves_with_an_open_far_list(B):
+@pytest.mark.parametrize("which", ["far", "near"])
+@pytest.mark.parametrize("n,leaf", [(1024, 128), (1000, 66)])
+def test_open_lists(B, n, leaf, which):
+    """A list that holds (j, i) without (i, j) at the leaves, with and without
+    padding of the FP32 arrays (leaves of 63 points)."""
     from oracle.construct import construct
     from oracle.instance import flatten
     from oracle.kernels import Kernel
-    n = 1024
-    H = construct(W.cube_points(n, 3), Kernel("yukawa_eps", diag_shift=1.0), 128, 1.0, 1e-8, 64, 256, 32)
+    H = construct(W.cube_points(n, 3), Kernel("yukawa_eps", diag_shift=1.0), leaf, 1.0, 1e-8, 0, 256, 32)
     flat = flatten(H)
     l = max(k for k in range(flat["L"] + 1) if len(flat["far"][k]))
-    flat["far"][l] = np.ascontiguousarray(flat["far"][l][:-1])  # (j, i) stays, (i, j) goes
-    S = B.H2Solver.from_instance(flat, kernel="yukawa_eps", leaf=128, eta=1.0, tol=1e-8, max_rank=64, far_samples=256,
+    pairs = flat[which][l]
+    q = np.flatnonzero(pairs[:, 0] != pairs[:, 1])[-1]
+    flat[which][l] = np.ascontiguousarray(np.delete(pairs, q, axis=0))
+    S = B.H2Solver.from_instance(flat, kernel="yukawa_eps", leaf=leaf, eta=1.0, tol=1e-8, far_samples=256,
                                  near_samples=32, diag_shift=1.0)
     check_arithmetics(S, n)
 
