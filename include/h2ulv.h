@@ -306,9 +306,11 @@ h2_status h2_matvec_noalloc(h2_ctx* c, const double* x, double* y);
  *                         inner iteration: substitution, matvec and
  *                         orthogonalization; the residual; one ULV
  *                         application), on a private stream, the first time
- *                         each is needed after a factorization or a change
- *                         of an option, and replayed; 0: plain launches.  A
- *                         capture that fails falls back to plain launches.
+ *                         each is needed, and replayed until the operand
+ *                         type, an option or the arrays change (a later
+ *                         factorization in the same arrays keeps them); 0:
+ *                         plain launches.  A capture that fails falls back to
+ *                         plain launches.
  *   H2_OPT_TC_KERNEL      the kernel form of the factorization's main-chain
  *                         tensor-core GEMMs (projection, Schur update;
  *                         process-wide, all contexts): 0 one CTA per batch

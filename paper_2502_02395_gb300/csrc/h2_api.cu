@@ -1370,9 +1370,9 @@ void matvec_t(h2_ctx* c, const T* A, T* const* X, T* const* S, T* xh, T* yh, con
 void matvec_impl(h2_ctx* c, const double* x, double* y) {
   matvec_t<double>(c, c->A64, c->X64p.data(), c->S64p.data(), c->xhat, c->yhat, x, y);
 }
-// The same product with the couplings and the leaf step in FP32-pair
-// arithmetic on the FP32 split of the FP64 matrix (about 2^-48 per entry);
-// the upward and downward passes stay FP64.
+// The same product in FP32-pair arithmetic throughout, on the FP32 split of the
+// FP64 matrix (about 2^-48 per entry): the input is split once, the basis
+// coefficients and partial products stay pairs, the output is FP64.
 void matvec_df(h2_ctx* c, const double* x, double* y) {
   const int L = c->L;
   cudaStream_t st = c->stream;
@@ -1752,7 +1752,6 @@ h2_status gmres_work(h2_ctx* c, GmresWork& W) {
   return H2_OK;
 }
 
-// r = b - A_H2 x in FP64; returns ||r||
 // r = b - A_H2 x in FP64 and its norm; pairs: the matvec in FP32-pair
 // arithmetic (matvec_df) instead of FP64 instructions.
 h2_status fp64_residual(h2_ctx* c, SolveTimer& tm, double& rnorm, bool pairs = false) {
@@ -2816,8 +2815,8 @@ h2_status h2_stats(const h2_ctx* c, char* json, size_t cap) {
     }
     // the projection's flops: the pairs actually projected (symmetric near
     // lists: the upper pairs i <= j; the lower ones are their transposes)
-    const bool up_only = (c->prec == H2_PREC_FP64) ? (d.near_sym && d.n_lw > 0)
-                                                   : ((int)c->f32.lv.size() > l && c->f32.lv[l].proj_sym);
+    const bool f32 = c->prec != H2_PREC_FP64 && (int)c->f32.lv.size() > l;
+    const bool up_only = (f32 && c->f32.lv[l].tc) ? c->f32.lv[l].proj_sym : (d.near_sym && d.n_lw > 0);
     const double npj = (double)(up_only ? d.n_up : d.NP);
     fl_proj += npj * 4.0 * D * D * D;
     // algorithmic bytes of the tensor-core projection: the 16-bit input
@@ -2830,7 +2829,8 @@ h2_status h2_stats(const h2_ctx* c, char* json, size_t cap) {
     }
     fl_lu += d.nb * 2.0 * R * R * R;
     fl_schur += d.nb * (2.0 * R * R * K + 2.0 * K * K * R);
-    fl_coup += d.FP * 4.0 * K * K * K;
+    // (couplings outside the tensor cores: the pairs i < j of a symmetric list)
+    fl_coup += (d.far_mirrored && !(f32 && c->f32.lv[l].tc_coup) ? d.n_fu : d.FP) * 4.0 * K * K * K;
     fl_qr += d.nb * (4.0 * D * K * K + 4.0 * D * D * K);
   }
   // algorithmic traffic of one substitution (Eq. 31 form; storage width w)
@@ -2845,7 +2845,9 @@ h2_status h2_stats(const h2_ctx* c, char* json, size_t cap) {
     const double wa = a16 ? 2.0 : w;
     // per box: M1 and U^S (fwd1), U (bwd2) and three reads of the inverse
     by_sub += wa * ((double)(d.NP - d.nb) * R * R + (double)d.NP * 2.0 * R * K) + w * d.nb * (2.0 * D * D + 3.0 * R * R);
-    by_mv += 8.0 * (2.0 * d.nb * D * K + (double)d.FP * K * K);
+    // (the mixed solve's matvecs read the stored halves of the couplings)
+    const double nfp = c->cb_ok && c->prec != H2_PREC_FP64 ? (double)c->pv[l].fpu : (double)d.FP;
+    by_mv += 8.0 * (2.0 * d.nb * D * K + nfp * K * K);
     fl_mv += 2.0 * (2.0 * d.nb * D * K + (double)d.FP * K * K);
   }
   double by_leaf32 = 0;

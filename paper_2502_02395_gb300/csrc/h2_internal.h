@@ -378,7 +378,7 @@ struct h2_ctx {
   // 2k + 1: A_k^T x_i with j = box), CSR over boxes.
   bool sym = false;
   int64_t npu = 0;
-  int32_t *sym_q = nullptr, *sym_i = nullptr, *sym_j = nullptr, *sym_ent = nullptr;
+  int32_t *sym_q = nullptr, *sym_ent = nullptr;
   int64_t* sym_ptr = nullptr;
   float* part32 = nullptr;   // npu * 2 D partial products (FP32 matvec)
   float* part32c = nullptr;  // coupling partial products of every level (beside the leaf's)
