@@ -33,6 +33,13 @@ thread_local std::string g_last_error;
     if (s_ != H2_OK) return s_;        \
   } while (0)
 
+// At the start of a call: no message, and no launch error that an earlier call
+// on this thread left by returning before it looked.
+void begin_call(h2_ctx* c) {
+  c->err.clear();
+  take_launch_error();
+}
+
 bool is_device_ptr(const void* p) {
   cudaPointerAttributes a{};
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -180,6 +187,7 @@ bool mirrors(const std::vector<int32_t>& pi, const std::vector<int32_t>& pj, con
 }
 
 h2_status setup_device(h2_ctx* c) {
+  begin_call(c);
   HostH2& H = c->host;
   c->L = H.L;
   c->N = H.N;
@@ -2250,7 +2258,7 @@ h2_status h2_import(h2_ctx** out, const h2_params* p, const h2_instance* in) {
 
 h2_status h2_factor(h2_ctx* c, int32_t prec) {
   if (!c) return H2_ERR_INVALID_ARG;
-  c->err.clear();
+  begin_call(c);
   if (prec < H2_PREC_FP64 || prec > H2_PREC_BF16) {
     c->err = "unknown precision";
     return H2_ERR_INVALID_ARG;
@@ -2269,7 +2277,7 @@ h2_status h2_factor(h2_ctx* c, int32_t prec) {
 
 h2_status h2_release_factorization(h2_ctx* c) {
   if (!c) return H2_ERR_INVALID_ARG;
-  c->err.clear();
+  begin_call(c);
   release_factor(c, c->f64);
   release_factor(c, c->f32);
   c->prec = -1;
@@ -2279,7 +2287,7 @@ h2_status h2_release_factorization(h2_ctx* c) {
 
 h2_status h2_ulv_apply(h2_ctx* c, const double* b, double* x) {
   if (!c || !b || !x) return H2_ERR_INVALID_ARG;
-  c->err.clear();
+  begin_call(c);
   if (!factor_ready(c)) { c->err = "no factorization"; return H2_ERR_STATE; }
   const DevLevel& lf = c->lv[c->L];
   const int64_t nslot = (int64_t)lf.nb * lf.D;
@@ -2295,7 +2303,7 @@ h2_status h2_ulv_apply(h2_ctx* c, const double* b, double* x) {
 
 h2_status h2_matvec(h2_ctx* c, const double* x, double* y) {
   if (!c || !x || !y) return H2_ERR_INVALID_ARG;
-  c->err.clear();
+  begin_call(c);
   if (!c->A64) { c->err = "the FP64 leaf blocks were released (H2_OPT_FP64_LEAF)"; return H2_ERR_STATE; }
   CKS(vec_in(c, x, c->x64));
   matvec_impl(c, c->x64, c->y64);
@@ -2331,7 +2339,7 @@ h2_status h2_matvec_many(h2_ctx* c, const double* X, double* Y, int32_t nrhs) {
 h2_status h2_solve(h2_ctx* c, const double* b, double* x, double target, int32_t max_iters, double* relres_out,
                    int32_t* iters_out) {
   if (!c || !b || !x || max_iters < 0) return H2_ERR_INVALID_ARG;
-  c->err.clear();
+  begin_call(c);
   if (!factor_ready(c)) { c->err = "no factorization"; return H2_ERR_STATE; }
   if (!c->A64 && c->resid64) {
     c->err = "the FP64 residual needs the FP64 leaf blocks, which were released (H2_OPT_FP64_LEAF)";
@@ -2423,7 +2431,7 @@ h2_status h2_set_refinement(h2_ctx* c, int32_t method, int32_t restart) {
 
 h2_status h2_set_option(h2_ctx* c, int32_t option, int64_t value) {
   if (!c) return H2_ERR_INVALID_ARG;
-  c->err.clear();
+  begin_call(c);
   if ((value != 0 && value != 1) && option != H2_OPT_TC_KERNEL && !(option == H2_OPT_BOX_STREAM && value == 2) &&
       option != H2_OPT_PAIR_CTAS && option != H2_OPT_BOX_CTAS) {
     c->err = "option value must be 0 or 1";
@@ -2491,7 +2499,7 @@ h2_status h2_set_option(h2_ctx* c, int32_t option, int64_t value) {
 
 h2_status h2_matvec_arith(h2_ctx* c, const double* x, double* y, int32_t arith) {
   if (!c || !x || !y) return H2_ERR_INVALID_ARG;
-  c->err.clear();
+  begin_call(c);
   if (arith < 0 || arith > 2) {
     c->err = "arith must be 0 (FP64), 1 (FP32) or 2 (FP32 pairs)";
     return H2_ERR_INVALID_ARG;
@@ -2523,7 +2531,7 @@ h2_status h2_matvec_arith(h2_ctx* c, const double* x, double* y, int32_t arith) 
 
 h2_status h2_autotune(h2_ctx* c, int32_t prec, char* json, size_t cap) {
   if (!c || (prec != H2_PREC_FP16 && prec != H2_PREC_BF16)) return H2_ERR_INVALID_ARG;
-  c->err.clear();
+  begin_call(c);
   std::ostringstream o;
   o.precision(6);
   // (1) the kernel form of the factorization's main-chain GEMMs: each form
@@ -2615,7 +2623,7 @@ h2_status h2_autotune(h2_ctx* c, int32_t prec, char* json, size_t cap) {
 
 h2_status h2_wait_selftest(h2_ctx* c, int64_t timeout_ns) {
   if (!c) return H2_ERR_INVALID_ARG;
-  c->err.clear();
+  begin_call(c);
   if (timeout_ns < 1 || timeout_ns > 10000000000ll) {
     c->err = "timeout_ns outside 1 .. 1e10";
     return H2_ERR_INVALID_ARG;
