@@ -582,7 +582,8 @@ std::string build_host(const h2_params& p, const double* pts, int64_t N, HostH2&
       }
       std::vector<char> ok(nb, 0);
       bool sketched = false;
-      if (gpu && gpu->supported(D, K) && p.near_samples > 0 && p.near_samples <= 64) {
+      // (levels with an empty box have rank 0: the plain pass below)
+      if (gpu && nmin > 0 && gpu->supported(D, K) && p.near_samples > 0 && p.near_samples <= 64) {
         // the level's sample lists for the GPU sketches
         job.nb = nb, job.D = D, job.K = K;
         job.m = std::min(160, ((K + 32 + 1) / 2) * 2);  // K + 26 sketch columns, 6 probes

@@ -58,3 +58,15 @@ def test_construction_shapes(B, n, leaf, kernel):
     assert eg <= max(4.0 * e0, 1e-9)
     S0.close()
     S.close()
+
+
+@pytest.mark.parametrize("n,leaf", [(3, 1), (15, 1), (21, 1)])
+def test_empty_boxes(B, n, leaf):
+    """More boxes than points: levels of rank 0, as the host construction has
+    them (the same blocks, so products equal to the last bits)."""
+    P = W.cube_points(n, 3)
+    kw = dict(kernel="yukawa_eps", diag_shift=1.0, leaf=leaf, eta=1.0, tol=1e-8, far_samples=64, near_samples=8)
+    G, H = B.H2Solver.build_gpu(P, **kw), B.H2Solver.build(P, **kw)
+    assert [d["K"] for d in G.stats()["levels"]] == [d["K"] for d in H.stats()["levels"]]
+    x = W.uniform_rhs(n, 4)
+    assert np.linalg.norm(G.matvec(x) - H.matvec(x)) <= 1e-14 * np.linalg.norm(H.matvec(x))
